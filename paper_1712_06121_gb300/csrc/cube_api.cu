@@ -857,8 +857,8 @@ static cube_status pk_enqueue(cube_ctx* c, int32_t n_bins, double* k, double* pk
     outk = part + (size_t)nb * 3 * n_bins;
     const double L = c->P.box;
     const double pfac = L * L * L / std::pow((double)g.N, 6);
-    launch_pk_bin(c->fft, c->mesh, g.S, n_bins, pfac, 2.0 * PI / L, part, c->st);
-    launch_pk_reduce(part, nb, n_bins, outk, outk + n_bins, outk + 2 * n_bins, c->st);
+    launch_pk_bin(c->fft, c->mesh, g.S, n_bins, part, c->st);
+    launch_pk_reduce(c->fft, part, n_bins, pfac, 2.0 * PI / L, outk, outk + n_bins, outk + 2 * n_bins, c->st);
     c->launches += 2;
     cube_status s = CUBE_OK;
     const bool hk = !is_device_ptr(k), hp = !is_device_ptr(pk), hn = !is_device_ptr(nmodes);

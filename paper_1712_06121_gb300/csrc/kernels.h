@@ -215,10 +215,9 @@ void fft_z(const FftPlan& p, float* mesh, int S, float g0, bool green, cudaStrea
 void fft_x_c2r(const FftPlan& p, float* mesh, int S, float* phig, cudaStream_t st,
                const Batch& bt = Batch{1, 0, nullptr, nullptr});                                      // rows: c2r into ghosted Phi
 int pk_blocks(int N);
-void launch_pk_bin(const FftPlan& p, const float* mesh, int S, int nbins, double pfac, double kfund,
-                   double* part, cudaStream_t st);
-void launch_pk_reduce(const double* part, int nblocks, int nbins, double* k, double* pk, double* nm,
-                      cudaStream_t st);
+void launch_pk_bin(const FftPlan& p, const float* mesh, int S, int nbins, double* part, cudaStream_t st);
+void launch_pk_reduce(const FftPlan& p, const double* part, int nbins, double pfac, double kfund, double* k, double* pk,
+                      double* nm, cudaStream_t st);
 void launch_unpad(const float* mesh, int N, int S, float* out, cudaStream_t st);
 // largest |component| of the FD4 gradient / 12 of the ghosted potential over
 // all mesh nodes (float bits): an upper bound of every particle's force

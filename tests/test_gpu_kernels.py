@@ -1,0 +1,57 @@
+"""Kernels at the sizes where their work split changes: edges of tiles,
+remainders and the smallest and largest of their ranges, against the oracle."""
+import numpy as np
+import pytest
+
+from oracle import pm
+
+from gpu_util import oracle_params, read_store
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(scope="module")
+def cube():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from conftest import build_lib
+    build_lib()
+    import paper_1712_06121_gb300 as c
+    torch.cuda.set_device(0)
+    return c
+
+
+def _random_particles(n, nf, seed):
+    rng = np.random.default_rng(seed)
+    pos = (rng.random((3, n)) * nf).astype(np.float32)
+    pos[pos >= nf] = 0.0
+    return pos, rng.normal(0.0, 0.3, (3, n)).astype(np.float32), np.arange(n, dtype=np.uint32)
+
+
+# ---------------------------------------------------------------- power spectrum
+# rows of 9 to 129 kx (one lane to several rounds of 32, a last round of one
+# lane), one bin, bins beyond the mesh's corner (empty: NaN).  Mode counts are
+# exact; |k| sums in pairs of floats (2^-46 per addition, fewer than 2^10
+# additions in a chain) stay within 1e-12; P carries the FP32 transform (1e-4).
+@pytest.mark.parametrize("nf,n_bins", [(16, 2048), (24, 21), (48, 1), (64, 60), (96, 84), (256, 128)])
+def test_power_spectrum_bins_at_the_edges(cube, nf, n_bins):
+    n = 5001
+    pos, vel, ids = _random_particles(n, nf, 1712201)
+    prm = cube.make_params(nf, n, x_bytes=2, v_bytes=1, box=50.0, omega_m=0.3, omega_l=0.7)
+    ctx = cube.cube_create(prm, torch.cuda.current_stream())
+    try:
+        cube.cube_encode(ctx, pos, vel, ids, 0.02, 0.5)
+        g = read_store(cube, ctx)
+        ref = pm.encode(oracle_params(pm, prm, g["brick"]), pos, vel, ids, 0.02, g["sigma"], snap=False)
+        k, p, m = (np.empty(n_bins) for _ in range(3))
+        cube.cube_power_spectrum(ctx, n_bins, k, p, m)
+        rk, rp, rm = pm.power_spectrum(ref, n_bins)
+        assert np.array_equal(m, rm)
+        full = rm > 0
+        assert np.all(np.isnan(k[~full])) and np.all(np.isnan(p[~full]))
+        assert np.allclose(k[full], rk[full], rtol=1e-12, atol=0.0)
+        assert np.allclose(p[full], rp[full], rtol=1e-4, atol=0.0)
+    finally:
+        cube.cube_destroy(ctx)
