@@ -293,7 +293,7 @@ typedef struct {
 cube_status cube_stats_get(cube_ctx* ctx, cube_stats* out);
 
 /* CIC density of the current store on the fine mesh, rho[z][y][x] floats
-   (N_f^3, mean 1).  Overwrites the FFT mesh.  Synchronises.
+   (N_f^3, mean 1).  May overwrite the FFT mesh.  Synchronises.
    Errors: CUBE_E_STATE. */
 cube_status cube_density(cube_ctx* ctx, float* rho);
 

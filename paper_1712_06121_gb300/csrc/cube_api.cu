@@ -691,16 +691,18 @@ static void mark(cube_ctx* c, int boundary) {
 
 static double particle_mass(const Geo& g) { return std::pow((double)g.N, 3) / (double)g.Np; }
 
-static void deposit(cube_ctx* c) {
-    const Geo& g = c->g;
+// density of the store on a mesh with rows of g.S floats (c->mesh, or any 16-byte aligned rows)
+static void deposit_on(cube_ctx* c, const Geo& g, float* mesh) {
     if (c->raw) {
-        cudaMemsetAsync(c->mesh, 0, (size_t)g.N * g.N * g.S * 4, c->st);
-        launch_raw_deposit(g, (const float*)c->chi[0], c->mesh, (float)particle_mass(g), c->st);
+        cudaMemsetAsync(mesh, 0, (size_t)g.N * g.N * g.S * 4, c->st);
+        launch_raw_deposit(g, (const float*)c->chi[0], mesh, (float)particle_mass(g), c->st);
     } else {
-        launch_deposit(g, c->store(c->cur), c->mesh, particle_mass(g) * std::ldexp(1.0, -3 * g.sbits), c->st);
+        launch_deposit(g, c->store(c->cur), mesh, particle_mass(g) * std::ldexp(1.0, -3 * g.sbits), c->st);
     }
     c->launches += 1;
 }
+
+static void deposit(cube_ctx* c) { deposit_on(c, c->g, c->mesh); }
 
 // density -> Phi on the mesh; boundaries 1..6 of the step's trace
 static void mesh_potential(cube_ctx* c) {
@@ -1205,7 +1207,11 @@ cube_status cube_stats_get(cube_ctx* c, cube_stats* out) {
     return latched(c);
 }
 
-// unpadded N^3 copy of the mesh (density) or of the ghosted Phi
+// The density (phi false) or the potential of the store as N^3 packed values
+// in dst.  The deposit writes whole rows of 16-byte pieces, so it writes the
+// packed rows itself where dst is on the device and aligned, or staged for the
+// host; otherwise the padded mesh is copied.  The potential is copied from
+// its ghosted rows, which later calls read.
 static cube_status mesh_out(cube_ctx* c, float* dst, bool phi) {
     const Geo& g = c->g;
     const size_t bytes = (size_t)g.N * g.N * g.N * 4;
@@ -1217,9 +1223,18 @@ static cube_status mesh_out(cube_ctx* c, float* dst, bool phi) {
         if (s != CUBE_OK) return s;
         d = (float*)p;
     }
-    if (phi) launch_unpad_phig(c->phig, g.N, d, c->st);
-    else launch_unpad(c->mesh, g.N, g.S, d, c->st);
-    c->launches += 1;
+    if (phi) {
+        launch_unpad_phig(c->phig, g.N, d, c->st);
+        c->launches += 1;
+    } else if (((uintptr_t)d & 15) == 0) {
+        Geo packed = g;
+        packed.S = g.N;
+        deposit_on(c, packed, d);
+    } else {
+        deposit(c);
+        launch_unpad(c->mesh, g.N, g.S, d, c->st);
+        c->launches += 1;
+    }
     if (host) CK(cudaMemcpyAsync(dst, d, bytes, cudaMemcpyDeviceToHost, c->st));
     CK(cudaGetLastError());
     return latched(c);
@@ -1228,7 +1243,6 @@ static cube_status mesh_out(cube_ctx* c, float* dst, bool phi) {
 cube_status cube_density(cube_ctx* c, float* rho) {
     if (!c || !rho) return fail(CUBE_E_ARG, "NULL argument");
     if (!c->encoded) return fail(CUBE_E_STATE, "no store: call cube_encode first");
-    deposit(c);
     return mesh_out(c, rho, false);
 }
 

@@ -55,3 +55,25 @@ def test_power_spectrum_bins_at_the_edges(cube, nf, n_bins):
         assert np.allclose(p[full], rp[full], rtol=1e-4, atol=0.0)
     finally:
         cube.cube_destroy(ctx)
+
+
+# packed meshes into 16-byte aligned and unaligned device memory and into host memory
+@pytest.mark.parametrize("nf", [16, 24, 96])
+def test_packed_meshes_do_not_depend_on_alignment(cube, nf):
+    n = 3000
+    pos, vel, ids = _random_particles(n, nf, 1712203)
+    prm = cube.make_params(nf, n, x_bytes=1, v_bytes=1, box=50.0, omega_m=0.3, omega_l=0.7)
+    ctx = cube.cube_create(prm, torch.cuda.current_stream())
+    try:
+        cube.cube_encode(ctx, pos, vel, ids, 0.02, 0.5)
+        for call in (cube.cube_density, cube.cube_potential):
+            host = np.empty((nf, nf, nf), dtype=np.float32)
+            call(ctx, host)
+            for shift in (0, 1, 2):
+                buf = torch.full((nf ** 3 + 8,), -1.0, device="cuda")
+                call(ctx, buf[shift:shift + nf ** 3])
+                got = buf.cpu().numpy()
+                assert np.array_equal(got[shift:shift + nf ** 3].reshape(nf, nf, nf), host)
+                assert np.all(got[:shift] == -1.0) and np.all(got[shift + nf ** 3:] == -1.0)
+    finally:
+        cube.cube_destroy(ctx)
