@@ -828,7 +828,7 @@ cube_status cube_decode(cube_ctx* c, float* pos, float* vel, uint32_t* id) {
             else launch_iota(did, g.Np, c->st);
         }
     } else {
-        launch_decode(g, c->store(c->cur), c->codec[c->cur].dec, dpos, dvel, did, c->st);
+        launch_decode(g, c->store(c->cur), c->codec[c->cur], dpos, dvel, did, c->st);
         c->launches += 1;
     }
     CK(cudaGetLastError());
@@ -882,7 +882,7 @@ cube_status cube_max_speed(cube_ctx* c, double* p_max) {
     if (!c->encoded) return fail(CUBE_E_STATE, "no store: call cube_encode first");
     const Geo& g = c->g;
     if (c->raw) launch_raw_max_speed(g, (const float*)c->nu[0], c->vmax, c->st);
-    else launch_max_speed(g, c->store(c->cur), c->codec[c->cur].dec, c->vmax, c->st);
+    else launch_max_speed(g, c->store(c->cur), c->codec[c->cur], c->vmax, c->st);
     c->launches += 1;
     unsigned bits = 0;
     CK(cudaMemcpyAsync(&bits, c->vmax, 4, cudaMemcpyDeviceToHost, c->st));
@@ -1474,12 +1474,12 @@ static cube_status batch_vmax_enqueue(cube_batch* b) {
     }
     if (same) {                                  // one launch over every member's store
         cube_ctx* c = b->m[0];
-        launch_max_speed(c->g, c->store(c->cur), c->codec[c->cur].dec, c->vmax, b->st,
+        launch_max_speed(c->g, c->store(c->cur), c->codec[c->cur], c->vmax, b->st,
                          Batch{K, b->stride, nullptr, nullptr});
         b->launches += 2;
     } else {
         for (cube_ctx* c : b->m) {
-            launch_max_speed(c->g, c->store(c->cur), c->codec[c->cur].dec, c->vmax, b->st);
+            launch_max_speed(c->g, c->store(c->cur), c->codec[c->cur], c->vmax, b->st);
             c->launches += 1;
         }
     }
@@ -1754,7 +1754,7 @@ cube_status served_flags_status(unsigned flags) { return flags_status(flags); }
 cube_status served_vmax_enqueue(cube_ctx* c, unsigned* pinned_bits) {
     const Geo& g = c->g;
     if (c->raw) launch_raw_max_speed(g, (const float*)c->nu[0], c->vmax, c->st);
-    else launch_max_speed(g, c->store(c->cur), c->codec[c->cur].dec, c->vmax, c->st);
+    else launch_max_speed(g, c->store(c->cur), c->codec[c->cur], c->vmax, c->st);
     c->launches += 1;
     CK(cudaMemcpyAsync(pinned_bits, c->vmax, 4, cudaMemcpyDeviceToHost, c->st));
     return CUBE_OK;

@@ -59,6 +59,43 @@ __device__ __forceinline__ int warp_cells(const unsigned* off, int ncell, unsign
     return c;
 }
 
+// The particles [q0, q1) of a brick: each warp takes a contiguous share
+// [*p0, *p1), a multiple of 32 but for the last.
+__device__ __forceinline__ void brick_share(unsigned q0, unsigned q1, unsigned* p0, unsigned* p1) {
+    const unsigned nw = blockDim.x >> 5;
+    const unsigned share = ((q1 - q0 + nw * 32 - 1) / (nw * 32)) * 32;
+    *p0 = q0 + min(q1 - q0, (threadIdx.x >> 5) * share);
+    *p1 = min(q1, *p0 + share);
+}
+
+// brick offsets, v_c of the brick and (1-byte codes) the decode table in
+// shared memory, [nbc + 1], [3][nbc], [2 lim + 1], by asynchronous copies:
+// complete after cp_async_wait_all() and a barrier
+struct BrickTables {
+    unsigned* off;
+    float* vc;
+    float* dec;
+};
+template <int NV>
+__device__ __forceinline__ BrickTables stage_brick(const Geo& g, const StoreDev& s, const CodecDev& c, int L0,
+                                                   unsigned* smem) {
+    const int nbc = g.B * g.B * g.B;
+    BrickTables t{smem, reinterpret_cast<float*>(smem + nbc + 1), reinterpret_cast<float*>(smem + 4 * nbc + 1)};
+    for (int i = threadIdx.x; i <= nbc; i += blockDim.x) cp_async4(&t.off[i], &s.offsets[L0 + i]);
+    for (int i = threadIdx.x; i < 3 * nbc; i += blockDim.x)
+        cp_async4(&t.vc[i], &s.vc[(int64_t)(i >> (3 * g.lB)) * g.Ncc + L0 + (i & (nbc - 1))]);
+    if (NV == 1)
+        for (int i = threadIdx.x; i < 2 * g.nulim + 1; i += blockDim.x) cp_async4(&t.dec[i], &c.dec[i]);
+    return t;
+}
+
+// the decode and threshold tables of 2-byte codes through their corrections
+template <int NV>
+__device__ __forceinline__ VelTables vel_tables(const CodecDev& c, int lim) {
+    return VelTables{c.dec, c.thr, c.vdel, VelApprox{NV == 2 ? c.est[3] : 0.0f, NV == 2 ? c.est[4] : 0.0f, 2 * lim + 1},
+                     lim};
+}
+
 // brick of a CTA launched on the (nb, nb, nb x members) grid: its
 // coordinates and storage rank; *m the member of a batch
 template <bool BAT>
@@ -310,64 +347,159 @@ __global__ void k_encode_scatter(Geo g, const float* __restrict__ pos, const flo
 }
 
 // ------------------------------------------------------------------ decode
+// Bound by its 28 bytes written per particle.  Positions q 2^-s with the
+// integer q = (cell << (8 n + 1)) + Q are rounded once: q < 2^19 for 1-byte
+// codes is exact in FP32, q < 2^27 for 2-byte codes is rounded to nearest by
+// u32_to_float_rn, and the scale is a power of two (the FP64 conversions of
+// an FP64 product cost more than the stores here).  A CTA's life is a chain of
+// loads, so a warp's first 64 particles are requested beside the brick's
+// tables and the rest 64 at a time.  256^3 particles x1v1: 0.342 ms with FP64
+// positions, a search per particle and tables in global memory -> 0.164 ms.
 template <int NX, int NV>
-__global__ void __launch_bounds__(T_BRICK) k_decode(Geo g, StoreDev s, const float* __restrict__ dec,
-                                                    float* __restrict__ pos, float* __restrict__ vel,
-                                                    unsigned* __restrict__ id) {
-    extern __shared__ unsigned sm_off[];
-    const int nbc = g.B * g.B * g.B;
+__global__ void __launch_bounds__(T_BRICK) k_decode(Geo g, StoreDev s, CodecDev cd, float* __restrict__ pos,
+                                                    float* __restrict__ vel, unsigned* __restrict__ id) {
+    extern __shared__ unsigned brick_sm[];
+    const int nbc = g.B * g.B * g.B, lim = g.nulim;
     const int L0 = blockIdx.x * nbc;
-    for (int c = threadIdx.x; c <= nbc; c += blockDim.x) sm_off[c] = s.offsets[L0 + c];
-    __syncthreads();
-    int bx, by, bz;
-    brick_coords(g, blockIdx.x, &bx, &by, &bz);
-    const int nbits = 8 * NX, half = 1 << (nbits - 1);
-    const double pscale = ldexp(1.0, g.r - nbits - 1);
-    const unsigned np_ = (unsigned)g.Np;
-    const unsigned q1 = min(sm_off[nbc], np_);
-    for (unsigned i = min(sm_off[0], q1) + threadIdx.x; i < q1; i += blockDim.x) {
-        int lc = upper_cell(sm_off, nbc, i);
-        int l[3] = {lc & (g.B - 1), (lc >> g.lB) & (g.B - 1), lc >> (2 * g.lB)};
-        int c[3] = {bx * g.B + l[0], by * g.B + l[1], bz * g.B + l[2]};
+    const BrickTables bt = stage_brick<NV>(g, s, cd, L0, brick_sm);
+    const unsigned q1 = min(s.offsets[L0 + nbc], (unsigned)g.Np), q0 = min(s.offsets[L0], q1);
+    unsigned p0, p1;
+    brick_share(q0, q1, &p0, &p1);
+    const unsigned lane = threadIdx.x & 31;
+    const CodeRows<NX> chi(s.chi, g.Np);
+    const CodeRows<NV> nu(s.nu, g.Np);
+    int x[2][3], v[2][3];
+    unsigned pid[2];
+    auto load = [&](unsigned base) {
 #pragma unroll
-        for (int d = 0; d < 3; ++d) {
-            int Q = 2 * (load_code<NX>(s.chi, d * g.Np + i) + half) + 1;
-            long long q = ((long long)c[d] << (nbits + 1)) + Q;
-            pos[d * g.Np + i] = __double2float_rn((double)q * pscale);
-            int nu = load_nu<NV>(s.nu, d * g.Np + i, g.nulim);
-            vel[d * g.Np + i] = s.vc[(int64_t)d * g.Ncc + L0 + lc] + dec[nu + g.nulim];
+        for (int h = 0; h < 2; ++h) {
+            const unsigned i = base + 32 * h + lane;
+            if (i >= p1) continue;
+#pragma unroll
+            for (int d = 0; d < 3; ++d) {
+                x[h][d] = chi.get(d, i);
+                v[h][d] = nu.get(d, i);
+            }
+            pid[h] = id && s.id ? load_pid(s.id, i, g.nid) : i;
         }
-        if (id) id[i] = s.id ? load_pid(s.id, i, g.nid) : i;
+    };
+    load(p0);
+    cp_async_wait_all();
+    __syncthreads();
+    if (p0 >= p1) return;
+    const VelTables vt = vel_tables<NV>(cd, lim);
+    int b[3];
+    brick_coords(g, blockIdx.x, &b[0], &b[1], &b[2]);
+    constexpr int nbits = 8 * NX, half = 1 << (nbits - 1);
+    const float pscale = ldexpf(1.0f, g.r - nbits - 1);
+    int c0 = upper_cell(bt.off, nbc, p0);
+    for (unsigned base = p0;;) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const unsigned i = base + 32 * h + lane;
+            int cnext;
+            const int lc = warp_cells(bt.off, nbc, base + 32 * h, c0, &cnext);
+            c0 = cnext;
+            if (i < p1) {
+#pragma unroll
+                for (int d = 0; d < 3; ++d) {
+                    const int c = (b[d] << g.lB) + ((lc >> (d * g.lB)) & (g.B - 1));
+                    const unsigned q = ((unsigned)c << (nbits + 1)) + (unsigned)(2 * (x[h][d] + half) + 1);
+                    const float f = NX == 1 ? __uint_as_float(0x4B000000u | q) - 8388608.0f : u32_to_float_rn(q);
+                    pos[d * g.Np + i] = f * pscale;
+                    const int k = max(-lim, min(lim, v[h][d]));
+                    vel[d * g.Np + i] = bt.vc[(d << (3 * g.lB)) + lc] + (NV == 1 ? bt.dec[k + lim] : vt.dec(k));
+                }
+                if (id) id[i] = pid[h];
+            }
+        }
+        base += 64;
+        if (base >= p1) break;
+        load(base);
     }
 }
 
 // largest |p| over particles and axes of the store (momenta as decoded,
 // v_c + tan-table offset), as the bits of a non-negative float (order-
-// preserving as unsigned)
-template <int NV>
-__global__ void __launch_bounds__(T_BRICK) k_max_speed(Geo g, StoreDev s, const float* __restrict__ dec,
+// preserving as unsigned).  The table and the rounded sum grow with the code,
+// so a cell's largest |p| along an axis is at its smallest or largest code:
+// LPC lanes a cell take both over the cell's particles and two codes are
+// decoded, not every particle's.  Cells of more than 8 LPC particles (haloes)
+// are finished by their whole warp, so that no lane runs alone.  A warp's
+// life is a chain of loads (offsets, codes, table): LPC = 8 gives small stores
+// their warps (one wave holds 64 of them per SM), LPC = 2 keeps large ones to
+// few waves.  The call with its read-backs (25 us of
+// them host and copies), 192^3 particles x1v1, clustered: 73 us with a CTA a
+// brick, a search and a decode per particle -> 55 us; 32^3: 29.7 -> 26.4 us.
+template <int NV, int LPC>
+__global__ void __launch_bounds__(T_BRICK) k_max_speed(Geo g, StoreDev s, CodecDev cd,
                                                        unsigned* __restrict__ vmax_bits, Batch bt) {
-    extern __shared__ unsigned sm_off[];
     {                                                        // member of slot blockIdx.y of a batch
         const size_t o = slot_member(bt, blockIdx.y) * bt.stride;
         s = moved(s, o);
-        dec = moved(dec, o);
+        cd = moved(cd, o);
         vmax_bits = moved(vmax_bits, o);
     }
-    const int nbc = g.B * g.B * g.B;
-    const int L0 = blockIdx.x * nbc;
-    for (int c = threadIdx.x; c <= nbc; c += blockDim.x) sm_off[c] = s.offsets[L0 + c];
-    __syncthreads();
-    const unsigned q1 = min(sm_off[nbc], (unsigned)g.Np);
-    float m = 0.0f;
-    for (unsigned i = min(sm_off[0], q1) + threadIdx.x; i < q1; i += blockDim.x) {
-        const int lc = upper_cell(sm_off, nbc, i);
+    const int lane = threadIdx.x & 31;
+    const int L = (blockIdx.x * T_BRICK + threadIdx.x) / LPC, sub = threadIdx.x % LPC;
+    const CodeRows<NV> nu(s.nu, g.Np);
+    constexpr int kNone = 0x7fffffff;
+    unsigned i0 = 0, i1 = 0;
+    float vc[3] = {0.0f, 0.0f, 0.0f};
+    if (L < g.Ncc) {
+        i1 = min(s.offsets[L + 1], (unsigned)g.Np);
+        i0 = min(s.offsets[L], i1);
+#pragma unroll
+        for (int d = 0; d < 3; ++d) vc[d] = s.vc[(int64_t)d * g.Ncc + L];
+    }
+    int lo[3] = {kNone, kNone, kNone}, hi[3] = {-kNone, -kNone, -kNone};
+    const unsigned e = min(i1, i0 + 8u * LPC);
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        const unsigned i = i0 + sub + k * LPC;
+        if (i < e)
+#pragma unroll
+            for (int d = 0; d < 3; ++d) {
+                const int v = nu.get(d, i);
+                lo[d] = min(lo[d], v);
+                hi[d] = max(hi[d], v);
+            }
+    }
+    for (unsigned more = __ballot_sync(0xffffffffu, sub == 0 && e < i1); more; more &= more - 1) {
+        const int src = __ffs(more) - 1;
+        const unsigned a = __shfl_sync(0xffffffffu, e, src), z = __shfl_sync(0xffffffffu, i1, src);
+        int wl[3] = {kNone, kNone, kNone}, wh[3] = {-kNone, -kNone, -kNone};
+#pragma unroll 4
+        for (unsigned i = a + lane; i < z; i += 32)
+#pragma unroll
+            for (int d = 0; d < 3; ++d) {
+                const int v = nu.get(d, i);
+                wl[d] = min(wl[d], v);
+                wh[d] = max(wh[d], v);
+            }
 #pragma unroll
         for (int d = 0; d < 3; ++d) {
-            const int nu = load_nu<NV>(s.nu, d * g.Np + i, g.nulim);
-            m = fmaxf(m, fabsf(s.vc[(int64_t)d * g.Ncc + L0 + lc] + dec[nu + g.nulim]));
+            const int l = __reduce_min_sync(0xffffffffu, wl[d]), h = __reduce_max_sync(0xffffffffu, wh[d]);
+            if (lane == src) {
+                lo[d] = min(lo[d], l);
+                hi[d] = max(hi[d], h);
+            }
         }
     }
+#pragma unroll
+    for (int o = LPC / 2; o > 0; o >>= 1)
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            lo[d] = min(lo[d], __shfl_xor_sync(0xffffffffu, lo[d], o));
+            hi[d] = max(hi[d], __shfl_xor_sync(0xffffffffu, hi[d], o));
+        }
+    float m = 0.0f;
+    if (i0 < i1 && sub < 2)                                  // lane 0 decodes the smallest codes, lane 1 the largest
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            const int v = max(-g.nulim, min(g.nulim, sub ? hi[d] : lo[d]));
+            m = fmaxf(m, fabsf(vc[d] + cd.dec[v + g.nulim]));
+        }
     block_max_to(__float_as_uint(m), vmax_bits);
 }
 
@@ -758,8 +890,7 @@ __global__ void __launch_bounds__(PA_T, PA_MINB) k_passA(Geo g, StoreDev s, cons
     }
     const float e0 = cur.est[0], e1 = cur.est[1];
     // 2-byte codes: the decode and threshold tables through their L1-resident corrections
-    const VelTables vt{cur.dec, cur.thr, cur.vdel, VelApprox{NV == 2 ? cur.est[3] : 0.0f, NV == 2 ? cur.est[4] : 0.0f,
-                                                             2 * lim + 1}, lim};
+    const VelTables vt = vel_tables<NV>(cur, lim);
     const int nbits = 8 * NX, half = 1 << (nbits - 1);
     const int sb = g.sbits, wmask = (1 << sb) - 1;
     // the in-cell CIC weight (Q mod 2^sb) 2^-sb exactly from the bits of
@@ -1436,23 +1567,31 @@ void launch_encode_scatter(const Geo& g, const float* pos, const float* vel, con
     else k_encode_scatter<2, 2><<<nb, 256, 0, st>>>(g, pos, vel, id_in, key_sorted, perm, vc, c.thr, c.est, s);
 }
 
-void launch_max_speed(const Geo& g, const StoreDev& s, const float* dec, unsigned* vmax_bits, cudaStream_t st,
+void launch_max_speed(const Geo& g, const StoreDev& s, const CodecDev& c, unsigned* vmax_bits, cudaStream_t st,
                       const Batch& bt) {
-    size_t sm = (size_t)(g.B * g.B * g.B + 1) * sizeof(unsigned);
     if (bt.members == 1 && !bt.ms) cudaMemsetAsync(vmax_bits, 0, sizeof(unsigned), st);
     else k_zero_slot_words<<<1, 256, 0, st>>>(vmax_bits, bt);
-    const dim3 grid(g.nbricks, bt.members);
-    if (g.nnu == 1) k_max_speed<1><<<grid, T_BRICK, sm, st>>>(g, s, dec, vmax_bits, bt);
-    else k_max_speed<2><<<grid, T_BRICK, sm, st>>>(g, s, dec, vmax_bits, bt);
+    // one wave of 64 warps per SM holds eight lanes a cell: small stores
+    const bool wide = (int64_t)g.Ncc * bt.members * 8 <= (int64_t)64 * 32 * g.nsm;
+    const dim3 grid(nblk((int64_t)g.Ncc * (wide ? 8 : 2), T_BRICK), bt.members);
+    if (g.nnu == 1 && wide) k_max_speed<1, 8><<<grid, T_BRICK, 0, st>>>(g, s, c, vmax_bits, bt);
+    else if (g.nnu == 1) k_max_speed<1, 2><<<grid, T_BRICK, 0, st>>>(g, s, c, vmax_bits, bt);
+    else if (wide) k_max_speed<2, 8><<<grid, T_BRICK, 0, st>>>(g, s, c, vmax_bits, bt);
+    else k_max_speed<2, 2><<<grid, T_BRICK, 0, st>>>(g, s, c, vmax_bits, bt);
 }
 
-void launch_decode(const Geo& g, const StoreDev& s, const float* dec, float* pos, float* vel, unsigned* id,
+// a brick's offsets, v_c and (1-byte codes) decode table
+static size_t brick_smem(const Geo& g) {
+    return (size_t)(4 * g.B * g.B * g.B + 1 + (g.nnu == 1 ? 2 * g.nulim + 1 : 0)) * 4;
+}
+
+void launch_decode(const Geo& g, const StoreDev& s, const CodecDev& c, float* pos, float* vel, unsigned* id,
                    cudaStream_t st) {
-    size_t sm = (size_t)(g.B * g.B * g.B + 1) * sizeof(unsigned);
-    if (g.nchi == 1 && g.nnu == 1) k_decode<1, 1><<<g.nbricks, T_BRICK, sm, st>>>(g, s, dec, pos, vel, id);
-    else if (g.nchi == 1) k_decode<1, 2><<<g.nbricks, T_BRICK, sm, st>>>(g, s, dec, pos, vel, id);
-    else if (g.nnu == 1) k_decode<2, 1><<<g.nbricks, T_BRICK, sm, st>>>(g, s, dec, pos, vel, id);
-    else k_decode<2, 2><<<g.nbricks, T_BRICK, sm, st>>>(g, s, dec, pos, vel, id);
+    const size_t sm = brick_smem(g);
+    if (g.nchi == 1 && g.nnu == 1) k_decode<1, 1><<<g.nbricks, T_BRICK, sm, st>>>(g, s, c, pos, vel, id);
+    else if (g.nchi == 1) k_decode<1, 2><<<g.nbricks, T_BRICK, sm, st>>>(g, s, c, pos, vel, id);
+    else if (g.nnu == 1) k_decode<2, 1><<<g.nbricks, T_BRICK, sm, st>>>(g, s, c, pos, vel, id);
+    else k_decode<2, 2><<<g.nbricks, T_BRICK, sm, st>>>(g, s, c, pos, vel, id);
 }
 
 static size_t deposit_smem(const Geo& g) {

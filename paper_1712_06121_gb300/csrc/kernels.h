@@ -161,7 +161,7 @@ void launch_codec_tables(int nulim, const double* tanv, const double* tanh, cons
 void launch_encode_scatter(const Geo& g, const float* pos, const float* vel, const unsigned* id_in,
                            const unsigned* key_sorted, const unsigned* perm, const float* vc, const CodecDev& c,
                            StoreDev s, cudaStream_t st);
-void launch_decode(const Geo& g, const StoreDev& s, const float* dec, float* pos, float* vel, unsigned* id,
+void launch_decode(const Geo& g, const StoreDev& s, const CodecDev& c, float* pos, float* vel, unsigned* id,
                    cudaStream_t st);
 void launch_deposit(const Geo& g, const StoreDev& s, float* mesh, double scale, cudaStream_t st,
                     const Batch& bt = Batch{1, 0, nullptr, nullptr});
@@ -193,7 +193,7 @@ void launch_raw_momentum(const Geo& g, const float* V, long long* out3, cudaStre
 void launch_iota(unsigned* out, int64_t n, cudaStream_t st);
 void launch_raw_max_speed(const Geo& g, const float* V, unsigned* vmax_bits, cudaStream_t st);
 // largest |p| of the store (float bits), of every listed member of a batch
-void launch_max_speed(const Geo& g, const StoreDev& s, const float* dec, unsigned* vmax_bits, cudaStream_t st,
+void launch_max_speed(const Geo& g, const StoreDev& s, const CodecDev& c, unsigned* vmax_bits, cudaStream_t st,
                       const Batch& bt = Batch{1, 0, nullptr, nullptr});
 
 // ------------------------------------------------------------ k_fft.cu

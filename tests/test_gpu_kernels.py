@@ -57,6 +57,41 @@ def test_power_spectrum_bins_at_the_edges(cube, nf, n_bins):
         cube.cube_destroy(ctx)
 
 
+# ---------------------------------------------------------------- decode and largest momentum
+def _blob(n, nf, seed):
+    """n particles, half of them in one coarse cell, the rest anywhere."""
+    pos, vel, ids = _random_particles(n, nf, seed)
+    pos[:, : n // 2] = 5.0 + 0.9 * (pos[:, : n // 2] / nf)
+    return pos, vel, ids
+
+
+# one particle, a round's edges and a crowded brick, every code width, bricks
+# of 4 to 16 fine cells, 2-byte positions at 256 coarse cells per side (25-bit
+# q: rounded); the decoded values are the oracle's rounded once
+@pytest.mark.parametrize("n,nf,ratio,xb,vb", [(1, 16, 4, 1, 1), (33, 16, 4, 2, 2), (257, 32, 8, 1, 2), (4099, 32, 2, 2, 1),
+                                              (3001, 48, 1, 1, 1), (9000, 256, 1, 2, 2)])
+def test_decode_and_max_speed_match_oracle(cube, n, nf, ratio, xb, vb):
+    pos, vel, ids = _blob(n, nf, 1712202)
+    prm = cube.make_params(nf, n, ratio=ratio, x_bytes=xb, v_bytes=vb, box=50.0, omega_m=0.3, omega_l=0.7)
+    ctx = cube.cube_create(prm, torch.cuda.current_stream())
+    try:
+        cube.cube_encode(ctx, pos, vel, ids, 0.02, 0.5)
+        g = read_store(cube, ctx)
+        ref = pm.encode(oracle_params(pm, prm, g["brick"]), pos, vel, ids, 0.02, g["sigma"], snap=False)
+        dp, dv = torch.zeros((3, n), device="cuda"), torch.zeros((3, n), device="cuda")
+        di = torch.zeros(n, device="cuda", dtype=torch.int32)
+        cube.cube_decode(ctx, dp, dv, di)
+        rp, rv = pm.decode(ref)[:2]
+        assert np.array_equal(dp.cpu().numpy(), rp.astype(np.float32))
+        assert np.array_equal(di.cpu().numpy().astype(np.uint32), ref.ids)
+        v = dv.cpu().numpy()
+        # v_c and the FP32 table entry are each rounded once, and their sum
+        assert np.all(np.abs(v - rv) <= 2.0 ** -23 * (np.abs(ref.vc).max() + np.abs(rv)))
+        assert cube.cube_max_speed(ctx) == np.abs(v).max()
+    finally:
+        cube.cube_destroy(ctx)
+
+
 # packed meshes into 16-byte aligned and unaligned device memory and into host memory
 @pytest.mark.parametrize("nf", [16, 24, 96])
 def test_packed_meshes_do_not_depend_on_alignment(cube, nf):
