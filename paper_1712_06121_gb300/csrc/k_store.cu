@@ -863,7 +863,7 @@ __global__ void __launch_bounds__(PA_T, PA_MINB) k_passA(Geo g, StoreDev s, cons
     const unsigned q1 = min(s.offsets[L0 + nbc], (unsigned)g.Np);
     const unsigned q0 = min(s.offsets[L0], q1);
     unsigned i = q0 + threadIdx.x;
-    if (threadIdx.x == 0 && q1 - q0 > (unsigned)PB_BIG) w.big[1 + atomicAdd(w.big, 1)] = brick;
+    if (NV == 1 && threadIdx.x == 0 && q1 - q0 > (unsigned)PB_BIG) w.big[1 + atomicAdd(w.big, 1)] = brick;
     const CodeRows<NX> chi_r(s.chi, g.Np);
     const CodeRows<NV> nu_r(s.nu, g.Np);
     int nchi[3] = {0, 0, 0}, nnu[3] = {0, 0, 0};
@@ -1084,17 +1084,26 @@ __global__ void k_cells(Geo g, StepScratch w, unsigned* __restrict__ off_new, fl
 }
 
 // ------------------------------------------------------------------ pass B
-// One warp per brick (8 bricks per CTA): the brick's particles are taken 32
-// at a time in index order; lanes moving to the same cell get consecutive
-// slots in lane order from the cell's running start (match + popc), so the
-// new order within a cell is the old index order.  No block barriers.
+// Two splits, chosen by passB_all:
 //
-// A brick holding more than PB_BIG particles (clustering: late epochs reach
-// ~30x the mean) would make its warp the kernel's tail.  Pass A lists those
-// bricks; the first CTAs of the grid take them whole, 256 particles per
-// round: each warp's per-cell counts go to a shared table, and a lane's slot
-// is the cell's running start + the counts of the lower warps + its rank in
-// its warp, which is again the old index order.
+// Large stores with 1-byte velocities: one warp per brick (8 bricks per CTA).
+// The brick's particles are taken 32 at a time in index order; lanes moving
+// to the same cell get consecutive slots in lane order from the cell's running
+// start (match + popc), so the new order within a cell is the old index
+// order.  No block barriers.  A brick holding more than PB_BIG particles
+// (clustering: late epochs reach ~30x the mean) would make its warp the
+// kernel's tail: pass A lists those bricks and the first CTAs of the grid take
+// them whole.
+//
+// A whole CTA per brick, 256 particles per round: each warp's per-cell counts
+// go to a shared table, and a lane's slot is the cell's running start + the
+// counts of the lower warps + its rank in its warp, which is again the old
+// index order.  Small stores take it because a warp's chain of 16 rounds is
+// the whole kernel there, and every store with 2-byte velocities, whose rounds
+// wait for their table reads.  Measured, us (warp a brick / CTA a brick), x1v1:
+// 64 bricks 25.9 / 10.2, 512: 27.2 / 14.3, 1728: 30.0 / 27.0, 4096: 45.6 /
+// 52.6, 13824: 102 / 159; x2v2: 64: 67 / 16, 512: 70 / 20, 1728: 78 / 42,
+// 4096: 122 / 81, 13824: 367 / 250, 32768: 770 / 565.
 constexpr int PB_WARPS = 8;
 
 // what pass B needs of one particle: its new cell in the brick's halo
@@ -1118,11 +1127,8 @@ struct PassB {
     int key0, lim;
     float dcs, e0, e1;     // dcs: the drift factor in bins of the position code (dc 2^(8n))
 
-    // lc: the particle's coarse cell in the brick; its velocity offsets are
-    // read from the table (1-byte codes) or given in coff (2-byte codes, read
-    // a round ahead)
-    __device__ __forceinline__ PbParticle move(int lc, const float* svc, const int* cchi, const int* cnu,
-                                               const float* coff) const {
+    // lc: the particle's coarse cell in the brick
+    __device__ __forceinline__ PbParticle move(int lc, const float* svc, const int* cchi, const int* cnu) const {
         const int Bh = g.Bh;
         const int nbits = 8 * NX, half = 1 << (nbits - 1), bmask = (1 << nbits) - 1;
         const int l[3] = {lc & (g.B - 1), (lc >> g.lB) & (g.B - 1), lc >> (2 * g.lB)};
@@ -1131,7 +1137,7 @@ struct PassB {
 #pragma unroll
         for (int d = 0; d < 3; ++d) {
             const int Q = 2 * (cchi[d] + half) + 1;
-            const float p2 = svc[(d << (3 * g.lB)) + lc] + (NV == 2 ? coff[d] : dec[cnu[d] + lim]);
+            const float p2 = svc[(d << (3 * g.lB)) + lc] + dec[cnu[d] + lim];
             float x;
             const int bin = drift_bin(Q, p2, dcs, &x);
             const int sh = max(-1, min(1, bin >> nbits));
@@ -1204,7 +1210,96 @@ __device__ __forceinline__ void passB_stage(const Geo& g, const StoreDev& so, co
     }
 }
 
-template <int NX, int NV, bool BAT, int PID>
+// One brick by the whole CTA, blockDim.x = 256 particles a round.  Shared
+// words `sm`: [nbc + 1] offsets, [H3] running starts, [3][nbc] v_c, [3][H3]
+// v_c*, [PB_WARPS][H3] per-warp cell counts.
+template <int NX, int NV, int PID>
+__device__ __forceinline__ void passB_cta_brick(const Geo& g, const PassB<NX, NV, PID>& pb, const StoreDev& so,
+                                                const unsigned* __restrict__ ghost, const float* __restrict__ vc_new,
+                                                int brick, unsigned* sm, unsigned* flags) {
+    const int nbc = g.B * g.B * g.B, H3 = g.Bh * g.Bh * g.Bh, lim = g.nulim;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const CodeRows<NX> chi_o(so.chi, g.Np);
+    const CodeRows<NV> nu_o(so.nu, g.Np);
+    unsigned* sm_off = sm;
+    unsigned* run = sm_off + nbc + 1;
+    float* svc = reinterpret_cast<float*>(run + H3);
+    float* svn = svc + 3 * nbc;
+    unsigned* wcnt = reinterpret_cast<unsigned*>(svn + 3 * H3);
+    // a round's codes and id, requested a round ahead (the first beside the staging)
+    const unsigned p1 = min(so.offsets[brick * nbc + nbc], (unsigned)g.Np), p0 = min(so.offsets[brick * nbc], p1);
+    int nchi[3] = {0, 0, 0}, nnu[3] = {0, 0, 0};
+    unsigned nid = 0;
+    auto fetch = [&](unsigned i) {
+        if (i >= p1) return;
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            nchi[d] = chi_o.get(d, i);
+            nnu[d] = nu_o.get(d, i);
+        }
+        if (pb.sn.id) nid = PID == 4 ? reinterpret_cast<const unsigned*>(so.id)[i] : load_pid(so.id, i, g.nid);
+    };
+    fetch(p0 + threadIdx.x);
+    __syncthreads();                         // a previous brick's tables are no longer read
+    for (int t = threadIdx.x; t < PB_WARPS * H3; t += blockDim.x) wcnt[t] = 0u;
+    passB_stage(g, so, ghost, vc_new, brick, threadIdx.x, blockDim.x, sm_off, run, svc, svn);
+    __syncthreads();
+    for (unsigned base = p0; base < p1; base += blockDim.x) {
+        const unsigned i = base + threadIdx.x;
+        const bool act = i < p1;
+        const unsigned am = __ballot_sync(0xffffffffu, act);
+        PbParticle q{};
+        unsigned peers = 0;
+        const unsigned cid = nid;
+        int leader = 0;
+        if (act) {
+            int cchi[3], cnu[3];
+#pragma unroll
+            for (int d = 0; d < 3; ++d) {
+                cchi[d] = nchi[d];
+                cnu[d] = max(-lim, min(lim, nnu[d]));
+            }
+            fetch(i + blockDim.x);
+            q = pb.move(upper_cell(sm_off, nbc, i), svc, cchi, cnu);
+            peers = __match_any_sync(am, q.ei);
+            leader = __ffs(peers) - 1;
+            if (lane == leader) wcnt[warp * H3 + q.ei] = (unsigned)__popc(peers);
+        }
+        __syncthreads();
+        unsigned start = 0, total = 0;
+        bool last = true;
+        if (act) {
+            if (lane == leader) {
+                start = run[q.ei];
+#pragma unroll
+                for (int v = 0; v < PB_WARPS; ++v) {
+                    const unsigned c = wcnt[v * H3 + q.ei];
+                    if (v < warp) start += c;
+                    if (v > warp && c) last = false;
+                    total += c;
+                }
+            }
+            start = __shfl_sync(peers, start, leader);
+        }
+        __syncthreads();                     // every read of run and wcnt is done
+        if (act) {
+            if (lane == leader) {
+                if (last) run[q.ei] += total;
+                wcnt[warp * H3 + q.ei] = 0u;
+            }
+            pb.put(q, svn, start + (unsigned)__popc(peers & ((1u << lane) - 1u)), cid, flags);
+        }
+    }
+}
+
+// the split of pass B: a CTA per brick when the bricks' warps would fill less
+// than 40% of the 40 resident per SM, or with 2-byte velocities
+static bool passB_all(const Geo& g, int members) {
+    return g.nnu == 2 || (int64_t)g.nbricks * members <= 16 * (int64_t)g.nsm;
+}
+
+// ALL: every brick by a whole CTA
+template <int NX, int NV, bool BAT, int PID, bool ALL>
 __global__ void __launch_bounds__(PB_WARPS * 32, 5) k_passB(Geo g, StoreDev so, StoreDev sn, CodecDev cur, CodecDev next,
                                                         float dc, const unsigned* __restrict__ ghost,
                                                         const float* __restrict__ vc_new, unsigned* flags,
@@ -1229,7 +1324,7 @@ __global__ void __launch_bounds__(PB_WARPS * 32, 5) k_passB(Geo g, StoreDev so, 
         flags = moved(flags, o);
         big = moved(big, o);
     }
-    const bool big_cta = (int)blockIdx.x < nbig_ctas;
+    const bool big_cta = !ALL && (int)blockIdx.x < nbig_ctas;
     const int nbig = big_cta ? big[0] : 0;
     if (big_cta && (int)blockIdx.x >= nbig) return;          // no crowded brick left for this CTA
     float* sdec = reinterpret_cast<float*>(pb_smem);                       // NV == 1: [2 lim + 1]
@@ -1251,135 +1346,70 @@ __global__ void __launch_bounds__(PB_WARPS * 32, 5) k_passB(Geo g, StoreDev so, 
         pb.thr = sthr;
         pb.key0 = __float_as_int(next.est[2]);
     }
-    if (big_cta) {
-        // whole CTA per crowded brick: [nbc + 1] offsets, [H3] running starts,
-        // [3][nbc] v_c, [3][H3] v_c*, [PB_WARPS][H3] per-warp cell counts
-        unsigned* sm_off = wbase;
-        unsigned* run = sm_off + nbc + 1;
-        float* svc = reinterpret_cast<float*>(run + H3);
-        float* svn = svc + 3 * nbc;
-        unsigned* wcnt = reinterpret_cast<unsigned*>(svn + 3 * H3);
-        for (int t = threadIdx.x; t < PB_WARPS * H3; t += blockDim.x) wcnt[t] = 0u;
-        for (int k = blockIdx.x; k < nbig; k += nbig_ctas) {
-            const int brick = big[1 + k];
-            __syncthreads();                 // the previous brick's tables are no longer read
-            passB_stage(g, so, ghost, vc_new, brick, threadIdx.x, blockDim.x, sm_off, run, svc, svn);
-            __syncthreads();
-            const unsigned p1 = min(sm_off[nbc], (unsigned)g.Np), p0 = min(sm_off[0], p1);
-            for (unsigned base = p0; base < p1; base += blockDim.x) {
-                const unsigned i = base + threadIdx.x;
-                const bool act = i < p1;
-                const unsigned am = __ballot_sync(0xffffffffu, act);
-                PbParticle q{};
-                unsigned cid = 0, peers = 0;
-                int leader = 0;
-                if (act) {
-                    int cchi[3], cnu[3];
-#pragma unroll
-                    for (int d = 0; d < 3; ++d) {
-                        cchi[d] = chi_o.get(d, i);
-                        cnu[d] = nu_o.get_nu(d, i, lim);
-                    }
-                    if (sn.id) cid = PID == 4 ? reinterpret_cast<const unsigned*>(so.id)[i] : load_pid(so.id, i, g.nid);
-                    float coff[3];
-#pragma unroll
-                    for (int d = 0; d < 3; ++d) coff[d] = NV == 2 ? pb.dec[cnu[d] + lim] : 0.0f;
-                    q = pb.move(upper_cell(sm_off, nbc, i), svc, cchi, cnu, coff);
-                    peers = __match_any_sync(am, q.ei);
-                    leader = __ffs(peers) - 1;
-                    if (lane == leader) wcnt[warp * H3 + q.ei] = (unsigned)__popc(peers);
-                }
-                __syncthreads();
-                unsigned start = 0, total = 0;
-                bool last = true;
-                if (act) {
-                    if (lane == leader) {
-                        start = run[q.ei];
-#pragma unroll
-                        for (int v = 0; v < PB_WARPS; ++v) {
-                            const unsigned c = wcnt[v * H3 + q.ei];
-                            if (v < warp) start += c;
-                            if (v > warp && c) last = false;
-                            total += c;
-                        }
-                    }
-                    start = __shfl_sync(peers, start, leader);
-                }
-                __syncthreads();                 // every read of run and wcnt is done
-                if (act) {
-                    if (lane == leader) {
-                        if (last) run[q.ei] += total;
-                        wcnt[warp * H3 + q.ei] = 0u;
-                    }
-                    pb.put(q, svn, start + (unsigned)__popc(peers & ((1u << lane) - 1u)), cid, flags);
-                }
-            }
+    if constexpr (ALL) {
+        passB_cta_brick<NX, NV, PID>(g, pb, so, ghost, vc_new, blockIdx.x, wbase, flags);
+    } else {
+        if (big_cta) {
+            for (int k = blockIdx.x; k < nbig; k += nbig_ctas)
+                passB_cta_brick<NX, NV, PID>(g, pb, so, ghost, vc_new, big[1 + k], wbase, flags);
+            return;
         }
-        return;
-    }
-    __syncthreads();
-    const int brick = ((int)blockIdx.x - nbig_ctas) * PB_WARPS + warp;
-    if (brick >= g.nbricks) return;
-    const int L0 = brick * nbc;
-    const unsigned p1 = min(so.offsets[L0 + nbc], (unsigned)g.Np), p0 = min(so.offsets[L0], p1);
-    if (p1 - p0 > (unsigned)PB_BIG) return;              // a crowded brick: taken by a whole CTA
-    unsigned* sm_off = wbase + warp * (4 * nbc + 1 + 4 * H3);               // [nbc + 1] per warp
-    unsigned* run = sm_off + nbc + 1;                                       // [H3] per warp
-    float* svc = reinterpret_cast<float*>(run + H3);                        // [3][nbc]: v_c of the brick
-    float* svn = svc + 3 * nbc;                                             // [3][H3]: v_c* of the halo region
-    // the first round's codes and ids first, so their latency overlaps the staging
-    int nchi[3] = {0, 0, 0}, nnu[3] = {0, 0, 0};
-    float noff[3] = {0.0f, 0.0f, 0.0f};        // 2-byte codes: the next round's decoded offsets
-    unsigned nid = 0;
-    if (p0 + lane < p1) {
-#pragma unroll
-        for (int d = 0; d < 3; ++d) {
-            nchi[d] = chi_o.get(d, p0 + lane);
-            nnu[d] = nu_o.get_nu(d, p0 + lane, lim);
-        }
-        if (sn.id)
-            nid = PID == 4 ? reinterpret_cast<const unsigned*>(so.id)[p0 + lane] : load_pid(so.id, p0 + lane, g.nid);
-        if (NV == 2)
-#pragma unroll
-            for (int d = 0; d < 3; ++d) noff[d] = pb.dec[nnu[d] + lim];
-    }
-    passB_stage(g, so, ghost, vc_new, brick, lane, 32, sm_off, run, svc, svn);
-    __syncwarp();
-    int c0 = upper_cell(sm_off, nbc, p0);      // the cell of each round's first particle
-    for (unsigned base = p0; base < p1; base += 32) {
-        const unsigned i = base + lane;
-        const bool act = i < p1;
-        const unsigned am = __ballot_sync(0xffffffffu, act);
-        // this round's codes; the next round's are requested now
-        const int cchi[3] = {nchi[0], nchi[1], nchi[2]}, cnu[3] = {nnu[0], nnu[1], nnu[2]};
-        const float coff[3] = {noff[0], noff[1], noff[2]};
-        const unsigned cid = nid;
-        if (i + 32 < p1) {
-#pragma unroll
+        __syncthreads();
+        const int brick = ((int)blockIdx.x - nbig_ctas) * PB_WARPS + warp;
+        if (brick >= g.nbricks) return;
+        const int L0 = brick * nbc;
+        const unsigned p1 = min(so.offsets[L0 + nbc], (unsigned)g.Np), p0 = min(so.offsets[L0], p1);
+        if (p1 - p0 > (unsigned)PB_BIG) return;              // a crowded brick: taken by a whole CTA
+        unsigned* sm_off = wbase + warp * (4 * nbc + 1 + 4 * H3);               // [nbc + 1] per warp
+        unsigned* run = sm_off + nbc + 1;                                       // [H3] per warp
+        float* svc = reinterpret_cast<float*>(run + H3);                        // [3][nbc]: v_c of the brick
+        float* svn = svc + 3 * nbc;                                             // [3][H3]: v_c* of the halo region
+        // the first round's codes and ids first, so their latency overlaps the staging
+        int nchi[3] = {0, 0, 0}, nnu[3] = {0, 0, 0};
+        unsigned nid = 0;
+        if (p0 + lane < p1) {
+    #pragma unroll
             for (int d = 0; d < 3; ++d) {
-                nchi[d] = chi_o.get(d, i + 32);
-                nnu[d] = nu_o.get_nu(d, i + 32, lim);
+                nchi[d] = chi_o.get(d, p0 + lane);
+                nnu[d] = nu_o.get_nu(d, p0 + lane, lim);
             }
             if (sn.id)
-                nid = PID == 4 ? reinterpret_cast<const unsigned*>(so.id)[i + 32] : load_pid(so.id, i + 32, g.nid);
+                nid = PID == 4 ? reinterpret_cast<const unsigned*>(so.id)[p0 + lane] : load_pid(so.id, p0 + lane, g.nid);
         }
-        int cnext;
-        const int lcell = warp_cells(sm_off, nbc, base, c0, &cnext);
-        c0 = cnext;
-        if (act) {
-            const PbParticle q = pb.move(lcell, svc, cchi, cnu, coff);
-            const unsigned peers = __match_any_sync(am, q.ei);
-            const int leader = __ffs(peers) - 1;
-            unsigned start = 0;
-            if (lane == leader) start = run[q.ei];
-            start = __shfl_sync(peers, start, leader);
-            if (lane == leader) run[q.ei] = start + (unsigned)__popc(peers);
-            pb.put(q, svn, start + (unsigned)__popc(peers & ((1u << lane) - 1u)), cid, flags);
-        }
-        if (NV == 2 && i + 32 < p1)                // the next round's offsets, its codes having arrived
-#pragma unroll
-            for (int d = 0; d < 3; ++d) noff[d] = pb.dec[nnu[d] + lim];
+        passB_stage(g, so, ghost, vc_new, brick, lane, 32, sm_off, run, svc, svn);
         __syncwarp();
+        int c0 = upper_cell(sm_off, nbc, p0);      // the cell of each round's first particle
+        for (unsigned base = p0; base < p1; base += 32) {
+            const unsigned i = base + lane;
+            const bool act = i < p1;
+            const unsigned am = __ballot_sync(0xffffffffu, act);
+            // this round's codes; the next round's are requested now
+            const int cchi[3] = {nchi[0], nchi[1], nchi[2]}, cnu[3] = {nnu[0], nnu[1], nnu[2]};
+            const unsigned cid = nid;
+            if (i + 32 < p1) {
+    #pragma unroll
+                for (int d = 0; d < 3; ++d) {
+                    nchi[d] = chi_o.get(d, i + 32);
+                    nnu[d] = nu_o.get_nu(d, i + 32, lim);
+                }
+                if (sn.id)
+                    nid = PID == 4 ? reinterpret_cast<const unsigned*>(so.id)[i + 32] : load_pid(so.id, i + 32, g.nid);
+            }
+            int cnext;
+            const int lcell = warp_cells(sm_off, nbc, base, c0, &cnext);
+            c0 = cnext;
+            if (act) {
+                const PbParticle q = pb.move(lcell, svc, cchi, cnu);
+                const unsigned peers = __match_any_sync(am, q.ei);
+                const int leader = __ffs(peers) - 1;
+                unsigned start = 0;
+                if (lane == leader) start = run[q.ei];
+                start = __shfl_sync(peers, start, leader);
+                if (lane == leader) run[q.ei] = start + (unsigned)__popc(peers);
+                pb.put(q, svn, start + (unsigned)__popc(peers & ((1u << lane) - 1u)), cid, flags);
+            }
+            __syncwarp();
+        }
     }
 }
 
@@ -1444,18 +1474,24 @@ struct Disp {
     }
     static void passB(const Geo& g, const StoreDev& so, const StoreDev& sn, const CodecDev& cur,
                       const CodecDev& next, float dc, const unsigned* ghost, const float* vcn, unsigned* flags,
-                      const int* big, size_t sm, cudaStream_t st, const Batch& bt) {
-        // CTAs for crowded bricks first (at most Np / (PB_BIG + 1) of them exist)
-        const int nbig_ctas = (int)std::min<int64_t>(2 * g.nsm, g.Np / (PB_BIG + 1));
-        const int grid = nbig_ctas + (g.nbricks + PB_WARPS - 1) / PB_WARPS;
-        const bool narrow = g.nid == 1 || g.nid == 2;
-        if (bt.members > 1 || bt.ms) {
-            const dim3 gb(grid, bt.members);
-            if (narrow) k_passB<NX, NV, true, 0><<<gb, PB_WARPS * 32, sm, st>>>(g, so, sn, cur, next, dc, ghost, vcn, flags, big, nbig_ctas, bt);
-            else k_passB<NX, NV, true, 4><<<gb, PB_WARPS * 32, sm, st>>>(g, so, sn, cur, next, dc, ghost, vcn, flags, big, nbig_ctas, bt);
-        } else {
-            if (narrow) k_passB<NX, NV, false, 0><<<grid, PB_WARPS * 32, sm, st>>>(g, so, sn, cur, next, dc, ghost, vcn, flags, big, nbig_ctas, bt);
-            else k_passB<NX, NV, false, 4><<<grid, PB_WARPS * 32, sm, st>>>(g, so, sn, cur, next, dc, ghost, vcn, flags, big, nbig_ctas, bt);
+                      const int* big, size_t sm, size_t sm_cta, cudaStream_t st, const Batch& bt) {
+        const bool narrow = g.nid == 1 || g.nid == 2, bat = bt.members > 1 || bt.ms;
+        if (passB_all(g, bt.members)) {
+            const dim3 gb(g.nbricks, bt.members);
+            if (bat && narrow) k_passB<NX, NV, true, 0, true><<<gb, PB_WARPS * 32, sm_cta, st>>>(g, so, sn, cur, next, dc, ghost, vcn, flags, big, 0, bt);
+            else if (bat) k_passB<NX, NV, true, 4, true><<<gb, PB_WARPS * 32, sm_cta, st>>>(g, so, sn, cur, next, dc, ghost, vcn, flags, big, 0, bt);
+            else if (narrow) k_passB<NX, NV, false, 0, true><<<gb, PB_WARPS * 32, sm_cta, st>>>(g, so, sn, cur, next, dc, ghost, vcn, flags, big, 0, bt);
+            else k_passB<NX, NV, false, 4, true><<<gb, PB_WARPS * 32, sm_cta, st>>>(g, so, sn, cur, next, dc, ghost, vcn, flags, big, 0, bt);
+            return;
+        }
+        if constexpr (NV == 1) {
+            // CTAs for crowded bricks first (at most Np / (PB_BIG + 1) of them exist)
+            const int nbig_ctas = (int)std::min<int64_t>(2 * g.nsm, g.Np / (PB_BIG + 1));
+            const dim3 gb(nbig_ctas + (g.nbricks + PB_WARPS - 1) / PB_WARPS, bt.members);
+            if (bat && narrow) k_passB<NX, NV, true, 0, false><<<gb, PB_WARPS * 32, sm, st>>>(g, so, sn, cur, next, dc, ghost, vcn, flags, big, nbig_ctas, bt);
+            else if (bat) k_passB<NX, NV, true, 4, false><<<gb, PB_WARPS * 32, sm, st>>>(g, so, sn, cur, next, dc, ghost, vcn, flags, big, nbig_ctas, bt);
+            else if (narrow) k_passB<NX, NV, false, 0, false><<<gb, PB_WARPS * 32, sm, st>>>(g, so, sn, cur, next, dc, ghost, vcn, flags, big, nbig_ctas, bt);
+            else k_passB<NX, NV, false, 4, false><<<gb, PB_WARPS * 32, sm, st>>>(g, so, sn, cur, next, dc, ghost, vcn, flags, big, nbig_ctas, bt);
         }
     }
 };
@@ -1469,10 +1505,10 @@ void set_smem_attrs() {
     cudaFuncSetAttribute(k_passA<NX, NV, 16, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
     cudaFuncSetAttribute(k_passA<NX, NV, 0, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
     cudaFuncSetAttribute(k_passA<NX, NV, 16, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-    cudaFuncSetAttribute(k_passB<NX, NV, false, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-    cudaFuncSetAttribute(k_passB<NX, NV, true, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-    cudaFuncSetAttribute(k_passB<NX, NV, false, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-    cudaFuncSetAttribute(k_passB<NX, NV, true, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+    if constexpr (NV == 1) cudaFuncSetAttribute(k_passB<NX, NV, false, 4, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+    if constexpr (NV == 1) cudaFuncSetAttribute(k_passB<NX, NV, true, 4, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+    if constexpr (NV == 1) cudaFuncSetAttribute(k_passB<NX, NV, false, 0, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+    if constexpr (NV == 1) cudaFuncSetAttribute(k_passB<NX, NV, true, 0, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
     cudaFuncSetAttribute(k_deposit<NX, 0, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
     cudaFuncSetAttribute(k_deposit<NX, 16, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
     cudaFuncSetAttribute(k_deposit<NX, 0, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
@@ -1653,21 +1689,22 @@ void launch_cells(const Geo& g, const StepScratch& w, unsigned* off_new, float* 
     else k_cells<false><<<nblk(g.Ncc, 256), 256, 0, st>>>(g, w, off_new, vc_new, bt);
 }
 
-static size_t passB_smem(const Geo& g) {
-    const int H3 = g.Bh * g.Bh * g.Bh, nbc = g.B * g.B * g.B;
-    size_t sm = (size_t)PB_WARPS * (4 * nbc + 1 + 4 * H3) * 4;
+// `words` of a CTA's brick tables after the staged 1-byte codec tables
+static size_t passB_smem(const Geo& g, int words) {
+    size_t sm = (size_t)words * 4;
     if (g.nnu == 1) sm += (size_t)(3 * g.nulim + 3) * 4 + VT_N;
     return (sm + 15) & ~(size_t)15;
 }
 
 void launch_passB(const Geo& g, const StoreDev& so, const StoreDev& sn, const CodecDev& cur, const CodecDev& next,
                   float dc, const StepScratch& w, cudaStream_t st, const Batch& bt) {
-    size_t sm = passB_smem(g);
+    const size_t sm = passB_smem(g, PB_WARPS * (4 * g.B * g.B * g.B + 1 + 4 * g.Bh * g.Bh * g.Bh));
+    const size_t sm_cta = passB_smem(g, 4 * g.B * g.B * g.B + 1 + (4 + PB_WARPS) * g.Bh * g.Bh * g.Bh);
     const float* vcn = sn.vc;
-    if (g.nchi == 1 && g.nnu == 1) { set_smem_attrs<1, 1>(); Disp<1, 1>::passB(g, so, sn, cur, next, dc, w.ghost, vcn, w.flags, w.big, sm, st, bt); }
-    else if (g.nchi == 1) { set_smem_attrs<1, 2>(); Disp<1, 2>::passB(g, so, sn, cur, next, dc, w.ghost, vcn, w.flags, w.big, sm, st, bt); }
-    else if (g.nnu == 1) { set_smem_attrs<2, 1>(); Disp<2, 1>::passB(g, so, sn, cur, next, dc, w.ghost, vcn, w.flags, w.big, sm, st, bt); }
-    else { set_smem_attrs<2, 2>(); Disp<2, 2>::passB(g, so, sn, cur, next, dc, w.ghost, vcn, w.flags, w.big, sm, st, bt); }
+    if (g.nchi == 1 && g.nnu == 1) { set_smem_attrs<1, 1>(); Disp<1, 1>::passB(g, so, sn, cur, next, dc, w.ghost, vcn, w.flags, w.big, sm, sm_cta, st, bt); }
+    else if (g.nchi == 1) { set_smem_attrs<1, 2>(); Disp<1, 2>::passB(g, so, sn, cur, next, dc, w.ghost, vcn, w.flags, w.big, sm, sm_cta, st, bt); }
+    else if (g.nnu == 1) { set_smem_attrs<2, 1>(); Disp<2, 1>::passB(g, so, sn, cur, next, dc, w.ghost, vcn, w.flags, w.big, sm, sm_cta, st, bt); }
+    else { set_smem_attrs<2, 2>(); Disp<2, 2>::passB(g, so, sn, cur, next, dc, w.ghost, vcn, w.flags, w.big, sm, sm_cta, st, bt); }
 }
 
 void launch_check_vel_tables(int lim, const CodecDev& c, long long* out2, cudaStream_t st) {

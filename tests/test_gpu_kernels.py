@@ -5,7 +5,7 @@ import pytest
 
 from oracle import pm
 
-from gpu_util import oracle_params, read_store
+from gpu_util import assert_store_equal, oracle_params, read_store
 
 pytestmark = pytest.mark.gpu
 
@@ -112,3 +112,73 @@ def test_packed_meshes_do_not_depend_on_alignment(cube, nf):
                 assert np.all(got[:shift] == -1.0) and np.all(got[shift + nf ** 3:] == -1.0)
     finally:
         cube.cube_destroy(ctx)
+
+
+# ---------------------------------------------------------------- pass B's split
+# epochs so close that the clump's force moves nothing, and momenta that cross
+# 0.7 fine cells (rms) in a step
+_EPOCHS = [0.5, 0.50005, 0.5001]
+_SPEED = 0.7 / (0.00005 / (0.5 ** 3 * 0.5 ** -1.5))
+
+
+def _mixed_particles(n, nf, seed, speed=_SPEED):
+    """Uniform random particles with 3000 of them in one brick."""
+    rng = np.random.default_rng(seed)
+    pos = rng.uniform(0.0, nf, (3, n))
+    pos[:, :3000] = 9.0 + 1.5 * rng.standard_normal((3, 3000))
+    vel = speed * rng.standard_normal((3, n))
+    return np.mod(pos, nf).astype(np.float32) % np.float32(nf), vel.astype(np.float32), np.arange(n, dtype=np.uint32)
+
+
+# more than 16 bricks per SM, 1-byte velocities: a warp per brick, crowded
+# bricks by whole CTAs, empty bricks, bricks of one cell; whole numbers, exact
+@pytest.mark.parametrize("nf,ratio,brick,n,xb,idb", [(256, 4, 4, 40000, 1, 4), (128, 4, 2, 33000, 2, 1),
+                                                     (64, 4, 1, 20001, 1, 2)])
+def test_resort_of_many_bricks_is_bit_exact(cube, nf, ratio, brick, n, xb, idb):
+    bricks = (nf // ratio // brick) ** 3
+    assert bricks > 16 * torch.cuda.get_device_properties(0).multi_processor_count
+    pos, vel, ids = _mixed_particles(n, nf, 1712204)
+    prm = cube.make_params(nf, n, ratio=ratio, x_bytes=xb, v_bytes=1, id_bytes=idb, brick=brick, box=50.0)
+    ctx = cube.cube_create(prm, torch.cuda.current_stream())
+    try:
+        a = _EPOCHS
+        cube.cube_encode(ctx, pos, vel, ids, a[0], 0.0)
+        cube.cube_keep_drifted(ctx, True)
+        for i in range(2):
+            before = read_store(cube, ctx)
+            cube.cube_pm_step(ctx, a[i], a[i + 1])
+            cell, u, p = np.empty((3, n), np.int32), np.empty((3, n), np.float32), np.empty((3, n), np.float32)
+            sig = cube.cube_debug_drifted(ctx, cell, u, p)
+            g = read_store(cube, ctx)
+            ref = pm.encode_drifted(oracle_params(pm, prm, g["brick"]), cell, u, p, before["ids"], sig, g["a"],
+                                    g["a_p"])
+            assert_store_equal(g, ref, f"step {i}")
+    finally:
+        cube.cube_destroy(ctx)
+
+
+# a batch whose members' bricks together pass the split gives each member's own run
+@pytest.mark.parametrize("vb", [1, 2])
+def test_batch_past_the_split_equals_members_alone(cube, vb):
+    nf, n, members = 128, 30000, 5
+    prm = cube.make_params(nf, n, v_bytes=vb, box=50.0)
+    batch = cube.cube_batch_create([prm] * members, torch.cuda.current_stream())
+    one = cube.cube_create(prm, torch.cuda.current_stream())
+    try:
+        sets = [_mixed_particles(n, nf, 1712205 + i) for i in range(members)]
+        ctxs = [cube.cube_batch_member(batch, i) for i in range(members)]
+        for c, s in zip(ctxs, sets):
+            cube.cube_encode(c, *s, _EPOCHS[0], 0.0)
+        for a0, a1 in zip(_EPOCHS, _EPOCHS[1:]):
+            cube.cube_batch_step(batch, [a0] * members, [a1] * members)
+        for c, s in zip(ctxs, sets):
+            cube.cube_encode(one, *s, _EPOCHS[0], 0.0)
+            for a0, a1 in zip(_EPOCHS, _EPOCHS[1:]):
+                cube.cube_pm_step(one, a0, a1)
+            x, y = read_store(cube, c), read_store(cube, one)
+            for k in ("counts", "offsets", "vc", "chi", "nu", "ids", "sigma"):
+                assert np.array_equal(x[k], y[k]), k
+            assert cube.cube_stats_get(c).max_migration == 1
+    finally:
+        cube.cube_destroy(one)
+        cube.cube_batch_destroy(batch)
