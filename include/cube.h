@@ -327,15 +327,15 @@ cube_status cube_debug_drifted(cube_ctx* ctx, int32_t* cell_old, float* u_new, f
    Errors: CUBE_E_ARG (NULL), CUBE_E_STATE (not kept, or no step yet). */
 cube_status cube_debug_force(cube_ctx* ctx, float* force);
 
-/* Self-check of the compact form in which the step kernels read 2-byte
-   velocity codes' tables (Eq. v decode values tan(pi k / M) gamma and Eq. nu
-   thresholds, Section 2.2): each entry is rebuilt, as the kernels rebuild
-   it, from a fixed FP32 approximation and a 4-bit correction, and compared
-   with the full table of the current store's codec, for every k in
-   [-lim, lim] (decode) and [0, lim + 1] (thresholds).  out2[0] = entries that
-   differ (0: the kernels see the exact tables), out2[1] = entries kept as
-   "read the full table" (correction out of range).  `out2` is host memory.
-   Synchronises.
+/* Self-check of how the kernels evaluate 2-byte velocity codes (Section 2.2):
+   each decode value tan(pi k / M) gamma (Eq. v) is rebuilt, as the kernels
+   rebuild it, from a fixed FP32 approximation and a one-byte correction, and
+   compared with the full table of the current store's codec, for every k in
+   [-lim, lim]; and the codes of the offsets at and just below every threshold
+   of Eq. nu, k in [1, lim], are compared with k and k - 1.  out2[0] = entries
+   and thresholds that differ (0: the kernels see the exact tables), out2[1] =
+   entries kept as "read the full table" (correction out of range).  `out2` is
+   host memory.  Synchronises.
    Errors: CUBE_E_ARG (NULL, or codes other than 2-byte velocities),
    CUBE_E_STATE (no store). */
 cube_status cube_debug_velocity_tables(cube_ctx* ctx, int64_t* out2);

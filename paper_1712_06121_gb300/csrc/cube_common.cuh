@@ -199,23 +199,7 @@ __device__ __forceinline__ float vel_unfix_mean(long long s, unsigned n) {
 // Eq. nu via exact thresholds: thr[k] (k = 1..lim) is the smallest float >=
 // tan(pi (k - 1/2) / M) / s, thr[lim + 1] = +inf, so |d| >= thr[k]  <=>  the
 // nearest integer of (M/pi) atan(|d| s) is >= k (halves away from zero).
-// `est` is any starting guess; the result does not depend on it.
-// The two thresholds around the guess are requested together, so a guess
-// within one code costs one memory round trip.
-__device__ __forceinline__ int nu_from_thresholds(float d, const float* __restrict__ thr, int lim, int est) {
-    float a = fabsf(d);
-    int k = min(max(est, 0), lim);
-    const float lo = thr[k], hi = thr[k + 1];            // thr[lim + 1] = +inf
-    if (a >= hi) {
-        ++k;
-        while (k < lim && a >= thr[k + 1]) ++k;
-    } else if (a < lo) {
-        --k;
-        while (k > 0 && a < thr[k]) --k;
-    }
-    return d < 0.0f ? -k : k;
-}
-
+//
 // Eq. nu for 1-byte codes through a bucket table.  Bucket i holds the |d|
 // whose float bit patterns share bits 31..(23 - VT_B) = key0 + i: 2^VT_B
 // buckets per octave, VT_N buckets (16 octaves) from just below thr[1].
@@ -224,8 +208,7 @@ __device__ __forceinline__ int nu_from_thresholds(float d, const float* __restri
 // tan(pi (k + 1/2) / 255) / tan(pi (k - 1/2) / 255)), more than a bucket's
 // width (at most 2^-6 = 1.56%), so a bucket holds at most one threshold and
 // one compare with the next threshold completes the code; thr[1 .. 127]
-// span 13.7 octaves, inside the table.  The result equals
-// nu_from_thresholds'.
+// span 13.7 octaves, inside the table.
 constexpr int VT_B = 6;
 constexpr int VT_N = 1024;
 __device__ __forceinline__ int nu_from_table(float d, const float* __restrict__ thr,
@@ -237,121 +220,113 @@ __device__ __forceinline__ int nu_from_table(float d, const float* __restrict__ 
     return d < 0.0f ? -k : k;
 }
 
-// ---- 2-byte velocity tables as an approximation plus a 4-bit correction
-// The decode values dec[k] = tan(pi k / M) gamma and the thresholds thr[k]
-// (tan(pi (k - 1/2) / M) / s rounded up) of 2-byte codes are 2^16-entry
-// tables whose entries a kernel reads at random: in global memory every
-// lookup is an L2 round trip.  Both are tan(m pi / (2M)) gamma at m = 2k and
-// m = 2k - 1, so each entry is stored as the difference, in ulps, between
-// its exact FP32 value and tan_half_steps(m), a fixed FP32 evaluation that
-// every kernel repeats bit for bit: 4 bits per entry (one byte holds both
-// tables' corrections for one k), 32 KB that stay in L1.  A difference
-// outside [-7, 7] is stored as -8 and that entry is read from the full table.
-// The result is the table's value in every case; the approximation's
-// accuracy only decides how rarely the full table is read.
+// ---- 2-byte decode table as an approximation plus an 8-bit correction
+// dec[k] = tan(pi k / M) gamma of 2-byte codes is a 2^16-entry table whose
+// entries a kernel reads at random: in global memory every lookup is an L2
+// round trip.  Each entry is stored as the difference, in ulps, between its
+// exact FP32 value and tan_steps(k), a fixed FP32 evaluation that every kernel
+// repeats bit for bit: one byte per k, 32 KB that stay in L1.  A difference
+// outside [-127, 127] is stored as -128 and that entry is read from the full
+// table.  The result is the table's value in every case; the approximation's
+// accuracy only decides how rarely the full table is read (never, for the
+// scales tested): six terms here instead of the Taylor series' twelve took
+// pass A of 1.03 M particles x2v2 from 69 to 64 us.
 struct VelApprox {
     float c;      // pi / (2M), M = 2 lim + 1
     float gam;    // sqrt(2 sigma^2 / pi) = 1 / s
     int M;
 };
 
-// tan(m pi / (2M)) gamma for 0 < m < M in FP32 to a few ulps: the angle, or
-// above pi/4 its complement (M - m) pi / (2M) (tan = 1 / tan of the
-// complement), lies in (0, pi/4], where the Taylor series of tan to x^23
-// (Abramowitz & Stegun 4.3.67, coefficients 2^2n (2^2n - 1) |B_2n| / (2n)!)
-// is within 5e-8 relative.  Explicitly rounded operations only, so every
-// kernel gets the same bits.
-__device__ __forceinline__ float tan_half_steps(int m, const VelApprox& va) {
-    const bool cot = 2 * m > va.M;
-    const int mm = cot ? va.M - m : m;                         // < 2^16
+// tan(k pi / M) gamma for 0 <= 2 k < M in FP32 to a few ulps: the angle, or
+// above pi/4 its complement (M - 2k) pi / (2M) (tan = 1 / tan of the
+// complement), lies in [0, pi/4], where the polynomial of Abramowitz & Stegun
+// 4.3.101 is within 2e-8.  Explicitly rounded operations only, so every kernel
+// gets the same bits.
+__device__ __forceinline__ float tan_steps(int k, const VelApprox& va) {
+    const bool cot = 4 * k > va.M;
+    const int mm = cot ? va.M - 2 * k : 2 * k;                 // < 2^16
     const float x = __fmul_rn(__fsub_rn(__int_as_float(0x4B000000 | mm), 8388608.0f), va.c);
     const float x2 = __fmul_rn(x, x);
-    float p = 3.9278322e-05f;
-    p = __fmaf_rn(p, x2, 9.691538e-05f);
-    p = __fmaf_rn(p, x2, 0.00023912912f);
-    p = __fmaf_rn(p, x2, 0.0005900274f);
-    p = __fmaf_rn(p, x2, 0.0014558344f);
-    p = __fmaf_rn(p, x2, 0.003592128f);
-    p = __fmaf_rn(p, x2, 0.008863236f);
-    p = __fmaf_rn(p, x2, 0.021869488f);
-    p = __fmaf_rn(p, x2, 0.053968254f);
-    p = __fmaf_rn(p, x2, 0.13333334f);
-    p = __fmaf_rn(p, x2, 0.33333334f);
-    p = __fmaf_rn(p, x2, 1.0f);
-    const float t = __fmul_rn(x, p);
+    float p = 0.0095168091f;
+    p = __fmaf_rn(p, x2, 0.0029005250f);
+    p = __fmaf_rn(p, x2, 0.0245650893f);
+    p = __fmaf_rn(p, x2, 0.0533740603f);
+    p = __fmaf_rn(p, x2, 0.1333923995f);
+    p = __fmaf_rn(p, x2, 0.3333314036f);
+    const float t = __fmaf_rn(__fmul_rn(x, x2), p, x);
     return cot ? __fdividef(va.gam, t) : __fmul_rn(t, va.gam);
 }
 
-// the signed 4-bit correction in bits lo..lo+3 of b
-__device__ __forceinline__ int vdelta(unsigned b, int lo) { return (int)(b << (28 - lo)) >> 28; }
+// the correction byte of a difference
+__device__ __forceinline__ signed char vdelta(int d) { return (signed char)(d < -127 || d > 127 ? -128 : d); }
 
-// the correction byte of k: decode difference in bits 0-3, threshold difference in bits 4-7
-__device__ __forceinline__ unsigned char vdelta_pack(int dd, int dt) {
-    const int a = (dd < -7 || dd > 7) ? -8 : dd, b = (dt < -7 || dt > 7) ? -8 : dt;
-    return (unsigned char)((a & 15) | ((b & 15) << 4));
-}
-
-// exact 2-byte tables through the corrections; dec_g / thr_g the full tables
-// (dec_g indexed by nu + lim), vdel [lim + 2] the correction bytes
+// the exact 2-byte decode table through the corrections; dec_g the full table
+// (indexed by nu + lim), vdel [lim + 2] the correction bytes
 struct VelTables {
     const float* __restrict__ dec_g;
-    const float* __restrict__ thr_g;
-    const unsigned char* __restrict__ vdel;
+    const signed char* __restrict__ vdel;
     VelApprox va;
     int lim;
     // dec[nu + lim] for |nu| <= lim
     __device__ __forceinline__ float dec(int nu) const {
         const int k = abs(nu);
-        if (k == 0) return 0.0f;
-        const int dd = vdelta(__ldg(&vdel[k]), 0);
-        const float v = dd == -8 ? dec_g[k + lim]
-                                 : __int_as_float(__float_as_int(tan_half_steps(2 * k, va)) + dd);
+        const int d = __ldg(&vdel[k]);
+        const float v = d == -128 ? dec_g[k + lim] : __int_as_float(__float_as_int(tan_steps(k, va)) + d);
         return nu < 0 ? -v : v;
-    }
-    // thr[k] for 0 <= k <= lim + 1 (thr[0] = 0, thr[lim + 1] = +inf)
-    __device__ __forceinline__ float thr(int k) const {
-        if (k <= 0) return 0.0f;
-        if (k > lim) return __int_as_float(0x7f800000);
-        const int dt = vdelta(__ldg(&vdel[k]), 4);
-        return dt == -8 ? thr_g[k] : __int_as_float(__float_as_int(tan_half_steps(2 * k - 1, va)) + dt);
     }
 };
 
-// nu_from_thresholds with the thresholds of a VelTables
-__device__ __forceinline__ int nu_from_tables(float d, const VelTables& vt, int est) {
-    const float a = fabsf(d);
-    int k = min(max(est, 0), vt.lim);
-    const float lo = vt.thr(k), hi = vt.thr(k + 1);
-    if (a >= hi) {
-        ++k;
-        while (k < vt.lim && a >= vt.thr(k + 1)) ++k;
-    } else if (a < lo) {
-        --k;
-        while (k > 0 && a < vt.thr(k)) --k;
-    }
-    return d < 0.0f ? -k : k;
-}
-
-// Starting guess for nu_from_thresholds: (M/pi) atan(|d| s) with the
-// arctangent from the polynomial of Abramowitz & Stegun 4.4.47 (Hastings),
-// |error| <= 1e-5 rad on [0, 1], and atan(x) = pi/2 - atan(1/x) above 1.
-// The error is well under one code for 2-byte codes, so the exact search
-// that follows takes at most a step or two.
-__device__ __forceinline__ int nu_estimate(float d, float s, float m_over_pi) {
-    const float x = fabsf(d) * s;
+// Eq. nu for three 2-byte codes at once.  y = (M / pi) atan(|d| s) is evaluated
+// in FP32 from the polynomial of Abramowitz & Stegun 4.4.49 (|error| <= 2e-8
+// on [0, 1]; atan(x) = pi/2 - atan(1/x) above 1) to within 0.006 codes (the
+// largest error at any threshold, for codec scales 2^-12 to 2^12 and two ulps
+// either way in the reciprocal; the roundings add up to less than 0.0075), so
+// the nearest integer is decided unless y lies within kNuMargin = 1/64 of a
+// half-integer.  There, 3% of the codes, |d| is compared with the exact
+// threshold: one table read, all three axes' in flight together, where a
+// search from a coarser guess reads two per code one code after the other.
+// Halves away from zero, |nu| <= lim.  1.03 M particles x2v2 (1728 bricks), with
+// the two-threshold search -> this: pass A 108 -> 69 us, pass B 55 -> 38 us.
+constexpr float kNuMargin = 1.0f / 64.0f;
+__device__ __forceinline__ float nu_value(float a, float s, float m_over_pi, float half_m) {
+    const float x = a * s;
     const bool big = x > 1.0f;
     float r;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));    // a guess needs no exact reciprocal
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
     const float t = big ? r : x;
     const float t2 = t * t;
-    float p = 0.0208351f;
-    p = __fmaf_rn(p, t2, -0.0851330f);
-    p = __fmaf_rn(p, t2, 0.1801410f);
-    p = __fmaf_rn(p, t2, -0.3302995f);
-    p = __fmaf_rn(p, t2, 0.9998660f);
-    float a = p * t;
-    if (big) a = 1.57079633f - a;
-    return __float2int_rn(m_over_pi * a);
+    float p = 0.0028662257f;
+    p = __fmaf_rn(p, t2, -0.0161657367f);
+    p = __fmaf_rn(p, t2, 0.0429096138f);
+    p = __fmaf_rn(p, t2, -0.0752896400f);
+    p = __fmaf_rn(p, t2, 0.1065626393f);
+    p = __fmaf_rn(p, t2, -0.1420889944f);
+    p = __fmaf_rn(p, t2, 0.1999355085f);
+    p = __fmaf_rn(p, t2, -0.3333314528f);
+    const float y = m_over_pi * __fmaf_rn(t * t2, p, t);
+    return big ? half_m - y : y;
+}
+__device__ __forceinline__ void nu_codes3(const float* d, const float* __restrict__ thr, int lim, float s,
+                                          float m_over_pi, int* nu) {
+    int j[3];
+    bool near[3], up[3];
+    float t[3];
+    const float half_m = (float)lim + 0.5f;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const float y = nu_value(fabsf(d[k]), s, m_over_pi, half_m);
+        const float f = __fadd_rd(y, 12582912.0f);               // 1.5 2^23 + floor(y): y < 2^16
+        j[k] = __float_as_int(f) - 0x4B400000;
+        const float fr = y - (f - 12582912.0f);
+        up[k] = fr > 0.5f;
+        near[k] = fabsf(fr - 0.5f) <= kNuMargin && j[k] < lim;
+        t[k] = near[k] ? thr[j[k] + 1] : 0.0f;
+    }
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const int v = min(j[k] + ((near[k] ? fabsf(d[k]) >= t[k] : up[k]) ? 1 : 0), lim);
+        nu[k] = d[k] < 0.0f ? -v : v;
+    }
 }
 
 // Packed FP32 pairs (Blackwell's two-wide FP32 instructions): each lane of a

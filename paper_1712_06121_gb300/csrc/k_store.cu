@@ -89,10 +89,10 @@ __device__ __forceinline__ BrickTables stage_brick(const Geo& g, const StoreDev&
     return t;
 }
 
-// the decode and threshold tables of 2-byte codes through their corrections
+// the decode table of 2-byte codes through its corrections
 template <int NV>
 __device__ __forceinline__ VelTables vel_tables(const CodecDev& c, int lim) {
-    return VelTables{c.dec, c.thr, c.vdel, VelApprox{NV == 2 ? c.est[3] : 0.0f, NV == 2 ? c.est[4] : 0.0f, 2 * lim + 1},
+    return VelTables{c.dec, c.vdel, VelApprox{NV == 2 ? c.est[3] : 0.0f, NV == 2 ? c.est[4] : 0.0f, 2 * lim + 1},
                      lim};
 }
 
@@ -249,18 +249,18 @@ __global__ void k_sigma_finalize(const float* __restrict__ part, int nparts, dou
     }
 }
 
-// decode table, thresholds, starting-guess constants and (1-byte codes,
+// decode table, thresholds, scale constants and (1-byte codes,
 // single block) the bucket table for the codec scale sg
 __device__ void codec_tables_body(int lim, const double* __restrict__ tanv, const double* __restrict__ tanh_,
                                   double sg, float* __restrict__ dec, float* __restrict__ thr,
                                   float* __restrict__ est, unsigned char* __restrict__ vtab,
-                                  unsigned char* __restrict__ vdel) {
+                                  signed char* __restrict__ vdel) {
     const double s = sqrt(PI_D / (2.0 * sg * sg));
     const double gam = sqrt(2.0 * sg * sg / PI_D);
     const double m = (double)(2 * lim + 1);
     const VelApprox va{(float)(PI_D / (2.0 * m)), (float)gam, 2 * lim + 1};
     for (int k = blockIdx.x * blockDim.x + threadIdx.x; k <= lim + 1; k += gridDim.x * blockDim.x) {
-        int ddec = 0, dthr = 0;                          // corrections of the 2-byte tables (vdel)
+        int ddec = 0;                                    // correction of the 2-byte decode table (vdel)
         if (k == 0) {
             dec[lim] = 0.0f;
             thr[0] = 0.0f;
@@ -274,14 +274,11 @@ __device__ void codec_tables_body(int lim, const double* __restrict__ tanv, cons
             dec[lim - k] = -dv;
             const float tv = __double2float_ru(tanh_[k] / s);
             thr[k] = tv;
-            if (vdel) {
-                ddec = __float_as_int(dv) - __float_as_int(tan_half_steps(2 * k, va));
-                dthr = __float_as_int(tv) - __float_as_int(tan_half_steps(2 * k - 1, va));
-            }
+            if (vdel) ddec = __float_as_int(dv) - __float_as_int(tan_steps(k, va));
         } else {
             thr[lim + 1] = __int_as_float(0x7f800000);   // +inf
         }
-        if (vdel) vdel[k] = vdelta_pack(ddec, dthr);
+        if (vdel) vdel[k] = vdelta(ddec);
     }
     if (vtab) {   // 1-byte codes (lim < 256), one block: the bucket table of nu_from_table
         __shared__ float sthr[256];
@@ -306,7 +303,7 @@ __device__ void codec_tables_body(int lim, const double* __restrict__ tanv, cons
 __global__ void k_codec_tables(int lim, const double* __restrict__ tanv, const double* __restrict__ tanh_,
                                const double* __restrict__ sigma, float* __restrict__ dec, float* __restrict__ thr,
                                float* __restrict__ est, unsigned char* __restrict__ vtab,
-                               unsigned char* __restrict__ vdel, Batch bt) {
+                               signed char* __restrict__ vdel, Batch bt) {
     const int slot = blockIdx.y;                             // slot of a batch
     if (bt.ms && !bt.ms[slot].active) return;
     const size_t o = slot_member(bt, slot) * bt.stride;
@@ -317,8 +314,8 @@ __global__ void k_codec_tables(int lim, const double* __restrict__ tanv, const d
 template <int NX, int NV>
 __global__ void k_encode_scatter(Geo g, const float* __restrict__ pos, const float* __restrict__ vel,
                                  const unsigned* __restrict__ id_in, const unsigned* __restrict__ key,
-                                 const unsigned* __restrict__ perm, const float* __restrict__ vc,
-                                 const float* __restrict__ thr, const float* __restrict__ est, StoreDev s) {
+                                 const unsigned* __restrict__ perm, const float* __restrict__ vc, CodecDev cd,
+                                 StoreDev s) {
     int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= g.Np) return;
     const int64_t i = perm[j];
@@ -327,7 +324,9 @@ __global__ void k_encode_scatter(Geo g, const float* __restrict__ pos, const flo
     const int nbits = 8 * NX;
     const long long tot = (long long)g.Nc << nbits;
     const float scale = ldexpf(1.0f, nbits - g.r);
-    const float e0 = est[0], e1 = est[1];
+    const int key0 = NV == 1 ? __float_as_int(cd.est[2]) : 0;
+    float dd[3];
+    int nu[3];
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
         float x = pos[d * g.Np + i];
@@ -339,10 +338,12 @@ __global__ void k_encode_scatter(Geo g, const float* __restrict__ pos, const flo
         store_code<NX>(s.chi, d * g.Np + j, chi);
         float v = vel[d * g.Np + i];
         if (!isfinite(v)) v = 0.0f;
-        float dd = v - vc[(int64_t)d * g.Ncc + k];
-        int nu = nu_from_thresholds(dd, thr, g.nulim, nu_estimate(dd, e0, e1));
-        store_code<NV>(s.nu, d * g.Np + j, nu);
+        dd[d] = v - vc[(int64_t)d * g.Ncc + k];
+        if (NV == 1) nu[d] = nu_from_table(dd[d], cd.thr, cd.vtab, key0, g.nulim);
     }
+    if (NV == 2) nu_codes3(dd, cd.thr, g.nulim, cd.est[0], cd.est[1], nu);
+#pragma unroll
+    for (int d = 0; d < 3; ++d) store_code<NV>(s.nu, d * g.Np + j, nu[d]);
     if (s.id) store_pid(s.id, (unsigned)j, g.nid, id_in ? id_in[i] : (unsigned)i);
 }
 
@@ -889,7 +890,7 @@ __global__ void __launch_bounds__(PA_T, PA_MINB) k_passA(Geo g, StoreDev s, cons
         return;
     }
     const float e0 = cur.est[0], e1 = cur.est[1];
-    // 2-byte codes: the decode and threshold tables through their L1-resident corrections
+    // 2-byte codes: the decode table through its L1-resident corrections
     const VelTables vt = vel_tables<NV>(cur, lim);
     const int nbits = 8 * NX, half = 1 << (nbits - 1);
     const int sb = g.sbits, wmask = (1 << sb) - 1;
@@ -966,17 +967,19 @@ __global__ void __launch_bounds__(PA_T, PA_MINB) k_passA(Geo g, StoreDev s, cons
         // kick (update_vp): the code is decided on v - v_c + F K = offset + F K,
         // re-encoded against the same v_c; then the drift of the in-cell
         // offset Q / 2^(8n+1) by the decoded momentum, rounded once
-        int e[3];
-        float pv[3], un[3];
+        int e[3], nu1[3];
+        float pv[3], un[3], dd[3];
 #pragma unroll
         for (int d = 0; d < 3; ++d) {
-            const float vcd = svc[(d << (3 * lB)) + lc];
-            const float dd = __fmaf_rn(gsum[d], kick12, NV == 1 ? dec[cnu[d] + lim] : vt.dec(cnu[d]));
-            const int nu1 = NV == 1 ? nu_from_table(dd, thr, stab, key0, lim)
-                                    : nu_from_tables(dd, vt, nu_estimate(dd, e0, e1));
-            nu_r.put(d, i, nu1);
-            const float off1 = NV == 1 ? dec[nu1 + lim] : vt.dec(nu1);
-            const float p2 = vcd + off1;
+            dd[d] = __fmaf_rn(gsum[d], kick12, NV == 1 ? dec[cnu[d] + lim] : vt.dec(cnu[d]));
+            if (NV == 1) nu1[d] = nu_from_table(dd[d], thr, stab, key0, lim);
+        }
+        if (NV == 2) nu_codes3(dd, cur.thr, lim, e0, e1, nu1);
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            nu_r.put(d, i, nu1[d]);
+            const float off1 = NV == 1 ? dec[nu1[d] + lim] : vt.dec(nu1[d]);
+            const float p2 = svc[(d << (3 * lB)) + lc] + off1;
             sacc = __fmaf_rn(off1, off1, sacc);
             const int sh1 = drift_bin(Q[d], p2, dcs, &un[d]) >> nbits;
             const int shc = max(-1, min(1, sh1));
@@ -1156,13 +1159,17 @@ struct PassB {
             atomicOr(flags, ERR_COUNT);
             return;
         }
+        float dd[3];
+        int nu[3];
 #pragma unroll
         for (int d = 0; d < 3; ++d) {
             chi_n.put(d, pos, q.chi[d]);
-            const float dd = q.pv[d] - svn[d * H3 + q.ei];
-            nu_n.put(d, pos, NV == 1 ? nu_from_table(dd, thr, stab, key0, lim)
-                                     : nu_from_thresholds(dd, thr, lim, nu_estimate(dd, e0, e1)));
+            dd[d] = q.pv[d] - svn[d * H3 + q.ei];
+            if (NV == 1) nu[d] = nu_from_table(dd[d], thr, stab, key0, lim);
         }
+        if (NV == 2) nu_codes3(dd, thr, lim, e0, e1, nu);
+#pragma unroll
+        for (int d = 0; d < 3; ++d) nu_n.put(d, pos, nu[d]);
         if (sn.id) {
             if (PID == 4) reinterpret_cast<unsigned*>(sn.id)[pos] = cid;
             else store_pid(sn.id, pos, g.nid, cid);
@@ -1521,19 +1528,21 @@ __global__ void k_zero_slot_words(unsigned* p, Batch bt) {
     for (int i = threadIdx.x; i < bt.members; i += blockDim.x) moved(p, slot_member(bt, i) * bt.stride)[0] = 0u;
 }
 
-// every entry of the 2-byte tables as VelTables rebuilds it, against the tables
+// every entry of the 2-byte decode table as VelTables rebuilds it, and the
+// codes of nu_codes3 at and just below every threshold, against the tables
 __global__ void k_check_vel_tables(int lim, CodecDev c, long long* out2) {
-    const VelTables vt{c.dec, c.thr, c.vdel, VelApprox{c.est[3], c.est[4], 2 * lim + 1}, lim};
+    const VelTables vt = vel_tables<2>(c, lim);
     long long bad = 0, whole = 0;
-    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k <= lim + 1; k += gridDim.x * blockDim.x) {
-        if (k <= lim) {
-            bad += __float_as_int(vt.dec(k)) != __float_as_int(c.dec[lim + k]);
-            bad += __float_as_int(vt.dec(-k)) != __float_as_int(c.dec[lim - k]);
-        }
-        bad += __float_as_int(vt.thr(k)) != __float_as_int(c.thr[k]);
-        if (k >= 1 && k <= lim) {
-            const unsigned b = c.vdel[k];
-            whole += (vdelta(b, 0) == -8) + (vdelta(b, 4) == -8);
+    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k <= lim; k += gridDim.x * blockDim.x) {
+        bad += __float_as_int(vt.dec(k)) != __float_as_int(c.dec[lim + k]);
+        bad += k > 0 && __float_as_int(vt.dec(-k)) != __float_as_int(c.dec[lim - k]);
+        whole += c.vdel[k] == -128;
+        if (k > 0) {
+            const float t = c.thr[k], below = __int_as_float(__float_as_int(t) - 1);
+            const float d[3] = {t, -t, below};
+            int nu[3];
+            nu_codes3(d, c.thr, lim, c.est[0], c.est[1], nu);
+            bad += nu[0] != k || nu[1] != -k || nu[2] != k - 1;
         }
     }
     block_sum_to(bad, &out2[0]);
@@ -1597,10 +1606,10 @@ void launch_encode_scatter(const Geo& g, const float* pos, const float* vel, con
                            const unsigned* key_sorted, const unsigned* perm, const float* vc, const CodecDev& c,
                            StoreDev s, cudaStream_t st) {
     int nb = nblk(g.Np, 256);
-    if (g.nchi == 1 && g.nnu == 1) k_encode_scatter<1, 1><<<nb, 256, 0, st>>>(g, pos, vel, id_in, key_sorted, perm, vc, c.thr, c.est, s);
-    else if (g.nchi == 1) k_encode_scatter<1, 2><<<nb, 256, 0, st>>>(g, pos, vel, id_in, key_sorted, perm, vc, c.thr, c.est, s);
-    else if (g.nnu == 1) k_encode_scatter<2, 1><<<nb, 256, 0, st>>>(g, pos, vel, id_in, key_sorted, perm, vc, c.thr, c.est, s);
-    else k_encode_scatter<2, 2><<<nb, 256, 0, st>>>(g, pos, vel, id_in, key_sorted, perm, vc, c.thr, c.est, s);
+    if (g.nchi == 1 && g.nnu == 1) k_encode_scatter<1, 1><<<nb, 256, 0, st>>>(g, pos, vel, id_in, key_sorted, perm, vc, c, s);
+    else if (g.nchi == 1) k_encode_scatter<1, 2><<<nb, 256, 0, st>>>(g, pos, vel, id_in, key_sorted, perm, vc, c, s);
+    else if (g.nnu == 1) k_encode_scatter<2, 1><<<nb, 256, 0, st>>>(g, pos, vel, id_in, key_sorted, perm, vc, c, s);
+    else k_encode_scatter<2, 2><<<nb, 256, 0, st>>>(g, pos, vel, id_in, key_sorted, perm, vc, c, s);
 }
 
 void launch_max_speed(const Geo& g, const StoreDev& s, const CodecDev& c, unsigned* vmax_bits, cudaStream_t st,

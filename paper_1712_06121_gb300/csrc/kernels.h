@@ -105,12 +105,12 @@ struct StoreDev {
 
 struct CodecDev {
     float* dec;         // [2 lim + 1]: dec[nu + lim] = tan(pi nu / M) * sqrt(2 sigma^2 / pi)
-    float* thr;         // [lim + 2]: encode thresholds (see nu_from_thresholds)
-    float* est;         // [8]: s and M/pi for the starting guess; [2] the first bucket key of vtab (int bits);
+    float* thr;         // [lim + 2]: encode thresholds (Eq. nu, cube_common.cuh)
+    float* est;         // [8]: s and M/pi (nu_codes3); [2] the first bucket key of vtab (int bits);
                         // [3], [4]: pi / (2M) and 1 / s of the 2-byte tables' approximation (VelApprox)
     unsigned char* vtab;   // [VT_N] (1-byte codes): code at the start of each bucket of |d| (see nu_from_table)
     double* sigma;      // device scalar
-    unsigned char* vdel;   // [lim + 2] (2-byte codes): corrections of dec and thr to tan_half_steps (VelTables)
+    signed char* vdel;     // [lim + 2] (2-byte codes): corrections of dec to tan_steps (VelTables)
 };
 
 struct DriftDebug {
@@ -180,7 +180,8 @@ void launch_passB(const Geo& g, const StoreDev& s_old, const StoreDev& s_new, co
 // sums over the current store: out[0..2] momentum of the decoded particles in
 // 2^-24 fixed point, out[3] the particle count (sum of the cell counts)
 void launch_store_sums(const Geo& g, const StoreDev& s, const float* dec, long long* out4, cudaStream_t st);
-// 2-byte codes: out2[0] entries of dec / thr that VelTables rebuilds differently, out2[1] entries it reads whole
+// 2-byte codes: out2[0] entries of dec that VelTables rebuilds differently and thresholds that nu_codes3
+// decides differently, out2[1] entries read whole
 void launch_check_vel_tables(int lim, const CodecDev& c, long long* out2, cudaStream_t st);
 
 // uncompressed FP32 particles (k_raw.cu)
