@@ -329,7 +329,8 @@ size_t work_layout(cube_ctx* c, char* base) {
     c->npart = std::max(g.nbricks, 1024);
     carve(base, off, c->part, (size_t)c->npart * 4);
     carve(base, off, c->scan_tmp,
-          (size_t)scan_tmp_words(std::max<int64_t>(g.Ncc + 1, (int64_t)g.nbricks * H3 + 1)) * 4 + 64);
+          (size_t)std::max(scan_tmp_words(std::max<int64_t>(g.Ncc + 1, (int64_t)g.nbricks * H3 + 1)),
+                           step_tmp_words(g)) * 4 + 64);
     c->stage_ws_bytes = c->raw ? 28 * (size_t)g.Np : encode_scratch_bytes(g, true);
     carve(base, off, c->stage_ws, c->stage_ws_bytes);
     return off;
@@ -676,8 +677,10 @@ cube_status cube_encode(cube_ctx* c, const float* pos, const float* vel, const u
     return encode_impl(c, pos, vel, id, a, sigma, true);
 }
 
-// kernels launched per phase of a step (see cube_phase_name)
-const int kPhaseKernels[CUBE_PHASES] = {0, 1, 1, 1, 1, 1, 1, 1, 2, 4, 1, 1};
+// kernels launched per phase of a step (see cube_phase_name): the codec
+// phase's kernel also sums the scan's tiles, the cells phase's kernel scans
+// them and builds the codec tables
+const int kPhaseKernels[CUBE_PHASES] = {0, 1, 1, 1, 1, 1, 1, 1, 1, 0, 1, 1};
 const char* kPhaseNames[CUBE_PHASES] = {"setup", "deposit", "fft_x_r2c", "fft_y_fwd", "fft_z_green", "fft_y_inv",
                                         "fft_x_c2r", "pass_a", "codec", "scan", "cells", "pass_b"};
 
@@ -692,22 +695,24 @@ static void mark(cube_ctx* c, int boundary) {
 static double particle_mass(const Geo& g) { return std::pow((double)g.N, 3) / (double)g.Np; }
 
 // density of the store on a mesh with rows of g.S floats (c->mesh, or any 16-byte aligned rows)
-static void deposit_on(cube_ctx* c, const Geo& g, float* mesh) {
+// step: the scratch of the step this deposit begins, cleared by the way
+static void deposit_on(cube_ctx* c, const Geo& g, float* mesh, const StepScratch* step = nullptr) {
     if (c->raw) {
         cudaMemsetAsync(mesh, 0, (size_t)g.N * g.N * g.S * 4, c->st);
         launch_raw_deposit(g, (const float*)c->chi[0], mesh, (float)particle_mass(g), c->st);
     } else {
-        launch_deposit(g, c->store(c->cur), mesh, particle_mass(g) * std::ldexp(1.0, -3 * g.sbits), c->st);
+        launch_deposit(g, c->store(c->cur), mesh, particle_mass(g) * std::ldexp(1.0, -3 * g.sbits), c->st, kSingle,
+                       step);
     }
     c->launches += 1;
 }
 
-static void deposit(cube_ctx* c) { deposit_on(c, c->g, c->mesh); }
+static void deposit(cube_ctx* c, const StepScratch* step = nullptr) { deposit_on(c, c->g, c->mesh, step); }
 
 // density -> Phi on the mesh; boundaries 1..6 of the step's trace
-static void mesh_potential(cube_ctx* c) {
+static void mesh_potential(cube_ctx* c, const StepScratch* step = nullptr) {
     const Geo& g = c->g;
-    deposit(c);
+    deposit(c, step);
     mark(c, 2);
     fft_x_r2c(c->fft, c->mesh, g.S, c->st);
     mark(c, 3);
@@ -765,26 +770,22 @@ cube_status cube_pm_step(cube_ctx* c, double a_from, double a_to) {
     }
     CK(cudaEventRecord(c->ev0, c->st));
     mark(c, 0);
-    CK(cudaMemsetAsync(c->vsum, 0, (size_t)g.Ncc * 24, c->st));
-    CK(cudaMemsetAsync(c->maxmig, 0, 8, c->st));     // max migration, crowded-brick count
     mark(c, 1);
-    mesh_potential(c);
-    c->phig_valid = true;
     StepScratch w{c->counts[kn], c->vsum, c->ghost, c->part, c->flags, c->maxmig, c->maxmig + 1};
+    mesh_potential(c, &w);
+    c->phig_valid = true;
     DriftDebug dbg{c->keep ? c->dbg_cell : nullptr, c->dbg_u, c->dbg_p, c->dbg_f};
     launch_passA(g, c->store(k), c->phig, c->tma ? &c->phig_map : nullptr, c->codec[k], kick, dc, w, dbg, c->st);
     mark(c, 8);
-    launch_sigma_finalize(c->part, g.nbricks, 3.0 * (double)g.Np, ratio, 0.0, c->codec[kn].sigma, c->st);
-    launch_codec_tables(g.nulim, c->tanv, c->tanh_, c->codec[kn], c->st);
+    launch_step_sums(g, w, ratio, c->codec[kn].sigma, c->scan_tmp, c->st);
     mark(c, 9);
-    exclusive_scan(c->ghost, c->ghost, (int64_t)g.nbricks * (g.Bh * g.Bh * g.Bh), c->scan_tmp, c->st);
     mark(c, 10);
-    launch_cells(g, w, c->offsets[kn], c->vc[kn], c->st);
+    launch_step_cells(g, w, c->offsets[kn], c->vc[kn], c->tanv, c->tanh_, c->codec[kn], c->scan_tmp, c->st);
     mark(c, 11);
     launch_passB(g, c->store(k), c->store(kn), c->codec[k], c->codec[kn], dc, w, c->st);
     mark(c, 12);
     CK(cudaEventRecord(c->ev1, c->st));
-    c->launches += 1 + 2 + 4 + 1 + 1;
+    c->launches += 4;
     if (c->prof_steps < c->prof_max) c->prof_steps += 1;
     CK(cudaGetLastError());
     c->cur = kn;

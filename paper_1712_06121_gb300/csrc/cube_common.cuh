@@ -164,8 +164,12 @@ __device__ __forceinline__ long long vel_fix(float v) {
 // is either an FP32 rounding midpoint or at least 2^-52 (relative) away from
 // every one -- more than FP64's half ulp -- so the FP64 rounding never moves
 // the FP32 result: it is the correctly rounded fl32(s / n * 2^-24), formed
-// here from a 64-bit integer quotient of 26-27 bits and a sticky bit (the
-// FP64 division is very slow on this part).  Larger inputs divide in FP64.
+// here from an integer quotient of 26-27 bits and a sticky bit.  The quotient
+// comes from an FP32 reciprocal: a first guess within 64 of it (a 32-bit
+// window of the numerator, three roundings of 2^-24), the guess's remainder
+// times the reciprocal (within one), one exact correction; FP64 division and
+// 64-bit integer division both cost several times as much on this part.
+// Larger inputs divide in FP64.
 __device__ __forceinline__ float vel_unfix_mean(long long s, unsigned n) {
     if (n == 0 || s == 0) return 0.0f;
     const unsigned long long a = s < 0 ? 0ull - (unsigned long long)s : (unsigned long long)s;
@@ -174,25 +178,33 @@ __device__ __forceinline__ float vel_unfix_mean(long long s, unsigned n) {
         return __double2float_rn(m * (1.0 / 16777216.0));
     }
     const int la = 63 - __clzll((long long)a), ln = 31 - __clz((int)n);
-    const int k = 26 - (la - ln);                      // shift giving a quotient in [2^25, 2^27)
-    unsigned long long q;
-    bool sticky;
-    int e;
-    if (k >= 0) {
-        const unsigned long long num = a << k;         // < 2^53
-        q = num / n;
-        sticky = num - q * n != 0;
-        e = -k;
-    } else {
-        q = a / n;
-        sticky = a - q * n != 0;
-        e = 0;
+    const int k = 26 - (la - ln);                      // the quotient (a 2^k) / n lies in [2^25, 2^27)
+    const unsigned long long num = k >= 0 ? a << k : a;                            // < 2^54
+    const unsigned long long den = k >= 0 ? (unsigned long long)n : (unsigned long long)n << -k;
+    // num / den = (num 2^-sh) / n 2^t: the top 32 bits of num, and n itself
+    const int sh = (k >= 0 ? 26 + ln : la) - 31;
+    const unsigned top = sh >= 0 ? (unsigned)(num >> sh) : (unsigned)(num << -sh);
+    const float rn = __frcp_rn(u32_to_float_rn(n));
+    const int t = k >= 0 ? sh : sh + k;                // -31 < t < 32
+    unsigned q = __float2uint_rz(__fmul_rn(__fmul_rn(u32_to_float_rn(top), rn), __int_as_float((127 + t) << 23)));
+    long long rem = (long long)(num - (unsigned long long)q * den);
+    const int dq = __float2int_rd(__fmul_rn(__fmul_rn(__ll2float_rn(rem), rn),
+                                            __int_as_float((127 + (k >= 0 ? 0 : k)) << 23)));
+    q += (unsigned)dq;
+    rem -= (long long)dq * (long long)den;
+    if (rem < 0) {
+        --q;
+        rem += (long long)den;
+    } else if (rem >= (long long)den) {
+        ++q;
+        rem -= (long long)den;
     }
-    const int t = 64 - __clzll((long long)q) - 24;     // bits below the 24 kept
-    const unsigned long long low = q & ((1ull << t) - 1), half = 1ull << (t - 1);
-    unsigned long long q24 = q >> t;
-    if (low > half || (low == half && (sticky || (q24 & 1)))) ++q24;   // nearest, ties to even
-    const float v = ldexpf((float)q24, e + t - 24);
+    const int drop = 8 - __clz((int)q);                // bits below the 24 kept (2 or 3)
+    const unsigned low = q & ((1u << drop) - 1u), half = 1u << (drop - 1);
+    unsigned q24 = q >> drop;
+    if (low > half || (low == half && (rem != 0 || (q24 & 1u)))) ++q24;    // nearest, ties to even
+    // q24 <= 2^24 is exact, and the result at least 2^-24 2^-27 in size: a normal float
+    const float v = __fmul_rn(u32_to_float_rn(q24), __int_as_float((127 + drop - 24 - k) << 23));
     return s < 0 ? -v : v;
 }
 

@@ -10,35 +10,6 @@ constexpr int SCAN_T = 1024;           // threads per scan block
 constexpr int SCAN_ITEMS = 4;          // items per thread
 constexpr int SCAN_TILE = SCAN_T * SCAN_ITEMS;
 
-// inclusive scan of one value per thread over the block; returns the
-// inclusive prefix, writes the block total to *total
-__device__ unsigned block_inclusive_scan(unsigned v, unsigned* smem_warp, unsigned* total) {
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int nw = blockDim.x >> 5;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        unsigned t = __shfl_up_sync(0xffffffffu, v, o);
-        if (lane >= o) v += t;
-    }
-    if (lane == 31) smem_warp[w] = v;
-    __syncthreads();
-    if (w == 0) {
-        unsigned s = lane < nw ? smem_warp[lane] : 0u;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            unsigned t = __shfl_up_sync(0xffffffffu, s, o);
-            if (lane >= o) s += t;
-        }
-        if (lane < nw) smem_warp[lane] = s;
-    }
-    __syncthreads();
-    unsigned add = w > 0 ? smem_warp[w - 1] : 0u;
-    unsigned tot = smem_warp[nw - 1];
-    __syncthreads();
-    *total = tot;
-    return v + add;
-}
-
 // SCAN_ITEMS = 4 consecutive items of one thread, as one 16-byte load when
 // the array is 16-byte aligned and the four items exist
 __device__ __forceinline__ void load4(const unsigned* __restrict__ in, int64_t base, int64_t n, bool vec,

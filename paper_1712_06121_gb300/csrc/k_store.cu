@@ -227,21 +227,23 @@ __global__ void k_encode_sigma(Geo g, const float* __restrict__ vel, const unsig
     if (threadIdx.x == 0) part[blockIdx.x] = (float)s;
 }
 
-__global__ void k_sigma_finalize(const float* __restrict__ part, int nparts, double count, double ratio,
-                                 double fixed, double* sigma_out, Batch bt) {
+// The codec scale from the partial sums of squared offsets, by a block of 1024
+// threads: strided FP32 sums per thread (coalesced loads, fixed order), then a
+// fixed tree in FP64
+__device__ __forceinline__ void sigma_body(const float* __restrict__ part, int nparts, double count, double ratio,
+                                           double fixed, double* sigma_out) {
     __shared__ double sh[32];
-    const int slot = blockIdx.x;                             // slot of a batch
-    if (bt.ms) {
-        if (!bt.ms[slot].active) return;
-        ratio = bt.ms[slot].ratio;
-    }
-    const int m = slot_member(bt, slot);
-    part = moved(part, m * bt.stride);
-    sigma_out = moved(sigma_out, m * bt.stride);
-    // strided FP32 sums per thread (coalesced loads, fixed order), then a fixed tree in FP64
     float acc = 0.0f;
-#pragma unroll 8
-    for (int i = threadIdx.x; i < nparts; i += blockDim.x) acc += part[i];
+    for (int i = threadIdx.x; i < nparts; i += 16 * blockDim.x) {
+        float v[16];                                     // 16 loads in flight, added in order
+#pragma unroll
+        for (int k = 0; k < 16; ++k) {
+            const int j = i + k * blockDim.x;
+            v[k] = j < nparts ? part[j] : 0.0f;
+        }
+#pragma unroll
+        for (int k = 0; k < 16; ++k) acc += v[k];        // (+ 0 past the end changes nothing: acc >= 0)
+    }
     double s = block_sum_double((double)acc, sh);
     if (threadIdx.x == 0) {
         double x = fixed > 0.0 ? fixed : sqrt(s / count) * ratio;
@@ -249,17 +251,28 @@ __global__ void k_sigma_finalize(const float* __restrict__ part, int nparts, dou
     }
 }
 
+__global__ void k_sigma_finalize(const float* __restrict__ part, int nparts, double count, double ratio,
+                                 double fixed, double* sigma_out, Batch bt) {
+    const int slot = blockIdx.x;                             // slot of a batch
+    if (bt.ms) {
+        if (!bt.ms[slot].active) return;
+        ratio = bt.ms[slot].ratio;
+    }
+    const int m = slot_member(bt, slot);
+    sigma_body(moved(part, m * bt.stride), nparts, count, ratio, fixed, moved(sigma_out, m * bt.stride));
+}
+
 // decode table, thresholds, scale constants and (1-byte codes,
 // single block) the bucket table for the codec scale sg
 __device__ void codec_tables_body(int lim, const double* __restrict__ tanv, const double* __restrict__ tanh_,
                                   double sg, float* __restrict__ dec, float* __restrict__ thr,
                                   float* __restrict__ est, unsigned char* __restrict__ vtab,
-                                  signed char* __restrict__ vdel) {
+                                  signed char* __restrict__ vdel, int block, int nblocks) {
     const double s = sqrt(PI_D / (2.0 * sg * sg));
     const double gam = sqrt(2.0 * sg * sg / PI_D);
     const double m = (double)(2 * lim + 1);
     const VelApprox va{(float)(PI_D / (2.0 * m)), (float)gam, 2 * lim + 1};
-    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k <= lim + 1; k += gridDim.x * blockDim.x) {
+    for (int k = block * blockDim.x + threadIdx.x; k <= lim + 1; k += nblocks * blockDim.x) {
         int ddec = 0;                                    // correction of the 2-byte decode table (vdel)
         if (k == 0) {
             dec[lim] = 0.0f;
@@ -308,7 +321,7 @@ __global__ void k_codec_tables(int lim, const double* __restrict__ tanv, const d
     if (bt.ms && !bt.ms[slot].active) return;
     const size_t o = slot_member(bt, slot) * bt.stride;
     codec_tables_body(lim, moved(tanv, o), moved(tanh_, o), *moved(sigma, o), moved(dec, o), moved(thr, o),
-                      moved(est, o), moved(vtab, o), moved(vdel, o));
+                      moved(est, o), moved(vtab, o), moved(vdel, o), blockIdx.x, gridDim.x);
 }
 
 template <int NX, int NV>
@@ -527,7 +540,7 @@ __host__ __device__ __forceinline__ int dep_acc_words(int F) {
 
 template <int NX, int FC, bool BAT>
 __global__ void __launch_bounds__(T_BRICK) k_deposit(Geo g, StoreDev s, float* __restrict__ mesh, float fscale,
-                                                     Batch bt) {
+                                                     long long* __restrict__ vsum, int* __restrict__ mig, Batch bt) {
     extern __shared__ unsigned long long dep_smem[];
     // FC > 0: the brick side in fine cells is the compile-time FC, else g.F
     const int lF = FC == 16 ? 4 : FC == 8 ? 3 : FC == 4 ? 2 : g.lF, F = 1 << lF, F3 = 1 << (3 * lF);
@@ -591,6 +604,14 @@ __global__ void __launch_bounds__(T_BRICK) k_deposit(Geo g, StoreDev s, float* _
         if (t == 0) cpref[0] = 0;
     }
     __syncthreads();
+    // a step's deposit clears what its pass A accumulates into: the brick's
+    // momentum sums, the largest migration and the number of crowded bricks
+    if (!BAT && vsum) {
+        const int nbc = g.B * g.B * g.B;
+        const int64_t L0 = (int64_t)(bx + g.nb * (by + g.nb * bz)) * nbc;
+        for (int i = t; i < 3 * nbc; i += T_BRICK) vsum[(int64_t)(i >> (3 * g.lB)) * g.Ncc + L0 + (i & (nbc - 1))] = 0;
+        if (blockIdx.x + blockIdx.y + blockIdx.z == 0 && t < 2) mig[t] = 0;
+    }
     const int nbits = 8 * NX, half = 1 << (nbits - 1);
     const int sb = g.sbits, wmask = (1 << sb) - 1, wone = 1 << sb;
     const unsigned total = min(cpref[E3], (unsigned)g.Np);   // bounded even for inconsistent offsets
@@ -1055,35 +1076,174 @@ __global__ void __launch_bounds__(PA_T, PA_MINB) k_passA(Geo g, StoreDev s, cons
 
 // ------------------------------------------------------------------ new cells
 // After the exclusive scan of the flattened histograms, a cell's first slot
-// holds offset*[c] and its slots span counts*[c] particles.  Also
-// v_c* = mean momentum of the cell's new particles (fixed point).
-template <bool BAT>
+// holds offset*[c] and its slots span counts*[c] particles; v_c* = mean
+// momentum of the cell's new particles (fixed point).
+__device__ __forceinline__ void store_cell(const Geo& g, const StepScratch& w, int L, unsigned off, unsigned cnt,
+                                           const long long* vs, unsigned* __restrict__ off_new,
+                                           float* __restrict__ vc_new) {
+    off_new[L] = off;
+    w.counts_new[L] = cnt;
+#pragma unroll
+    for (int d = 0; d < 3; ++d) vc_new[(int64_t)d * g.Ncc + L] = vel_unfix_mean(vs[d], cnt);
+}
+// the end of the offsets, checked against the particle count
+__device__ __forceinline__ void store_total(const Geo& g, const StepScratch& w, unsigned total,
+                                            unsigned* __restrict__ off_new) {
+    off_new[g.Ncc] = total;
+    if (total != (unsigned)g.Np) atomicOr(w.flags, ERR_COUNT);
+}
+
+// the cells of a batch (blockIdx.y its slot)
 __global__ void k_cells(Geo g, StepScratch w, unsigned* __restrict__ off_new, float* __restrict__ vc_new, Batch bt) {
     const int L = blockIdx.x * blockDim.x + threadIdx.x;
     if (L >= g.Ncc) return;
-    if constexpr (BAT) {                                     // slot blockIdx.y of a batch
-        if (bt.ms && !bt.ms[blockIdx.y].active) return;
-        const int m = slot_member(bt, blockIdx.y);
-        w = moved(w, m * bt.stride);
-        off_new = moved(off_new, m * bt.stride);
-        vc_new = moved(vc_new, m * bt.stride);
-    }
-    const int nbc = g.B * g.B * g.B;
-    const int hb = L / nbc, lc = L - hb * nbc;
-    const int l[3] = {lc % g.B, (lc / g.B) % g.B, lc / (g.B * g.B)};
-    const int64_t base = flat_base(g, hb, l);
+    if (bt.ms && !bt.ms[blockIdx.y].active) return;
+    const int m = slot_member(bt, blockIdx.y);
+    w = moved(w, m * bt.stride);
+    off_new = moved(off_new, m * bt.stride);
+    vc_new = moved(vc_new, m * bt.stride);
+    const int lc = L & ((1 << (3 * g.lB)) - 1), bm = g.B - 1;
+    const int l[3] = {lc & bm, (lc >> g.lB) & bm, lc >> (2 * g.lB)};
+    const int64_t base = flat_base(g, L >> (3 * g.lB), l);
     const int n = ncand(l[0], g.B) * ncand(l[1], g.B) * ncand(l[2], g.B);
+    const long long vs[3] = {w.vsum_new[L], w.vsum_new[(int64_t)g.Ncc + L], w.vsum_new[2 * (int64_t)g.Ncc + L]};
     const unsigned off = w.ghost[base];
-    const unsigned cnt = w.ghost[base + n] - off;
-    off_new[L] = off;
-    w.counts_new[L] = cnt;
-    if (L == g.Ncc - 1) {
-        const unsigned total = w.ghost[(int64_t)g.nbricks * (g.Bh * g.Bh * g.Bh)];
-        off_new[g.Ncc] = total;
-        if (total != (unsigned)g.Np) atomicOr(w.flags, ERR_COUNT);
+    store_cell(g, w, L, off, w.ghost[base + n] - off, vs, off_new, vc_new);
+    if (L == g.Ncc - 1) store_total(g, w, w.ghost[(int64_t)g.nbricks * (g.Bh * g.Bh * g.Bh)], off_new);
+}
+
+// A single context's step runs two kernels between its passes, over tiles of
+// whole bricks (16, 64 or 128 of them: at most 4096 histogram slots, eight a
+// thread, and 1024 cells, two a thread): k_step_sums adds each tile's slots up, k_step_cells starts from the
+// sum of the tiles before its own, scans its slots in place and, with the
+// scanned values in shared memory, finishes the cells of its bricks.  The
+// codec rides along: one block of the first kernel finds the next scale, a few
+// blocks of the second build its tables.  Eight launches before (scale,
+// tables, four of the scan, cells, and the clearing of the momentum sums, now
+// in the deposit), each a few microseconds of launch and drain and the cells
+// a second pass over the histograms: per step (with the clearing) 51 us at 32^3
+// particles and 125 us at 256^3 -> 23 and 70 us.
+constexpr int SC_T = 512, SC_ITEMS = 8;
+__host__ __device__ __forceinline__ int tile_bricks(const Geo& g) { return g.B == 4 ? 16 : g.B == 2 ? 64 : 128; }
+__host__ __device__ __forceinline__ int step_tiles(const Geo& g) {
+    return (g.nbricks + tile_bricks(g) - 1) / tile_bricks(g);
+}
+
+// the eight slots of this thread in tile `tile` (zero past the last brick), of *count
+__device__ __forceinline__ void tile_slots(const Geo& g, const unsigned* __restrict__ ghost, int tile, int* count,
+                                           unsigned* v) {
+    const int S3 = g.Bh * g.Bh * g.Bh, tb = tile_bricks(g);
+    const int n = min(tb, g.nbricks - tile * tb) * S3, i = SC_ITEMS * (int)threadIdx.x;
+    const unsigned* p = ghost + (int64_t)tile * tb * S3 + i;     // 16-byte aligned: tb S3 is a multiple of 4
+    *count = n;
+    if (i + SC_ITEMS <= n) {
+        const uint4 a = reinterpret_cast<const uint4*>(p)[0], b = reinterpret_cast<const uint4*>(p)[1];
+        v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
+        v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+    } else {
+#pragma unroll
+        for (int k = 0; k < SC_ITEMS; ++k) v[k] = i + k < n ? p[k] : 0u;
+    }
+}
+
+__global__ void __launch_bounds__(1024) k_step_sums(Geo g, StepScratch w, double ratio, double* sigma_out,
+                                                    unsigned* __restrict__ tsum) {
+    if (blockIdx.x == 0) {
+        sigma_body(w.part, g.nbricks, 3.0 * (double)g.Np, ratio, 0.0, sigma_out);
+        return;
+    }
+    __shared__ unsigned sw[32];
+    // two tiles a block, 512 threads each
+    const int tile = 2 * ((int)blockIdx.x - 1) + ((int)threadIdx.x >= SC_T), t = threadIdx.x & (SC_T - 1);
+    const int S3 = g.Bh * g.Bh * g.Bh, tb = tile_bricks(g);
+    const int n = max(0, min(tb, g.nbricks - tile * tb)) * S3;
+    const unsigned* p = w.ghost + (int64_t)tile * tb * S3;
+    unsigned s = 0;
+    for (int i = 4 * t; i < n; i += 4 * SC_T) {
+        if (i + 3 < n) {
+            const uint4 q = *reinterpret_cast<const uint4*>(p + i);
+            s += q.x + q.y + q.z + q.w;
+        } else {
+            for (int k = i; k < n; ++k) s += p[k];
+        }
+    }
+    s = __reduce_add_sync(0xffffffffu, s);
+    if ((threadIdx.x & 31) == 0) sw[threadIdx.x >> 5] = s;
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        s = sw[threadIdx.x];
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if ((threadIdx.x & 15) == 0) {
+            const int k = 2 * ((int)blockIdx.x - 1) + ((int)threadIdx.x >> 4);
+            if (k < step_tiles(g)) tsum[k] = s;
+        }
+    }
+}
+
+__global__ void __launch_bounds__(SC_T) k_step_cells(Geo g, StepScratch w, const unsigned* __restrict__ tsum,
+                                                     unsigned* __restrict__ off_new, float* __restrict__ vc_new,
+                                                     const double* __restrict__ tanv, const double* __restrict__ tanh_,
+                                                     CodecDev next, int ntab) {
+    if ((int)blockIdx.x < ntab) {                            // the next codec's tables
+        codec_tables_body(g.nulim, tanv, tanh_, *next.sigma, next.dec, next.thr, next.est,
+                          g.nnu == 1 ? next.vtab : nullptr, g.nnu == 1 ? nullptr : next.vdel, blockIdx.x, ntab);
+        return;
+    }
+    __shared__ unsigned sw[32];
+    __shared__ __align__(16) unsigned ex[SC_ITEMS * SC_T + 4];   // the tile's scanned slots and their end
+    const int tile = blockIdx.x - ntab, tb = tile_bricks(g), S3 = g.Bh * g.Bh * g.Bh;
+    const int nbc = 1 << (3 * g.lB), L0 = tile * tb * nbc, bm = g.B - 1;
+    unsigned v[SC_ITEMS];
+    int n;
+    tile_slots(g, w.ghost, tile, &n, v);
+    const int ncell = (n / S3) * nbc;
+    // the momentum sums of this thread's cells (at most two), in flight during the scan
+    long long vs[2][3];
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            const int c = (int)threadIdx.x + h * SC_T;
+            vs[h][d] = c < ncell ? w.vsum_new[(int64_t)d * g.Ncc + L0 + c] : 0;
+        }
+    unsigned before = 0;
+    for (int j = threadIdx.x; j < tile; j += SC_T) before += tsum[j];
+    unsigned s = 0;
+#pragma unroll
+    for (int k = 0; k < SC_ITEMS; ++k) s += v[k];
+    unsigned start, total;
+    block_inclusive_scan(before, sw, &start);
+    unsigned e = start + block_inclusive_scan(s, sw, &total) - s;
+#pragma unroll
+    for (int k = 0; k < SC_ITEMS; ++k) {
+        const unsigned c = v[k];
+        v[k] = e;
+        e += c;
+    }
+    const int i = SC_ITEMS * (int)threadIdx.x;
+    *reinterpret_cast<uint4*>(&ex[i]) = make_uint4(v[0], v[1], v[2], v[3]);
+    *reinterpret_cast<uint4*>(&ex[i + 4]) = make_uint4(v[4], v[5], v[6], v[7]);
+    if (threadIdx.x == 0) ex[SC_ITEMS * SC_T] = start + total;
+    __syncthreads();
+    // coalesced write-back; slots past the last are zero, so ex[n] holds the end as well
+    unsigned* p = w.ghost + (int64_t)tile * tb * S3;
+    for (int k = 4 * (int)threadIdx.x; k < n; k += 4 * SC_T) {
+        if (k + 3 < n) *reinterpret_cast<uint4*>(p + k) = *reinterpret_cast<const uint4*>(&ex[k]);
+        else
+            for (int j = k; j < n; ++j) p[j] = ex[j];
     }
 #pragma unroll
-    for (int d = 0; d < 3; ++d) vc_new[(int64_t)d * g.Ncc + L] = vel_unfix_mean(w.vsum_new[(int64_t)d * g.Ncc + L], cnt);
+    for (int h = 0; h < 2; ++h) {
+        const int c = (int)threadIdx.x + h * SC_T;
+        if (c >= ncell) continue;
+        const int lc = c & (nbc - 1);
+        const int l[3] = {lc & bm, (lc >> g.lB) & bm, lc >> (2 * g.lB)};
+        const int base = (int)flat_base(g, c >> (3 * g.lB), l);
+        const int k = ncand(l[0], g.B) * ncand(l[1], g.B) * ncand(l[2], g.B);
+        store_cell(g, w, L0 + c, ex[base], ex[base + k] - ex[base], vs[h], off_new, vc_new);
+    }
+    if (threadIdx.x == 0 && L0 + ncell == g.Ncc) store_total(g, w, start + total, off_new);
 }
 
 // ------------------------------------------------------------------ pass B
@@ -1644,28 +1804,31 @@ static size_t deposit_smem(const Geo& g) {
     return (size_t)dep_acc_words(g.F) * 4 + (size_t)(3 * E3 + 1) * 4 + DEP_QCAP;
 }
 
-void launch_deposit(const Geo& g, const StoreDev& s, float* mesh, double scale, cudaStream_t st, const Batch& bt) {
+void launch_deposit(const Geo& g, const StoreDev& s, float* mesh, double scale, cudaStream_t st, const Batch& bt,
+                    const StepScratch* step) {
     size_t sm = deposit_smem(g);
     const bool f16 = g.F == 16, bat = bt.members > 1 || bt.ms;
     const dim3 grid(g.nb, g.nb, g.nb * bt.members);
     const float fs = (float)scale;
+    long long* vs = step ? step->vsum_new : nullptr;
+    int* mig = step ? step->maxmig : nullptr;
     if (g.nchi == 1) {
         set_smem_attrs<1, 1>(); set_smem_attrs<1, 2>();
         if (f16) {
-            if (bat) k_deposit<1, 16, true><<<grid, T_BRICK, sm, st>>>(g, s, mesh, fs, bt);
-            else k_deposit<1, 16, false><<<grid, T_BRICK, sm, st>>>(g, s, mesh, fs, bt);
+            if (bat) k_deposit<1, 16, true><<<grid, T_BRICK, sm, st>>>(g, s, mesh, fs, vs, mig, bt);
+            else k_deposit<1, 16, false><<<grid, T_BRICK, sm, st>>>(g, s, mesh, fs, vs, mig, bt);
         } else {
-            if (bat) k_deposit<1, 0, true><<<grid, T_BRICK, sm, st>>>(g, s, mesh, fs, bt);
-            else k_deposit<1, 0, false><<<grid, T_BRICK, sm, st>>>(g, s, mesh, fs, bt);
+            if (bat) k_deposit<1, 0, true><<<grid, T_BRICK, sm, st>>>(g, s, mesh, fs, vs, mig, bt);
+            else k_deposit<1, 0, false><<<grid, T_BRICK, sm, st>>>(g, s, mesh, fs, vs, mig, bt);
         }
     } else {
         set_smem_attrs<2, 1>(); set_smem_attrs<2, 2>();
         if (f16) {
-            if (bat) k_deposit<2, 16, true><<<grid, T_BRICK, sm, st>>>(g, s, mesh, fs, bt);
-            else k_deposit<2, 16, false><<<grid, T_BRICK, sm, st>>>(g, s, mesh, fs, bt);
+            if (bat) k_deposit<2, 16, true><<<grid, T_BRICK, sm, st>>>(g, s, mesh, fs, vs, mig, bt);
+            else k_deposit<2, 16, false><<<grid, T_BRICK, sm, st>>>(g, s, mesh, fs, vs, mig, bt);
         } else {
-            if (bat) k_deposit<2, 0, true><<<grid, T_BRICK, sm, st>>>(g, s, mesh, fs, bt);
-            else k_deposit<2, 0, false><<<grid, T_BRICK, sm, st>>>(g, s, mesh, fs, bt);
+            if (bat) k_deposit<2, 0, true><<<grid, T_BRICK, sm, st>>>(g, s, mesh, fs, vs, mig, bt);
+            else k_deposit<2, 0, false><<<grid, T_BRICK, sm, st>>>(g, s, mesh, fs, vs, mig, bt);
         }
     }
 }
@@ -1694,8 +1857,20 @@ void launch_passA(const Geo& g, const StoreDev& s, const float* phig, const CUte
 
 void launch_cells(const Geo& g, const StepScratch& w, unsigned* off_new, float* vc_new, cudaStream_t st,
                   const Batch& bt) {
-    if (bt.members > 1 || bt.ms) k_cells<true><<<dim3(nblk(g.Ncc, 256), bt.members), 256, 0, st>>>(g, w, off_new, vc_new, bt);
-    else k_cells<false><<<nblk(g.Ncc, 256), 256, 0, st>>>(g, w, off_new, vc_new, bt);
+    k_cells<<<dim3(nblk(g.Ncc, 256), bt.members), 256, 0, st>>>(g, w, off_new, vc_new, bt);
+}
+
+int step_tmp_words(const Geo& g) { return step_tiles(g); }
+
+void launch_step_sums(const Geo& g, const StepScratch& w, double ratio, double* sigma_out, unsigned* tmp,
+                      cudaStream_t st) {
+    k_step_sums<<<1 + (step_tiles(g) + 1) / 2, 1024, 0, st>>>(g, w, ratio, sigma_out, tmp);
+}
+
+void launch_step_cells(const Geo& g, const StepScratch& w, unsigned* off_new, float* vc_new, const double* tanv,
+                       const double* tanh, const CodecDev& next, const unsigned* tmp, cudaStream_t st) {
+    const int ntab = g.nnu == 1 ? 1 : nblk(g.nulim + 2, SC_T);
+    k_step_cells<<<ntab + step_tiles(g), SC_T, 0, st>>>(g, w, tmp, off_new, vc_new, tanv, tanh, next, ntab);
 }
 
 // `words` of a CTA's brick tables after the staged 1-byte codec tables

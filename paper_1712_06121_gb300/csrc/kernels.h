@@ -45,6 +45,35 @@ __device__ __forceinline__ int stable_round_rank(int digit, bool active, unsigne
     return pos;
 }
 
+// inclusive scan of one value per thread over the block; returns the
+// inclusive prefix, writes the block total to *total
+__device__ __forceinline__ unsigned block_inclusive_scan(unsigned v, unsigned* smem_warp, unsigned* total) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int nw = blockDim.x >> 5;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        unsigned t = __shfl_up_sync(0xffffffffu, v, o);
+        if (lane >= o) v += t;
+    }
+    if (lane == 31) smem_warp[w] = v;
+    __syncthreads();
+    if (w == 0) {
+        unsigned s = lane < nw ? smem_warp[lane] : 0u;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            unsigned t = __shfl_up_sync(0xffffffffu, s, o);
+            if (lane >= o) s += t;
+        }
+        if (lane < nw) smem_warp[lane] = s;
+    }
+    __syncthreads();
+    unsigned add = w > 0 ? smem_warp[w - 1] : 0u;
+    unsigned tot = smem_warp[nw - 1];
+    __syncthreads();
+    *total = tot;
+    return v + add;
+}
+
 // ------------------------------------------------------------ batches
 // A batched launch steps several members (simulations with the same
 // geometry) at once: member m's device buffers are member 0's plus m * stride
@@ -163,8 +192,9 @@ void launch_encode_scatter(const Geo& g, const float* pos, const float* vel, con
                            StoreDev s, cudaStream_t st);
 void launch_decode(const Geo& g, const StoreDev& s, const CodecDev& c, float* pos, float* vel, unsigned* id,
                    cudaStream_t st);
+// (step: the step's scratch that pass A accumulates into, cleared by the way, or null)
 void launch_deposit(const Geo& g, const StoreDev& s, float* mesh, double scale, cudaStream_t st,
-                    const Batch& bt = Batch{1, 0, nullptr, nullptr});
+                    const Batch& bt = Batch{1, 0, nullptr, nullptr}, const StepScratch* step = nullptr);
 // phig: ghosted Phi; tmap: TMA map of phig with the brick's tile as its box, or NULL (cp.async loads)
 // (tmap: a 4-D map over (x, y, z, member) of the members' ghosted Phi)
 void launch_passA(const Geo& g, const StoreDev& s, const float* phig, const CUtensorMap* tmap, const CodecDev& cur,
@@ -172,8 +202,17 @@ void launch_passA(const Geo& g, const StoreDev& s, const float* phig, const CUte
                   const Batch& bt = Batch{1, 0, nullptr, nullptr});
 // a batch step's cleared scratch (momentum sums, migration words) of its stepped members
 void launch_batch_clear(const Geo& g, long long* vsum, int* maxmig, cudaStream_t st, const Batch& bt);
+// a single context's kernels between the passes: the histograms' tile sums and
+// the next codec scale, then the scanned histograms, the new cells' counts,
+// offsets and v_c, and the next codec's tables.  tmp: step_tmp_words words
+int step_tmp_words(const Geo& g);
+void launch_step_sums(const Geo& g, const StepScratch& w, double ratio, double* sigma_out, unsigned* tmp,
+                      cudaStream_t st);
+void launch_step_cells(const Geo& g, const StepScratch& w, unsigned* off_new, float* vc_new, const double* tanv,
+                       const double* tanh, const CodecDev& next, const unsigned* tmp, cudaStream_t st);
+// the new cells of a batch, from the scanned histograms
 void launch_cells(const Geo& g, const StepScratch& w, unsigned* off_new, float* vc_new, cudaStream_t st,
-                  const Batch& bt = Batch{1, 0, nullptr, nullptr});
+                  const Batch& bt);
 void launch_passB(const Geo& g, const StoreDev& s_old, const StoreDev& s_new, const CodecDev& cur,
                   const CodecDev& next, float dc, const StepScratch& w, cudaStream_t st,
                   const Batch& bt = Batch{1, 0, nullptr, nullptr});
