@@ -5,15 +5,27 @@
 // (kx = 0..N/2) with complex stride S/2.  Transforms are unnormalised; the
 // 1/N^3 of the inverse is folded into the Green's function.
 //
-// Each kernel transforms one tile of NC = 16 columns of length n in shared
-// memory with a mixed-radix (8, 4, 2, 3) Stockham autosort FFT: every pass
-// reads each element once and writes it once, through registers.
+// Each kernel transforms one tile of 16 columns of length n in shared memory
+// with a mixed-radix (8, 4, 2, 3) Stockham autosort FFT: every pass reads each
+// element once and writes it once, through registers.
 //   x sweep : 16 rows per CTA, r2c / c2r by the even-odd packing into an
-//             N/2-point complex transform (layout [k][row], XOR-swizzled so
+//             N/2-point complex transform (layout [k][row pair], XOR-swizzled so
 //             row-wise and column-wise accesses are both conflict-free)
 //   y sweep : 16 consecutive kx columns of one z-slab
 //   z sweep : 16 consecutive kx columns of one ky line; forward, times
 //             -(3/2) Om / k^2 / W(k)^p / N^3, inverse, in one pass.
+//
+// The sweeps are bound by instruction issue before they are bound by memory,
+// so a thread transforms two columns at once: a tile element is (re, re, im,
+// im) of a column pair, one 16-byte access, and every operation is one packed
+// FP32 instruction on the pair; twiddles (one address and one load for both
+// columns) are staged as (re, re, im, im) too.  Each lane of a packed operation
+// is rounded as the scalar one, and sums of products are written as the fused
+// operations the scalar expressions contract to, so the results are those of
+// one column at a time, bit for bit.  512^3, us, one column a thread with two
+// barriers a pass -> this: x r2c 210 -> 184, y 222 -> 209, z 373 -> 322, inverse
+// y 234 -> 206, c2r 234 -> 227; 384^3: 113 -> 107, 119 -> 92, 180 -> 146, 115 ->
+// 84, 111 -> 108.
 #include <cmath>
 
 #include "kernels.h"
@@ -23,109 +35,165 @@ namespace cube {
 namespace {
 
 constexpr int NC = 16;          // columns per tile
-constexpr int LOG_NC = 4;
-constexpr int FFT_T = 512;      // threads per CTA of the column (y, z) sweeps
-constexpr int XFFT_T = 256;     // threads per CTA of the row (x) sweeps
+constexpr int NP = NC / 2;      // column pairs per tile
+constexpr int LOG_NP = 3;
 
-__device__ __forceinline__ float2 cmul(float2 a, float2 b) {
-    return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
+// Threads of a CTA: one radix-8 butterfly of a column pair each, at least a
+// warp; launch bounds keep 64 registers a thread (1024 threads per SM)
+constexpr int fft_threads(int n) { return n < 32 ? 32 : n > 1024 ? 1024 : n; }
+constexpr int fft_blocks(int n) { return 1024 / fft_threads(n) > 16 ? 16 : 1024 / fft_threads(n); }
+
+// a pair of complex numbers: (re, re), (im, im) of two columns
+struct C2 {
+    float2 x, y;
+};
+__device__ __forceinline__ C2 c2(float4 f) { return C2{make_float2(f.x, f.y), make_float2(f.z, f.w)}; }
+__device__ __forceinline__ float4 pack4(const C2& a) { return make_float4(a.x.x, a.x.y, a.y.x, a.y.y); }
+// two complex numbers in memory order (re0, im0, re1, im1)
+__device__ __forceinline__ C2 from_columns(float4 f) { return C2{make_float2(f.x, f.z), make_float2(f.y, f.w)}; }
+__device__ __forceinline__ float4 to_columns(const C2& a) { return make_float4(a.x.x, a.y.x, a.x.y, a.y.y); }
+__device__ __forceinline__ C2 from_rows(float2 a, float2 b) { return C2{make_float2(a.x, b.x), make_float2(a.y, b.y)}; }
+__device__ __forceinline__ float2 row_of(const C2& a, int r) {
+    return r ? make_float2(a.x.y, a.y.y) : make_float2(a.x.x, a.y.x);
 }
-__device__ __forceinline__ float2 cadd(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
-__device__ __forceinline__ float2 csub(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
-__device__ __forceinline__ float2 cconj(float2 a) { return make_float2(a.x, -a.y); }
-// multiply by -i (forward) or +i (inverse)
+__device__ __forceinline__ C2 cadd(const C2& a, const C2& b) { return C2{padd(a.x, b.x), padd(a.y, b.y)}; }
+__device__ __forceinline__ C2 csub(const C2& a, const C2& b) { return C2{psub(a.x, b.x), psub(a.y, b.y)}; }
+// a + r b and a - r b, r = -i (forward) or +i (inverse)
 template <bool INV>
-__device__ __forceinline__ float2 rot90(float2 a) {
-    return INV ? make_float2(-a.y, a.x) : make_float2(a.y, -a.x);
+__device__ __forceinline__ C2 cadd_rot(const C2& a, const C2& b) {
+    return INV ? C2{psub(a.x, b.y), padd(a.y, b.x)} : C2{padd(a.x, b.y), psub(a.y, b.x)};
+}
+template <bool INV>
+__device__ __forceinline__ C2 csub_rot(const C2& a, const C2& b) {
+    return cadd_rot<!INV>(a, b);
+}
+// f a, each lane by its own factor; scalar products, which nothing fuses
+__device__ __forceinline__ C2 scaled(const C2& a, float2 f) {
+    return C2{make_float2(__fmul_rn(a.x.x, f.x), __fmul_rn(a.x.y, f.y)),
+              make_float2(__fmul_rn(a.y.x, f.x), __fmul_rn(a.y.y, f.y))};
+}
+// a w (forward) or a w* (inverse), w the same for both columns.  One product of
+// each sum is rounded first: of the imaginary part the second, or (YX) the first
+template <bool INV, bool YX = INV>
+__device__ __forceinline__ C2 cmul_tw(const C2& a, float2 w) {
+    const float2 wx = pk2(w.x), wy = pk2(w.y), nwy = pk2(-w.y);
+    const float2 im = YX ? pfma(a.y, wx, pmul(a.x, INV ? nwy : wy)) : pfma(a.x, INV ? nwy : wy, pmul(a.y, wx));
+    return C2{INV ? pfma(a.x, wx, pmul(a.y, wy)) : pfma(a.x, wx, pmul(a.y, nwy)), im};
 }
 
-// Tile layout: element k of column (row) c at k NC + c, or, swizzled (x
-// sweeps), at k NC + (c ^ ((k ^ (k >> 3)) mod NC)).  The swizzle keeps both
-// thread mappings bank-conflict free: one k across the 16 columns, and one
-// column across 16 values of k, whether consecutive or with the strides of
-// the Stockham passes (checked exhaustively for n/2 = 128 ... 512).
+// w a or (CONJ) w* a, the product's terms in the order of a scalar w a
+template <bool CONJ>
+__device__ __forceinline__ C2 cmul_by(float2 w, const C2& a) {
+    const float2 wx = pk2(w.x), wy = pk2(w.y), nwy = pk2(-w.y);
+    return CONJ ? C2{pfma(wx, a.x, pmul(wy, a.y)), pfma(wx, a.y, pmul(nwy, a.x))}
+                : C2{pfma(wx, a.x, pmul(nwy, a.y)), pfma(wx, a.y, pmul(wy, a.x))};
+}
+
+// Tile layout: element k of column (row) pair p at k NP + p, or, swizzled (x
+// sweeps), at k NP + (p ^ ((k ^ (k >> 3)) mod NP)).  A 16-byte access is served
+// eight lanes at a time: eight pairs of one k fill a 128-byte row, and with the
+// swizzle so do eight values of k of one pair, whether consecutive or with the
+// strides of the Stockham passes.
 template <bool SWZ>
-__device__ __forceinline__ int sidx(int k, int c) {
-    return SWZ ? (k << LOG_NC) + (c ^ ((k ^ (k >> 3)) & (NC - 1))) : (k << LOG_NC) + c;
+__device__ __forceinline__ int sidx(int k, int p) {
+    return SWZ ? (k << LOG_NP) + (p ^ ((k ^ (k >> 3)) & (NP - 1))) : (k << LOG_NP) + p;
 }
 
-// sidx(k_lo + k_hi, c) from base = sidx(k_lo, c) when the set bits of the
+// sidx(k_lo + k_hi, p) from base = sidx(k_lo, p) when the set bits of the
 // compile-time k_hi lie above those of k_lo: the swizzle is XOR-linear in k,
 // so the sum is base XOR a constant plus a constant (one logic op and an
 // immediate offset per access)
 template <bool SWZ>
 __device__ __forceinline__ int sidx_add(int base, int k_hi) {
-    return SWZ ? (base ^ ((k_hi ^ (k_hi >> 3)) & (NC - 1))) + (k_hi << LOG_NC) : base + (k_hi << LOG_NC);
+    return SWZ ? (base ^ ((k_hi ^ (k_hi >> 3)) & (NP - 1))) + (k_hi << LOG_NP) : base + (k_hi << LOG_NP);
 }
 
 constexpr bool pow2(int x) { return x > 0 && (x & (x - 1)) == 0; }
 
 template <int RAD, bool INV>
-__device__ __forceinline__ void dft(float2* v) {
+__device__ __forceinline__ void dft(C2* v);
+
+// the radix-4 DFTs of a[m] = x[m] + x[m + 4] and of b[m] w8^m, b[m] = x[m] -
+// x[m + 4], w8 = e^{-+ 2 pi i / 8}: the even and odd outputs of a radix-8 DFT.
+// w8^2 is a rotation, and with w8 b1 = r (u1, w1), w8^3 b3 = r (u3, w3) the
+// sum and difference are formed as r u1 + (r u3) and so on, one rounding
+// after a product.
+template <bool INV>
+__device__ __forceinline__ void dft8_tail(C2* a, const C2* b, C2* v) {
+    const float2 r = pk2(0.70710678118654752f), n = pk2(-0.70710678118654752f);
+    dft<4, INV>(a);
+    const float2 u1 = INV ? psub(b[1].x, b[1].y) : padd(b[1].x, b[1].y);
+    const float2 w1 = INV ? padd(b[1].x, b[1].y) : psub(b[1].y, b[1].x);
+    const float2 u3 = INV ? padd(b[3].x, b[3].y) : psub(b[3].y, b[3].x);    // inverse: -u3
+    const float2 w3 = INV ? psub(b[3].x, b[3].y) : padd(b[3].x, b[3].y);    // forward: -w3
+    const float2 ru = pmul(INV ? n : r, u3), nu = pmul(INV ? r : n, u3);
+    const float2 rw = pmul(INV ? r : n, w3), nw = pmul(INV ? n : r, w3);
+    const C2 s{pfma(r, u1, ru), pfma(r, w1, rw)}, d{pfma(r, u1, nu), pfma(r, w1, nw)};
+    const C2 a0 = cadd_rot<INV>(b[0], b[2]), a1 = csub_rot<INV>(b[0], b[2]);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) v[2 * k] = a[k];
+    v[1] = cadd(a0, s);
+    v[3] = cadd_rot<INV>(a1, d);
+    v[5] = csub(a0, s);
+    v[7] = csub_rot<INV>(a1, d);
+}
+
+template <int RAD, bool INV>
+__device__ __forceinline__ void dft(C2* v) {
     if (RAD == 2) {
-        float2 a = v[0], b = v[1];
+        const C2 a = v[0], b = v[1];
         v[0] = cadd(a, b);
         v[1] = csub(a, b);
     } else if (RAD == 3) {
         const float h = 0.86602540378443865f;   // sqrt(3)/2
-        float2 t1 = cadd(v[1], v[2]);
-        float2 t2 = make_float2(v[0].x - 0.5f * t1.x, v[0].y - 0.5f * t1.y);
-        float2 d = csub(v[1], v[2]);
-        float2 t3 = make_float2(h * d.x, h * d.y);
-        float2 r = rot90<INV>(t3);               // -+ i * t3
+        const C2 t1 = cadd(v[1], v[2]), d = csub(v[1], v[2]);
+        const C2 t2 = C2{pfma(pk2(-0.5f), t1.x, v[0].x), pfma(pk2(-0.5f), t1.y, v[0].y)};
         v[0] = cadd(v[0], t1);
-        v[1] = cadd(t2, r);
-        v[2] = csub(t2, r);
+        // t2 -+ i h d
+        const float2 p = pk2(h), m = pk2(-h);
+        const C2 up = C2{pfma(m, d.y, t2.x), pfma(p, d.x, t2.y)}, dn = C2{pfma(p, d.y, t2.x), pfma(m, d.x, t2.y)};
+        v[1] = INV ? up : dn;
+        v[2] = INV ? dn : up;
     } else if (RAD == 4) {
-        float2 a0 = cadd(v[0], v[2]), a1 = csub(v[0], v[2]);
-        float2 b0 = cadd(v[1], v[3]), b1 = rot90<INV>(csub(v[1], v[3]));
+        const C2 a0 = cadd(v[0], v[2]), a1 = csub(v[0], v[2]);
+        const C2 b0 = cadd(v[1], v[3]), b1 = csub(v[1], v[3]);
         v[0] = cadd(a0, b0);
-        v[1] = cadd(a1, b1);
+        v[1] = cadd_rot<INV>(a1, b1);
         v[2] = csub(a0, b0);
-        v[3] = csub(a1, b1);
+        v[3] = csub_rot<INV>(a1, b1);
     } else {   // 8 = 2 x 4
-        const float r = 0.70710678118654752f;
-        float2 a[4], b[4];
+        C2 a[4], b[4];
 #pragma unroll
         for (int m = 0; m < 4; ++m) {
             a[m] = cadd(v[m], v[m + 4]);
             b[m] = csub(v[m], v[m + 4]);
         }
-        // b[m] *= w8^m,  w8 = e^{-+ 2 pi i / 8}
-        b[1] = INV ? make_float2(r * (b[1].x - b[1].y), r * (b[1].x + b[1].y))
-                   : make_float2(r * (b[1].x + b[1].y), r * (b[1].y - b[1].x));
-        b[2] = rot90<INV>(b[2]);
-        b[3] = INV ? make_float2(-r * (b[3].x + b[3].y), r * (b[3].x - b[3].y))
-                   : make_float2(r * (b[3].y - b[3].x), -r * (b[3].x + b[3].y));
-        dft<4, INV>(a);
-        dft<4, INV>(b);
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            v[2 * k] = a[k];
-            v[2 * k + 1] = b[k];
-        }
+        dft8_tail<INV>(a, b, v);
     }
 }
 
-// one Stockham pass of radix R over the NC-column tile of length n, span Ns;
-// twiddles come from a table of TWN = n * TWM entries e^{-2 pi i k / TWN}
-template <int n, int Ns, int R, int TWM, bool INV, bool SWZ, int T = FFT_T>
-__device__ __forceinline__ void fft_pass(float2* buf, const float2* tw) {
+// the radices 8, 4, 2, 3 taken greedily
+constexpr int radix_of(int rem) { return rem % 8 == 0 ? 8 : rem % 4 == 0 ? 4 : rem % 2 == 0 ? 2 : 3; }
+
+// one Stockham pass of radix R over the tile of length n, span Ns; twiddles
+// come from a table of TWN = n * TWM entries e^{-2 pi i k / TWN}
+template <int n, int Ns, int R, int TWM, bool INV, bool SWZ, int T>
+__device__ __forceinline__ void fft_pass(float4* buf, const float2* tw) {
     constexpr int nq = n / R;
-    constexpr int nbf = nq * NC;
+    constexpr int nbf = nq * NP;
     constexpr int KMAX = (nbf + T - 1) / T;
     constexpr int step = TWM * (n / (Ns * R));
     constexpr bool lin = pow2(nq) && pow2(Ns) && pow2(R);   // bit-disjoint element offsets
-    float2 v[KMAX][R];
+    C2 v[KMAX][R];
 #pragma unroll
     for (int q = 0; q < KMAX; ++q) {
         const int b = threadIdx.x + q * T;
         if (nbf % T == 0 || b < nbf) {
-            const int c = b & (NC - 1), j = b >> LOG_NC;
-            const int base = sidx<SWZ>(j, c);
+            const int p = b & (NP - 1), j = b >> LOG_NP;
+            const int base = sidx<SWZ>(j, p);
 #pragma unroll
             for (int m = 0; m < R; ++m)
-                v[q][m] = buf[lin ? sidx_add<SWZ>(base, m * nq) : sidx<SWZ>(j + m * nq, c)];
+                v[q][m] = c2(buf[lin ? sidx_add<SWZ>(base, m * nq) : sidx<SWZ>(j + m * nq, p)]);
         }
     }
     __syncthreads();
@@ -133,320 +201,285 @@ __device__ __forceinline__ void fft_pass(float2* buf, const float2* tw) {
     for (int q = 0; q < KMAX; ++q) {
         const int b = threadIdx.x + q * T;
         if (nbf % T == 0 || b < nbf) {
-            const int c = b & (NC - 1), j = b >> LOG_NC;
+            const int p = b & (NP - 1), j = b >> LOG_NP;
             const int k = j % Ns;
             if (Ns > 1) {                                  // span 1: all twiddles are 1
 #pragma unroll
-                for (int m = 1; m < R; ++m) {
-                    float2 w = tw[k * m * step];
-                    if (INV) w.y = -w.y;
-                    v[q][m] = cmul(v[q][m], w);
-                }
+                for (int m = 1; m < R; ++m) v[q][m] = cmul_tw<INV>(v[q][m], tw[k * m * step]);
             }
             dft<R, INV>(v[q]);
             const int idxD = (j / Ns) * Ns * R + k;
-            const int base = sidx<SWZ>(idxD, c);
+            const int base = sidx<SWZ>(idxD, p);
 #pragma unroll
             for (int m = 0; m < R; ++m)
-                buf[lin ? sidx_add<SWZ>(base, m * Ns) : sidx<SWZ>(idxD + m * Ns, c)] = v[q][m];
+                buf[lin ? sidx_add<SWZ>(base, m * Ns) : sidx<SWZ>(idxD + m * Ns, p)] = pack4(v[q][m]);
         }
     }
     __syncthreads();
 }
 
-// all passes of a length-n transform, radices 8, 4, 2, 3 taken greedily
-template <int n, int Ns, int TWM, bool INV, bool SWZ, int T = FFT_T>
-__device__ __forceinline__ void tile_fft(float2* buf, const float2* tw) {
+// all passes from span Ns on
+template <int n, int Ns, int TWM, bool INV, bool SWZ, int T>
+__device__ __forceinline__ void tile_fft(float4* buf, const float2* tw) {
     if constexpr (Ns < n) {
-        constexpr int rem = n / Ns;
-        constexpr int R = rem % 8 == 0 ? 8 : rem % 4 == 0 ? 4 : rem % 2 == 0 ? 2 : 3;
-        static_assert(rem % R == 0, "length must be 2^a 3^b");
+        constexpr int R = radix_of(n / Ns);
+        static_assert((n / Ns) % R == 0, "length must be 2^a 3^b");
         fft_pass<n, Ns, R, TWM, INV, SWZ, T>(buf, tw);
         tile_fft<n, Ns * R, TWM, INV, SWZ, T>(buf, tw);
     }
 }
 
-// First pass (span 1, no twiddles) of a column tile straight from global
-// memory: column c of element j + m n/R is src[(j + m n/R) rs + (c0 + c) cs],
-// zero at or past column ncol.  pack_off > 0: column 0 of the tile (c0 = 0)
-// becomes X + i Y, X its own values and Y those of the column pack_off
-// further (two real sequences in one complex transform).  The caller's
-// cp.async copies (twiddles, tables) are waited for before the closing
-// barrier.
-// UNR = 1 keeps one butterfly's loads in flight per thread (fewer
-// registers); UNR = KMAX issues all of them first (more loads in flight)
-template <int n, int R, bool INV, int UNR = 1>
-__device__ __forceinline__ void fft_pass_load(float2* buf, const float2* __restrict__ src, int64_t rs, int c0,
-                                              int ncol, int64_t cs = 1, int pack_off = 0) {
-    constexpr int nq = n / R;
-    constexpr int nbf = nq * NC;
-    constexpr int KMAX = (nbf + FFT_T - 1) / FFT_T;
-#pragma unroll UNR
-    for (int q = 0; q < KMAX; ++q) {
-        const int b = threadIdx.x + q * FFT_T;
-        if (nbf % FFT_T == 0 || b < nbf) {
-            const int c = b & (NC - 1), j = b >> LOG_NC;
-            const bool ok = c0 + c < ncol;
-            const float2* p = src + (int64_t)j * rs + (int64_t)(c0 + c) * cs;
-            float2 v[R];
-#pragma unroll
-            for (int m = 0; m < R; ++m) v[m] = ok ? p[(int64_t)m * nq * rs] : make_float2(0.f, 0.f);
-            if (pack_off > 0 && c0 + c == 0)
-#pragma unroll
-                for (int m = 0; m < R; ++m) {
-                    const float2 y = p[(int64_t)m * nq * rs + pack_off];
-                    v[m] = make_float2(v[m].x - y.y, v[m].y + y.x);
-                }
-            dft<R, INV>(v);
-#pragma unroll
-            for (int m = 0; m < R; ++m) buf[sidx<false>(j * R + m, c)] = v[m];
-        }
-    }
-    cp_async_wait_all();
-    __syncthreads();
-}
-
-// Last pass of a column tile: results (natural order, element j + m Ns) go
-// straight to dst[(j + m Ns) rs + (c0 + c) cs] for columns below ncol, each
-// first passed through post(element, column, value).  split_off > 0: column
-// 0 of the tile (c0 = 0) holds x + i y of two real sequences; x goes to
-// column 0 and y to the column split_off further, both as (value, 0).
-// Shared memory is only read: the caller synchronises before reusing it.
-template <int n, int Ns, int R, int TWM, bool INV, class Post, int UNR = 1>
-__device__ __forceinline__ void fft_pass_store(const float2* buf, const float2* tw, float2* dst, int64_t rs, int c0,
-                                               int ncol, Post post, int64_t cs = 1, int split_off = 0) {
-    constexpr int nq = n / R;
-    static_assert(nq == Ns, "the last pass has span n / R");
-    constexpr int nbf = nq * NC;
-    constexpr int KMAX = (nbf + FFT_T - 1) / FFT_T;
-    constexpr int step = TWM * (n / (Ns * R));
-#pragma unroll UNR
-    for (int q = 0; q < KMAX; ++q) {
-        const int b = threadIdx.x + q * FFT_T;
-        if (nbf % FFT_T == 0 || b < nbf) {
-            const int c = b & (NC - 1), j = b >> LOG_NC;
-            float2 v[R];
-#pragma unroll
-            for (int m = 0; m < R; ++m) v[m] = buf[sidx<false>(j + m * nq, c)];
-            if (Ns > 1) {
-#pragma unroll
-                for (int m = 1; m < R; ++m) {
-                    float2 w = tw[j * m * step];
-                    if (INV) w.y = -w.y;
-                    v[m] = cmul(v[m], w);
-                }
-            }
-            dft<R, INV>(v);
-            if (split_off > 0 && c0 + c == 0) {
-                float2* p = dst + (int64_t)j * rs;
-#pragma unroll
-                for (int m = 0; m < R; ++m) {
-                    p[(int64_t)m * Ns * rs] = make_float2(v[m].x, 0.f);
-                    p[(int64_t)m * Ns * rs + split_off] = make_float2(v[m].y, 0.f);
-                }
-            } else if (c0 + c < ncol) {
-                float2* p = dst + (int64_t)j * rs + (int64_t)(c0 + c) * cs;
-#pragma unroll
-                for (int m = 0; m < R; ++m) p[(int64_t)m * Ns * rs] = post(j + m * Ns, c, v[m]);
-            }
-        }
-    }
-}
-
-struct NoPost {
-    __device__ __forceinline__ float2 operator()(int, int, float2 v) const { return v; }
-};
-
-// passes from span Ns on, the last one through fft_pass_store
-template <int n, int Ns, int TWM, bool INV, class Post, int UNR = 1>
-__device__ __forceinline__ void tile_fft_to_global(float2* buf, const float2* tw, float2* dst, int64_t rs, int c0,
-                                                   int ncol, Post post, int64_t cs = 1, int split_off = 0) {
-    constexpr int rem = n / Ns;
-    constexpr int R = rem % 8 == 0 ? 8 : rem % 4 == 0 ? 4 : rem % 2 == 0 ? 2 : 3;
-    static_assert(rem % R == 0, "length must be 2^a 3^b");
-    if constexpr (Ns * R == n) {
-        fft_pass_store<n, Ns, R, TWM, INV, Post, UNR>(buf, tw, dst, rs, c0, ncol, post, cs, split_off);
-    } else {
-        fft_pass<n, Ns, R, TWM, INV, false>(buf, tw);
-        tile_fft_to_global<n, Ns * R, TWM, INV, Post, UNR>(buf, tw, dst, rs, c0, ncol, post, cs, split_off);
-    }
-}
-
-// passes from span Ns up to (not including) the last, in shared memory
-template <int n, int Ns, int TWM, bool INV, bool SWZ = false, int T = FFT_T>
-__device__ __forceinline__ void tile_fft_but_last(float2* buf, const float2* tw) {
-    constexpr int rem = n / Ns;
-    constexpr int R = rem % 8 == 0 ? 8 : rem % 4 == 0 ? 4 : rem % 2 == 0 ? 2 : 3;
+// passes from span Ns up to (not including) the last
+template <int n, int Ns, int TWM, bool INV, bool SWZ, int T>
+__device__ __forceinline__ void tile_fft_but_last(float4* buf, const float2* tw) {
+    constexpr int R = radix_of(n / Ns);
     if constexpr (Ns * R < n) {
         fft_pass<n, Ns, R, TWM, INV, SWZ, T>(buf, tw);
         tile_fft_but_last<n, Ns * R, TWM, INV, SWZ, T>(buf, tw);
     }
 }
 
-template <int n>
-constexpr int first_radix() {
-    return n % 8 == 0 ? 8 : n % 4 == 0 ? 4 : n % 2 == 0 ? 2 : 3;
+template <int n, int ns0 = 1>
+constexpr int last_span() {   // span of the last pass of tile_fft<n, ns0, ...>
+    int ns = ns0;
+    while (ns * radix_of(n / ns) != n) ns *= radix_of(n / ns);
+    return ns;
+}
+
+// ---- column tiles, in place
+// A pass's butterfly writes its results where it read its inputs, so passes
+// are separated by one barrier and hold nothing across it.  With radices R_1 ..
+// R_q (P_i = R_1 .. R_i), pass i turns digit d_i of the input index
+// sum d_l n / P_l into digit k_i of the output index sum k_l P_{l-1}, at the
+// slot whose digits are the k's done and the d's to do.  Forward transforms
+// weigh digit l by P_{l-1} (the output ends in natural order), inverse ones by
+// n / P_l (the input begins in natural order).  A slot is a 128-byte row of 8
+// pairs, so every order of the butterflies is free of bank conflicts; those of
+// one twiddle are neighbours.
+constexpr int rad(int n, int i) {                // R_i
+    for (int l = 1; l < i; ++l) n /= radix_of(n);
+    return radix_of(n);
+}
+constexpr int pre(int n, int i) {                // P_i
+    int p = 1;
+    for (int l = 1; l <= i; ++l) p *= rad(n, l);
+    return p;
+}
+constexpr int npass(int n) {
+    int q = 0;
+    for (int m = n; m > 1; m /= radix_of(m)) ++q;
+    return q;
+}
+// sum_{l = 1 .. I} k_l n / P_l of kk = sum k_l P_{l-1}
+template <int n, int I>
+__device__ __forceinline__ int rev_k(int kk) {
+    if constexpr (I == 0) return 0;
+    else return rev_k<n, I - 1>(kk) + (kk / pre(n, I - 1)) % rad(n, I) * (n / pre(n, I));
+}
+// sum_{l = 2 .. I} d_l P_{l-1} of j = sum_{l >= 2} d_l n / P_l
+template <int n, int I>
+__device__ __forceinline__ int rev_d(int j) {
+    if constexpr (I <= 1) return 0;
+    else return rev_d<n, I - 1>(j) + (j / (n / pre(n, I))) % rad(n, I) * pre(n, I - 1);
+}
+// slot of butterfly j's input 0 in pass I, and the distance to the next
+template <int n, int I, bool INV>
+__device__ __forceinline__ int slot0(int kk, int dd) {
+    return INV ? rev_k<n, I - 1>(kk) + dd : kk + pre(n, I) * dd;
+}
+template <int n, int I, bool INV>
+constexpr int slot_step() {
+    return INV ? n / pre(n, I) : pre(n, I - 1);
+}
+
+// runs fn(pair, butterfly) over the tile's butterflies of radix R
+template <int n, int R, int T, class Fn>
+__device__ __forceinline__ void for_butterflies(Fn fn) {
+    constexpr int nbf = n / R * NP;
+#pragma unroll
+    for (int b0 = 0; b0 < nbf; b0 += T) {
+        const int b = b0 + threadIdx.x;
+        if (nbf % T == 0 || b < nbf) fn(b & (NP - 1), b >> LOG_NP);
+    }
+}
+
+// inputs of butterfly (kk, dd) of pass I, times their twiddles, transformed
+template <int n, int I, bool INV, bool YX = INV>
+__device__ __forceinline__ void butterfly(const float4* buf, const float2* tw, int p, int kk, int dd, C2* v) {
+    constexpr int R = rad(n, I), step = n / pre(n, I);
+    const float4* s = buf + (slot0<n, I, INV>(kk, dd) << LOG_NP) + p;
+#pragma unroll
+    for (int m = 0; m < R; ++m) v[m] = c2(s[(m * slot_step<n, I, INV>()) << LOG_NP]);
+    if (I > 1) {                                           // pass 1: all twiddles are 1
+#pragma unroll
+        for (int m = 1; m < R; ++m) v[m] = cmul_tw<INV, YX>(v[m], tw[kk * m * step]);
+    }
+}
+
+// pass I in shared memory
+template <int n, int I, bool INV, int T>
+__device__ __forceinline__ void col_pass(float4* buf, const float2* tw) {
+    constexpr int R = rad(n, I), D = n / pre(n, I);
+    for_butterflies<n, R, T>([&](int p, int j) {
+        const int kk = j / D, dd = j % D;
+        C2 v[R];
+        butterfly<n, I, INV>(buf, tw, p, kk, dd, v);
+        dft<R, INV>(v);
+        float4* s = buf + (slot0<n, I, INV>(kk, dd) << LOG_NP) + p;
+#pragma unroll
+        for (int m = 0; m < R; ++m) s[(m * slot_step<n, I, INV>()) << LOG_NP] = pack4(v[m]);
+    });
+    __syncthreads();
+}
+// passes I .. L
+template <int n, int I, int L, bool INV, int T>
+__device__ __forceinline__ void col_passes(float4* buf, const float2* tw) {
+    if constexpr (I <= L) {
+        col_pass<n, I, INV, T>(buf, tw);
+        col_passes<n, I + 1, L, INV, T>(buf, tw);
+    }
+}
+
+// First pass (no twiddles) of a column tile straight from global memory:
+// element r of the pair of columns c0 + 2 p, + 1 is the 16 bytes at
+// src[r rs + c0 + 2 p], zero when the pair starts at or past column ncol (a last
+// column without a partner is paired with the row's padding slot, whose values
+// go nowhere).  pack_off > 0: column 0 of the tile (c0 = 0) becomes X + i Y, X
+// its own values and Y those of the column pack_off further (two real
+// sequences in one complex transform).  Ends with a barrier.
+template <int n, bool INV, int T>
+__device__ __forceinline__ void col_load(float4* buf, const float2* __restrict__ src, int64_t rs, int c0, int ncol,
+                                         int pack_off = 0) {
+    constexpr int R = rad(n, 1), nq = n / R;
+    for_butterflies<n, R, T>([&](int p, int j) {
+        const bool ok = c0 + 2 * p < ncol;
+        const float2* s = src + (int64_t)j * rs + c0 + 2 * p;
+        float4 f[R];
+#pragma unroll
+        for (int m = 0; m < R; ++m)
+            f[m] = ok ? *reinterpret_cast<const float4*>(s + (int64_t)m * nq * rs) : make_float4(0.f, 0.f, 0.f, 0.f);
+        if (pack_off > 0 && c0 + p == 0)
+#pragma unroll
+            for (int m = 0; m < R; ++m) {
+                const float2 y = s[(int64_t)m * nq * rs + pack_off];
+                f[m].x -= y.y;
+                f[m].y += y.x;
+            }
+        C2 v[R];
+#pragma unroll
+        for (int m = 0; m < R; ++m) v[m] = from_columns(f[m]);
+        dft<R, INV>(v);
+        float4* d = buf + ((INV ? j : rev_d<n, npass(n)>(j)) << LOG_NP) + p;
+#pragma unroll
+        for (int m = 0; m < R; ++m) d[(m * slot_step<n, 1, INV>()) << LOG_NP] = pack4(v[m]);
+    });
+    __syncthreads();
+}
+
+// Last pass of a column tile: results go straight to dst[k rs + c0 + 2 p] for
+// pairs starting below ncol.  split_off > 0: column 0 of the tile (c0 = 0) holds
+// x + i y of two real sequences; x goes to column 0 and y to the column
+// split_off further, both as (value, 0).
+template <int n, bool INV, int T>
+__device__ __forceinline__ void col_store(const float4* buf, const float2* tw, float2* dst, int64_t rs, int c0,
+                                          int ncol, int split_off = 0) {
+    constexpr int q = npass(n), R = rad(n, q), nq = n / R;
+    for_butterflies<n, R, T>([&](int p, int j) {
+        C2 v[R];
+        butterfly<n, q, INV>(buf, tw, p, j, 0, v);
+        dft<R, INV>(v);
+        float2* d = dst + (int64_t)j * rs + c0 + 2 * p;
+        if (split_off > 0 && c0 + p == 0) {
+#pragma unroll
+            for (int m = 0; m < R; ++m) {
+                *reinterpret_cast<float4*>(d + (int64_t)m * nq * rs) = make_float4(v[m].x.x, 0.f, v[m].x.y, v[m].y.y);
+                d[(int64_t)m * nq * rs + split_off] = make_float2(v[m].y.x, 0.f);
+            }
+        } else if (c0 + 2 * p < ncol) {
+#pragma unroll
+            for (int m = 0; m < R; ++m) *reinterpret_cast<float4*>(d + (int64_t)m * nq * rs) = to_columns(v[m]);
+        }
+    });
+}
+
+// The last forward pass, times post(element, pair) (the Green's function), in
+// place (natural order).  Where the last forward and the first inverse pass
+// have the same radix (8), both act on the same elements: FUSE runs the first
+// inverse pass before the results are written.
+template <int n, bool FUSE, int T, class Post>
+__device__ __forceinline__ void col_pass_post(float4* buf, const float2* tw, Post post) {
+    constexpr int q = npass(n), R = rad(n, q), nq = n / R;
+    static_assert(!FUSE || R == rad(n, 1), "one radix");
+    for_butterflies<n, R, T>([&](int p, int j) {
+        C2 v[R];
+        butterfly<n, q, false, FUSE>(buf, tw, p, j, 0, v);
+        dft<R, false>(v);
+#pragma unroll
+        for (int m = 0; m < R; ++m) v[m] = scaled(v[m], post(j + m * nq, p));
+        if (FUSE) dft<R, true>(v);
+        float4* s = buf + (j << LOG_NP) + p;
+#pragma unroll
+        for (int m = 0; m < R; ++m) s[(m * nq) << LOG_NP] = pack4(v[m]);
+    });
+    __syncthreads();
 }
 
 // first radix of the row transforms: never the whole length, so that the
 // first (load) and last (store) passes are distinct
 template <int n>
 constexpr int x_first_radix() {
-    return first_radix<n>() < n ? first_radix<n>() : (n % 4 == 0 && n > 4 ? 4 : 2);
+    return radix_of(n) < n ? radix_of(n) : (n % 4 == 0 && n > 4 ? 4 : 2);
 }
 
-template <int n, int ns0 = 1>
-constexpr int last_span() {   // span of the last pass of tile_fft<n, ns0, ...>
-    int ns = ns0;
-    while (true) {
-        const int rem = n / ns;
-        const int r = rem % 8 == 0 ? 8 : rem % 4 == 0 ? 4 : rem % 2 == 0 ? 2 : 3;
-        if (ns * r == n) return ns;
-        ns *= r;
-    }
-}
-
-// last pass in shared memory, each result passed through post(element, column, value)
-template <int n, int Ns, int R, int TWM, bool INV, class Post>
-__device__ __forceinline__ void fft_pass_post(float2* buf, const float2* tw, Post post) {
-    constexpr int nq = n / R;
-    constexpr int nbf = nq * NC;
-    constexpr int KMAX = (nbf + FFT_T - 1) / FFT_T;
-    constexpr int step = TWM * (n / (Ns * R));
-    float2 v[KMAX][R];
+// twiddle table into shared memory; the tile's first barrier publishes it
+template <int N, int T>
+__device__ __forceinline__ void load_tw(float2* stw, const float2* __restrict__ tw) {
 #pragma unroll
-    for (int q = 0; q < KMAX; ++q) {
-        const int b = threadIdx.x + q * FFT_T;
-        if (nbf % FFT_T == 0 || b < nbf) {
-            const int c = b & (NC - 1), j = b >> LOG_NC;
-#pragma unroll
-            for (int m = 0; m < R; ++m) v[q][m] = buf[sidx<false>(j + m * nq, c)];
-        }
-    }
-    __syncthreads();
-#pragma unroll
-    for (int q = 0; q < KMAX; ++q) {
-        const int b = threadIdx.x + q * FFT_T;
-        if (nbf % FFT_T == 0 || b < nbf) {
-            const int c = b & (NC - 1), j = b >> LOG_NC;
-            if (Ns > 1) {
-#pragma unroll
-                for (int m = 1; m < R; ++m) {
-                    float2 w = tw[j * m * step];
-                    if (INV) w.y = -w.y;
-                    v[q][m] = cmul(v[q][m], w);
-                }
-            }
-            dft<R, INV>(v[q]);
-#pragma unroll
-            for (int m = 0; m < R; ++m) buf[sidx<false>(j + m * Ns, c)] = post(j + m * Ns, c, v[q][m]);
-        }
-    }
-    __syncthreads();
-}
-
-// The last forward pass (span n / R) and the first inverse pass (span 1)
-// of the same radix R touch the same R elements per thread (j + m n/R), so
-// they run back to back in registers: forward pass, post(element, column,
-// value) (the Green's function), inverse radix-R DFT, written where the
-// inverse first pass writes (j R + m).
-template <int n, int Ns, int R, int TWM, class Post>
-__device__ __forceinline__ void fft_pass_fwd_post_inv(float2* buf, const float2* tw, Post post) {
-    constexpr int nq = n / R;
-    static_assert(nq == Ns, "the last forward pass has span n / R");
-    constexpr int nbf = nq * NC;
-    constexpr int KMAX = (nbf + FFT_T - 1) / FFT_T;
-    constexpr int step = TWM * (n / (Ns * R));
-    float2 v[KMAX][R];
-#pragma unroll
-    for (int q = 0; q < KMAX; ++q) {
-        const int b = threadIdx.x + q * FFT_T;
-        if (nbf % FFT_T == 0 || b < nbf) {
-            const int c = b & (NC - 1), j = b >> LOG_NC;
-#pragma unroll
-            for (int m = 0; m < R; ++m) v[q][m] = buf[sidx<false>(j + m * nq, c)];
-        }
-    }
-    __syncthreads();
-#pragma unroll
-    for (int q = 0; q < KMAX; ++q) {
-        const int b = threadIdx.x + q * FFT_T;
-        if (nbf % FFT_T == 0 || b < nbf) {
-            const int c = b & (NC - 1), j = b >> LOG_NC;
-#pragma unroll
-            for (int m = 1; m < R; ++m) v[q][m] = cmul(v[q][m], tw[j * m * step]);
-            dft<R, false>(v[q]);
-#pragma unroll
-            for (int m = 0; m < R; ++m) v[q][m] = post(j + m * Ns, c, v[q][m]);
-            dft<R, true>(v[q]);
-#pragma unroll
-            for (int m = 0; m < R; ++m) buf[sidx<false>(j * R + m, c)] = v[q][m];
-        }
-    }
-    __syncthreads();
-}
-
-// twiddle table into shared memory (asynchronous; waited for with the tile)
-__device__ __forceinline__ void load_tw(float2* stw, const float2* tw, int N) {
-    for (int i = threadIdx.x; i < N; i += blockDim.x) cp_async8(&stw[i], &tw[i]);
-}
-
-// NC-column tile of rows 0..n-1 (row stride `rs` complex) into buf[row][NC]:
-// 16-byte copies of column pairs; pairs starting at or past `ncol` are zeroed
-// instead of read (the second column of the last pair may be the row's
-// padding slot, which exists in memory and is never written back)
-__device__ __forceinline__ void load_columns(float2* buf, const float2* src, int n, int64_t rs, int c0, int ncol) {
-    for (int q = threadIdx.x; q < n * (NC / 2); q += blockDim.x) {
-        const int r = q / (NC / 2), cp = 2 * (q % (NC / 2));
-        float2* d = &buf[(r << LOG_NC) + cp];
-        if (c0 + cp < ncol) cp_async16(d, src + r * rs + c0 + cp);
-        else d[0] = d[1] = make_float2(0.f, 0.f);
-    }
+    for (int i = threadIdx.x; i < N; i += T) stw[i] = __ldg(&tw[i]);
 }
 
 // ------------------------------------------------------------ x sweeps
-// NC = 16 rows per CTA.  The first and last passes run with threads along
-// the row (j fastest), so they read and write global memory in coalesced
-// runs; the middle passes run across the 16 rows.
+// NC = 16 rows per CTA, two a thread.  The first and last passes run with
+// threads along the row (j fastest), so they read and write global memory in
+// coalesced runs; the middle passes run across the 8 row pairs.
 
 // First pass (span 1) of the n = N/2-point transforms of rows row0 .. row0 +
 // NC - 1, straight from global memory.  PACK (c2r): the input row holds the
 // half spectrum X[0 .. n] and the transform input is Z[k] = E + i O with
 // E = X[k] + X*[n-k], O = W^-k (X[k] - X*[n-k]), W = e^{-2 pi i / N} (twiddles
 // read from global memory: the shared copy may still be in flight).
-template <int n, int R, bool INV, bool PACK>
-__device__ __forceinline__ void xpass_load(float2* buf, const float* mesh, int64_t row0, int S,
+template <int n, int R, bool INV, bool PACK, int T>
+__device__ __forceinline__ void xpass_load(float4* buf, const float* mesh, int64_t row0, int S,
                                            const float2* __restrict__ gtw) {
     constexpr int nq = n / R;
-    constexpr int nbf = nq * NC;
-    constexpr int KMAX = (nbf + XFFT_T - 1) / XFFT_T;
+    constexpr int nbf = nq * NP;
+    constexpr int KMAX = (nbf + T - 1) / T;
 #pragma unroll
     for (int q = 0; q < KMAX; ++q) {
-        const int b = threadIdx.x + q * XFFT_T;
-        if (nbf % XFFT_T == 0 || b < nbf) {
-            const int j = b % nq, c = b / nq;
-            const float2* row = reinterpret_cast<const float2*>(mesh + (row0 + c) * S);
-            float2 v[R];
+        const int b = threadIdx.x + q * T;
+        if (nbf % T == 0 || b < nbf) {
+            const int j = b % nq, p = b / nq;
+            const float2* r0 = reinterpret_cast<const float2*>(mesh + (row0 + 2 * p) * S);
+            const float2* r1 = reinterpret_cast<const float2*>(mesh + (row0 + 2 * p + 1) * S);
+            C2 v[R];
 #pragma unroll
             for (int m = 0; m < R; ++m) {
                 const int k = j + m * nq;
                 if (!PACK) {
-                    v[m] = row[k];
+                    v[m] = from_rows(r0[k], r1[k]);
                 } else {
-                    const float2 xk = row[k], xm = row[n - k];
-                    const float2 e = make_float2(xk.x + xm.x, xk.y - xm.y);
-                    const float2 d = make_float2(xk.x - xm.x, xk.y + xm.y);
-                    const float2 o = cmul(cconj(gtw[k]), d);
-                    v[m] = make_float2(e.x - o.y, e.y + o.x);
+                    const C2 xk = from_rows(r0[k], r1[k]), xm = from_rows(r0[n - k], r1[n - k]);
+                    const C2 e{padd(xk.x, xm.x), psub(xk.y, xm.y)}, d{psub(xk.x, xm.x), padd(xk.y, xm.y)};
+                    const C2 o = cmul_by<true>(gtw[k], d);
+                    v[m] = C2{psub(e.x, o.y), padd(e.y, o.x)};
                 }
             }
             dft<R, INV>(v);
-            const int base = sidx<true>(j * R, c);
+            const int base = sidx<true>(j * R, p);
 #pragma unroll
-            for (int m = 0; m < R; ++m) buf[pow2(R) ? sidx_add<true>(base, m) : sidx<true>(j * R + m, c)] = v[m];
+            for (int m = 0; m < R; ++m) buf[pow2(R) ? sidx_add<true>(base, m) : sidx<true>(j * R + m, p)] = pack4(v[m]);
         }
     }
-    cp_async_wait_all();
     __syncthreads();
 }
 
@@ -454,51 +487,50 @@ __device__ __forceinline__ void xpass_load(float2* buf, const float* mesh, int64
 // the ghosted copy of Phi: every row lands at its place and, within the
 // ghost layers, at its periodic images (rows y < 3 also at y + N, y >= N - 2
 // also at y - N, the same in z; x < 4 also at x + N, x >= N - 4 at x - N).
-template <int n, int Ns, int R, int TWM, bool INV>
-__device__ __forceinline__ void xpass_store(const float2* buf, const float2* tw, float* phig, int64_t row0) {
+template <int n, int Ns, int R, int TWM, bool INV, int T>
+__device__ __forceinline__ void xpass_store(const float4* buf, const float2* tw, float* phig, int64_t row0) {
     constexpr int N = 2 * n;
     constexpr int nq = n / R;
     static_assert(nq == Ns, "the last pass has span n / R");
-    constexpr int nbf = nq * NC;
-    constexpr int KMAX = (nbf + XFFT_T - 1) / XFFT_T;
+    constexpr int nbf = nq * NP;
+    constexpr int KMAX = (nbf + T - 1) / T;
     constexpr int step = TWM * (n / (Ns * R));
 #pragma unroll
     for (int q = 0; q < KMAX; ++q) {
-        const int b = threadIdx.x + q * XFFT_T;
-        if (nbf % XFFT_T == 0 || b < nbf) {
-            const int j = b % nq, c = b / nq;
-            float2 v[R];
-            const int base = sidx<true>(j, c);
+        const int b = threadIdx.x + q * T;
+        if (nbf % T == 0 || b < nbf) {
+            const int j = b % nq, p = b / nq;
+            C2 v[R];
+            const int base = sidx<true>(j, p);
 #pragma unroll
             for (int m = 0; m < R; ++m)
-                v[m] = buf[pow2(nq) ? sidx_add<true>(base, m * nq) : sidx<true>(j + m * nq, c)];
+                v[m] = c2(buf[pow2(nq) ? sidx_add<true>(base, m * nq) : sidx<true>(j + m * nq, p)]);
             if (Ns > 1) {
 #pragma unroll
-                for (int m = 1; m < R; ++m) {
-                    float2 w = tw[j * m * step];
-                    if (INV) w.y = -w.y;
-                    v[m] = cmul(v[m], w);
-                }
+                for (int m = 1; m < R; ++m) v[m] = cmul_tw<INV>(v[m], tw[j * m * step]);
             }
             dft<R, INV>(v);
-            const int64_t r = row0 + c;
-            const int z = (int)(r / N), y = (int)(r - (int64_t)z * N);
-            // element k = j + m Ns holds reals 2k, 2k + 1; k < 2 only for m = 0,
-            // k >= n - 2 only for m = R - 1 (Ns >= 2)
-            auto put = [&](int yy, int zz) {
-                float2* row = reinterpret_cast<float2*>(phig + phig_index(N, 0, yy, zz));
 #pragma unroll
-                for (int m = 0; m < R; ++m) row[j + m * Ns] = v[m];
-                if (j < 2) row[j + n] = v[0];
-                if (j >= Ns - 2) row[j + (R - 1) * Ns - n] = v[R - 1];
-            };
-            put(y, z);
-            const bool gy = y < 3 || y >= N - 2, gz = z < 3 || z >= N - 2;
-            if (gy || gz) {                      // rows with periodic images in the ghost layers
-                const int y2 = y < 3 ? y + N : y - N, z2 = z < 3 ? z + N : z - N;
-                if (gy) put(y2, z);
-                if (gz) put(y, z2);
-                if (gy && gz) put(y2, z2);
+            for (int h = 0; h < 2; ++h) {
+                const int64_t r = row0 + 2 * p + h;
+                const int z = (int)(r / N), y = (int)(r - (int64_t)z * N);
+                // element k = j + m Ns holds reals 2k, 2k + 1; k < 2 only for m = 0,
+                // k >= n - 2 only for m = R - 1 (Ns >= 2)
+                auto put = [&](int yy, int zz) {
+                    float2* row = reinterpret_cast<float2*>(phig + phig_index(N, 0, yy, zz));
+#pragma unroll
+                    for (int m = 0; m < R; ++m) row[j + m * Ns] = row_of(v[m], h);
+                    if (j < 2) row[j + n] = row_of(v[0], h);
+                    if (j >= Ns - 2) row[j + (R - 1) * Ns - n] = row_of(v[R - 1], h);
+                };
+                put(y, z);
+                const bool gy = y < 3 || y >= N - 2, gz = z < 3 || z >= N - 2;
+                if (gy || gz) {                  // rows with periodic images in the ghost layers
+                    const int y2 = y < 3 ? y + N : y - N, z2 = z < 3 ? z + N : z - N;
+                    if (gy) put(y2, z);
+                    if (gz) put(y, z2);
+                    if (gy && gz) put(y2, z2);
+                }
             }
         }
     }
@@ -507,42 +539,47 @@ __device__ __forceinline__ void xpass_store(const float2* buf, const float2* tw,
 // r2c: the N reals of a row as N/2 complex z[k] = x[2k] + i x[2k+1], an
 // N/2-point FFT Z, then X[k] = (Z[k] + Z*[h-k])/2 - i W^k (Z[k] - Z*[h-k])/2
 template <int N, bool BAT>
-__global__ void __launch_bounds__(XFFT_T) k_fft_x_r2c(float* mesh, int S, const float2* __restrict__ tw, Batch bt) {
-    extern __shared__ float2 fsm[];
+__global__ void __launch_bounds__(fft_threads(N / 2), fft_blocks(N / 2))
+    k_fft_x_r2c(float* mesh, int S, const float2* __restrict__ tw, Batch bt) {
+    extern __shared__ float4 fsm[];
     if constexpr (BAT) {                                     // slot blockIdx.y of a batch
         if (bt.ms && !bt.ms[blockIdx.y].active) return;
         mesh = moved(mesh, slot_member(bt, blockIdx.y) * bt.stride);
     }
-    constexpr int h = N / 2;
-    float2* stw = fsm;               // [N]
-    float2* buf = fsm + N;           // [h][NC]
-    load_tw(stw, tw, N);
+    constexpr int h = N / 2, T = fft_threads(h);
+    float4* buf = fsm;                                       // [h][NP]
+    float2* stw = reinterpret_cast<float2*>(buf + h * NP);   // [N]
+    load_tw<N, T>(stw, tw);
     const int64_t row0 = (int64_t)blockIdx.x * NC;
     constexpr int R1 = x_first_radix<h>();
-    xpass_load<h, R1, false, false>(buf, mesh, row0, S, tw);
-    tile_fft<h, R1, 2, false, true, XFFT_T>(buf, stw);
-    // X[k] and X[h - k] from Z[k] and Z[h - k], k = 0 .. h / 2: the warps
-    // take k < h / 2 of one row at a time, so that (h / 2 a multiple of 16)
-    // each half-warp's Z[k] are one 16-element block of the swizzled tile,
-    // free of bank conflicts; the self-paired k = h / 2 of the 16 rows last
-    for (int t = threadIdx.x; t < (h / 2) * NC + NC; t += XFFT_T) {
-        const bool mid = t >= (h / 2) * NC;
-        const int k = mid ? h / 2 : t % (h / 2), c = mid ? t - (h / 2) * NC : t / (h / 2);
-        float2* dst = reinterpret_cast<float2*>(mesh + (row0 + c) * S);
-        const float2 zk = buf[sidx<true>(k % h, c)];
-        const float2 zm = buf[sidx<true>((h - k) % h, c)];
+    xpass_load<h, R1, false, false, T>(buf, mesh, row0, S, tw);
+    tile_fft<h, R1, 2, false, true, T>(buf, stw);
+    // X[k] and X[h - k] from Z[k] and Z[h - k], k = 0 .. h / 2: threads along k
+    // of one row pair, the self-paired k = h / 2 of the 8 pairs last
+    for (int t = threadIdx.x; t < (h / 2) * NP + NP; t += T) {
+        const bool mid = t >= (h / 2) * NP;
+        const int k = mid ? h / 2 : t % (h / 2), p = mid ? t - (h / 2) * NP : t / (h / 2);
+        float2* d0 = reinterpret_cast<float2*>(mesh + (row0 + 2 * p) * S);
+        float2* d1 = reinterpret_cast<float2*>(mesh + (row0 + 2 * p + 1) * S);
+        const C2 zk = c2(buf[sidx<true>(k % h, p)]);
+        const C2 zm = c2(buf[sidx<true>((h - k) % h, p)]);
+        const float2 hf = pk2(0.5f);
         {
-            float2 e = make_float2(0.5f * (zk.x + zm.x), 0.5f * (zk.y - zm.y));
-            float2 o = make_float2(0.5f * (zk.x - zm.x), 0.5f * (zk.y + zm.y));   // (Z - Z*) / 2
-            float2 wo = cmul(stw[k], o);
-            dst[k] = make_float2(e.x + wo.y, e.y - wo.x);                         // e - i wo
+            const C2 e{pmul(hf, padd(zk.x, zm.x)), pmul(hf, psub(zk.y, zm.y))};
+            const C2 o{pmul(hf, psub(zk.x, zm.x)), pmul(hf, padd(zk.y, zm.y))};   // (Z - Z*) / 2
+            const C2 wo = cmul_by<false>(stw[k], o);
+            const C2 x{padd(e.x, wo.y), psub(e.y, wo.x)};                         // e - i wo
+            d0[k] = row_of(x, 0);
+            d1[k] = row_of(x, 1);
         }
         if (k != h - k) {
             const int km = h - k;
-            float2 e = make_float2(0.5f * (zm.x + zk.x), 0.5f * (zm.y - zk.y));
-            float2 o = make_float2(0.5f * (zm.x - zk.x), 0.5f * (zm.y + zk.y));
-            float2 wo = cmul(stw[km], o);
-            dst[km] = make_float2(e.x + wo.y, e.y - wo.x);
+            const C2 e{pmul(hf, padd(zm.x, zk.x)), pmul(hf, psub(zm.y, zk.y))};
+            const C2 o{pmul(hf, psub(zm.x, zk.x)), pmul(hf, padd(zm.y, zk.y))};
+            const C2 wo = cmul_by<false>(stw[km], o);
+            const C2 x{padd(e.x, wo.y), psub(e.y, wo.x)};
+            d0[km] = row_of(x, 0);
+            d1[km] = row_of(x, 1);
         }
     }
 }
@@ -550,25 +587,25 @@ __global__ void __launch_bounds__(XFFT_T) k_fft_x_r2c(float* mesh, int S, const 
 // c2r: the packing above inverted inside the first pass, the N/2-point
 // inverse FFT, and the last pass writing the row's N reals
 template <int N, bool BAT>
-__global__ void __launch_bounds__(XFFT_T) k_fft_x_c2r(const float* mesh, int S, const float2* __restrict__ tw,
-                                                     float* __restrict__ phig, Batch bt) {
-    extern __shared__ float2 fsm[];
+__global__ void __launch_bounds__(fft_threads(N / 2), fft_blocks(N / 2))
+    k_fft_x_c2r(const float* mesh, int S, const float2* __restrict__ tw, float* __restrict__ phig, Batch bt) {
+    extern __shared__ float4 fsm[];
     if constexpr (BAT) {                                     // slot blockIdx.y of a batch
         if (bt.ms && !bt.ms[blockIdx.y].active) return;
         const int m = slot_member(bt, blockIdx.y);
         mesh = moved(mesh, m * bt.stride);
         phig = moved(phig, m * bt.stride);
     }
-    constexpr int h = N / 2;
-    float2* stw = fsm;               // [N]
-    float2* buf = fsm + N;           // [h][NC]
-    load_tw(stw, tw, N);
+    constexpr int h = N / 2, T = fft_threads(h);
+    float4* buf = fsm;                                       // [h][NP]
+    float2* stw = reinterpret_cast<float2*>(buf + h * NP);   // [N]
+    load_tw<N, T>(stw, tw);
     const int64_t row0 = (int64_t)blockIdx.x * NC;
     constexpr int R1 = x_first_radix<h>();
-    xpass_load<h, R1, true, true>(buf, mesh, row0, S, tw);
-    tile_fft_but_last<h, R1, 2, true, true, XFFT_T>(buf, stw);
+    xpass_load<h, R1, true, true, T>(buf, mesh, row0, S, tw);
+    tile_fft_but_last<h, R1, 2, true, true, T>(buf, stw);
     constexpr int Ns = last_span<h, R1>();
-    xpass_store<h, Ns, h / Ns, 2, true>(buf, stw, phig, row0);
+    xpass_store<h, Ns, h / Ns, 2, true, T>(buf, stw, phig, row0);
 }
 
 // ------------------------------------------------------------ y sweep
@@ -582,100 +619,99 @@ template <int N>
 constexpr int ntile_x() { return (N / 2 + NC - 1) / NC; }
 
 template <int N, bool INV, bool BAT>
-__global__ void __launch_bounds__(FFT_T, N <= 512 ? 2 : 1) k_fft_y(float* mesh, int S, const float2* __restrict__ tw,
-                                                                    Batch bt) {
-    extern __shared__ float2 fsm[];
+__global__ void __launch_bounds__(fft_threads(N), fft_blocks(N))
+    k_fft_y(float* mesh, int S, const float2* __restrict__ tw, Batch bt) {
+    extern __shared__ float4 fsm[];
     if constexpr (BAT) {                                     // slot blockIdx.z of a batch
         if (bt.ms && !bt.ms[blockIdx.z].active) return;
         mesh = moved(mesh, slot_member(bt, blockIdx.z) * bt.stride);
     }
-    constexpr int h = N / 2;
-    float2* stw = fsm;
-    float2* buf = fsm + N;
-    load_tw(stw, tw, N);
+    constexpr int h = N / 2, T = fft_threads(N);
+    float4* buf = fsm;
+    float2* stw = reinterpret_cast<float2*>(buf + N * NP);
+    load_tw<N, T>(stw, tw);
     const int Sc = S / 2;
     const int c0 = blockIdx.x * NC;
     float2* slab = reinterpret_cast<float2*>(mesh) + (int64_t)blockIdx.y * N * Sc;
-    constexpr int R1 = first_radix<N>(), KMAX1 = (N / R1 * NC + FFT_T - 1) / FFT_T;
-    fft_pass_load<N, R1, INV, INV ? 1 : KMAX1>(buf, slab, Sc, c0, h, 1, h);
-    if (INV) {
-        tile_fft_to_global<N, first_radix<N>(), 1, INV>(buf, stw, slab, Sc, c0, h, NoPost{}, 1, h);
-    } else if (blockIdx.x > 0) {
-        constexpr int KL = (last_span<N>() * NC + FFT_T - 1) / FFT_T;
-        tile_fft_to_global<N, first_radix<N>(), 1, INV, NoPost, KL>(buf, stw, slab, Sc, c0, h, NoPost{});
+    constexpr int q = npass(N);
+    col_load<N, INV, T>(buf, slab, Sc, c0, h, h);
+    if (INV || blockIdx.x > 0) {
+        col_passes<N, 2, q - 1, INV, T>(buf, stw);
+        col_store<N, INV, T>(buf, stw, slab, Sc, c0, h, INV ? h : 0);
     } else {
-        tile_fft<N, first_radix<N>(), 1, INV, false>(buf, stw);
-        for (int t = threadIdx.x; t < N * NC; t += FFT_T) {
-            const int c = t & (NC - 1), ky = t >> LOG_NC;
+        col_passes<N, 2, q, INV, T>(buf, stw);
+        for (int t = threadIdx.x; t < N * NP; t += T) {
+            const int p = t & (NP - 1), ky = t >> LOG_NP;
+            if (2 * p >= h) continue;
             float2* row = slab + (int64_t)ky * Sc;
-            if (c == 0) {
-                const float2 zk = buf[sidx<false>(ky, 0)];
-                const float2 zm = buf[sidx<false>((N - ky) % N, 0)];
-                row[0] = make_float2(0.5f * (zk.x + zm.x), 0.5f * (zk.y - zm.y));
+            const C2 z = c2(buf[sidx<false>(ky, p)]);
+            float4 f = to_columns(z);
+            if (p == 0) {
+                const float2 zk = row_of(z, 0), zm = row_of(c2(buf[sidx<false>((N - ky) % N, 0)]), 0);
+                f.x = 0.5f * (zk.x + zm.x);
+                f.y = 0.5f * (zk.y - zm.y);
                 row[h] = make_float2(0.5f * (zk.y + zm.y), 0.5f * (zm.x - zk.x));
-            } else if (c < h) {
-                row[c] = buf[sidx<false>(ky, c)];
             }
+            *reinterpret_cast<float4*>(row + 2 * p) = f;
         }
     }
 }
 
 // ------------------------------------------------------------ z sweep (+ Green)
-// Green's function -(3/2) Om / k^2 / W(k)^p / N^3 of one column (kx, ky), kz = z
+// Green's function -(3/2) Om / k^2 / W(k)^p / N^3 of a pair of columns (kx, ky),
+// (kx + 1, ky), kz = z
 struct GreenPost {
     const float* sk2;
     const float* swd;
     float g0, ky2, wy;
-    int c0, ky, ncol;
-    __device__ __forceinline__ float2 operator()(int z, int c, float2 v) const {
-        const int kx = c0 + c;
-        if (kx >= ncol) return v;
+    int c0, ky;
+    __device__ __forceinline__ float at(int z, int kx) const {
         const float kk = sk2[kx] + ky2 + sk2[z];
         // approximate division: within 2 ulp for kk below 2^126 (here kk < 3 pi^2)
-        const float gr = (kx == 0 && ky == 0 && z == 0) ? 0.0f : __fdividef(g0, kk) * (swd[kx] * wy * swd[z]);
-        return make_float2(v.x * gr, v.y * gr);
+        return (kx == 0 && ky == 0 && z == 0) ? 0.0f : __fdividef(g0, kk) * (swd[kx] * wy * swd[z]);
+    }
+    __device__ __forceinline__ float2 operator()(int z, int p) const {
+        const int kx = c0 + 2 * p;
+        return make_float2(at(z, kx), at(z, kx + 1));
     }
 };
 
 // One tile of 16 consecutive kx (0 .. N/2) at one ky.
 template <int N, int MODE, bool BAT>   // MODE 0: forward only, 1: forward, Green, inverse
-__global__ void __launch_bounds__(FFT_T, N <= 512 ? 2 : 1) k_fft_z(float* mesh, int S, const float2* __restrict__ tw,
-                                                 const float* __restrict__ k2, const float* __restrict__ wdec, float g0,
-                                                 Batch bt) {
-    extern __shared__ float2 fsm[];
+__global__ void __launch_bounds__(fft_threads(N), fft_blocks(N))
+    k_fft_z(float* mesh, int S, const float2* __restrict__ tw, const float* __restrict__ k2,
+            const float* __restrict__ wdec, float g0, Batch bt) {
+    extern __shared__ float4 fsm[];
     if constexpr (BAT) {                                     // slot blockIdx.z of a batch
         if (bt.ms && !bt.ms[blockIdx.z].active) return;
         mesh = moved(mesh, slot_member(bt, blockIdx.z) * bt.stride);
     }
-    constexpr int ncol = N / 2 + 1;
-    float2* stw = fsm;
-    float2* buf = fsm + N;
-    float* sk2 = reinterpret_cast<float*>(buf + N * NC + NC);     // [N]
-    float* swd = sk2 + N;                                          // [N]
-    load_tw(stw, tw, N);
+    constexpr int ncol = N / 2 + 1, T = fft_threads(N), q = npass(N);
+    float4* buf = fsm;
+    float2* stw = reinterpret_cast<float2*>(buf + N * NP);
+    // [N + NC]: a last pair's padding column stays inside
+    float* sk2 = reinterpret_cast<float*>(stw + N);
+    float* swd = sk2 + N + NC;
+    load_tw<N, T>(stw, tw);
     const int Sc = S / 2;
     const int64_t zs = (int64_t)N * Sc;
     const int c0 = blockIdx.x * NC, ky = blockIdx.y;
     float2* base = reinterpret_cast<float2*>(mesh) + (int64_t)ky * Sc;
     if (MODE == 1)
-        for (int i = threadIdx.x; i < N; i += blockDim.x) {
-            cp_async4(&sk2[i], &k2[i]);
-            cp_async4(&swd[i], &wdec[i]);
+        for (int i = threadIdx.x; i < N + NC; i += T) {
+            sk2[i] = i < N ? __ldg(&k2[i]) : 1.0f;
+            swd[i] = i < N ? __ldg(&wdec[i]) : 1.0f;
         }
-    fft_pass_load<N, first_radix<N>(), false>(buf, base, zs, c0, ncol);
+    col_load<N, false, T>(buf, base, zs, c0, ncol);
+    col_passes<N, 2, q - 1, false, T>(buf, stw);
     if (MODE == 1) {
-        tile_fft_but_last<N, first_radix<N>(), 1, false>(buf, stw);
-        constexpr int Ns = last_span<N>();
-        const GreenPost gp{sk2, swd, g0, sk2[ky], swd[ky], c0, ky, ncol};
-        if constexpr (N / Ns == first_radix<N>()) {     // last forward radix = first inverse radix
-            fft_pass_fwd_post_inv<N, Ns, N / Ns, 1>(buf, stw, gp);
-            tile_fft_to_global<N, first_radix<N>(), 1, true>(buf, stw, base, zs, c0, ncol, NoPost{});
-        } else {
-            fft_pass_post<N, Ns, N / Ns, 1, false>(buf, stw, gp);
-            tile_fft_to_global<N, 1, 1, true>(buf, stw, base, zs, c0, ncol, NoPost{});
-        }
+        const GreenPost gp{sk2, swd, g0, sk2[ky], swd[ky], c0, ky};
+        constexpr bool fuse = rad(N, 1) == rad(N, q);
+        col_pass_post<N, fuse, T>(buf, stw, gp);
+        col_passes<N, fuse ? 2 : 1, q - 1, true, T>(buf, stw);
+        col_store<N, true, T>(buf, stw, base, zs, c0, ncol);
     } else {
-        tile_fft_to_global<N, first_radix<N>(), 1, false>(buf, stw, base, zs, c0, ncol, NoPost{});
+        col_store<N, false, T>(buf, stw, base, zs, c0, ncol);
     }
 }
 
@@ -918,8 +954,10 @@ __global__ void __launch_bounds__(256) k_unpad(const float* __restrict__ src, in
     }
 }
 
-// twiddles (N) + tile (n x NC) + one spare column + Green tables (2 x N floats)
-size_t tile_smem(int N, int n) { return (size_t)(N + n * NC + NC) * sizeof(float2) + (size_t)2 * N * sizeof(float); }
+// twiddles (N) + tile (n x NP pairs)
+size_t tile_smem(int N, int n) { return (size_t)N * sizeof(float2) + (size_t)n * NP * sizeof(float4); }
+// the z sweep's, with the Green's function tables
+size_t ztile_smem(int N) { return tile_smem(N, N) + (size_t)2 * (N + NC) * sizeof(float); }
 
 template <int N>
 struct Sweeps {
@@ -927,13 +965,13 @@ struct Sweeps {
     static void attrs_for() {
         if constexpr (BAT && !(N <= 256)) return;
         else {
-        const int big = (int)tile_smem(N, N), half = (int)tile_smem(N, N / 2);
+        const int big = (int)tile_smem(N, N), half = (int)tile_smem(N, N / 2), bigz = (int)ztile_smem(N);
         cudaFuncSetAttribute(k_fft_x_r2c<N, BAT>, cudaFuncAttributeMaxDynamicSharedMemorySize, half);
         cudaFuncSetAttribute(k_fft_x_c2r<N, BAT>, cudaFuncAttributeMaxDynamicSharedMemorySize, half);
         cudaFuncSetAttribute(k_fft_y<N, false, BAT>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
         cudaFuncSetAttribute(k_fft_y<N, true, BAT>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
-        cudaFuncSetAttribute(k_fft_z<N, 0, BAT>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
-        cudaFuncSetAttribute(k_fft_z<N, 1, BAT>, cudaFuncAttributeMaxDynamicSharedMemorySize, big);
+        cudaFuncSetAttribute(k_fft_z<N, 0, BAT>, cudaFuncAttributeMaxDynamicSharedMemorySize, bigz);
+        cudaFuncSetAttribute(k_fft_z<N, 1, BAT>, cudaFuncAttributeMaxDynamicSharedMemorySize, bigz);
         }
     }
     // instances with a member dimension exist for the small meshes, where a
@@ -957,13 +995,13 @@ struct Sweeps {
         attrs();
         if constexpr (kBatchable) {
             if (batched(bt)) {
-                k_fft_x_r2c<N, true><<<dim3((N * N) / NC, bt.members), XFFT_T, tile_smem(N, N / 2), st>>>(mesh, S,
+                k_fft_x_r2c<N, true><<<dim3((N * N) / NC, bt.members), fft_threads(N / 2), tile_smem(N, N / 2), st>>>(mesh, S,
                                                                                                          p.tw, bt);
                 return;
             }
         }
         per_member(bt, [&](size_t o) {
-            k_fft_x_r2c<N, false><<<(N * N) / NC, XFFT_T, tile_smem(N, N / 2), st>>>(moved(mesh, o), S, p.tw, kSingle);
+            k_fft_x_r2c<N, false><<<(N * N) / NC, fft_threads(N / 2), tile_smem(N, N / 2), st>>>(moved(mesh, o), S, p.tw, kSingle);
         });
     }
     static void y(const FftPlan& p, float* mesh, int S, bool inv, cudaStream_t st, const Batch& bt) {
@@ -972,45 +1010,45 @@ struct Sweeps {
         if constexpr (kBatchable) {
             if (batched(bt)) {
                 const dim3 gy(ntile_x<N>(), N, bt.members);
-                if (inv) k_fft_y<N, true, true><<<gy, FFT_T, sm, st>>>(mesh, S, p.tw, bt);
-                else k_fft_y<N, false, true><<<gy, FFT_T, sm, st>>>(mesh, S, p.tw, bt);
+                if (inv) k_fft_y<N, true, true><<<gy, fft_threads(N), sm, st>>>(mesh, S, p.tw, bt);
+                else k_fft_y<N, false, true><<<gy, fft_threads(N), sm, st>>>(mesh, S, p.tw, bt);
                 return;
             }
         }
         const dim3 gy(ntile_x<N>(), N);
         per_member(bt, [&](size_t o) {
-            if (inv) k_fft_y<N, true, false><<<gy, FFT_T, sm, st>>>(moved(mesh, o), S, p.tw, kSingle);
-            else k_fft_y<N, false, false><<<gy, FFT_T, sm, st>>>(moved(mesh, o), S, p.tw, kSingle);
+            if (inv) k_fft_y<N, true, false><<<gy, fft_threads(N), sm, st>>>(moved(mesh, o), S, p.tw, kSingle);
+            else k_fft_y<N, false, false><<<gy, fft_threads(N), sm, st>>>(moved(mesh, o), S, p.tw, kSingle);
         });
     }
     static void z(const FftPlan& p, float* mesh, int S, float g0, bool green, cudaStream_t st, const Batch& bt) {
         attrs();
-        const size_t sm = tile_smem(N, N);
+        const size_t sm = ztile_smem(N);
         if constexpr (kBatchable) {
             if (batched(bt)) {
                 const dim3 gz((N / 2 + NC) / NC, N, bt.members);
-                if (green) k_fft_z<N, 1, true><<<gz, FFT_T, sm, st>>>(mesh, S, p.tw, p.k2, p.wdec, g0, bt);
-                else k_fft_z<N, 0, true><<<gz, FFT_T, sm, st>>>(mesh, S, p.tw, p.k2, p.wdec, g0, bt);
+                if (green) k_fft_z<N, 1, true><<<gz, fft_threads(N), sm, st>>>(mesh, S, p.tw, p.k2, p.wdec, g0, bt);
+                else k_fft_z<N, 0, true><<<gz, fft_threads(N), sm, st>>>(mesh, S, p.tw, p.k2, p.wdec, g0, bt);
                 return;
             }
         }
         const dim3 gz((N / 2 + NC) / NC, N);
         per_member(bt, [&](size_t o) {
-            if (green) k_fft_z<N, 1, false><<<gz, FFT_T, sm, st>>>(moved(mesh, o), S, p.tw, p.k2, p.wdec, g0, kSingle);
-            else k_fft_z<N, 0, false><<<gz, FFT_T, sm, st>>>(moved(mesh, o), S, p.tw, p.k2, p.wdec, g0, kSingle);
+            if (green) k_fft_z<N, 1, false><<<gz, fft_threads(N), sm, st>>>(moved(mesh, o), S, p.tw, p.k2, p.wdec, g0, kSingle);
+            else k_fft_z<N, 0, false><<<gz, fft_threads(N), sm, st>>>(moved(mesh, o), S, p.tw, p.k2, p.wdec, g0, kSingle);
         });
     }
     static void x_c2r(const FftPlan& p, float* mesh, int S, float* phig, cudaStream_t st, const Batch& bt) {
         attrs();
         if constexpr (kBatchable) {
             if (batched(bt)) {
-                k_fft_x_c2r<N, true><<<dim3((N * N) / NC, bt.members), XFFT_T, tile_smem(N, N / 2), st>>>(mesh, S,
+                k_fft_x_c2r<N, true><<<dim3((N * N) / NC, bt.members), fft_threads(N / 2), tile_smem(N, N / 2), st>>>(mesh, S,
                                                                                                          p.tw, phig, bt);
                 return;
             }
         }
         per_member(bt, [&](size_t o) {
-            k_fft_x_c2r<N, false><<<(N * N) / NC, XFFT_T, tile_smem(N, N / 2), st>>>(moved(mesh, o), S, p.tw,
+            k_fft_x_c2r<N, false><<<(N * N) / NC, fft_threads(N / 2), tile_smem(N, N / 2), st>>>(moved(mesh, o), S, p.tw,
                                                                                      moved(phig, o), kSingle);
         });
     }
