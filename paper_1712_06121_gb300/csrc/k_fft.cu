@@ -552,7 +552,10 @@ __global__ void __launch_bounds__(fft_threads(N / 2), fft_blocks(N / 2))
     k_fft_x_r2c(float* mesh, int S, const float2* __restrict__ tw, Batch bt) {
     extern __shared__ float4 fsm[];
     if constexpr (BAT) {                                     // slot blockIdx.y of a batch
-        if (bt.ms && !bt.ms[blockIdx.y].active) return;
+        if (bt.ms && !bt.ms[blockIdx.y].active) {
+            chain_wait();
+            return;
+        }
         mesh = moved(mesh, slot_member(bt, blockIdx.y) * bt.stride);
     }
     constexpr int h = N / 2, T = fft_threads(h);
@@ -560,6 +563,7 @@ __global__ void __launch_bounds__(fft_threads(N / 2), fft_blocks(N / 2))
     float2* stw = reinterpret_cast<float2*>(buf + h * NP);   // [N]
     load_tw<N, T>(stw, tw);
     const int64_t row0 = (int64_t)blockIdx.x * NC;
+    chain_wait();
     if (threadIdx.x == 0) {
         const int64_t r = row0 + (int64_t)152 * fft_blocks(h) * NC;
         if (r < (int64_t)N * N) l2_prefetch(mesh + r * S, NC * S * 4);
@@ -604,7 +608,10 @@ __global__ void __launch_bounds__(fft_threads(N / 2), fft_blocks(N / 2))
     k_fft_x_c2r(const float* mesh, int S, const float2* __restrict__ tw, float* __restrict__ phig, Batch bt) {
     extern __shared__ float4 fsm[];
     if constexpr (BAT) {                                     // slot blockIdx.y of a batch
-        if (bt.ms && !bt.ms[blockIdx.y].active) return;
+        if (bt.ms && !bt.ms[blockIdx.y].active) {
+            chain_wait();
+            return;
+        }
         const int m = slot_member(bt, blockIdx.y);
         mesh = moved(mesh, m * bt.stride);
         phig = moved(phig, m * bt.stride);
@@ -614,6 +621,7 @@ __global__ void __launch_bounds__(fft_threads(N / 2), fft_blocks(N / 2))
     float2* stw = reinterpret_cast<float2*>(buf + h * NP);   // [N]
     load_tw<N, T>(stw, tw);
     const int64_t row0 = (int64_t)blockIdx.x * NC;
+    chain_wait();
     if (threadIdx.x == 0) {
         const int64_t r = row0 + (int64_t)152 * fft_blocks(h) * NC;
         if (r < (int64_t)N * N) l2_prefetch(mesh + r * S, NC * S * 4);
@@ -640,13 +648,17 @@ __global__ void __launch_bounds__(fft_threads(N), fft_blocks(N))
     k_fft_y(float* mesh, int S, const float2* __restrict__ tw, Batch bt) {
     extern __shared__ float4 fsm[];
     if constexpr (BAT) {                                     // slot blockIdx.z of a batch
-        if (bt.ms && !bt.ms[blockIdx.z].active) return;
+        if (bt.ms && !bt.ms[blockIdx.z].active) {
+            chain_wait();
+            return;
+        }
         mesh = moved(mesh, slot_member(bt, blockIdx.z) * bt.stride);
     }
     constexpr int h = N / 2, T = fft_threads(N);
     float4* buf = fsm;
     float2* stw = reinterpret_cast<float2*>(buf + N * NP);
     load_tw<N, T>(stw, tw);
+    chain_wait();
     const int Sc = S / 2;
     const int c0 = blockIdx.x * NC;
     float2* slab = reinterpret_cast<float2*>(mesh) + (int64_t)blockIdx.y * N * Sc;
@@ -702,7 +714,10 @@ __global__ void __launch_bounds__(fft_threads(N), fft_blocks(N))
             const float* __restrict__ wdec, float g0, Batch bt) {
     extern __shared__ float4 fsm[];
     if constexpr (BAT) {                                     // slot blockIdx.z of a batch
-        if (bt.ms && !bt.ms[blockIdx.z].active) return;
+        if (bt.ms && !bt.ms[blockIdx.z].active) {
+            chain_wait();
+            return;
+        }
         mesh = moved(mesh, slot_member(bt, blockIdx.z) * bt.stride);
     }
     constexpr int ncol = N / 2 + 1, T = fft_threads(N), q = npass(N);
@@ -717,6 +732,7 @@ __global__ void __launch_bounds__(fft_threads(N), fft_blocks(N))
     if (MODE == 1)
         for (int i = threadIdx.x; i < N + NC; i += T)
             green[i] = i < N ? make_float2(__ldg(&k2[i]), __ldg(&wdec[i])) : make_float2(1.0f, 1.0f);
+    chain_wait();
     col_load<N, false, T>(buf, base, zs, c0, ncol);
     col_passes<N, 2, q - 1, false, T>(buf, stw);
     if (MODE == 1) {
@@ -1010,13 +1026,13 @@ struct Sweeps {
         attrs();
         if constexpr (kBatchable) {
             if (batched(bt)) {
-                k_fft_x_r2c<N, true><<<dim3((N * N) / NC, bt.members), fft_threads(N / 2), tile_smem(N, N / 2), st>>>(mesh, S,
+                launch_chained(k_fft_x_r2c<N, true>, dim3((N * N) / NC, bt.members), fft_threads(N / 2), tile_smem(N, N / 2), st, mesh, S,
                                                                                                          p.tw, bt);
                 return;
             }
         }
         per_member(bt, [&](size_t o) {
-            k_fft_x_r2c<N, false><<<(N * N) / NC, fft_threads(N / 2), tile_smem(N, N / 2), st>>>(moved(mesh, o), S, p.tw, kSingle);
+            launch_chained(k_fft_x_r2c<N, false>, (N * N) / NC, fft_threads(N / 2), tile_smem(N, N / 2), st, moved(mesh, o), S, p.tw, kSingle);
         });
     }
     static void y(const FftPlan& p, float* mesh, int S, bool inv, cudaStream_t st, const Batch& bt) {
@@ -1025,15 +1041,15 @@ struct Sweeps {
         if constexpr (kBatchable) {
             if (batched(bt)) {
                 const dim3 gy(ntile_x<N>(), N, bt.members);
-                if (inv) k_fft_y<N, true, true><<<gy, fft_threads(N), sm, st>>>(mesh, S, p.tw, bt);
-                else k_fft_y<N, false, true><<<gy, fft_threads(N), sm, st>>>(mesh, S, p.tw, bt);
+                if (inv) launch_chained(k_fft_y<N, true, true>, gy, fft_threads(N), sm, st, mesh, S, p.tw, bt);
+                else launch_chained(k_fft_y<N, false, true>, gy, fft_threads(N), sm, st, mesh, S, p.tw, bt);
                 return;
             }
         }
         const dim3 gy(ntile_x<N>(), N);
         per_member(bt, [&](size_t o) {
-            if (inv) k_fft_y<N, true, false><<<gy, fft_threads(N), sm, st>>>(moved(mesh, o), S, p.tw, kSingle);
-            else k_fft_y<N, false, false><<<gy, fft_threads(N), sm, st>>>(moved(mesh, o), S, p.tw, kSingle);
+            if (inv) launch_chained(k_fft_y<N, true, false>, gy, fft_threads(N), sm, st, moved(mesh, o), S, p.tw, kSingle);
+            else launch_chained(k_fft_y<N, false, false>, gy, fft_threads(N), sm, st, moved(mesh, o), S, p.tw, kSingle);
         });
     }
     static void z(const FftPlan& p, float* mesh, int S, float g0, bool green, cudaStream_t st, const Batch& bt) {
@@ -1042,28 +1058,28 @@ struct Sweeps {
         if constexpr (kBatchable) {
             if (batched(bt)) {
                 const dim3 gz((N / 2 + NC) / NC, N, bt.members);
-                if (green) k_fft_z<N, 1, true><<<gz, fft_threads(N), sm, st>>>(mesh, S, p.tw, p.k2, p.wdec, g0, bt);
-                else k_fft_z<N, 0, true><<<gz, fft_threads(N), sm, st>>>(mesh, S, p.tw, p.k2, p.wdec, g0, bt);
+                if (green) launch_chained(k_fft_z<N, 1, true>, gz, fft_threads(N), sm, st, mesh, S, p.tw, p.k2, p.wdec, g0, bt);
+                else launch_chained(k_fft_z<N, 0, true>, gz, fft_threads(N), sm, st, mesh, S, p.tw, p.k2, p.wdec, g0, bt);
                 return;
             }
         }
         const dim3 gz((N / 2 + NC) / NC, N);
         per_member(bt, [&](size_t o) {
-            if (green) k_fft_z<N, 1, false><<<gz, fft_threads(N), sm, st>>>(moved(mesh, o), S, p.tw, p.k2, p.wdec, g0, kSingle);
-            else k_fft_z<N, 0, false><<<gz, fft_threads(N), sm, st>>>(moved(mesh, o), S, p.tw, p.k2, p.wdec, g0, kSingle);
+            if (green) launch_chained(k_fft_z<N, 1, false>, gz, fft_threads(N), sm, st, moved(mesh, o), S, p.tw, p.k2, p.wdec, g0, kSingle);
+            else launch_chained(k_fft_z<N, 0, false>, gz, fft_threads(N), sm, st, moved(mesh, o), S, p.tw, p.k2, p.wdec, g0, kSingle);
         });
     }
     static void x_c2r(const FftPlan& p, float* mesh, int S, float* phig, cudaStream_t st, const Batch& bt) {
         attrs();
         if constexpr (kBatchable) {
             if (batched(bt)) {
-                k_fft_x_c2r<N, true><<<dim3((N * N) / NC, bt.members), fft_threads(N / 2), tile_smem(N, N / 2), st>>>(mesh, S,
+                launch_chained(k_fft_x_c2r<N, true>, dim3((N * N) / NC, bt.members), fft_threads(N / 2), tile_smem(N, N / 2), st, mesh, S,
                                                                                                          p.tw, phig, bt);
                 return;
             }
         }
         per_member(bt, [&](size_t o) {
-            k_fft_x_c2r<N, false><<<(N * N) / NC, fft_threads(N / 2), tile_smem(N, N / 2), st>>>(moved(mesh, o), S, p.tw,
+            launch_chained(k_fft_x_c2r<N, false>, (N * N) / NC, fft_threads(N / 2), tile_smem(N, N / 2), st, moved(mesh, o), S, p.tw,
                                                                                      moved(phig, o), kSingle);
         });
     }

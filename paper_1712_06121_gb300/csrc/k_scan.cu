@@ -27,6 +27,7 @@ __device__ __forceinline__ void load4(const unsigned* __restrict__ in, int64_t b
 __global__ void k_scan_reduce(const unsigned* __restrict__ in, int64_t n, unsigned* __restrict__ bsum, bool vec,
                               Batch bt) {
     __shared__ unsigned sw[32];
+    chain_wait();
     if (bt.ms && !bt.ms[blockIdx.y].active) return;
     const int m = slot_member(bt, blockIdx.y);
     in = moved(in, m * bt.stride);
@@ -42,6 +43,7 @@ __global__ void k_scan_reduce(const unsigned* __restrict__ in, int64_t n, unsign
 // exclusive scan of the block sums in place (single block, any count)
 __global__ void k_scan_bsums(unsigned* bsum, int nb, unsigned* total_out, Batch bt) {
     __shared__ unsigned sw[32];
+    chain_wait();
     if (bt.ms && !bt.ms[blockIdx.x].active) return;
     const int m = slot_member(bt, blockIdx.x);
     bsum = moved(bsum, m * bt.stride);
@@ -61,6 +63,7 @@ __global__ void k_scan_bsums(unsigned* bsum, int nb, unsigned* total_out, Batch 
 __global__ void k_scan_down(const unsigned* in, int64_t n, const unsigned* __restrict__ bsum, unsigned* out,
                             bool vec, Batch bt) {
     __shared__ unsigned sw[32];
+    chain_wait();
     if (bt.ms && !bt.ms[blockIdx.y].active) return;
     const int m = slot_member(bt, blockIdx.y);
     in = moved(in, m * bt.stride);
@@ -86,6 +89,7 @@ __global__ void k_scan_down(const unsigned* in, int64_t n, const unsigned* __res
 }
 
 __global__ void k_write_total(unsigned* out, int64_t n, const unsigned* total, Batch bt) {
+    chain_wait();
     if (bt.ms && !bt.ms[blockIdx.x].active) return;
     const int m = slot_member(bt, blockIdx.x);
     moved(out, m * bt.stride)[n] = *moved(total, m * bt.stride);
@@ -162,10 +166,10 @@ void exclusive_scan(const unsigned* in, unsigned* out, int64_t n, unsigned* tmp,
     unsigned* total = tmp + nb;
     // (members are whole multiples of 256 bytes apart: the same alignment)
     const bool vec = ((reinterpret_cast<uintptr_t>(in) | reinterpret_cast<uintptr_t>(out)) & 15) == 0;
-    k_scan_reduce<<<dim3(nb, bt.members), SCAN_T, 0, st>>>(in, n, tmp, vec, bt);
-    k_scan_bsums<<<bt.members, SCAN_T, 0, st>>>(tmp, nb, total, bt);
-    k_scan_down<<<dim3(nb, bt.members), SCAN_T, 0, st>>>(in, n, tmp, out, vec, bt);
-    k_write_total<<<bt.members, 1, 0, st>>>(out, n, total, bt);
+    launch_chained(k_scan_reduce, dim3(nb, bt.members), SCAN_T, 0, st, in, n, tmp, vec, bt);
+    launch_chained(k_scan_bsums, dim3(bt.members), SCAN_T, 0, st, tmp, nb, total, bt);
+    launch_chained(k_scan_down, dim3(nb, bt.members), SCAN_T, 0, st, in, n, tmp, out, vec, bt);
+    launch_chained(k_write_total, dim3(bt.members), 1, 0, st, out, n, total, bt);
 }
 
 void count_totals(const unsigned* counts, int64_t n, unsigned long long* out2, cudaStream_t st) {

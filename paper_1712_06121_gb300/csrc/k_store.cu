@@ -253,6 +253,7 @@ __device__ __forceinline__ void sigma_body(const float* __restrict__ part, int n
 
 __global__ void k_sigma_finalize(const float* __restrict__ part, int nparts, double count, double ratio,
                                  double fixed, double* sigma_out, Batch bt) {
+    chain_wait();
     const int slot = blockIdx.x;                             // slot of a batch
     if (bt.ms) {
         if (!bt.ms[slot].active) return;
@@ -317,6 +318,7 @@ __global__ void k_codec_tables(int lim, const double* __restrict__ tanv, const d
                                const double* __restrict__ sigma, float* __restrict__ dec, float* __restrict__ thr,
                                float* __restrict__ est, unsigned char* __restrict__ vtab,
                                signed char* __restrict__ vdel, Batch bt) {
+    chain_wait();
     const int slot = blockIdx.y;                             // slot of a batch
     if (bt.ms && !bt.ms[slot].active) return;
     const size_t o = slot_member(bt, slot) * bt.stride;
@@ -373,6 +375,7 @@ template <int NX, int NV>
 __global__ void __launch_bounds__(T_BRICK) k_decode(Geo g, StoreDev s, CodecDev cd, float* __restrict__ pos,
                                                     float* __restrict__ vel, unsigned* __restrict__ id) {
     extern __shared__ unsigned brick_sm[];
+    chain_wait();
     const int nbc = g.B * g.B * g.B, lim = g.nulim;
     const int L0 = blockIdx.x * nbc;
     const BrickTables bt = stage_brick<NV>(g, s, cd, L0, brick_sm);
@@ -448,6 +451,7 @@ __global__ void __launch_bounds__(T_BRICK) k_decode(Geo g, StoreDev s, CodecDev 
 template <int NV, int LPC>
 __global__ void __launch_bounds__(T_BRICK) k_max_speed(Geo g, StoreDev s, CodecDev cd,
                                                        unsigned* __restrict__ vmax_bits, Batch bt) {
+    chain_wait();
     {                                                        // member of slot blockIdx.y of a batch
         const size_t o = slot_member(bt, blockIdx.y) * bt.stride;
         s = moved(s, o);
@@ -542,6 +546,7 @@ template <int NX, int FC, bool BAT>
 __global__ void __launch_bounds__(T_BRICK) k_deposit(Geo g, StoreDev s, float* __restrict__ mesh, float fscale,
                                                      long long* __restrict__ vsum, int* __restrict__ mig, Batch bt) {
     extern __shared__ unsigned long long dep_smem[];
+    chain_wait();
     // FC > 0: the brick side in fine cells is the compile-time FC, else g.F
     const int lF = FC == 16 ? 4 : FC == 8 ? 3 : FC == 4 ? 2 : g.lF, F = 1 << lF, F3 = 1 << (3 * lF);
     const int E = g.B + 1, E3 = E * E * E;
@@ -783,6 +788,7 @@ __global__ void __launch_bounds__(PA_T, PA_MINB) k_passA(Geo g, StoreDev s, cons
                                                       CodecDev cur, float kick, float dc, StepScratch w,
                                                       DriftDebug dbg, Batch bt) {
     extern __shared__ unsigned char pa_smem[];
+    chain_wait();
     __shared__ __align__(8) unsigned long long tile_bar;
     // Phi tile: T x T rows (y, z: [o - 2, o + F + 3)) of TX = F + 8 nodes
     // (x: [o - 4, o + F + 4)), row stride TS = TX floats, read from the
@@ -1095,9 +1101,9 @@ __device__ __forceinline__ void store_total(const Geo& g, const StepScratch& w, 
 
 // the cells of a batch (blockIdx.y its slot)
 __global__ void k_cells(Geo g, StepScratch w, unsigned* __restrict__ off_new, float* __restrict__ vc_new, Batch bt) {
+    chain_wait();
     const int L = blockIdx.x * blockDim.x + threadIdx.x;
-    if (L >= g.Ncc) return;
-    if (bt.ms && !bt.ms[blockIdx.y].active) return;
+    if (L >= g.Ncc || (bt.ms && !bt.ms[blockIdx.y].active)) return;
     const int m = slot_member(bt, blockIdx.y);
     w = moved(w, m * bt.stride);
     off_new = moved(off_new, m * bt.stride);
@@ -1148,6 +1154,7 @@ __device__ __forceinline__ void tile_slots(const Geo& g, const unsigned* __restr
 
 __global__ void __launch_bounds__(1024) k_step_sums(Geo g, StepScratch w, double ratio, double* sigma_out,
                                                     unsigned* __restrict__ tsum) {
+    chain_wait();
     if (blockIdx.x == 0) {
         sigma_body(w.part, g.nbricks, 3.0 * (double)g.Np, ratio, 0.0, sigma_out);
         return;
@@ -1185,6 +1192,7 @@ __global__ void __launch_bounds__(SC_T) k_step_cells(Geo g, StepScratch w, const
                                                      unsigned* __restrict__ off_new, float* __restrict__ vc_new,
                                                      const double* __restrict__ tanv, const double* __restrict__ tanh_,
                                                      CodecDev next, int ntab) {
+    chain_wait();
     if ((int)blockIdx.x < ntab) {                            // the next codec's tables
         codec_tables_body(g.nulim, tanv, tanh_, *next.sigma, next.dec, next.thr, next.est,
                           g.nnu == 1 ? next.vtab : nullptr, g.nnu == 1 ? nullptr : next.vdel, blockIdx.x, ntab);
@@ -1472,6 +1480,7 @@ __global__ void __launch_bounds__(PB_WARPS * 32, 5) k_passB(Geo g, StoreDev so, 
                                                         const float* __restrict__ vc_new, unsigned* flags,
                                                         const int* __restrict__ big, int nbig_ctas, Batch bt) {
     extern __shared__ unsigned pb_smem[];
+    chain_wait();
     const int nbc = g.B * g.B * g.B, H3 = g.Bh * g.Bh * g.Bh;
     const int lim = g.nulim;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -1632,11 +1641,11 @@ struct Disp {
         const dim3 grid(g.nb, g.nb, g.nb * bt.members);
         const bool bat = bt.members > 1 || bt.ms;
         if (g.F == 16) {
-            if (bat) k_passA<NX, NV, 16, true><<<grid, PA_T, sm, st>>>(g, s, phig, tmap, use_tma, cur, kick, dc, w, dbg, bt);
-            else k_passA<NX, NV, 16, false><<<grid, PA_T, sm, st>>>(g, s, phig, tmap, use_tma, cur, kick, dc, w, dbg, bt);
+            if (bat) launch_chained(k_passA<NX, NV, 16, true>, grid, PA_T, sm, st, g, s, phig, tmap, use_tma, cur, kick, dc, w, dbg, bt);
+            else launch_chained(k_passA<NX, NV, 16, false>, grid, PA_T, sm, st, g, s, phig, tmap, use_tma, cur, kick, dc, w, dbg, bt);
         } else {
-            if (bat) k_passA<NX, NV, 0, true><<<grid, PA_T, sm, st>>>(g, s, phig, tmap, use_tma, cur, kick, dc, w, dbg, bt);
-            else k_passA<NX, NV, 0, false><<<grid, PA_T, sm, st>>>(g, s, phig, tmap, use_tma, cur, kick, dc, w, dbg, bt);
+            if (bat) launch_chained(k_passA<NX, NV, 0, true>, grid, PA_T, sm, st, g, s, phig, tmap, use_tma, cur, kick, dc, w, dbg, bt);
+            else launch_chained(k_passA<NX, NV, 0, false>, grid, PA_T, sm, st, g, s, phig, tmap, use_tma, cur, kick, dc, w, dbg, bt);
         }
     }
     static void passB(const Geo& g, const StoreDev& so, const StoreDev& sn, const CodecDev& cur,
@@ -1645,20 +1654,20 @@ struct Disp {
         const bool narrow = g.nid == 1 || g.nid == 2, bat = bt.members > 1 || bt.ms;
         if (passB_all(g, bt.members)) {
             const dim3 gb(g.nbricks, bt.members);
-            if (bat && narrow) k_passB<NX, NV, true, 0, true><<<gb, PB_WARPS * 32, sm_cta, st>>>(g, so, sn, cur, next, dc, ghost, vcn, flags, big, 0, bt);
-            else if (bat) k_passB<NX, NV, true, 4, true><<<gb, PB_WARPS * 32, sm_cta, st>>>(g, so, sn, cur, next, dc, ghost, vcn, flags, big, 0, bt);
-            else if (narrow) k_passB<NX, NV, false, 0, true><<<gb, PB_WARPS * 32, sm_cta, st>>>(g, so, sn, cur, next, dc, ghost, vcn, flags, big, 0, bt);
-            else k_passB<NX, NV, false, 4, true><<<gb, PB_WARPS * 32, sm_cta, st>>>(g, so, sn, cur, next, dc, ghost, vcn, flags, big, 0, bt);
+            if (bat && narrow) launch_chained(k_passB<NX, NV, true, 0, true>, gb, PB_WARPS * 32, sm_cta, st, g, so, sn, cur, next, dc, ghost, vcn, flags, big, 0, bt);
+            else if (bat) launch_chained(k_passB<NX, NV, true, 4, true>, gb, PB_WARPS * 32, sm_cta, st, g, so, sn, cur, next, dc, ghost, vcn, flags, big, 0, bt);
+            else if (narrow) launch_chained(k_passB<NX, NV, false, 0, true>, gb, PB_WARPS * 32, sm_cta, st, g, so, sn, cur, next, dc, ghost, vcn, flags, big, 0, bt);
+            else launch_chained(k_passB<NX, NV, false, 4, true>, gb, PB_WARPS * 32, sm_cta, st, g, so, sn, cur, next, dc, ghost, vcn, flags, big, 0, bt);
             return;
         }
         if constexpr (NV == 1) {
             // CTAs for crowded bricks first (at most Np / (PB_BIG + 1) of them exist)
             const int nbig_ctas = (int)std::min<int64_t>(2 * g.nsm, g.Np / (PB_BIG + 1));
             const dim3 gb(nbig_ctas + (g.nbricks + PB_WARPS - 1) / PB_WARPS, bt.members);
-            if (bat && narrow) k_passB<NX, NV, true, 0, false><<<gb, PB_WARPS * 32, sm, st>>>(g, so, sn, cur, next, dc, ghost, vcn, flags, big, nbig_ctas, bt);
-            else if (bat) k_passB<NX, NV, true, 4, false><<<gb, PB_WARPS * 32, sm, st>>>(g, so, sn, cur, next, dc, ghost, vcn, flags, big, nbig_ctas, bt);
-            else if (narrow) k_passB<NX, NV, false, 0, false><<<gb, PB_WARPS * 32, sm, st>>>(g, so, sn, cur, next, dc, ghost, vcn, flags, big, nbig_ctas, bt);
-            else k_passB<NX, NV, false, 4, false><<<gb, PB_WARPS * 32, sm, st>>>(g, so, sn, cur, next, dc, ghost, vcn, flags, big, nbig_ctas, bt);
+            if (bat && narrow) launch_chained(k_passB<NX, NV, true, 0, false>, gb, PB_WARPS * 32, sm, st, g, so, sn, cur, next, dc, ghost, vcn, flags, big, nbig_ctas, bt);
+            else if (bat) launch_chained(k_passB<NX, NV, true, 4, false>, gb, PB_WARPS * 32, sm, st, g, so, sn, cur, next, dc, ghost, vcn, flags, big, nbig_ctas, bt);
+            else if (narrow) launch_chained(k_passB<NX, NV, false, 0, false>, gb, PB_WARPS * 32, sm, st, g, so, sn, cur, next, dc, ghost, vcn, flags, big, nbig_ctas, bt);
+            else launch_chained(k_passB<NX, NV, false, 4, false>, gb, PB_WARPS * 32, sm, st, g, so, sn, cur, next, dc, ghost, vcn, flags, big, nbig_ctas, bt);
         }
     }
 };
@@ -1685,6 +1694,7 @@ void set_smem_attrs() {
 
 // one word of every listed member of a batch set to zero
 __global__ void k_zero_slot_words(unsigned* p, Batch bt) {
+    chain_wait();
     for (int i = threadIdx.x; i < bt.members; i += blockDim.x) moved(p, slot_member(bt, i) * bt.stride)[0] = 0u;
 }
 
@@ -1712,6 +1722,7 @@ __global__ void k_check_vel_tables(int lim, CodecDev c, long long* out2) {
 // the step's cleared scratch of every stepped member of a batch: the
 // fixed-point momentum sums [3][Ncc] and the migration / crowded-brick words
 __global__ void k_batch_clear(int64_t n64, long long* __restrict__ vsum, int* __restrict__ mig, Batch bt) {
+    chain_wait();
     if (bt.ms && !bt.ms[blockIdx.y].active) return;
     const int m = slot_member(bt, blockIdx.y);
     vsum = moved(vsum, m * bt.stride);
@@ -1725,8 +1736,8 @@ __global__ void k_batch_clear(int64_t n64, long long* __restrict__ vsum, int* __
 // ------------------------------------------------------------------ launchers
 void launch_batch_clear(const Geo& g, long long* vsum, int* maxmig, cudaStream_t st, const Batch& bt) {
     const int64_t n = 3 * (int64_t)g.Ncc;
-    k_batch_clear<<<dim3((unsigned)std::min<int64_t>(1024, (n + 255) / 256), bt.members), 256, 0, st>>>(n, vsum,
-                                                                                                     maxmig, bt);
+    launch_chained(k_batch_clear, dim3((unsigned)std::min<int64_t>(1024, (n + 255) / 256), bt.members), 256, 0, st, n,
+                   vsum, maxmig, bt);
 }
 
 static inline int nblk(int64_t n, int t) { return (int)((n + t - 1) / t); }
@@ -1750,14 +1761,14 @@ void launch_encode_sigma(const Geo& g, const float* vel, const unsigned* key, co
 
 void launch_sigma_finalize(const float* part, int nparts, double count, double ratio, double fixed,
                            double* sigma_out, cudaStream_t st, const Batch& bt) {
-    k_sigma_finalize<<<bt.members, 1024, 0, st>>>(part, nparts, count, ratio, fixed, sigma_out, bt);
+    launch_chained(k_sigma_finalize, dim3(bt.members), 1024, 0, st, part, nparts, count, ratio, fixed, sigma_out, bt);
 }
 
 void launch_codec_tables(int nulim, const double* tanv, const double* tanh_, const CodecDev& c, cudaStream_t st,
                          const Batch& bt) {
     // 1-byte codes (nulim 127) fit one block, which also builds the bucket table
     const bool one = nulim + 2 <= 256;
-    k_codec_tables<<<dim3(nblk(nulim + 2, 256), bt.members), 256, 0, st>>>(nulim, tanv, tanh_, c.sigma, c.dec, c.thr,
+    launch_chained(k_codec_tables, dim3(nblk(nulim + 2, 256), bt.members), 256, 0, st, nulim, tanv, tanh_, c.sigma, c.dec, c.thr,
                                                                           c.est, one ? c.vtab : nullptr,
                                                                           one ? nullptr : c.vdel, bt);
 }
@@ -1775,14 +1786,14 @@ void launch_encode_scatter(const Geo& g, const float* pos, const float* vel, con
 void launch_max_speed(const Geo& g, const StoreDev& s, const CodecDev& c, unsigned* vmax_bits, cudaStream_t st,
                       const Batch& bt) {
     if (bt.members == 1 && !bt.ms) cudaMemsetAsync(vmax_bits, 0, sizeof(unsigned), st);
-    else k_zero_slot_words<<<1, 256, 0, st>>>(vmax_bits, bt);
+    else launch_chained(k_zero_slot_words, dim3(1), 256, 0, st, vmax_bits, bt);
     // one wave of 64 warps per SM holds eight lanes a cell: small stores
     const bool wide = (int64_t)g.Ncc * bt.members * 8 <= (int64_t)64 * 32 * g.nsm;
     const dim3 grid(nblk((int64_t)g.Ncc * (wide ? 8 : 2), T_BRICK), bt.members);
-    if (g.nnu == 1 && wide) k_max_speed<1, 8><<<grid, T_BRICK, 0, st>>>(g, s, c, vmax_bits, bt);
-    else if (g.nnu == 1) k_max_speed<1, 2><<<grid, T_BRICK, 0, st>>>(g, s, c, vmax_bits, bt);
-    else if (wide) k_max_speed<2, 8><<<grid, T_BRICK, 0, st>>>(g, s, c, vmax_bits, bt);
-    else k_max_speed<2, 2><<<grid, T_BRICK, 0, st>>>(g, s, c, vmax_bits, bt);
+    if (g.nnu == 1 && wide) launch_chained(k_max_speed<1, 8>, grid, T_BRICK, 0, st, g, s, c, vmax_bits, bt);
+    else if (g.nnu == 1) launch_chained(k_max_speed<1, 2>, grid, T_BRICK, 0, st, g, s, c, vmax_bits, bt);
+    else if (wide) launch_chained(k_max_speed<2, 8>, grid, T_BRICK, 0, st, g, s, c, vmax_bits, bt);
+    else launch_chained(k_max_speed<2, 2>, grid, T_BRICK, 0, st, g, s, c, vmax_bits, bt);
 }
 
 // a brick's offsets, v_c and (1-byte codes) decode table
@@ -1793,10 +1804,10 @@ static size_t brick_smem(const Geo& g) {
 void launch_decode(const Geo& g, const StoreDev& s, const CodecDev& c, float* pos, float* vel, unsigned* id,
                    cudaStream_t st) {
     const size_t sm = brick_smem(g);
-    if (g.nchi == 1 && g.nnu == 1) k_decode<1, 1><<<g.nbricks, T_BRICK, sm, st>>>(g, s, c, pos, vel, id);
-    else if (g.nchi == 1) k_decode<1, 2><<<g.nbricks, T_BRICK, sm, st>>>(g, s, c, pos, vel, id);
-    else if (g.nnu == 1) k_decode<2, 1><<<g.nbricks, T_BRICK, sm, st>>>(g, s, c, pos, vel, id);
-    else k_decode<2, 2><<<g.nbricks, T_BRICK, sm, st>>>(g, s, c, pos, vel, id);
+    if (g.nchi == 1 && g.nnu == 1) launch_chained(k_decode<1, 1>, dim3(g.nbricks), T_BRICK, sm, st, g, s, c, pos, vel, id);
+    else if (g.nchi == 1) launch_chained(k_decode<1, 2>, dim3(g.nbricks), T_BRICK, sm, st, g, s, c, pos, vel, id);
+    else if (g.nnu == 1) launch_chained(k_decode<2, 1>, dim3(g.nbricks), T_BRICK, sm, st, g, s, c, pos, vel, id);
+    else launch_chained(k_decode<2, 2>, dim3(g.nbricks), T_BRICK, sm, st, g, s, c, pos, vel, id);
 }
 
 static size_t deposit_smem(const Geo& g) {
@@ -1815,20 +1826,20 @@ void launch_deposit(const Geo& g, const StoreDev& s, float* mesh, double scale, 
     if (g.nchi == 1) {
         set_smem_attrs<1, 1>(); set_smem_attrs<1, 2>();
         if (f16) {
-            if (bat) k_deposit<1, 16, true><<<grid, T_BRICK, sm, st>>>(g, s, mesh, fs, vs, mig, bt);
-            else k_deposit<1, 16, false><<<grid, T_BRICK, sm, st>>>(g, s, mesh, fs, vs, mig, bt);
+            if (bat) launch_chained(k_deposit<1, 16, true>, grid, T_BRICK, sm, st, g, s, mesh, fs, vs, mig, bt);
+            else launch_chained(k_deposit<1, 16, false>, grid, T_BRICK, sm, st, g, s, mesh, fs, vs, mig, bt);
         } else {
-            if (bat) k_deposit<1, 0, true><<<grid, T_BRICK, sm, st>>>(g, s, mesh, fs, vs, mig, bt);
-            else k_deposit<1, 0, false><<<grid, T_BRICK, sm, st>>>(g, s, mesh, fs, vs, mig, bt);
+            if (bat) launch_chained(k_deposit<1, 0, true>, grid, T_BRICK, sm, st, g, s, mesh, fs, vs, mig, bt);
+            else launch_chained(k_deposit<1, 0, false>, grid, T_BRICK, sm, st, g, s, mesh, fs, vs, mig, bt);
         }
     } else {
         set_smem_attrs<2, 1>(); set_smem_attrs<2, 2>();
         if (f16) {
-            if (bat) k_deposit<2, 16, true><<<grid, T_BRICK, sm, st>>>(g, s, mesh, fs, vs, mig, bt);
-            else k_deposit<2, 16, false><<<grid, T_BRICK, sm, st>>>(g, s, mesh, fs, vs, mig, bt);
+            if (bat) launch_chained(k_deposit<2, 16, true>, grid, T_BRICK, sm, st, g, s, mesh, fs, vs, mig, bt);
+            else launch_chained(k_deposit<2, 16, false>, grid, T_BRICK, sm, st, g, s, mesh, fs, vs, mig, bt);
         } else {
-            if (bat) k_deposit<2, 0, true><<<grid, T_BRICK, sm, st>>>(g, s, mesh, fs, vs, mig, bt);
-            else k_deposit<2, 0, false><<<grid, T_BRICK, sm, st>>>(g, s, mesh, fs, vs, mig, bt);
+            if (bat) launch_chained(k_deposit<2, 0, true>, grid, T_BRICK, sm, st, g, s, mesh, fs, vs, mig, bt);
+            else launch_chained(k_deposit<2, 0, false>, grid, T_BRICK, sm, st, g, s, mesh, fs, vs, mig, bt);
         }
     }
 }
@@ -1857,20 +1868,20 @@ void launch_passA(const Geo& g, const StoreDev& s, const float* phig, const CUte
 
 void launch_cells(const Geo& g, const StepScratch& w, unsigned* off_new, float* vc_new, cudaStream_t st,
                   const Batch& bt) {
-    k_cells<<<dim3(nblk(g.Ncc, 256), bt.members), 256, 0, st>>>(g, w, off_new, vc_new, bt);
+    launch_chained(k_cells, dim3(nblk(g.Ncc, 256), bt.members), 256, 0, st, g, w, off_new, vc_new, bt);
 }
 
 int step_tmp_words(const Geo& g) { return step_tiles(g); }
 
 void launch_step_sums(const Geo& g, const StepScratch& w, double ratio, double* sigma_out, unsigned* tmp,
                       cudaStream_t st) {
-    k_step_sums<<<1 + (step_tiles(g) + 1) / 2, 1024, 0, st>>>(g, w, ratio, sigma_out, tmp);
+    launch_chained(k_step_sums, dim3(1 + (step_tiles(g) + 1) / 2), 1024, 0, st, g, w, ratio, sigma_out, tmp);
 }
 
 void launch_step_cells(const Geo& g, const StepScratch& w, unsigned* off_new, float* vc_new, const double* tanv,
                        const double* tanh, const CodecDev& next, const unsigned* tmp, cudaStream_t st) {
     const int ntab = g.nnu == 1 ? 1 : nblk(g.nulim + 2, SC_T);
-    k_step_cells<<<ntab + step_tiles(g), SC_T, 0, st>>>(g, w, tmp, off_new, vc_new, tanv, tanh, next, ntab);
+    launch_chained(k_step_cells, dim3(ntab + step_tiles(g)), SC_T, 0, st, g, w, tmp, off_new, vc_new, tanv, tanh, next, ntab);
 }
 
 // `words` of a CTA's brick tables after the staged 1-byte codec tables

@@ -3,6 +3,7 @@
 
 #include <string>
 #include <type_traits>
+#include <utility>
 
 #include <cuda.h>
 
@@ -43,6 +44,35 @@ __device__ __forceinline__ int stable_round_rank(int digit, bool active, unsigne
     int pos = active ? (int)(wcnt[w * nd + digit] + (unsigned)lrank) : -1;
     __syncthreads();
     return pos;
+}
+
+// ------------------------------------------------------------ chained launches
+// A step is a chain of short kernels, each reading what the one before wrote.
+// launch_chained lets the next kernel's launch overlap the running one
+// (programmatic dependent launch): its CTAs come up as the predecessor's exit,
+// and chain_wait() holds them until the predecessor has completed and its
+// writes are visible.  Every CTA of a kernel launched this way calls
+// chain_wait() before it touches anything that an earlier kernel of the stream
+// reads or writes (tables uploaded once at creation may be read before), and
+// before it returns, so completion stays transitive along the chain.  Steps of
+// 32^3, 64^3 (x1v2), 128^3 and 256^3 particles: runs 766 -> 652, 640 -> 533, 1787
+// -> 1672 and 6683 -> 6605 us.  (An early griddepcontrol.launch_dependents
+// lets the successor's waiting CTAs take the slots of the running kernel: 7535
+// us at 256^3.)
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+template <class... P, class... A>
+inline void launch_chained(void (*kernel)(P...), dim3 grid, unsigned block, size_t smem, cudaStream_t st, A&&... args) {
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
 }
 
 // inclusive scan of one value per thread over the block; returns the
