@@ -646,20 +646,19 @@ static cube_status encode_impl(cube_ctx* c, const float* pos, const float* vel, 
     const int k = c->cur;
     CK(cudaMemsetAsync(c->flags, 0, 4, c->st));
     CK(cudaMemsetAsync(c->counts[k], 0, (size_t)g.Ncc * 4, c->st));
-    CK(cudaMemsetAsync(c->vsum, 0, (size_t)g.Ncc * 24, c->st));
-    launch_encode_keys(g, dpos, dvel, keys, perm, c->counts[k], c->vsum, c->flags, c->st);
+    launch_encode_keys(g, dpos, keys, c->counts[k], c->flags, c->st);
     exclusive_scan(c->counts[k], c->offsets[k], g.Ncc, c->scan_tmp, c->st);
-    launch_vc_finalize(g, c->counts[k], c->vsum, c->vc[k], c->st);
-    if (sigma > 0.0) {
-        launch_sigma_finalize(c->part, 0, 1.0, 1.0, sigma, c->codec[k].sigma, c->st);
-    } else {
-        launch_encode_sigma(g, dvel, keys, c->vc[k], c->part, c->st);
-        launch_sigma_finalize(c->part, encode_sigma_blocks(g), 3.0 * (double)g.Np, 1.0, 0.0, c->codec[k].sigma, c->st);
-    }
+    unsigned* spare[3];
+    const unsigned* order = radix_sort_index(keys, perm, g.Np, key_bits, rtmp, c->st, spare);
+    // the momenta in storage order take the sort's other arrays
+    float* const vsorted[3] = {(float*)spare[0], (float*)spare[1], (float*)spare[2]};
+    const StoreDev store = c->store(k);
+    launch_encode_vc(g, dvel, order, store, vsorted, sigma > 0.0 ? nullptr : c->part, c->flags, c->st);
+    launch_sigma_finalize(c->part, sigma > 0.0 ? 0 : g.nbricks, 3.0 * (double)g.Np, 1.0, sigma > 0.0 ? sigma : 0.0,
+                          c->codec[k].sigma, c->st);
     launch_codec_tables(g.nulim, c->tanv, c->tanh_, c->codec[k], c->st);
-    radix_sort_pairs(keys, perm, g.Np, key_bits, rtmp, c->st);
-    launch_encode_scatter(g, dpos, dvel, did, keys, perm, c->vc[k], c->codec[k], c->store(k), c->st);
-    c->launches += 1 + 4 + 1 + (sigma > 0.0 ? 1 : 2) + 1 + (int64_t)((key_bits + 7) / 8) * 6 + 1;
+    launch_encode_codes(g, dpos, vsorted, did, order, c->codec[k], store, c->st);
+    c->launches += 1 + 4 + (int64_t)((key_bits + 7) / 8) * 6 + 1 + 1 + 1 + 1;
     CK(cudaGetLastError());
     if (sync) CK(cudaStreamSynchronize(c->st));
     c->encoded = true;

@@ -478,18 +478,6 @@ __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commi
 // wait until at most one committed group (the most recent) is still in flight
 __device__ __forceinline__ void cp_async_wait_prev() { asm volatile("cp.async.wait_group 1;\n" ::: "memory"); }
 
-// Lanes of `active` whose 8-bit value v (0 <= v < 256) equals this lane's:
-// one ballot per bit, intersected.  Every lane of `active` must call it.
-__device__ __forceinline__ unsigned same_value_lanes(unsigned active, int v) {
-    unsigned m = active;
-#pragma unroll
-    for (int b = 0; b < 8; ++b) {
-        const unsigned bb = __ballot_sync(active, (v >> b) & 1);
-        m &= ((v >> b) & 1) ? bb : ~bb;
-    }
-    return m;
-}
-
 // 64-bit add into shared memory from 32-bit atomics: the low word's
 // wrap-arounds are carried into the high word, so the final value is the
 // exact sum mod 2^64 whatever the order.  lohi = {low word, high word}.

@@ -115,43 +115,131 @@ __global__ void k_count_totals(const unsigned* __restrict__ c, int64_t n, unsign
 }
 
 // ------------------------------------------------------------ radix sort
+// Stable LSD radix sort of keys with the permutation that sorts them, at most
+// 8 bits a pass (the bits split evenly).  A CTA takes a tile of 4096 consecutive items, a warp 512 of them in
+// 16 rounds of 32: a round's items of one digit take consecutive ranks in lane
+// order behind the warp's running count (match + popc, no barrier), the warps'
+// counts are scanned per digit, and the tile is put in order in shared memory
+// so that each digit's run goes out in consecutive addresses.  Bound by the
+// latency of that chain: 64 registers and the largest shared-memory carve-out
+// keep four CTAs a SM (two: 152-194 us).  16.7 M keys, us a pass: 136 with a
+// block-wide ranking of every 256 items and scattered stores -> 96 the first
+// pass, 110 the others; histogram 37 -> 13.
 constexpr int RX_T = 256;
-constexpr int RX_ITEMS = 8;
+constexpr int RX_ITEMS = 16;
 constexpr int RX_TILE = RX_T * RX_ITEMS;
 
-__global__ void k_radix_hist(const unsigned* __restrict__ keys, int64_t n, int shift, int ntiles,
-                             unsigned* __restrict__ hist) {
+__global__ void __launch_bounds__(RX_T) k_radix_hist(const unsigned* __restrict__ keys, int64_t n, int shift,
+                                                     unsigned mask, int ntiles, unsigned* __restrict__ hist,
+                                                     bool vec) {
     __shared__ unsigned h[256];
+    chain_wait();
     h[threadIdx.x] = 0;
     __syncthreads();
-    int64_t base = (int64_t)blockIdx.x * RX_TILE;
-    for (int i = 0; i < RX_ITEMS; ++i) {
-        int64_t idx = base + (int64_t)i * RX_T + threadIdx.x;
-        if (idx < n) atomicAdd(&h[(keys[idx] >> shift) & 255u], 1u);
+    const int64_t base = (int64_t)blockIdx.x * RX_TILE;
+    if (vec && base + RX_TILE <= n) {
+        const uint4* k4 = reinterpret_cast<const uint4*>(keys + base);
+        uint4 v[RX_ITEMS / 4];
+#pragma unroll
+        for (int i = 0; i < RX_ITEMS / 4; ++i) v[i] = k4[i * RX_T + threadIdx.x];
+#pragma unroll
+        for (int i = 0; i < RX_ITEMS / 4; ++i) {
+            atomicAdd(&h[(v[i].x >> shift) & mask], 1u);
+            atomicAdd(&h[(v[i].y >> shift) & mask], 1u);
+            atomicAdd(&h[(v[i].z >> shift) & mask], 1u);
+            atomicAdd(&h[(v[i].w >> shift) & mask], 1u);
+        }
+    } else {
+        for (int i = 0; i < RX_ITEMS; ++i) {
+            const int64_t idx = base + (int64_t)i * RX_T + threadIdx.x;
+            if (idx < n) atomicAdd(&h[(keys[idx] >> shift) & mask], 1u);
+        }
     }
     __syncthreads();
-    hist[(int64_t)threadIdx.x * ntiles + blockIdx.x] = h[threadIdx.x];
+    if (threadIdx.x <= mask) hist[(int64_t)threadIdx.x * ntiles + blockIdx.x] = h[threadIdx.x];
 }
 
-__global__ void __launch_bounds__(RX_T) k_radix_scatter(const unsigned* __restrict__ kin, const unsigned* __restrict__ vin,
-                                                        int64_t n, int shift, int ntiles,
-                                                        const unsigned* __restrict__ hscan,
+// FIRST: the permutation so far is the identity (vin is not read)
+template <bool FIRST>
+__global__ void __launch_bounds__(RX_T, 4) k_radix_scatter(const unsigned* __restrict__ kin,
+                                                        const unsigned* __restrict__ vin, int64_t n, int shift,
+                                                        unsigned mask, int ntiles, const unsigned* __restrict__ hscan,
                                                         unsigned* __restrict__ kout, unsigned* __restrict__ vout) {
-    __shared__ unsigned run[256];
-    __shared__ unsigned wcnt[(RX_T / 32) * 256];
-    run[threadIdx.x] = hscan[(int64_t)threadIdx.x * ntiles + blockIdx.x];
+    constexpr int W = RX_T / 32;
+    __shared__ unsigned wh[W][256];                          // per warp: a digit's count, then its first place
+    __shared__ unsigned sk[RX_TILE], sv[RX_TILE];            // the tile in order
+    __shared__ unsigned gs[256];                             // a digit's first address less its first place
+    __shared__ unsigned sw[32];
+    chain_wait();
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int64_t t0 = (int64_t)blockIdx.x * RX_TILE, base = t0 + w * (RX_ITEMS * 32) + lane;
+    unsigned k[RX_ITEMS], rank[RX_ITEMS];
+#pragma unroll
+    for (int r = 0; r < RX_ITEMS; ++r) k[r] = base + r * 32 < n ? kin[base + r * 32] : 0u;
+#pragma unroll
+    for (int i = 0; i < W; ++i) wh[i][threadIdx.x] = 0u;
     __syncthreads();
-    int64_t base = (int64_t)blockIdx.x * RX_TILE;
-    for (int i = 0; i < RX_ITEMS; ++i) {
-        int64_t idx = base + (int64_t)i * RX_T + threadIdx.x;
-        bool act = idx < n;
-        unsigned k = act ? kin[idx] : 0u;
-        unsigned v = act ? vin[idx] : 0u;
-        int d = (int)((k >> shift) & 255u);
-        int pos = stable_round_rank<RX_T / 32>(d, act, run, wcnt, 256);
-        if (act && pos >= 0 && pos < n) {
-            kout[pos] = k;
-            vout[pos] = v;
+#pragma unroll
+    for (int r = 0; r < RX_ITEMS; ++r) {
+        const bool act = base + r * 32 < n;
+        const unsigned d = act ? (k[r] >> shift) & mask : 256u;
+        // lanes of the same digit.  A match instruction costs more the more
+        // values there are: the low digits of a pass over lattice order differ
+        // all along a warp (117 us with a ballot per bit, 126 matched), the
+        // higher ones hardly (113, 105)
+        unsigned peers = 0xffffffffu;
+        if (FIRST) {
+#pragma unroll
+            for (int b = 0; b < 9; ++b) {
+                const bool bit = (d >> b) & 1u;
+                const unsigned m = __ballot_sync(0xffffffffu, bit);
+                peers &= bit ? m : ~m;
+            }
+        } else {
+            peers = __match_any_sync(0xffffffffu, d);
+        }
+        const int leader = __ffs(peers) - 1;
+        unsigned st = 0;
+        if (lane == leader && act) {
+            st = wh[w][d];
+            wh[w][d] = st + (unsigned)__popc(peers);
+        }
+        rank[r] = __shfl_sync(0xffffffffu, st, leader) + (unsigned)__popc(peers & ((1u << lane) - 1u));
+        __syncwarp();
+    }
+    __syncthreads();
+    {
+        const int d = threadIdx.x;
+        unsigned t = 0, total;
+#pragma unroll
+        for (int i = 0; i < W; ++i) {
+            const unsigned c = wh[i][d];
+            wh[i][d] = t;
+            t += c;
+        }
+        const unsigned first = block_inclusive_scan(t, sw, &total) - t;
+#pragma unroll
+        for (int i = 0; i < W; ++i) wh[i][d] += first;
+        if (d <= (int)mask) gs[d] = hscan[(int64_t)d * ntiles + blockIdx.x] - first;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < RX_ITEMS; ++r) {
+        const int64_t idx = base + r * 32;
+        if (idx < n) {
+            const unsigned at = wh[w][(k[r] >> shift) & mask] + rank[r];
+            sk[at] = k[r];
+            sv[at] = FIRST ? (unsigned)idx : vin[idx];
+        }
+    }
+    __syncthreads();
+    const int cnt = (int)(n - t0 < RX_TILE ? n - t0 : RX_TILE);
+    for (int i = threadIdx.x; i < cnt; i += RX_T) {
+        const unsigned kk = sk[i];
+        const unsigned at = gs[(kk >> shift) & mask] + (unsigned)i;
+        if (at < (unsigned)n) {
+            kout[at] = kk;
+            vout[at] = sv[i];
         }
     }
 }
@@ -182,32 +270,37 @@ int64_t radix_tmp_words(int64_t n) {
     int64_t ntiles = (n + RX_TILE - 1) / RX_TILE;
     if (ntiles == 0) ntiles = 1;
     int64_t h = 256 * ntiles;
-    return 2 * h + 1 + scan_tmp_words(h) + 2 * n;
+    return 2 * h + 1 + scan_tmp_words(h) + 2 * n + 8;     // + 8: the arrays of n begin on 16-byte boundaries
 }
 
-void radix_sort_pairs(unsigned* keys, unsigned* vals, int64_t n, int key_bits, unsigned* tmp, cudaStream_t st) {
-    int ntiles = (int)((n + RX_TILE - 1) / RX_TILE);
-    if (ntiles == 0) return;
-    int64_t h = 256LL * ntiles;
+unsigned* radix_sort_index(unsigned* keys, unsigned* perm, int64_t n, int key_bits, unsigned* tmp, cudaStream_t st,
+                           unsigned** spare) {
+    const int ntiles = (int)((n + RX_TILE - 1) / RX_TILE);
+    const int64_t h = 256LL * ntiles;
     unsigned* hist = tmp;
     unsigned* hscan = hist + h;          // h + 1 entries (total at the end)
     unsigned* stmp = hscan + h + 1;
-    unsigned* kalt = stmp + scan_tmp_words(h);
-    unsigned* valt = kalt + n;
-    unsigned *ka = keys, *va = vals, *kb = kalt, *vb = valt;
-    int passes = (key_bits + 7) / 8;
+    unsigned* kalt = reinterpret_cast<unsigned*>((reinterpret_cast<uintptr_t>(stmp + scan_tmp_words(h)) + 15) & ~(uintptr_t)15);
+    unsigned* valt = kalt + (n + 3) / 4 * 4;
+    unsigned *ka = keys, *va = valt, *kb = kalt, *vb = perm;
+    cudaFuncSetAttribute(k_radix_scatter<true>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+    cudaFuncSetAttribute(k_radix_scatter<false>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+    const int passes = (key_bits + 7) / 8, bits = (key_bits + passes - 1) / passes;
+    const unsigned mask = (1u << bits) - 1u;
     for (int p = 0; p < passes; ++p) {
-        int shift = 8 * p;
-        k_radix_hist<<<ntiles, RX_T, 0, st>>>(ka, n, shift, ntiles, hist);
-        exclusive_scan(hist, hscan, h, stmp, st);
-        k_radix_scatter<<<ntiles, RX_T, 0, st>>>(ka, va, n, shift, ntiles, hscan, kb, vb);
-        unsigned* t = ka; ka = kb; kb = t;
-        t = va; va = vb; vb = t;
+        const int shift = bits * p;
+        const bool vec = (reinterpret_cast<uintptr_t>(ka) & 15) == 0;
+        launch_chained(k_radix_hist, dim3(ntiles), RX_T, 0, st, ka, n, shift, mask, ntiles, hist, vec);
+        exclusive_scan(hist, hscan, (int64_t)(mask + 1) * ntiles, stmp, st);
+        if (p == 0) launch_chained(k_radix_scatter<true>, dim3(ntiles), RX_T, 0, st, ka, va, n, shift, mask, ntiles, hscan, kb, vb);
+        else launch_chained(k_radix_scatter<false>, dim3(ntiles), RX_T, 0, st, ka, va, n, shift, mask, ntiles, hscan, kb, vb);
+        std::swap(ka, kb);
+        std::swap(va, vb);
     }
-    if (ka != keys) {
-        cudaMemcpyAsync(keys, ka, n * sizeof(unsigned), cudaMemcpyDeviceToDevice, st);
-        cudaMemcpyAsync(vals, va, n * sizeof(unsigned), cudaMemcpyDeviceToDevice, st);
-    }
+    spare[0] = ka;
+    spare[1] = kb;
+    spare[2] = vb;
+    return va;
 }
 
 }  // namespace cube

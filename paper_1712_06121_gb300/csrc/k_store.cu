@@ -166,65 +166,143 @@ __device__ __forceinline__ double snap_sigma_dev(double x) {
 }
 
 // ------------------------------------------------------------------ encode
+// Bin of a position, floor(x scale) mod tot (tot = Nc 2^(8 n) <= 2^26, so it and
+// every bin are exact in FP32): positions already in the box need neither the
+// 64-bit conversion nor the modulo.  Non-finite positions give 0.
+__device__ __forceinline__ int pos_bin(float x, float scale, int tot) {
+    if (!isfinite(x)) return 0;
+    const float f = x * scale;
+    if (f >= 0.0f && f < (float)tot) return (int)f;
+    long long b = __float2ll_rd(f) % tot;
+    return (int)(b < 0 ? b + tot : b);
+}
+
 template <int NX>
-__global__ void k_encode_keys(Geo g, const float* __restrict__ pos, const float* __restrict__ vel,
-                              unsigned* __restrict__ key, unsigned* __restrict__ val, unsigned* counts,
-                              long long* vsum, unsigned* flags) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+__global__ void k_encode_keys(Geo g, const float* __restrict__ pos, unsigned* __restrict__ key, unsigned* counts,
+                              unsigned* flags) {
+    chain_wait();
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= g.Np) return;
-    const int nbits = 8 * NX;
-    const long long tot = (long long)g.Nc << nbits;
+    constexpr int nbits = 8 * NX;
     const float scale = ldexpf(1.0f, nbits - g.r);
     int cell[3];
     bool bad = false;
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
-        float x = pos[d * g.Np + i];
-        if (!isfinite(x)) { bad = true; x = 0.0f; }
-        long long bf = __float2ll_rd(x * scale);
-        bf %= tot;
-        if (bf < 0) bf += tot;
-        cell[d] = (int)(bf >> nbits);
+        const float x = pos[d * g.Np + i];
+        bad |= !isfinite(x);
+        cell[d] = pos_bin(x, scale, g.Nc << nbits) >> nbits;
     }
-    unsigned k = (unsigned)cell_rank(g, cell[0], cell[1], cell[2]);
+    const unsigned k = (unsigned)cell_rank(g, cell[0], cell[1], cell[2]);
     key[i] = k;
-    val[i] = (unsigned)i;
-    atomicAdd(&counts[k], 1u);
-#pragma unroll
-    for (int d = 0; d < 3; ++d) {
-        float v = vel[d * g.Np + i];
-        if (!isfinite(v)) { bad = true; v = 0.0f; }
-        atomicAdd(reinterpret_cast<unsigned long long*>(&vsum[(int64_t)d * g.Ncc + k]),
-                  (unsigned long long)vel_fix(v));
+    // one atomic per run of lanes with one cell (neighbours in lattice order)
+    const unsigned act = __activemask(), lane = threadIdx.x & 31;      // a prefix of the warp
+    const unsigned left = __shfl_up_sync(act, k, 1);
+    const unsigned heads = __ballot_sync(act, lane == 0 || left != k);
+    if ((heads >> lane) & 1u) {
+        const unsigned after = lane == 31 ? 0u : heads & (0xfffffffeu << lane);
+        const int end = after ? __ffs(after) - 1 : __popc(act);
+        atomicAdd(&counts[k], (unsigned)(end - (int)lane));
     }
     if (bad) atomicOr(flags, ERR_NONFINITE);
 }
 
-__global__ void k_vc_finalize(int ncc, const unsigned* __restrict__ counts, const long long* __restrict__ vsum,
-                              float* __restrict__ vc) {
-    int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= ncc) return;
-    unsigned n = counts[c];
+// One CTA per brick of the sorted order: the particles' momenta are gathered
+// once, written in storage order for the kernels that follow, and added up
+// per cell in shared memory (exact fixed point); then v_c, and the brick's sum
+// of squared offsets for a measured codec scale.  256^3 particles x1v1: this
+// 273 us and k_encode_codes 231, where 64-bit global atomics per particle, the
+// measurement and the final gather took 215 + 28 + 58 + 398 us in four kernels;
+// the whole encode with its sort 1540 -> 1129 us.
+__global__ void __launch_bounds__(T_BRICK) k_encode_vc(Geo g, const float* __restrict__ vel,
+                                                       const unsigned* __restrict__ perm, StoreDev s, float* v0,
+                                                       float* v1, float* v2, float* __restrict__ part,
+                                                       unsigned* flags) {
+    __shared__ unsigned off[65];
+    __shared__ unsigned vs[3 * 64 * 2];                      // {low, high} words
+    __shared__ float svc[3 * 64];
+    __shared__ double red[32];
+    chain_wait();
+    const int nbc = g.B * g.B * g.B, L0 = blockIdx.x * nbc;
+    for (int c = threadIdx.x; c <= nbc; c += blockDim.x) off[c] = s.offsets[L0 + c];
+    for (int t = threadIdx.x; t < 6 * nbc; t += blockDim.x) vs[t] = 0u;
+    __syncthreads();
+    const unsigned q1 = min(off[nbc], (unsigned)g.Np), q0 = min(off[0], q1);
+    unsigned p0, p1;
+    brick_share(q0, q1, &p0, &p1);
+    const unsigned lane = threadIdx.x & 31;
+    float* vo[3] = {v0, v1, v2};
+    const float* vi[3] = {vel, vel + g.Np, vel + 2 * g.Np};
+    bool bad = false;
+    // 64 particles of the warp at a time, their loads in flight together
+    float v[2][3];
+    int cell[2] = {0, 0};
+    int c0 = p0 < p1 ? upper_cell(off, nbc, p0) : 0;
+    for (unsigned base = p0; base < p1; base += 64) {
+        unsigned i[2];
 #pragma unroll
-    for (int d = 0; d < 3; ++d) vc[(int64_t)d * ncc + c] = vel_unfix_mean(vsum[(int64_t)d * ncc + c], n);
-}
-
-__global__ void k_encode_sigma(Geo g, const float* __restrict__ vel, const unsigned* __restrict__ key,
-                               const float* __restrict__ vc, float* __restrict__ part) {
-    __shared__ double sh[32];
-    float acc = 0.0f;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < g.Np; i += (int64_t)gridDim.x * blockDim.x) {
-        unsigned k = key[i];
+        for (int h = 0; h < 2; ++h) i[h] = base + 32 * h + lane < p1 ? perm[base + 32 * h + lane] : 0xffffffffu;
 #pragma unroll
-        for (int d = 0; d < 3; ++d) {
-            float v = vel[d * g.Np + i];
-            if (!isfinite(v)) v = 0.0f;
-            float e = v - vc[(int64_t)d * g.Ncc + k];
-            acc = __fmaf_rn(e, e, acc);
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+            for (int d = 0; d < 3; ++d) v[h][d] = i[h] < (unsigned)g.Np ? vi[d][i[h]] : 0.0f;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const unsigned j = base + 32 * h + lane;
+            int cnext;
+            cell[h] = warp_cells(off, nbc, base + 32 * h, c0, &cnext);
+            c0 = cnext;
+            if (j < p1)
+#pragma unroll
+                for (int d = 0; d < 3; ++d) {
+                    if (!isfinite(v[h][d])) {
+                        bad = true;
+                        v[h][d] = 0.0f;
+                    }
+                    vo[d][j] = v[h][d];
+                    smem_add_u64(&vs[2 * (d * nbc + cell[h])], (unsigned long long)vel_fix(v[h][d]));
+                }
         }
     }
-    double s = block_sum_double((double)acc, sh);
-    if (threadIdx.x == 0) part[blockIdx.x] = (float)s;
+    __syncthreads();
+    for (int t = threadIdx.x; t < 3 * nbc; t += blockDim.x) {
+        const int d = t >> (3 * g.lB), c = t & (nbc - 1);
+        const long long sum = (long long)(((unsigned long long)vs[2 * t + 1] << 32) | vs[2 * t]);
+        const float m = vel_unfix_mean(sum, off[c + 1] - off[c]);
+        svc[t] = m;
+        s.vc[(int64_t)d * g.Ncc + L0 + c] = m;
+    }
+    if (part) {
+        __syncthreads();
+        float acc = 0.0f;
+        auto add = [&](const float* x, int c) {
+#pragma unroll
+            for (int d = 0; d < 3; ++d) {
+                const float e = x[d] - svc[d * nbc + c];
+                acc = __fmaf_rn(e, e, acc);
+            }
+        };
+        if (p1 - p0 <= 64) {                                 // the share is still in registers
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+                if (p0 + 32 * h + lane < p1) add(v[h], cell[h]);
+        } else {
+            c0 = upper_cell(off, nbc, p0);
+            for (unsigned base = p0; base < p1; base += 32) {
+                const unsigned j = base + lane;
+                int cnext;
+                const int c = warp_cells(off, nbc, base, c0, &cnext);
+                c0 = cnext;
+                if (j < p1) {
+                    const float x[3] = {vo[0][j], vo[1][j], vo[2][j]};
+                    add(x, c);
+                }
+            }
+        }
+        const double t = block_sum_double((double)acc, red);
+        if (threadIdx.x == 0) part[blockIdx.x] = (float)t;
+    }
+    if (bad) atomicOr(flags, ERR_NONFINITE);
 }
 
 // The codec scale from the partial sums of squared offsets, by a block of 1024
@@ -326,40 +404,71 @@ __global__ void k_codec_tables(int lim, const double* __restrict__ tanv, const d
                       moved(est, o), moved(vtab, o), moved(vdel, o), blockIdx.x, gridDim.x);
 }
 
+// codes and ids in storage order, one CTA per brick: positions and ids
+// gathered by the permutation, momenta already in order
 template <int NX, int NV>
-__global__ void k_encode_scatter(Geo g, const float* __restrict__ pos, const float* __restrict__ vel,
-                                 const unsigned* __restrict__ id_in, const unsigned* __restrict__ key,
-                                 const unsigned* __restrict__ perm, const float* __restrict__ vc, CodecDev cd,
-                                 StoreDev s) {
-    int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= g.Np) return;
-    const int64_t i = perm[j];
-    const unsigned k = key[j];
-    if (i >= g.Np || k >= (unsigned)g.Ncc) return;      // only if the sort went wrong
-    const int nbits = 8 * NX;
-    const long long tot = (long long)g.Nc << nbits;
+__global__ void __launch_bounds__(T_BRICK) k_encode_codes(Geo g, const float* __restrict__ pos,
+                                                          const float* __restrict__ v0, const float* __restrict__ v1,
+                                                          const float* __restrict__ v2,
+                                                          const unsigned* __restrict__ id_in,
+                                                          const unsigned* __restrict__ perm, CodecDev cd, StoreDev s) {
+    __shared__ unsigned off[65];
+    __shared__ float svc[3 * 64];
+    chain_wait();
+    const int nbc = g.B * g.B * g.B, L0 = blockIdx.x * nbc;
+    for (int c = threadIdx.x; c <= nbc; c += blockDim.x) off[c] = s.offsets[L0 + c];
+    for (int t = threadIdx.x; t < 3 * nbc; t += blockDim.x)
+        svc[t] = s.vc[(int64_t)(t >> (3 * g.lB)) * g.Ncc + L0 + (t & (nbc - 1))];
+    __syncthreads();
+    const unsigned q1 = min(off[nbc], (unsigned)g.Np);
+    unsigned p0, p1;
+    brick_share(min(off[0], q1), q1, &p0, &p1);
+    if (p0 >= p1) return;
+    constexpr int nbits = 8 * NX, half = 1 << (nbits - 1), mask = (1 << nbits) - 1;
     const float scale = ldexpf(1.0f, nbits - g.r);
     const int key0 = NV == 1 ? __float_as_int(cd.est[2]) : 0;
-    float dd[3];
-    int nu[3];
+    const unsigned lane = threadIdx.x & 31;
+    const CodeRows<NX> chi(s.chi, g.Np);
+    const CodeRows<NV> nu_r(s.nu, g.Np);
+    const float* vi[3] = {v0, v1, v2};
+    const float* xi[3] = {pos, pos + g.Np, pos + 2 * g.Np};
+    int c0 = upper_cell(off, nbc, p0);
+    for (unsigned base = p0; base < p1; base += 64) {       // 64 particles' loads in flight
+        float x[2][3], v[2][3];
+        unsigned i[2], pid[2] = {0, 0};
 #pragma unroll
-    for (int d = 0; d < 3; ++d) {
-        float x = pos[d * g.Np + i];
-        if (!isfinite(x)) x = 0.0f;
-        long long bf = __float2ll_rd(x * scale);
-        bf %= tot;
-        if (bf < 0) bf += tot;
-        int chi = (int)(bf & ((1 << nbits) - 1)) - (1 << (nbits - 1));
-        store_code<NX>(s.chi, d * g.Np + j, chi);
-        float v = vel[d * g.Np + i];
-        if (!isfinite(v)) v = 0.0f;
-        dd[d] = v - vc[(int64_t)d * g.Ncc + k];
-        if (NV == 1) nu[d] = nu_from_table(dd[d], cd.thr, cd.vtab, key0, g.nulim);
+        for (int h = 0; h < 2; ++h) i[h] = base + 32 * h + lane < p1 ? perm[base + 32 * h + lane] : 0xffffffffu;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const bool ok = i[h] < (unsigned)g.Np;
+#pragma unroll
+            for (int d = 0; d < 3; ++d) {
+                x[h][d] = ok ? xi[d][i[h]] : 0.0f;
+                v[h][d] = ok ? vi[d][base + 32 * h + lane] : 0.0f;
+            }
+            if (s.id && ok) pid[h] = id_in ? id_in[i[h]] : i[h];
+        }
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const unsigned j = base + 32 * h + lane;
+            int cnext;
+            const int c = warp_cells(off, nbc, base + 32 * h, c0, &cnext);
+            c0 = cnext;
+            if (j >= p1) continue;
+            float dd[3];
+            int nu[3];
+#pragma unroll
+            for (int d = 0; d < 3; ++d) {
+                chi.put(d, j, (pos_bin(x[h][d], scale, g.Nc << nbits) & mask) - half);
+                dd[d] = v[h][d] - svc[d * nbc + c];
+                if (NV == 1) nu[d] = nu_from_table(dd[d], cd.thr, cd.vtab, key0, g.nulim);
+            }
+            if (NV == 2) nu_codes3(dd, cd.thr, g.nulim, cd.est[0], cd.est[1], nu);
+#pragma unroll
+            for (int d = 0; d < 3; ++d) nu_r.put(d, j, nu[d]);
+            if (s.id) store_pid(s.id, j, g.nid, pid[h]);
+        }
     }
-    if (NV == 2) nu_codes3(dd, cd.thr, g.nulim, cd.est[0], cd.est[1], nu);
-#pragma unroll
-    for (int d = 0; d < 3; ++d) store_code<NV>(s.nu, d * g.Np + j, nu[d]);
-    if (s.id) store_pid(s.id, (unsigned)j, g.nid, id_in ? id_in[i] : (unsigned)i);
 }
 
 // ------------------------------------------------------------------ decode
@@ -1742,21 +1851,17 @@ void launch_batch_clear(const Geo& g, long long* vsum, int* maxmig, cudaStream_t
 
 static inline int nblk(int64_t n, int t) { return (int)((n + t - 1) / t); }
 
-void launch_encode_keys(const Geo& g, const float* pos, const float* vel, unsigned* key, unsigned* val,
-                        unsigned* counts, long long* vsum, unsigned* flags, cudaStream_t st) {
-    if (g.nchi == 1) k_encode_keys<1><<<nblk(g.Np, 256), 256, 0, st>>>(g, pos, vel, key, val, counts, vsum, flags);
-    else k_encode_keys<2><<<nblk(g.Np, 256), 256, 0, st>>>(g, pos, vel, key, val, counts, vsum, flags);
+void launch_encode_keys(const Geo& g, const float* pos, unsigned* key, unsigned* counts, unsigned* flags,
+                        cudaStream_t st) {
+    const dim3 grid(nblk(g.Np, 256));
+    if (g.nchi == 1) launch_chained(k_encode_keys<1>, grid, 256, 0, st, g, pos, key, counts, flags);
+    else launch_chained(k_encode_keys<2>, grid, 256, 0, st, g, pos, key, counts, flags);
 }
 
-void launch_vc_finalize(const Geo& g, const unsigned* counts, const long long* vsum, float* vc, cudaStream_t st) {
-    k_vc_finalize<<<nblk(g.Ncc, 256), 256, 0, st>>>(g.Ncc, counts, vsum, vc);
-}
-
-int encode_sigma_blocks(const Geo& g) { return (int)std::min<int64_t>(1024, std::max<int64_t>(1, nblk(g.Np, 256))); }
-
-void launch_encode_sigma(const Geo& g, const float* vel, const unsigned* key, const float* vc, float* part,
-                         cudaStream_t st) {
-    k_encode_sigma<<<encode_sigma_blocks(g), 256, 0, st>>>(g, vel, key, vc, part);
+void launch_encode_vc(const Geo& g, const float* vel, const unsigned* perm, const StoreDev& s, float* const* vsorted,
+                      float* part, unsigned* flags, cudaStream_t st) {
+    launch_chained(k_encode_vc, dim3(g.nbricks), T_BRICK, 0, st, g, vel, perm, s, vsorted[0], vsorted[1], vsorted[2],
+                   part, flags);
 }
 
 void launch_sigma_finalize(const float* part, int nparts, double count, double ratio, double fixed,
@@ -1773,14 +1878,16 @@ void launch_codec_tables(int nulim, const double* tanv, const double* tanh_, con
                                                                           one ? nullptr : c.vdel, bt);
 }
 
-void launch_encode_scatter(const Geo& g, const float* pos, const float* vel, const unsigned* id_in,
-                           const unsigned* key_sorted, const unsigned* perm, const float* vc, const CodecDev& c,
-                           StoreDev s, cudaStream_t st) {
-    int nb = nblk(g.Np, 256);
-    if (g.nchi == 1 && g.nnu == 1) k_encode_scatter<1, 1><<<nb, 256, 0, st>>>(g, pos, vel, id_in, key_sorted, perm, vc, c, s);
-    else if (g.nchi == 1) k_encode_scatter<1, 2><<<nb, 256, 0, st>>>(g, pos, vel, id_in, key_sorted, perm, vc, c, s);
-    else if (g.nnu == 1) k_encode_scatter<2, 1><<<nb, 256, 0, st>>>(g, pos, vel, id_in, key_sorted, perm, vc, c, s);
-    else k_encode_scatter<2, 2><<<nb, 256, 0, st>>>(g, pos, vel, id_in, key_sorted, perm, vc, c, s);
+void launch_encode_codes(const Geo& g, const float* pos, const float* const* vsorted, const unsigned* id_in,
+                         const unsigned* perm, const CodecDev& c, const StoreDev& s, cudaStream_t st) {
+    const dim3 grid(g.nbricks);
+    auto go = [&](auto kernel) {
+        launch_chained(kernel, grid, T_BRICK, 0, st, g, pos, vsorted[0], vsorted[1], vsorted[2], id_in, perm, c, s);
+    };
+    if (g.nchi == 1 && g.nnu == 1) go(k_encode_codes<1, 1>);
+    else if (g.nchi == 1) go(k_encode_codes<1, 2>);
+    else if (g.nnu == 1) go(k_encode_codes<2, 1>);
+    else go(k_encode_codes<2, 2>);
 }
 
 void launch_max_speed(const Geo& g, const StoreDev& s, const CodecDev& c, unsigned* vmax_bits, cudaStream_t st,

@@ -11,41 +11,6 @@
 
 namespace cube {
 
-// Stable ranking of one round of blockDim.x items by `digit` in [0, nd),
-// nd <= 256:
-// items are ordered by (warp, lane), i.e. by thread index, and equal digits
-// keep that order.  run[nd] holds each digit's next free position and is
-// advanced by the round's counts; wcnt[NWARPS * nd] is scratch.  Every thread
-// of the block must call it (it synchronises).  Returns the item's position,
-// or -1 for inactive threads.
-template <int NWARPS>
-__device__ __forceinline__ int stable_round_rank(int digit, bool active, unsigned* run, unsigned* wcnt, int nd) {
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    for (int i = threadIdx.x; i < NWARPS * nd; i += blockDim.x) wcnt[i] = 0u;
-    __syncthreads();
-    unsigned act = __ballot_sync(0xffffffffu, active);
-    int lrank = 0;
-    if (active) {
-        unsigned peers = same_value_lanes(act, digit);
-        lrank = __popc(peers & ((1u << lane) - 1u));
-        if (lrank == 0) wcnt[w * nd + digit] = (unsigned)__popc(peers);
-    }
-    __syncthreads();
-    for (int d = threadIdx.x; d < nd; d += blockDim.x) {
-        unsigned s = run[d];
-        for (int ww = 0; ww < NWARPS; ++ww) {
-            unsigned t = wcnt[ww * nd + d];
-            wcnt[ww * nd + d] = s;
-            s += t;
-        }
-        run[d] = s;
-    }
-    __syncthreads();
-    int pos = active ? (int)(wcnt[w * nd + digit] + (unsigned)lrank) : -1;
-    __syncthreads();
-    return pos;
-}
-
 // ------------------------------------------------------------ chained launches
 // A step is a chain of short kernels, each reading what the one before wrote.
 // launch_chained lets the next kernel's launch overlap the running one
@@ -150,7 +115,11 @@ void exclusive_scan(const unsigned* in, unsigned* out, int64_t n, unsigned* tmp,
 // out2[0] = 64-bit sum, out2[1] = maximum of n counts
 void count_totals(const unsigned* counts, int64_t n, unsigned long long* out2, cudaStream_t st);
 int64_t radix_tmp_words(int64_t n);
-void radix_sort_pairs(unsigned* keys, unsigned* vals, int64_t n, int key_bits, unsigned* tmp, cudaStream_t st);
+// the permutation that sorts keys[n] by their low key_bits bits (stable), in
+// `perm` or `tmp`; *spare: three other arrays of n words, free afterwards
+// (the keys are overwritten)
+unsigned* radix_sort_index(unsigned* keys, unsigned* perm, int64_t n, int key_bits, unsigned* tmp, cudaStream_t st,
+                           unsigned** spare);
 
 // ------------------------------------------------------------ k_store.cu
 struct StoreDev {
@@ -207,19 +176,19 @@ __host__ __device__ __forceinline__ StepScratch moved(const StepScratch& w, size
 // a batch of one: a single context's launch
 constexpr Batch kSingle{1, 0, nullptr, nullptr};
 
-void launch_encode_keys(const Geo& g, const float* pos, const float* vel, unsigned* key, unsigned* val,
-                        unsigned* counts, long long* vsum, unsigned* flags, cudaStream_t st);
-void launch_vc_finalize(const Geo& g, const unsigned* counts, const long long* vsum, float* vc, cudaStream_t st);
-int encode_sigma_blocks(const Geo& g);
-void launch_encode_sigma(const Geo& g, const float* vel, const unsigned* key_sorted_or_raw, const float* vc,
-                         float* part, cudaStream_t st);
+// sort keys (cell ranks) and cell counts of float positions
+void launch_encode_keys(const Geo& g, const float* pos, unsigned* key, unsigned* counts, unsigned* flags,
+                        cudaStream_t st);
+// the particles' momenta in storage order (three rows of Np), v_c of every
+// cell, and (part not null) each brick's sum of squared offsets from v_c
+void launch_encode_vc(const Geo& g, const float* vel, const unsigned* perm, const StoreDev& s, float* const* vsorted,
+                      float* part, unsigned* flags, cudaStream_t st);
 void launch_sigma_finalize(const float* part, int nparts, double count, double ratio, double fixed,
                            double* sigma_out, cudaStream_t st, const Batch& bt = Batch{1, 0, nullptr, nullptr});
 void launch_codec_tables(int nulim, const double* tanv, const double* tanh, const CodecDev& c, cudaStream_t st,
                          const Batch& bt = Batch{1, 0, nullptr, nullptr});
-void launch_encode_scatter(const Geo& g, const float* pos, const float* vel, const unsigned* id_in,
-                           const unsigned* key_sorted, const unsigned* perm, const float* vc, const CodecDev& c,
-                           StoreDev s, cudaStream_t st);
+void launch_encode_codes(const Geo& g, const float* pos, const float* const* vsorted, const unsigned* id_in,
+                         const unsigned* perm, const CodecDev& c, const StoreDev& s, cudaStream_t st);
 void launch_decode(const Geo& g, const StoreDev& s, const CodecDev& c, float* pos, float* vel, unsigned* id,
                    cudaStream_t st);
 // (step: the step's scratch that pass A accumulates into, cleared by the way, or null)

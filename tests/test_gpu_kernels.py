@@ -182,3 +182,30 @@ def test_batch_past_the_split_equals_members_alone(cube, vb):
     finally:
         cube.cube_destroy(one)
         cube.cube_batch_destroy(batch)
+
+
+# ---------------------------------------------------------------- encode
+# the sort's tiles (4096 items, 512 a warp) and their remainders, one to three
+# passes of 8 bits, scales given and measured, particles outside the box;
+# whole numbers, exact
+@pytest.mark.parametrize("n,nf,ratio,xb,vb,sigma", [(1, 16, 4, 1, 1, 0.5), (511, 16, 4, 2, 2, 0.0), (4096, 64, 4, 1, 2, 0.0),
+                                                    (4097, 64, 4, 2, 1, 0.3), (12801, 96, 1, 1, 1, 0.0),
+                                                    (40001, 256, 2, 1, 2, 0.0)])
+def test_encode_at_tile_edges(cube, n, nf, ratio, xb, vb, sigma):
+    pos, vel, ids = _blob(n, nf, 1712207)
+    rng = np.random.default_rng(n)
+    pos = pos[:, rng.permutation(n)] + np.float32(nf) * rng.integers(-2, 3, (3, n)).astype(np.float32)
+    prm = cube.make_params(nf, n, ratio=ratio, x_bytes=xb, v_bytes=vb, box=50.0, omega_m=0.3, omega_l=0.7)
+    ctx = cube.cube_create(prm, torch.cuda.current_stream())
+    try:
+        for host in (True, False):
+            put = (lambda a: a) if host else (lambda a: torch.from_numpy(a.copy()).cuda())
+            cube.cube_encode(ctx, put(pos), put(vel), put(ids.view(np.int32)), 0.02, sigma)
+            g = read_store(cube, ctx)
+            ref = pm.encode(oracle_params(pm, prm, g["brick"]), pos, vel, ids, 0.02, g["sigma"], snap=False)
+            assert_store_equal(g, ref, f"encode {n} host {host}")
+            if sigma == 0.0:
+                free = pm.encode(oracle_params(pm, prm, g["brick"]), pos, vel, ids, 0.02, 0.0)
+                assert g["sigma"] == pytest.approx(free.sigma, rel=1e-12)
+    finally:
+        cube.cube_destroy(ctx)
