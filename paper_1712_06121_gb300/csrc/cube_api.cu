@@ -5,6 +5,7 @@
 #include <cstring>
 #include <functional>
 #include <map>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -175,6 +176,55 @@ bool is_device_ptr(const void* p) {
     return at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged;
 }
 
+// 64-byte lines of pinned host memory for the contexts' small read-backs, from
+// 4 KB chunks: creating and releasing a context (a server does so while others
+// run) neither allocates pinned memory nor frees it, both of which can wait for
+// the device.  One empty chunk at most is kept.  Every use of a line ends with
+// a stream synchronisation, so a returned line has no copy in flight.
+struct LineChunk {
+    char* base;
+    uint64_t used;                       // bit i: line i is taken
+};
+std::mutex g_lines_mu;
+std::vector<LineChunk> g_lines;
+
+cudaError_t pinned_line(unsigned** out) {
+    std::lock_guard<std::mutex> lock(g_lines_mu);
+    for (LineChunk& ch : g_lines)
+        if (~ch.used) {
+            const int i = __builtin_ctzll(~ch.used);
+            ch.used |= 1ull << i;
+            *out = (unsigned*)(ch.base + 64 * i);
+            return cudaSuccess;
+        }
+    char* p = nullptr;
+    const cudaError_t e = cudaHostAlloc((void**)&p, 4096, cudaHostAllocPortable);
+    if (e != cudaSuccess) return e;
+    g_lines.push_back(LineChunk{p, 1ull});
+    *out = (unsigned*)p;
+    return cudaSuccess;
+}
+
+void return_line(unsigned* line) {
+    char* freed = nullptr;
+    {
+        std::lock_guard<std::mutex> lock(g_lines_mu);
+        int empty = 0;
+        for (const LineChunk& ch : g_lines) empty += ch.used == 0;
+        for (size_t k = 0; k < g_lines.size(); ++k) {
+            LineChunk& ch = g_lines[k];
+            if ((char*)line < ch.base || (char*)line >= ch.base + 4096) continue;
+            ch.used &= ~(1ull << (((char*)line - ch.base) / 64));
+            if (ch.used == 0 && empty) {
+                freed = ch.base;
+                g_lines.erase(g_lines.begin() + k);
+            }
+            break;
+        }
+    }
+    if (freed) cudaFreeHost(freed);
+}
+
 bool is_2a3b(int n) {
     if (n <= 0) return false;
     while (n % 2 == 0) n /= 2;
@@ -213,6 +263,7 @@ struct cube_ctx {
     float* part = nullptr;
     int npart = 0;
     unsigned* flags = nullptr;
+    unsigned* line = nullptr;       // pinned, 64 bytes: small read-backs
     int* maxmig = nullptr;
     bool phig_valid = false;        // phig holds the potential of the last step or cube_potential call
     unsigned* scan_tmp = nullptr;
@@ -296,10 +347,10 @@ size_t state_layout(cube_ctx* c, char* base) {
     }
     carve(base, off, c->tanv, (size_t)(g.nulim + 1) * 8);
     carve(base, off, c->tanh_, (size_t)(g.nulim + 2) * 8);
-    carve(base, off, c->flags, 4);
+    carve(base, off, c->flags, 8);                               // error flags, then vmax: one read-back
+    c->vmax = base ? c->flags + 1 : nullptr;
     carve(base, off, c->maxmig, ((size_t)g.nbricks + 2) * 4);    // [0] max migration, [1 ..] crowded-brick list
     carve(base, off, c->mom, 4 * 8);
-    carve(base, off, c->vmax, 4);
     FftPlan& f = c->fft;
     carve(base, off, f.tw, (size_t)g.N * 8);
     carve(base, off, f.k2, (size_t)g.N * 4);
@@ -360,11 +411,26 @@ cube_status flags_status(unsigned f) {
     return CUBE_OK;
 }
 
-cube_status latched(cube_ctx* c) {
-    unsigned f = 0;
-    CK(cudaMemcpyAsync(&f, c->flags, sizeof(unsigned), cudaMemcpyDeviceToHost, c->st));
+// `bytes` (at most 64) of src in the context's pinned line, stream-ordered and waited for
+cube_status read_back(cube_ctx* c, const void* src, size_t bytes) {
+    CK(cudaMemcpyAsync(c->line, src, bytes, cudaMemcpyDefault, c->st));
     CK(cudaStreamSynchronize(c->st));
-    return flags_status(f);
+    return CUBE_OK;
+}
+
+cube_status latched(cube_ctx* c) {
+    cube_status s = read_back(c, c->flags, 4);
+    return s == CUBE_OK ? flags_status(c->line[0]) : s;
+}
+
+// the maximum in vmax (float bits) and the latched errors, in one copy
+cube_status read_vmax(cube_ctx* c, double* out) {
+    cube_status s = read_back(c, c->flags, 8);
+    if (s != CUBE_OK) return s;
+    float f;
+    std::memcpy(&f, &c->line[1], 4);
+    *out = f;
+    return flags_status(c->line[0]);
 }
 
 // TMA descriptor of the ghosted Phi: a 3-D float tensor (x, y, z extents
@@ -484,6 +550,7 @@ cube_status cube_destroy(cube_ctx* c) {
     if (c->dbg_p) cudaFree(c->dbg_p);
     if (c->dbg_f) cudaFree(c->dbg_f);
     for (cudaEvent_t e : c->prof_ev) cudaEventDestroy(e);
+    if (c->line) return_line(c->line);
     if (c->ev0) cudaEventDestroy(c->ev0);
     if (c->ev1) cudaEventDestroy(c->ev1);
     delete c;
@@ -563,6 +630,7 @@ static cube_status create_ctx(const cube_params* params, void* cuda_stream, bool
         if (e == cudaSuccess) e = cudaMemcpyAsync(c->tanv, tv.data(), tv.size() * 8, cudaMemcpyHostToDevice, c->st);
         if (e == cudaSuccess) e = cudaMemcpyAsync(c->tanh_, th.data(), th.size() * 8, cudaMemcpyHostToDevice, c->st);
         if (e == cudaSuccess) e = cudaMemsetAsync(c->flags, 0, 4, c->st);
+        if (e == cudaSuccess) e = pinned_line(&c->line);
         if (e == cudaSuccess) e = cudaEventCreate(&c->ev0);
         if (e == cudaSuccess) e = cudaEventCreate(&c->ev1);
         if (e != cudaSuccess) return bad(e, "table upload");
@@ -884,13 +952,7 @@ cube_status cube_max_speed(cube_ctx* c, double* p_max) {
     if (c->raw) launch_raw_max_speed(g, (const float*)c->nu[0], c->vmax, c->st);
     else launch_max_speed(g, c->store(c->cur), c->codec[c->cur], c->vmax, c->st);
     c->launches += 1;
-    unsigned bits = 0;
-    CK(cudaMemcpyAsync(&bits, c->vmax, 4, cudaMemcpyDeviceToHost, c->st));
-    cube_status s = latched(c);
-    float f;
-    std::memcpy(&f, &bits, 4);
-    *p_max = f;
-    return s;
+    return read_vmax(c, p_max);
 }
 
 // largest a_to <= a_max with p * int_a^a_to da / (a^3 E) <= cells coarse cells
@@ -911,13 +973,7 @@ cube_status cube_max_force(cube_ctx* c, double* f_max) {
     if (!c->phig_valid) return CUBE_OK;
     launch_grad_max(c->phig, c->g.N, c->vmax, c->st);
     c->launches += 1;
-    unsigned bits = 0;
-    CK(cudaMemcpyAsync(&bits, c->vmax, 4, cudaMemcpyDeviceToHost, c->st));
-    cube_status s = latched(c);
-    float f;
-    std::memcpy(&f, &bits, 4);
-    *f_max = f;
-    return s;
+    return read_vmax(c, f_max);
 }
 
 static cube_status check_limits(const cube_step_limits* lim) {
@@ -1096,8 +1152,9 @@ cube_status cube_checkpoint_load(cube_ctx* c, const void* buf) {
     if (!c || !buf) return fail(CUBE_E_ARG, "NULL argument");
     const Geo& g = c->g;
     CkptHeader h{};
-    CK(cudaMemcpyAsync(&h, buf, sizeof(h), cudaMemcpyDefault, c->st));
-    CK(cudaStreamSynchronize(c->st));
+    cube_status hs = read_back(c, buf, sizeof(h));
+    if (hs != CUBE_OK) return hs;
+    std::memcpy(&h, c->line, sizeof(h));
     if (std::memcmp(h.magic, "CUBECKP1", 8) != 0) return fail(CUBE_E_ARG, "not a checkpoint (magic)");
     if (h.n_fine != g.N || h.ratio != g.R || h.n_particles != g.Np || h.brick != g.B ||
         h.x_bytes != (c->raw ? 4 : g.nchi) || h.v_bytes != (c->raw ? 4 : g.nnu) || h.id_bytes != c->P.id_bytes)
@@ -1134,10 +1191,11 @@ cube_status cube_checkpoint_load(cube_ctx* c, const void* buf) {
     if (!c->raw) {
         count_totals(c->counts[k], g.Ncc, reinterpret_cast<unsigned long long*>(c->mom), c->st);
         c->launches += 1;
-        CK(cudaMemcpyAsync(tot, c->mom, sizeof(tot), cudaMemcpyDeviceToHost, c->st));
     }
     CK(cudaGetLastError());
-    CK(cudaStreamSynchronize(c->st));
+    hs = read_back(c, c->mom, sizeof(tot));
+    if (hs != CUBE_OK) return hs;
+    if (!c->raw) std::memcpy(tot, c->line, sizeof(tot));
     c->phig_valid = false;
     c->a = h.a;
     c->a_p = h.a_p;
