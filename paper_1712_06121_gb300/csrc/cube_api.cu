@@ -225,6 +225,16 @@ void return_line(unsigned* line) {
     if (freed) cudaFreeHost(freed);
 }
 
+// p can be read and written by kernels of `device`, 16 bytes at a time
+bool kernel_aligned(const void* p, int device) {
+    cudaPointerAttributes at;
+    if (((uintptr_t)p & 15) || cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return at.type == cudaMemoryTypeManaged || (at.type == cudaMemoryTypeDevice && at.device == device);
+}
+
 bool is_2a3b(int n) {
     if (n <= 0) return false;
     while (n % 2 == 0) n /= 2;
@@ -347,9 +357,10 @@ size_t state_layout(cube_ctx* c, char* base) {
     }
     carve(base, off, c->tanv, (size_t)(g.nulim + 1) * 8);
     carve(base, off, c->tanh_, (size_t)(g.nulim + 2) * 8);
-    carve(base, off, c->flags, 8);                               // error flags, then vmax: one read-back
+    // error flags and vmax (one read-back), largest migration, crowded-brick list
+    carve(base, off, c->flags, ((size_t)g.nbricks + 4) * 4);
     c->vmax = base ? c->flags + 1 : nullptr;
-    carve(base, off, c->maxmig, ((size_t)g.nbricks + 2) * 4);    // [0] max migration, [1 ..] crowded-brick list
+    c->maxmig = base ? (int*)(c->flags + 2) : nullptr;
     carve(base, off, c->mom, 4 * 8);
     FftPlan& f = c->fft;
     carve(base, off, f.tw, (size_t)g.N * 8);
@@ -726,7 +737,7 @@ static cube_status encode_impl(cube_ctx* c, const float* pos, const float* vel, 
                           c->codec[k].sigma, c->st);
     launch_codec_tables(g.nulim, c->tanv, c->tanh_, c->codec[k], c->st);
     launch_encode_codes(g, dpos, vsorted, did, order, c->codec[k], store, c->st);
-    c->launches += 1 + 4 + (int64_t)((key_bits + 7) / 8) * 6 + 1 + 1 + 1 + 1;
+    c->launches += 1 + scan_launches(g.Ncc) + radix_launches(g.Np, key_bits) + 4;
     CK(cudaGetLastError());
     if (sync) CK(cudaStreamSynchronize(c->st));
     c->encoded = true;
@@ -1097,6 +1108,24 @@ size_t ckpt_layout(const Geo& g, bool raw, int id_bytes, size_t sec[5]) {
     return off;
 }
 
+// the checkpoint's sections between buf and the store's buffer k
+SectionCopy sections(cube_ctx* c, int k, char* buf, const size_t sec[5], bool save) {
+    const Geo& g = c->g;
+    const int64_t N = g.Np, Ncc = g.Ncc;
+    char* own[5] = {c->raw ? (char*)c->chi[0] : (char*)c->counts[k], c->raw ? (char*)c->nu[0] : (char*)c->vc[k],
+                    (char*)c->chi[k], (char*)c->nu[k], (char*)c->id[k]};
+    const int64_t sz[5] = {c->raw ? 12 * N : 4 * Ncc, 12 * (c->raw ? N : Ncc), c->raw ? 0 : 3 * N * g.nchi,
+                           c->raw ? 0 : 3 * N * g.nnu, c->P.id_bytes * N};
+    SectionCopy cp{};
+    for (int i = 0; i < 5; ++i) {
+        if (!sz[i]) continue;
+        cp.dst[cp.n] = save ? buf + sec[i] : own[i];
+        cp.src[cp.n] = save ? own[i] : buf + sec[i];
+        cp.bytes[cp.n++] = sz[i];
+    }
+    return cp;
+}
+
 }  // namespace
 
 cube_status cube_checkpoint_size(const cube_params* params, int64_t* bytes) {
@@ -1130,10 +1159,20 @@ cube_status cube_checkpoint_save(cube_ctx* c, void* buf) {
     h.a = c->a;
     h.a_p = c->a_p;
     h.sigma = 0.0;
-    if (!c->raw) CK(cudaMemcpyAsync(&h.sigma, c->codec[k].sigma, 8, cudaMemcpyDeviceToHost, c->st));
-    CK(cudaStreamSynchronize(c->st));
     char* b = (char*)buf;
     const size_t N = (size_t)g.Np, Ncc = (size_t)g.Ncc;
+    if (kernel_aligned(buf, c->device)) {          // one launch, the scale from the device
+        SectionCopy cp = sections(c, k, b, sec, true);
+        cp.header_to = b;
+        std::memcpy(cp.header, &h, sizeof(h));
+        cp.sigma_from = c->raw ? nullptr : c->codec[k].sigma;
+        launch_section_copy(cp, c->st);
+        c->launches += 1;
+        CK(cudaGetLastError());
+        return latched(c);
+    }
+    if (!c->raw) CK(cudaMemcpyAsync(&h.sigma, c->codec[k].sigma, 8, cudaMemcpyDeviceToHost, c->st));
+    CK(cudaStreamSynchronize(c->st));
     CK(cudaMemcpyAsync(b, &h, sizeof(h), cudaMemcpyDefault, c->st));
     if (c->raw) {
         CK(cudaMemcpyAsync(b + sec[0], c->chi[0], 12 * N, cudaMemcpyDefault, c->st));
@@ -1168,29 +1207,40 @@ cube_status cube_checkpoint_load(cube_ctx* c, const void* buf) {
     c->cur = 0;                          // a loaded store starts in buffer 0, as an encoded one
     const int k = c->cur;
     c->encoded = false;                  // until the whole store is in place
-    if (c->raw) {
-        CK(cudaMemcpyAsync(c->chi[0], b + sec[0], 12 * N, cudaMemcpyDefault, c->st));
-        CK(cudaMemcpyAsync(c->nu[0], b + sec[1], 12 * N, cudaMemcpyDefault, c->st));
+    // the sections, the scale, and the latched errors and sums cleared
+    if (kernel_aligned(buf, c->device)) {          // in one launch
+        SectionCopy cp = sections(c, k, const_cast<char*>(b), sec, false);
+        cp.sigma_to = c->raw ? nullptr : c->codec[k].sigma;
+        cp.sigma = h.sigma;
+        cp.zero = c->flags;
+        cp.nzero = 3;
+        cp.zero64 = c->mom;
+        launch_section_copy(cp, c->st);
+        c->launches += 1;
     } else {
-        CK(cudaMemcpyAsync(c->counts[k], b + sec[0], 4 * Ncc, cudaMemcpyDefault, c->st));
-        CK(cudaMemcpyAsync(c->vc[k], b + sec[1], 12 * Ncc, cudaMemcpyDefault, c->st));
-        CK(cudaMemcpyAsync(c->chi[k], b + sec[2], 3 * N * g.nchi, cudaMemcpyDefault, c->st));
-        CK(cudaMemcpyAsync(c->nu[k], b + sec[3], 3 * N * g.nnu, cudaMemcpyDefault, c->st));
-        exclusive_scan(c->counts[k], c->offsets[k], g.Ncc, c->scan_tmp, c->st);
-        c->stage_sigma = h.sigma;
-        CK(cudaMemcpyAsync(c->codec[k].sigma, &c->stage_sigma, 8, cudaMemcpyHostToDevice, c->st));
-        launch_codec_tables(g.nulim, c->tanv, c->tanh_, c->codec[k], c->st);
-        c->launches += 4 + 1;
+        if (c->raw) {
+            CK(cudaMemcpyAsync(c->chi[0], b + sec[0], 12 * N, cudaMemcpyDefault, c->st));
+            CK(cudaMemcpyAsync(c->nu[0], b + sec[1], 12 * N, cudaMemcpyDefault, c->st));
+        } else {
+            CK(cudaMemcpyAsync(c->counts[k], b + sec[0], 4 * Ncc, cudaMemcpyDefault, c->st));
+            CK(cudaMemcpyAsync(c->vc[k], b + sec[1], 12 * Ncc, cudaMemcpyDefault, c->st));
+            CK(cudaMemcpyAsync(c->chi[k], b + sec[2], 3 * N * g.nchi, cudaMemcpyDefault, c->st));
+            CK(cudaMemcpyAsync(c->nu[k], b + sec[3], 3 * N * g.nnu, cudaMemcpyDefault, c->st));
+            c->stage_sigma = h.sigma;
+            CK(cudaMemcpyAsync(c->codec[k].sigma, &c->stage_sigma, 8, cudaMemcpyHostToDevice, c->st));
+        }
+        if (c->P.id_bytes) CK(cudaMemcpyAsync(c->id[k], b + sec[4], (size_t)c->P.id_bytes * N, cudaMemcpyDefault, c->st));
+        CK(cudaMemsetAsync(c->flags, 0, 12, c->st));                  // flags, vmax, largest migration
+        CK(cudaMemsetAsync(c->mom, 0, 16, c->st));
     }
-    if (c->P.id_bytes) CK(cudaMemcpyAsync(c->id[k], b + sec[4], (size_t)c->P.id_bytes * N, cudaMemcpyDefault, c->st));
-    CK(cudaMemsetAsync(c->flags, 0, 4, c->st));
-    CK(cudaMemsetAsync(c->maxmig, 0, 4, c->st));
     // the counts must add up to N_p in 64 bits, none above N_p (a sum that
     // only matches modulo 2^32 would pass a 32-bit check)
     unsigned long long tot[2] = {(unsigned long long)g.Np, 0ull};
     if (!c->raw) {
+        exclusive_scan(c->counts[k], c->offsets[k], g.Ncc, c->scan_tmp, c->st);
+        launch_codec_tables(g.nulim, c->tanv, c->tanh_, c->codec[k], c->st);
         count_totals(c->counts[k], g.Ncc, reinterpret_cast<unsigned long long*>(c->mom), c->st);
-        c->launches += 1;
+        c->launches += scan_launches(g.Ncc) + 2;
     }
     CK(cudaGetLastError());
     hs = read_back(c, c->mom, sizeof(tot));

@@ -60,6 +60,9 @@ __global__ void k_scan_bsums(unsigned* bsum, int nb, unsigned* total_out, Batch 
     if (threadIdx.x == 0 && total_out) *total_out = carry;
 }
 
+// SUMS: bsum holds the tiles' sums, not their scan: a block adds the ones
+// before its own, and the last one writes the total to out[n]
+template <bool SUMS>
 __global__ void k_scan_down(const unsigned* in, int64_t n, const unsigned* __restrict__ bsum, unsigned* out,
                             bool vec, Batch bt) {
     __shared__ unsigned sw[32];
@@ -73,10 +76,18 @@ __global__ void k_scan_down(const unsigned* in, int64_t n, const unsigned* __res
     unsigned v[SCAN_ITEMS];
     load4(in, base, n, vec, v);
     const unsigned s = v[0] + v[1] + v[2] + v[3];
-    unsigned tot;
+    unsigned tot, start;
+    if (SUMS) {
+        unsigned before = 0;
+        for (int j = threadIdx.x; j < (int)blockIdx.x; j += SCAN_T) before += bsum[j];
+        block_inclusive_scan(before, sw, &start);
+    } else {
+        start = bsum[blockIdx.x];
+    }
     const unsigned inc = block_inclusive_scan(s, sw, &tot);
+    if (SUMS && threadIdx.x == 0 && blockIdx.x == gridDim.x - 1) out[n] = start + tot;
     unsigned e[SCAN_ITEMS];
-    e[0] = bsum[blockIdx.x] + inc - s;
+    e[0] = start + inc - s;
 #pragma unroll
     for (int i = 1; i < SCAN_ITEMS; ++i) e[i] = e[i - 1] + v[i - 1];
     if (vec && base + 3 < n) {
@@ -97,6 +108,7 @@ __global__ void k_write_total(unsigned* out, int64_t n, const unsigned* total, B
 
 // 64-bit sum and maximum of n 32-bit counts: out2[0] += sum, out2[1] = max(out2[1], max)
 __global__ void k_count_totals(const unsigned* __restrict__ c, int64_t n, unsigned long long* out2) {
+    chain_wait();
     unsigned long long s = 0;
     unsigned m = 0;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
@@ -248,6 +260,8 @@ __global__ void __launch_bounds__(RX_T, 4) k_radix_scatter(const unsigned* __res
 
 int scan_tmp_words(int64_t n) { return (int)((n + SCAN_TILE - 1) / SCAN_TILE) + 1; }
 
+int scan_launches(int64_t n) { return (n + SCAN_TILE - 1) / SCAN_TILE <= 2048 ? 2 : 4; }
+
 void exclusive_scan(const unsigned* in, unsigned* out, int64_t n, unsigned* tmp, cudaStream_t st, const Batch& bt) {
     int nb = (int)((n + SCAN_TILE - 1) / SCAN_TILE);
     if (nb == 0) nb = 1;
@@ -255,15 +269,20 @@ void exclusive_scan(const unsigned* in, unsigned* out, int64_t n, unsigned* tmp,
     // (members are whole multiples of 256 bytes apart: the same alignment)
     const bool vec = ((reinterpret_cast<uintptr_t>(in) | reinterpret_cast<uintptr_t>(out)) & 15) == 0;
     launch_chained(k_scan_reduce, dim3(nb, bt.members), SCAN_T, 0, st, in, n, tmp, vec, bt);
+    // up to 2048 tiles (8 M items) the blocks add the earlier tiles' sums
+    // themselves: two launches instead of four.  (A batch keeps the four.)
+    if (nb <= 2048 && bt.members == 1 && !bt.ms) {
+        launch_chained(k_scan_down<true>, dim3(nb), SCAN_T, 0, st, in, n, tmp, out, vec, bt);
+        return;
+    }
     launch_chained(k_scan_bsums, dim3(bt.members), SCAN_T, 0, st, tmp, nb, total, bt);
-    launch_chained(k_scan_down, dim3(nb, bt.members), SCAN_T, 0, st, in, n, tmp, out, vec, bt);
+    launch_chained(k_scan_down<false>, dim3(nb, bt.members), SCAN_T, 0, st, in, n, tmp, out, vec, bt);
     launch_chained(k_write_total, dim3(bt.members), 1, 0, st, out, n, total, bt);
 }
 
 void count_totals(const unsigned* counts, int64_t n, unsigned long long* out2, cudaStream_t st) {
-    cudaMemsetAsync(out2, 0, 2 * sizeof(unsigned long long), st);
     const int64_t nb = (n + 255) / 256;
-    k_count_totals<<<(int)(nb < 1024 ? (nb < 1 ? 1 : nb) : 1024), 256, 0, st>>>(counts, n, out2);
+    launch_chained(k_count_totals, dim3((unsigned)(nb < 1024 ? (nb < 1 ? 1 : nb) : 1024)), 256, 0, st, counts, n, out2);
 }
 
 int64_t radix_tmp_words(int64_t n) {
@@ -271,6 +290,11 @@ int64_t radix_tmp_words(int64_t n) {
     if (ntiles == 0) ntiles = 1;
     int64_t h = 256 * ntiles;
     return 2 * h + 1 + scan_tmp_words(h) + 2 * n + 8;     // + 8: the arrays of n begin on 16-byte boundaries
+}
+
+int radix_launches(int64_t n, int key_bits) {
+    const int passes = (key_bits + 7) / 8, bits = (key_bits + passes - 1) / passes;
+    return passes * (2 + scan_launches((n + RX_TILE - 1) / RX_TILE << bits));
 }
 
 unsigned* radix_sort_index(unsigned* keys, unsigned* perm, int64_t n, int key_bits, unsigned* tmp, cudaStream_t st,

@@ -1840,9 +1840,45 @@ __global__ void k_batch_clear(int64_t n64, long long* __restrict__ vsum, int* __
     if (blockIdx.x == 0 && threadIdx.x < 2) moved(mig, m * bt.stride)[threadIdx.x] = 0;
 }
 
+__global__ void __launch_bounds__(256) k_section_copy(const __grid_constant__ SectionCopy c) {
+    const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, nt = (int64_t)gridDim.x * blockDim.x;
+    if (blockIdx.x == 0) {
+        if (c.header_to && threadIdx.x < 16) {
+            unsigned w = c.header[threadIdx.x];
+            if (threadIdx.x >= 14 && c.sigma_from) w = reinterpret_cast<const unsigned*>(c.sigma_from)[threadIdx.x - 14];
+            reinterpret_cast<unsigned*>(c.header_to)[threadIdx.x] = w;
+        }
+        if (c.sigma_to && threadIdx.x == 0) *c.sigma_to = c.sigma;
+        if ((int)threadIdx.x < c.nzero) c.zero[threadIdx.x] = 0u;
+        if (c.zero64 && threadIdx.x < 2) c.zero64[threadIdx.x] = 0;
+    }
+    for (int s = 0; s < c.n; ++s) {
+        const int64_t q = c.bytes[s] >> 4;
+        const uint4* a = reinterpret_cast<const uint4*>(c.src[s]);
+        uint4* b = reinterpret_cast<uint4*>(c.dst[s]);
+        int64_t i = t0;
+        for (; i + 3 * nt < q; i += 4 * nt) {                // four 16-byte loads in flight
+            const uint4 v0 = a[i], v1 = a[i + nt], v2 = a[i + 2 * nt], v3 = a[i + 3 * nt];
+            b[i] = v0;
+            b[i + nt] = v1;
+            b[i + 2 * nt] = v2;
+            b[i + 3 * nt] = v3;
+        }
+        for (; i < q; i += nt) b[i] = a[i];
+        if (t0 < (c.bytes[s] & 15)) c.dst[s][16 * q + t0] = c.src[s][16 * q + t0];
+    }
+}
+
 }  // namespace
 
 // ------------------------------------------------------------------ launchers
+void launch_section_copy(const SectionCopy& c, cudaStream_t st) {
+    int64_t total = 0;
+    for (int s = 0; s < c.n; ++s) total += c.bytes[s];
+    const int64_t nb = (total / 64 + 255) / 256;
+    k_section_copy<<<(unsigned)std::min<int64_t>(152 * 8, std::max<int64_t>(1, nb)), 256, 0, st>>>(c);
+}
+
 void launch_batch_clear(const Geo& g, long long* vsum, int* maxmig, cudaStream_t st, const Batch& bt) {
     const int64_t n = 3 * (int64_t)g.Ncc;
     launch_chained(k_batch_clear, dim3((unsigned)std::min<int64_t>(1024, (n + 255) / 256), bt.members), 256, 0, st, n,

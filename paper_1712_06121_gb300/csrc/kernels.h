@@ -110,11 +110,13 @@ void set_last_error(const std::string& msg);     // message for cube_last_error(
 
 // ------------------------------------------------------------ k_scan.cu
 int scan_tmp_words(int64_t n);
+int scan_launches(int64_t n);              // kernels of exclusive_scan for one context
 void exclusive_scan(const unsigned* in, unsigned* out, int64_t n, unsigned* tmp, cudaStream_t st,
                     const Batch& bt = Batch{1, 0, nullptr, nullptr});
-// out2[0] = 64-bit sum, out2[1] = maximum of n counts
+// out2[0] += 64-bit sum, out2[1] = max(out2[1], maximum) of n counts
 void count_totals(const unsigned* counts, int64_t n, unsigned long long* out2, cudaStream_t st);
 int64_t radix_tmp_words(int64_t n);
+int radix_launches(int64_t n, int key_bits);   // kernels of radix_sort_index
 // the permutation that sorts keys[n] by their low key_bits bits (stable), in
 // `perm` or `tmp`; *spare: three other arrays of n words, free afterwards
 // (the keys are overwritten)
@@ -215,6 +217,25 @@ void launch_cells(const Geo& g, const StepScratch& w, unsigned* off_new, float* 
 void launch_passB(const Geo& g, const StoreDev& s_old, const StoreDev& s_new, const CodecDev& cur,
                   const CodecDev& next, float dc, const StepScratch& w, cudaStream_t st,
                   const Batch& bt = Batch{1, 0, nullptr, nullptr});
+// Up to five arrays copied in one launch (a checkpoint's sections): array i is
+// bytes[i] long, both ends 16-byte aligned.  By the way, any of: a 64-byte
+// header written to `header_to` with *sigma_from at byte 56; sigma_to = sigma;
+// zero[0 .. nzero) and zero64[0 .. 1] cleared.
+struct SectionCopy {
+    char* dst[5];
+    const char* src[5];
+    int64_t bytes[5];
+    int n;
+    char* header_to;
+    unsigned header[16];
+    const double* sigma_from;
+    double* sigma_to;
+    double sigma;
+    unsigned* zero;
+    int nzero;
+    long long* zero64;
+};
+void launch_section_copy(const SectionCopy& c, cudaStream_t st);
 // sums over the current store: out[0..2] momentum of the decoded particles in
 // 2^-24 fixed point, out[3] the particle count (sum of the cell counts)
 void launch_store_sums(const Geo& g, const StoreDev& s, const float* dec, long long* out4, cudaStream_t st);

@@ -209,3 +209,38 @@ def test_encode_at_tile_edges(cube, n, nf, ratio, xb, vb, sigma):
                 assert g["sigma"] == pytest.approx(free.sigma, rel=1e-12)
     finally:
         cube.cube_destroy(ctx)
+
+
+# ---------------------------------------------------------------- checkpoint sections
+# section lengths with every remainder of 16 bytes, buffers the copy kernel
+# takes (aligned, on the device) and those it does not: the same bytes, and the
+# same store from each of them
+@pytest.mark.parametrize("n,xb,vb,idb", [(1, 1, 1, 1), (1003, 2, 1, 2), (777, 1, 2, 4), (513, 4, 4, 4), (100, 1, 1, 0)])
+def test_checkpoint_buffers_hold_the_same_bytes(cube, n, xb, vb, idb):
+    nf = 32
+    pos, vel, ids = _random_particles(n, nf, 1712208)
+    prm = cube.make_params(nf, n, x_bytes=xb, v_bytes=vb, id_bytes=idb, box=50.0)
+    ctx = cube.cube_create(prm, torch.cuda.current_stream())
+    try:
+        cube.cube_encode(ctx, pos, vel, ids, 0.02, 0.5)
+        size = cube.cube_checkpoint_size(prm)
+        host = np.full(size, 7, dtype=np.uint8)
+        cube.cube_checkpoint_save(ctx, host)
+        bufs = [torch.full((size + 16,), 7, device="cuda", dtype=torch.uint8) for _ in range(2)]
+        views = [bufs[0][:size], bufs[1][8:8 + size]]
+        for v in views:
+            cube.cube_checkpoint_save(ctx, v)
+            assert np.array_equal(v.cpu().numpy(), host)
+        assert bool((bufs[0][size:] == 7).all()) and bool((bufs[1][:8] == 7).all())
+        out = [np.empty((3, n), np.float32) for _ in range(2)]
+        cube.cube_decode(ctx, *out)
+        for b in (host, *views):
+            other = [np.empty((3, n), np.float32) for _ in range(2)]
+            cube.cube_encode(ctx, pos[:, ::-1].copy(), vel, ids, 0.03, 0.7)
+            cube.cube_checkpoint_load(ctx, b)
+            cube.cube_decode(ctx, *other)
+            assert all(np.array_equal(x, y) for x, y in zip(out, other))
+            st = cube.cube_stats_get(ctx)
+            assert st.error_flags == 0 and st.a == 0.02
+    finally:
+        cube.cube_destroy(ctx)
