@@ -341,24 +341,23 @@ __device__ __forceinline__ void col_passes(float4* buf, const float2* tw) {
 }
 
 // First pass (no twiddles) of a column tile straight from global memory:
-// element r of the pair of columns c0 + 2 p, + 1 is the 16 bytes at
-// src[r rs + c0 + 2 p], zero when the pair starts at or past column ncol (a last
-// column without a partner is paired with the row's padding slot, whose values
-// go nowhere).  pack_off > 0: column 0 of the tile (c0 = 0) becomes X + i Y, X
-// its own values and Y those of the column pack_off further (two real
-// sequences in one complex transform).  Ends with a barrier.
+// element r of pair p (columns c and c + 1) is the 16 bytes at src[r rs + p ps],
+// zero from pair np on (a last column without a partner is paired with the
+// row's padding slot, whose values go nowhere).  pack_off > 0: column 0 of pair
+// 0 becomes X + i Y, X its own values and Y those of the column pack_off
+// further (two real sequences in one complex transform).  Ends with a barrier.
 template <int n, bool INV, int T>
-__device__ __forceinline__ void col_load(float4* buf, const float2* __restrict__ src, int64_t rs, int c0, int ncol,
+__device__ __forceinline__ void col_load(float4* buf, const float2* __restrict__ src, int64_t rs, int ps, int np,
                                          int pack_off = 0) {
     constexpr int R = rad(n, 1), nq = n / R;
     for_butterflies<n, R, T>([&](int p, int j) {
-        const bool ok = c0 + 2 * p < ncol;
-        const float2* s = src + (int64_t)j * rs + c0 + 2 * p;
+        const bool ok = p < np;
+        const float2* s = src + (int64_t)j * rs + p * ps;
         float4 f[R];
 #pragma unroll
         for (int m = 0; m < R; ++m)
             f[m] = ok ? *reinterpret_cast<const float4*>(s + (int64_t)m * nq * rs) : make_float4(0.f, 0.f, 0.f, 0.f);
-        if (pack_off > 0 && c0 + p == 0)
+        if (pack_off > 0 && p == 0)
 #pragma unroll
             for (int m = 0; m < R; ++m) {
                 const float2 y = s[(int64_t)m * nq * rs + pack_off];
@@ -376,26 +375,26 @@ __device__ __forceinline__ void col_load(float4* buf, const float2* __restrict__
     __syncthreads();
 }
 
-// Last pass of a column tile: results go straight to dst[k rs + c0 + 2 p] for
-// pairs starting below ncol.  split_off > 0: column 0 of the tile (c0 = 0) holds
-// x + i y of two real sequences; x goes to column 0 and y to the column
-// split_off further, both as (value, 0).
+// Last pass of a column tile: results go straight to dst[k rs + p ps] for pairs
+// below np.  split_off > 0: column 0 of pair 0 holds x + i y of two real
+// sequences; x goes to column 0 and y to the column split_off further, both as
+// (value, 0).
 template <int n, bool INV, int T>
-__device__ __forceinline__ void col_store(const float4* buf, const float2* tw, float2* dst, int64_t rs, int c0,
-                                          int ncol, int split_off = 0) {
+__device__ __forceinline__ void col_store(const float4* buf, const float2* tw, float2* dst, int64_t rs, int ps,
+                                          int np, int split_off = 0) {
     constexpr int q = npass(n), R = rad(n, q), nq = n / R;
     for_butterflies<n, R, T>([&](int p, int j) {
         C2 v[R];
         butterfly<n, q, INV>(buf, tw, p, j, 0, v);
         dft<R, INV>(v);
-        float2* d = dst + (int64_t)j * rs + c0 + 2 * p;
-        if (split_off > 0 && c0 + p == 0) {
+        float2* d = dst + (int64_t)j * rs + p * ps;
+        if (split_off > 0 && p == 0) {
 #pragma unroll
             for (int m = 0; m < R; ++m) {
                 *reinterpret_cast<float4*>(d + (int64_t)m * nq * rs) = make_float4(v[m].x.x, 0.f, v[m].x.y, v[m].y.y);
                 d[(int64_t)m * nq * rs + split_off] = make_float2(v[m].y.x, 0.f);
             }
-        } else if (c0 + 2 * p < ncol) {
+        } else if (p < np) {
 #pragma unroll
             for (int m = 0; m < R; ++m) *reinterpret_cast<float4*>(d + (int64_t)m * nq * rs) = to_columns(v[m]);
         }
@@ -663,10 +662,11 @@ __global__ void __launch_bounds__(fft_threads(N), fft_blocks(N))
     const int c0 = blockIdx.x * NC;
     float2* slab = reinterpret_cast<float2*>(mesh) + (int64_t)blockIdx.y * N * Sc;
     constexpr int q = npass(N);
-    col_load<N, INV, T>(buf, slab, Sc, c0, h, h);
+    const int np = h % NC == 0 ? NP : min(NP, (h - c0) / 2), packed = blockIdx.x == 0 ? h : 0;
+    col_load<N, INV, T>(buf, slab + c0, Sc, 2, np, packed);
     if (INV || blockIdx.x > 0) {
         col_passes<N, 2, q - 1, INV, T>(buf, stw);
-        col_store<N, INV, T>(buf, stw, slab, Sc, c0, h, INV ? h : 0);
+        col_store<N, INV, T>(buf, stw, slab + c0, Sc, 2, np, packed);
     } else {
         col_passes<N, 2, q, INV, T>(buf, stw);
         for (int t = threadIdx.x; t < N * NP; t += T) {
@@ -687,62 +687,78 @@ __global__ void __launch_bounds__(fft_threads(N), fft_blocks(N))
 }
 
 // ------------------------------------------------------------ z sweep (+ Green)
-// Green's function -(3/2) Om / k^2 / W(k)^p / N^3 of a pair of columns (kx, ky),
-// (kx + 1, ky), kz = z
+// Green's function -(3/2) Om / k^2 / W(k)^p / N^3 of a pair's columns, kz = z
 struct GreenPost {
     const float2* tab;           // (k^2, window factor) of each index
-    float g0, ky2, wy;
-    int c0, ky;
-    __device__ __forceinline__ float at(float2 x, float2 z, bool origin) const {
-        const float kk = x.x + ky2 + z.x;
+    float g0;
+    int kx0, ky0;                // pair p: columns kx0 + 2 p, + 1 at ky0, or (edge) column kx0 at ky0 + p
+    bool edge;
+    __device__ __forceinline__ float at(float2 x, float2 y, float2 z, bool origin) const {
+        const float kk = x.x + y.x + z.x;
         // approximate division: within 2 ulp for kk below 2^126 (here kk < 3 pi^2)
-        return origin ? 0.0f : __fdividef(g0, kk) * (x.y * wy * z.y);
+        return origin ? 0.0f : __fdividef(g0, kk) * (x.y * y.y * z.y);
     }
     __device__ __forceinline__ float2 operator()(int z, int p) const {
-        const int kx = c0 + 2 * p;
+        const int kx = edge ? kx0 : kx0 + 2 * p, ky = edge ? ky0 + p : ky0;
         const float4 x = *reinterpret_cast<const float4*>(&tab[kx]);
-        const float2 tz = tab[z];
-        return make_float2(at(make_float2(x.x, x.y), tz, kx == 0 && ky == 0 && z == 0),
-                           at(make_float2(x.z, x.w), tz, false));
+        const float2 y = tab[ky], tz = tab[z];
+        return make_float2(at(make_float2(x.x, x.y), y, tz, kx == 0 && ky == 0 && z == 0),
+                           at(make_float2(x.z, x.w), y, tz, false));
     }
 };
 
-// One tile of 16 consecutive kx (0 .. N/2) at one ky.
+// Tiles of 16 consecutive kx at one ky.  The column kx = N/2 would fill a tile
+// of its own with one column of 16 at every ky, so up to N = 384 it goes, for
+// eight consecutive ky at a time, into edge tiles, the first of the grid (z of
+// 12 meshes of 128^3 55 -> 50 us, 192^3 20.5 -> 18.6, 256^3 41 -> 38, 384^3 145
+// -> 139; at 512^3 the edge tiles' scattered 16-byte pieces cost more than the
+// 6% they save: 312 -> 320).
+template <int N>
+constexpr int nedge() { return N <= 384 ? N / NP : 0; }
+template <int N>
+constexpr int ntile_z() { return nedge<N>() ? ntile_x<N>() : (N / 2 + NC) / NC; }
+template <int N>
+constexpr int ztiles() { return nedge<N>() + ntile_z<N>() * N; }
+
 template <int N, int MODE, bool BAT>   // MODE 0: forward only, 1: forward, Green, inverse
 __global__ void __launch_bounds__(fft_threads(N), fft_blocks(N))
     k_fft_z(float* mesh, int S, const float2* __restrict__ tw, const float* __restrict__ k2,
             const float* __restrict__ wdec, float g0, Batch bt) {
     extern __shared__ float4 fsm[];
-    if constexpr (BAT) {                                     // slot blockIdx.z of a batch
-        if (bt.ms && !bt.ms[blockIdx.z].active) {
+    if constexpr (BAT) {                                     // slot blockIdx.y of a batch
+        if (bt.ms && !bt.ms[blockIdx.y].active) {
             chain_wait();
             return;
         }
-        mesh = moved(mesh, slot_member(bt, blockIdx.z) * bt.stride);
+        mesh = moved(mesh, slot_member(bt, blockIdx.y) * bt.stride);
     }
-    constexpr int ncol = N / 2 + 1, T = fft_threads(N), q = npass(N);
+    constexpr int h = N / 2, T = fft_threads(N), q = npass(N);
     float4* buf = fsm;
     float2* stw = reinterpret_cast<float2*>(buf + N * NP);
     float2* green = stw + N;     // [N + NC]: a last pair's padding column stays inside
     load_tw<N, T>(stw, tw);
     const int Sc = S / 2;
     const int64_t zs = (int64_t)N * Sc;
-    const int c0 = blockIdx.x * NC, ky = blockIdx.y;
-    float2* base = reinterpret_cast<float2*>(mesh) + (int64_t)ky * Sc;
+    constexpr int ne = nedge<N>(), ncol = ne ? h : h + 1;    // columns of the 16-column tiles
+    const bool edge = (int)blockIdx.x < ne;
+    const int t = (int)blockIdx.x - ne;
+    const int ky = edge ? (int)blockIdx.x * NP : t / ntile_z<N>(), c0 = edge ? h : t % ntile_z<N>() * NC;
+    const int ps = edge ? Sc : 2, np = ne && h % NC == 0 ? NP : edge ? NP : min(NP, (ncol - c0 + 1) / 2);
+    float2* base = reinterpret_cast<float2*>(mesh) + (int64_t)ky * Sc + c0;
     if (MODE == 1)
         for (int i = threadIdx.x; i < N + NC; i += T)
             green[i] = i < N ? make_float2(__ldg(&k2[i]), __ldg(&wdec[i])) : make_float2(1.0f, 1.0f);
     chain_wait();
-    col_load<N, false, T>(buf, base, zs, c0, ncol);
+    col_load<N, false, T>(buf, base, zs, ps, np);
     col_passes<N, 2, q - 1, false, T>(buf, stw);
     if (MODE == 1) {
-        const GreenPost gp{green, g0, green[ky].x, green[ky].y, c0, ky};
+        const GreenPost gp{green, g0, c0, ky, edge};
         constexpr bool fuse = rad(N, 1) == rad(N, q);
         col_pass_post<N, fuse, T>(buf, stw, gp);
         col_passes<N, fuse ? 2 : 1, q - 1, true, T>(buf, stw);
-        col_store<N, true, T>(buf, stw, base, zs, c0, ncol);
+        col_store<N, true, T>(buf, stw, base, zs, ps, np);
     } else {
-        col_store<N, false, T>(buf, stw, base, zs, c0, ncol);
+        col_store<N, false, T>(buf, stw, base, zs, ps, np);
     }
 }
 
@@ -1057,13 +1073,13 @@ struct Sweeps {
         const size_t sm = ztile_smem(N);
         if constexpr (kBatchable) {
             if (batched(bt)) {
-                const dim3 gz((N / 2 + NC) / NC, N, bt.members);
+                const dim3 gz(ztiles<N>(), bt.members);
                 if (green) launch_chained(k_fft_z<N, 1, true>, gz, fft_threads(N), sm, st, mesh, S, p.tw, p.k2, p.wdec, g0, bt);
                 else launch_chained(k_fft_z<N, 0, true>, gz, fft_threads(N), sm, st, mesh, S, p.tw, p.k2, p.wdec, g0, bt);
                 return;
             }
         }
-        const dim3 gz((N / 2 + NC) / NC, N);
+        const dim3 gz(ztiles<N>());
         per_member(bt, [&](size_t o) {
             if (green) launch_chained(k_fft_z<N, 1, false>, gz, fft_threads(N), sm, st, moved(mesh, o), S, p.tw, p.k2, p.wdec, g0, kSingle);
             else launch_chained(k_fft_z<N, 0, false>, gz, fft_threads(N), sm, st, moved(mesh, o), S, p.tw, p.k2, p.wdec, g0, kSingle);
