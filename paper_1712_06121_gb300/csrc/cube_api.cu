@@ -733,7 +733,7 @@ static cube_status encode_impl(cube_ctx* c, const float* pos, const float* vel, 
     float* const vsorted[3] = {(float*)spare[0], (float*)spare[1], (float*)spare[2]};
     const StoreDev store = c->store(k);
     launch_encode_vc(g, dvel, order, store, vsorted, sigma > 0.0 ? nullptr : c->part, c->flags, c->st);
-    launch_sigma_finalize(c->part, sigma > 0.0 ? 0 : g.nbricks, 3.0 * (double)g.Np, 1.0, sigma > 0.0 ? sigma : 0.0,
+    launch_sigma_finalize(c->part, sigma > 0.0 ? 0 : encode_groups(g), 3.0 * (double)g.Np, 1.0, sigma > 0.0 ? sigma : 0.0,
                           c->codec[k].sigma, c->st);
     launch_codec_tables(g.nulim, c->tanv, c->tanh_, c->codec[k], c->st);
     launch_encode_codes(g, dpos, vsorted, did, order, c->codec[k], store, c->st);

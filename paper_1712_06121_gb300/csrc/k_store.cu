@@ -6,7 +6,7 @@
 //   (identical drift, stable scatter by new cell,
 //   Eq. chi / Eq. nu encode against the new v_c; Fig. update_xp second loop).
 //
-// Every per-particle pass runs one CTA per storage brick: the brick's cells
+// The per-particle passes of a step run one CTA per storage brick: the brick's cells
 // are contiguous in the store, so the CTA reads a contiguous particle range
 // and finds each particle's cell by binary search in the brick's offsets.
 #include <algorithm>
@@ -207,9 +207,14 @@ __global__ void k_encode_keys(Geo g, const float* __restrict__ pos, unsigned* __
     if (bad) atomicOr(flags, ERR_NONFINITE);
 }
 
-// One CTA per brick of the sorted order: the particles' momenta are gathered
+// Cells of a CTA of the two kernels below: consecutive in storage order, so
+// their particles are too, whatever the brick (the encode of 128^3 particles
+// in bricks of one cell: 482 us with a CTA a brick -> 184; of 64 cells 183)
+constexpr int ENC_CELLS = 64;
+
+// One CTA per 64 cells of the sorted order: the particles' momenta are gathered
 // once, written in storage order for the kernels that follow, and added up
-// per cell in shared memory (exact fixed point); then v_c, and the brick's sum
+// per cell in shared memory (exact fixed point); then v_c, and the cells' sum
 // of squared offsets for a measured codec scale.  256^3 particles x1v1: this
 // 273 us and k_encode_codes 231, where 64-bit global atomics per particle, the
 // measurement and the final gather took 215 + 28 + 58 + 398 us in four kernels;
@@ -218,16 +223,16 @@ __global__ void __launch_bounds__(T_BRICK) k_encode_vc(Geo g, const float* __res
                                                        const unsigned* __restrict__ perm, StoreDev s, float* v0,
                                                        float* v1, float* v2, float* __restrict__ part,
                                                        unsigned* flags) {
-    __shared__ unsigned off[65];
-    __shared__ unsigned vs[3 * 64 * 2];                      // {low, high} words
-    __shared__ float svc[3 * 64];
+    __shared__ unsigned off[ENC_CELLS + 1];
+    __shared__ unsigned vs[3 * ENC_CELLS * 2];               // {low, high} words
+    __shared__ float svc[3 * ENC_CELLS];
     __shared__ double red[32];
     chain_wait();
-    const int nbc = g.B * g.B * g.B, L0 = blockIdx.x * nbc;
-    for (int c = threadIdx.x; c <= nbc; c += blockDim.x) off[c] = s.offsets[L0 + c];
-    for (int t = threadIdx.x; t < 6 * nbc; t += blockDim.x) vs[t] = 0u;
+    const int L0 = blockIdx.x * ENC_CELLS, nc = min(ENC_CELLS, g.Ncc - L0);
+    for (int c = threadIdx.x; c <= nc; c += blockDim.x) off[c] = s.offsets[L0 + c];
+    for (int t = threadIdx.x; t < 6 * ENC_CELLS; t += blockDim.x) vs[t] = 0u;
     __syncthreads();
-    const unsigned q1 = min(off[nbc], (unsigned)g.Np), q0 = min(off[0], q1);
+    const unsigned q1 = min(off[nc], (unsigned)g.Np), q0 = min(off[0], q1);
     unsigned p0, p1;
     brick_share(q0, q1, &p0, &p1);
     const unsigned lane = threadIdx.x & 31;
@@ -237,7 +242,7 @@ __global__ void __launch_bounds__(T_BRICK) k_encode_vc(Geo g, const float* __res
     // 64 particles of the warp at a time, their loads in flight together
     float v[2][3];
     int cell[2] = {0, 0};
-    int c0 = p0 < p1 ? upper_cell(off, nbc, p0) : 0;
+    int c0 = p0 < p1 ? upper_cell(off, nc, p0) : 0;
     for (unsigned base = p0; base < p1; base += 64) {
         unsigned i[2];
 #pragma unroll
@@ -250,7 +255,7 @@ __global__ void __launch_bounds__(T_BRICK) k_encode_vc(Geo g, const float* __res
         for (int h = 0; h < 2; ++h) {
             const unsigned j = base + 32 * h + lane;
             int cnext;
-            cell[h] = warp_cells(off, nbc, base + 32 * h, c0, &cnext);
+            cell[h] = warp_cells(off, nc, base + 32 * h, c0, &cnext);
             c0 = cnext;
             if (j < p1)
 #pragma unroll
@@ -260,13 +265,14 @@ __global__ void __launch_bounds__(T_BRICK) k_encode_vc(Geo g, const float* __res
                         v[h][d] = 0.0f;
                     }
                     vo[d][j] = v[h][d];
-                    smem_add_u64(&vs[2 * (d * nbc + cell[h])], (unsigned long long)vel_fix(v[h][d]));
+                    smem_add_u64(&vs[2 * (d * ENC_CELLS + cell[h])], (unsigned long long)vel_fix(v[h][d]));
                 }
         }
     }
     __syncthreads();
-    for (int t = threadIdx.x; t < 3 * nbc; t += blockDim.x) {
-        const int d = t >> (3 * g.lB), c = t & (nbc - 1);
+    for (int t = threadIdx.x; t < 3 * ENC_CELLS; t += blockDim.x) {
+        const int d = t / ENC_CELLS, c = t % ENC_CELLS;
+        if (c >= nc) continue;
         const long long sum = (long long)(((unsigned long long)vs[2 * t + 1] << 32) | vs[2 * t]);
         const float m = vel_unfix_mean(sum, off[c + 1] - off[c]);
         svc[t] = m;
@@ -278,7 +284,7 @@ __global__ void __launch_bounds__(T_BRICK) k_encode_vc(Geo g, const float* __res
         auto add = [&](const float* x, int c) {
 #pragma unroll
             for (int d = 0; d < 3; ++d) {
-                const float e = x[d] - svc[d * nbc + c];
+                const float e = x[d] - svc[d * ENC_CELLS + c];
                 acc = __fmaf_rn(e, e, acc);
             }
         };
@@ -287,11 +293,11 @@ __global__ void __launch_bounds__(T_BRICK) k_encode_vc(Geo g, const float* __res
             for (int h = 0; h < 2; ++h)
                 if (p0 + 32 * h + lane < p1) add(v[h], cell[h]);
         } else {
-            c0 = upper_cell(off, nbc, p0);
+            c0 = upper_cell(off, nc, p0);
             for (unsigned base = p0; base < p1; base += 32) {
                 const unsigned j = base + lane;
                 int cnext;
-                const int c = warp_cells(off, nbc, base, c0, &cnext);
+                const int c = warp_cells(off, nc, base, c0, &cnext);
                 c0 = cnext;
                 if (j < p1) {
                     const float x[3] = {vo[0][j], vo[1][j], vo[2][j]};
@@ -404,7 +410,7 @@ __global__ void k_codec_tables(int lim, const double* __restrict__ tanv, const d
                       moved(est, o), moved(vtab, o), moved(vdel, o), blockIdx.x, gridDim.x);
 }
 
-// codes and ids in storage order, one CTA per brick: positions and ids
+// codes and ids in storage order, one CTA per 64 cells: positions and ids
 // gathered by the permutation, momenta already in order
 template <int NX, int NV>
 __global__ void __launch_bounds__(T_BRICK) k_encode_codes(Geo g, const float* __restrict__ pos,
@@ -412,15 +418,15 @@ __global__ void __launch_bounds__(T_BRICK) k_encode_codes(Geo g, const float* __
                                                           const float* __restrict__ v2,
                                                           const unsigned* __restrict__ id_in,
                                                           const unsigned* __restrict__ perm, CodecDev cd, StoreDev s) {
-    __shared__ unsigned off[65];
-    __shared__ float svc[3 * 64];
+    __shared__ unsigned off[ENC_CELLS + 1];
+    __shared__ float svc[3 * ENC_CELLS];
     chain_wait();
-    const int nbc = g.B * g.B * g.B, L0 = blockIdx.x * nbc;
-    for (int c = threadIdx.x; c <= nbc; c += blockDim.x) off[c] = s.offsets[L0 + c];
-    for (int t = threadIdx.x; t < 3 * nbc; t += blockDim.x)
-        svc[t] = s.vc[(int64_t)(t >> (3 * g.lB)) * g.Ncc + L0 + (t & (nbc - 1))];
+    const int L0 = blockIdx.x * ENC_CELLS, nc = min(ENC_CELLS, g.Ncc - L0);
+    for (int c = threadIdx.x; c <= nc; c += blockDim.x) off[c] = s.offsets[L0 + c];
+    for (int t = threadIdx.x; t < 3 * ENC_CELLS; t += blockDim.x)
+        if (t % ENC_CELLS < nc) svc[t] = s.vc[(int64_t)(t / ENC_CELLS) * g.Ncc + L0 + t % ENC_CELLS];
     __syncthreads();
-    const unsigned q1 = min(off[nbc], (unsigned)g.Np);
+    const unsigned q1 = min(off[nc], (unsigned)g.Np);
     unsigned p0, p1;
     brick_share(min(off[0], q1), q1, &p0, &p1);
     if (p0 >= p1) return;
@@ -432,7 +438,7 @@ __global__ void __launch_bounds__(T_BRICK) k_encode_codes(Geo g, const float* __
     const CodeRows<NV> nu_r(s.nu, g.Np);
     const float* vi[3] = {v0, v1, v2};
     const float* xi[3] = {pos, pos + g.Np, pos + 2 * g.Np};
-    int c0 = upper_cell(off, nbc, p0);
+    int c0 = upper_cell(off, nc, p0);
     for (unsigned base = p0; base < p1; base += 64) {       // 64 particles' loads in flight
         float x[2][3], v[2][3];
         unsigned i[2], pid[2] = {0, 0};
@@ -452,7 +458,7 @@ __global__ void __launch_bounds__(T_BRICK) k_encode_codes(Geo g, const float* __
         for (int h = 0; h < 2; ++h) {
             const unsigned j = base + 32 * h + lane;
             int cnext;
-            const int c = warp_cells(off, nbc, base + 32 * h, c0, &cnext);
+            const int c = warp_cells(off, nc, base + 32 * h, c0, &cnext);
             c0 = cnext;
             if (j >= p1) continue;
             float dd[3];
@@ -460,7 +466,7 @@ __global__ void __launch_bounds__(T_BRICK) k_encode_codes(Geo g, const float* __
 #pragma unroll
             for (int d = 0; d < 3; ++d) {
                 chi.put(d, j, (pos_bin(x[h][d], scale, g.Nc << nbits) & mask) - half);
-                dd[d] = v[h][d] - svc[d * nbc + c];
+                dd[d] = v[h][d] - svc[d * ENC_CELLS + c];
                 if (NV == 1) nu[d] = nu_from_table(dd[d], cd.thr, cd.vtab, key0, g.nulim);
             }
             if (NV == 2) nu_codes3(dd, cd.thr, g.nulim, cd.est[0], cd.est[1], nu);
@@ -1000,7 +1006,7 @@ __global__ void __launch_bounds__(PA_T, PA_MINB) k_passA(Geo g, StoreDev s, cons
     const unsigned q1 = min(s.offsets[L0 + nbc], (unsigned)g.Np);
     const unsigned q0 = min(s.offsets[L0], q1);
     unsigned i = q0 + threadIdx.x;
-    if (NV == 1 && threadIdx.x == 0 && q1 - q0 > (unsigned)PB_BIG) w.big[1 + atomicAdd(w.big, 1)] = brick;
+    if (threadIdx.x == 0 && q1 - q0 > (unsigned)PB_BIG) w.big[1 + atomicAdd(w.big, 1)] = brick;
     const CodeRows<NX> chi_r(s.chi, g.Np);
     const CodeRows<NV> nu_r(s.nu, g.Np);
     int nchi[3] = {0, 0, 0}, nnu[3] = {0, 0, 0};
@@ -1366,7 +1372,7 @@ __global__ void __launch_bounds__(SC_T) k_step_cells(Geo g, StepScratch w, const
 // ------------------------------------------------------------------ pass B
 // Two splits, chosen by passB_all:
 //
-// Large stores with 1-byte velocities: one warp per brick (8 bricks per CTA).
+// Large stores: one warp per brick (8 bricks per CTA).
 // The brick's particles are taken 32 at a time in index order; lanes moving
 // to the same cell get consecutive slots in lane order from the cell's running
 // start (match + popc), so the new order within a cell is the old index
@@ -1379,8 +1385,8 @@ __global__ void __launch_bounds__(SC_T) k_step_cells(Geo g, StepScratch w, const
 // go to a shared table, and a lane's slot is the cell's running start + the
 // counts of the lower warps + its rank in its warp, which is again the old
 // index order.  Small stores take it because a warp's chain of 16 rounds is
-// the whole kernel there, and every store with 2-byte velocities, whose rounds
-// wait for their table reads.  Measured, us (warp a brick / CTA a brick), x1v1:
+// the whole kernel there, and bricks of side 4 with 2-byte velocities, whose
+// rounds wait for their table reads.  Measured, us (warp a brick / CTA a brick), x1v1:
 // 64 bricks 25.9 / 10.2, 512: 27.2 / 14.3, 1728: 30.0 / 27.0, 4096: 45.6 /
 // 52.6, 13824: 102 / 159; x2v2: 64: 67 / 16, 512: 70 / 20, 1728: 78 / 42,
 // 4096: 122 / 81, 13824: 367 / 250, 32768: 770 / 565.
@@ -1577,9 +1583,12 @@ __device__ __forceinline__ void passB_cta_brick(const Geo& g, const PassB<NX, NV
 }
 
 // the split of pass B: a CTA per brick when the bricks' warps would fill less
-// than 40% of the 40 resident per SM, or with 2-byte velocities
+// than 40% of the 40 resident per SM, or with 2-byte velocities when a brick
+// holds some warps' worth of particles (bricks of side 4; a smaller brick's few
+// particles leave most of a CTA idle: the step of 128^3 particles x2v2 with
+// bricks of 8 cells takes 622 us by warps, of 64 cells 359 us by CTAs)
 static bool passB_all(const Geo& g, int members) {
-    return g.nnu == 2 || (int64_t)g.nbricks * members <= 16 * (int64_t)g.nsm;
+    return (int64_t)g.nbricks * members <= 16 * (int64_t)g.nsm || (g.nnu == 2 && g.Np >= 96 * (int64_t)g.nbricks);
 }
 
 // ALL: every brick by a whole CTA
@@ -1769,15 +1778,13 @@ struct Disp {
             else launch_chained(k_passB<NX, NV, false, 4, true>, gb, PB_WARPS * 32, sm_cta, st, g, so, sn, cur, next, dc, ghost, vcn, flags, big, 0, bt);
             return;
         }
-        if constexpr (NV == 1) {
-            // CTAs for crowded bricks first (at most Np / (PB_BIG + 1) of them exist)
-            const int nbig_ctas = (int)std::min<int64_t>(2 * g.nsm, g.Np / (PB_BIG + 1));
-            const dim3 gb(nbig_ctas + (g.nbricks + PB_WARPS - 1) / PB_WARPS, bt.members);
-            if (bat && narrow) launch_chained(k_passB<NX, NV, true, 0, false>, gb, PB_WARPS * 32, sm, st, g, so, sn, cur, next, dc, ghost, vcn, flags, big, nbig_ctas, bt);
-            else if (bat) launch_chained(k_passB<NX, NV, true, 4, false>, gb, PB_WARPS * 32, sm, st, g, so, sn, cur, next, dc, ghost, vcn, flags, big, nbig_ctas, bt);
-            else if (narrow) launch_chained(k_passB<NX, NV, false, 0, false>, gb, PB_WARPS * 32, sm, st, g, so, sn, cur, next, dc, ghost, vcn, flags, big, nbig_ctas, bt);
-            else launch_chained(k_passB<NX, NV, false, 4, false>, gb, PB_WARPS * 32, sm, st, g, so, sn, cur, next, dc, ghost, vcn, flags, big, nbig_ctas, bt);
-        }
+        // CTAs for crowded bricks first (at most Np / (PB_BIG + 1) of them exist)
+        const int nbig_ctas = (int)std::min<int64_t>(2 * g.nsm, g.Np / (PB_BIG + 1));
+        const dim3 gb(nbig_ctas + (g.nbricks + PB_WARPS - 1) / PB_WARPS, bt.members);
+        if (bat && narrow) launch_chained(k_passB<NX, NV, true, 0, false>, gb, PB_WARPS * 32, sm, st, g, so, sn, cur, next, dc, ghost, vcn, flags, big, nbig_ctas, bt);
+        else if (bat) launch_chained(k_passB<NX, NV, true, 4, false>, gb, PB_WARPS * 32, sm, st, g, so, sn, cur, next, dc, ghost, vcn, flags, big, nbig_ctas, bt);
+        else if (narrow) launch_chained(k_passB<NX, NV, false, 0, false>, gb, PB_WARPS * 32, sm, st, g, so, sn, cur, next, dc, ghost, vcn, flags, big, nbig_ctas, bt);
+        else launch_chained(k_passB<NX, NV, false, 4, false>, gb, PB_WARPS * 32, sm, st, g, so, sn, cur, next, dc, ghost, vcn, flags, big, nbig_ctas, bt);
     }
 };
 
@@ -1790,10 +1797,10 @@ void set_smem_attrs() {
     cudaFuncSetAttribute(k_passA<NX, NV, 16, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
     cudaFuncSetAttribute(k_passA<NX, NV, 0, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
     cudaFuncSetAttribute(k_passA<NX, NV, 16, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-    if constexpr (NV == 1) cudaFuncSetAttribute(k_passB<NX, NV, false, 4, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-    if constexpr (NV == 1) cudaFuncSetAttribute(k_passB<NX, NV, true, 4, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-    if constexpr (NV == 1) cudaFuncSetAttribute(k_passB<NX, NV, false, 0, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-    if constexpr (NV == 1) cudaFuncSetAttribute(k_passB<NX, NV, true, 0, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+    cudaFuncSetAttribute(k_passB<NX, NV, false, 4, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+    cudaFuncSetAttribute(k_passB<NX, NV, true, 4, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+    cudaFuncSetAttribute(k_passB<NX, NV, false, 0, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+    cudaFuncSetAttribute(k_passB<NX, NV, true, 0, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
     cudaFuncSetAttribute(k_deposit<NX, 0, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
     cudaFuncSetAttribute(k_deposit<NX, 16, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
     cudaFuncSetAttribute(k_deposit<NX, 0, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
@@ -1885,6 +1892,10 @@ void launch_batch_clear(const Geo& g, long long* vsum, int* maxmig, cudaStream_t
                    vsum, maxmig, bt);
 }
 
+// threads of a decode CTA: four a cell, a warp at least (128^3 particles in
+// bricks of one cell: 673 us with 256 -> 151; of eight 127 -> 41)
+static inline unsigned brick_threads(const Geo& g) { return std::max(32, std::min(T_BRICK, 4 * g.B * g.B * g.B)); }
+
 static inline int nblk(int64_t n, int t) { return (int)((n + t - 1) / t); }
 
 void launch_encode_keys(const Geo& g, const float* pos, unsigned* key, unsigned* counts, unsigned* flags,
@@ -1894,9 +1905,11 @@ void launch_encode_keys(const Geo& g, const float* pos, unsigned* key, unsigned*
     else launch_chained(k_encode_keys<2>, grid, 256, 0, st, g, pos, key, counts, flags);
 }
 
+int encode_groups(const Geo& g) { return nblk(g.Ncc, ENC_CELLS); }
+
 void launch_encode_vc(const Geo& g, const float* vel, const unsigned* perm, const StoreDev& s, float* const* vsorted,
                       float* part, unsigned* flags, cudaStream_t st) {
-    launch_chained(k_encode_vc, dim3(g.nbricks), T_BRICK, 0, st, g, vel, perm, s, vsorted[0], vsorted[1], vsorted[2],
+    launch_chained(k_encode_vc, dim3(encode_groups(g)), T_BRICK, 0, st, g, vel, perm, s, vsorted[0], vsorted[1], vsorted[2],
                    part, flags);
 }
 
@@ -1916,7 +1929,7 @@ void launch_codec_tables(int nulim, const double* tanv, const double* tanh_, con
 
 void launch_encode_codes(const Geo& g, const float* pos, const float* const* vsorted, const unsigned* id_in,
                          const unsigned* perm, const CodecDev& c, const StoreDev& s, cudaStream_t st) {
-    const dim3 grid(g.nbricks);
+    const dim3 grid(encode_groups(g));
     auto go = [&](auto kernel) {
         launch_chained(kernel, grid, T_BRICK, 0, st, g, pos, vsorted[0], vsorted[1], vsorted[2], id_in, perm, c, s);
     };
@@ -1947,10 +1960,10 @@ static size_t brick_smem(const Geo& g) {
 void launch_decode(const Geo& g, const StoreDev& s, const CodecDev& c, float* pos, float* vel, unsigned* id,
                    cudaStream_t st) {
     const size_t sm = brick_smem(g);
-    if (g.nchi == 1 && g.nnu == 1) launch_chained(k_decode<1, 1>, dim3(g.nbricks), T_BRICK, sm, st, g, s, c, pos, vel, id);
-    else if (g.nchi == 1) launch_chained(k_decode<1, 2>, dim3(g.nbricks), T_BRICK, sm, st, g, s, c, pos, vel, id);
-    else if (g.nnu == 1) launch_chained(k_decode<2, 1>, dim3(g.nbricks), T_BRICK, sm, st, g, s, c, pos, vel, id);
-    else launch_chained(k_decode<2, 2>, dim3(g.nbricks), T_BRICK, sm, st, g, s, c, pos, vel, id);
+    if (g.nchi == 1 && g.nnu == 1) launch_chained(k_decode<1, 1>, dim3(g.nbricks), brick_threads(g), sm, st, g, s, c, pos, vel, id);
+    else if (g.nchi == 1) launch_chained(k_decode<1, 2>, dim3(g.nbricks), brick_threads(g), sm, st, g, s, c, pos, vel, id);
+    else if (g.nnu == 1) launch_chained(k_decode<2, 1>, dim3(g.nbricks), brick_threads(g), sm, st, g, s, c, pos, vel, id);
+    else launch_chained(k_decode<2, 2>, dim3(g.nbricks), brick_threads(g), sm, st, g, s, c, pos, vel, id);
 }
 
 static size_t deposit_smem(const Geo& g) {

@@ -182,7 +182,9 @@ constexpr Batch kSingle{1, 0, nullptr, nullptr};
 void launch_encode_keys(const Geo& g, const float* pos, unsigned* key, unsigned* counts, unsigned* flags,
                         cudaStream_t st);
 // the particles' momenta in storage order (three rows of Np), v_c of every
-// cell, and (part not null) each brick's sum of squared offsets from v_c
+// cell, and (part not null) the sums of squared offsets from v_c of
+// encode_groups runs of cells
+int encode_groups(const Geo& g);
 void launch_encode_vc(const Geo& g, const float* vel, const unsigned* perm, const StoreDev& s, float* const* vsorted,
                       float* part, unsigned* flags, cudaStream_t st);
 void launch_sigma_finalize(const float* part, int nparts, double count, double ratio, double fixed,

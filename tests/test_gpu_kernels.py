@@ -244,3 +244,28 @@ def test_checkpoint_buffers_hold_the_same_bytes(cube, n, xb, vb, idb):
             assert st.error_flags == 0 and st.a == 0.02
     finally:
         cube.cube_destroy(ctx)
+
+
+# 64 cells a CTA whatever the brick: bricks of one cell and of eight, a last
+# CTA of 24 cells, 2-byte velocities past the re-sort's split with crowded
+# bricks; whole numbers, exact
+@pytest.mark.parametrize("nf,ratio,brick,n,xb,vb", [(24, 4, 1, 4001, 1, 1), (64, 4, 1, 20001, 2, 2), (128, 4, 2, 33000, 1, 2)])
+def test_small_bricks_are_bit_exact(cube, nf, ratio, brick, n, xb, vb):
+    pos, vel, ids = _mixed_particles(n, nf, 1712209)
+    prm = cube.make_params(nf, n, ratio=ratio, x_bytes=xb, v_bytes=vb, brick=brick, box=50.0)
+    ctx = cube.cube_create(prm, torch.cuda.current_stream())
+    try:
+        a = _EPOCHS
+        cube.cube_encode(ctx, pos, vel, ids, a[0], 0.0)
+        before = read_store(cube, ctx)
+        assert_store_equal(before, pm.encode(oracle_params(pm, prm, brick), pos, vel, ids, a[0], before["sigma"],
+                                             snap=False), "encode")
+        cube.cube_keep_drifted(ctx, True)
+        cube.cube_pm_step(ctx, a[0], a[1])
+        cell, u, p = np.empty((3, n), np.int32), np.empty((3, n), np.float32), np.empty((3, n), np.float32)
+        sig = cube.cube_debug_drifted(ctx, cell, u, p)
+        g = read_store(cube, ctx)
+        ref = pm.encode_drifted(oracle_params(pm, prm, brick), cell, u, p, before["ids"], sig, g["a"], g["a_p"])
+        assert_store_equal(g, ref, "step")
+    finally:
+        cube.cube_destroy(ctx)
