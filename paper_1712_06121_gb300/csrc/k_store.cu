@@ -229,7 +229,9 @@ __global__ void __launch_bounds__(T_BRICK) k_encode_vc(Geo g, const float* __res
     __shared__ double red[32];
     chain_wait();
     const int L0 = blockIdx.x * ENC_CELLS, nc = min(ENC_CELLS, g.Ncc - L0);
+#pragma unroll 1
     for (int c = threadIdx.x; c <= nc; c += blockDim.x) off[c] = s.offsets[L0 + c];
+#pragma unroll 1
     for (int t = threadIdx.x; t < 6 * ENC_CELLS; t += blockDim.x) vs[t] = 0u;
     __syncthreads();
     const unsigned q1 = min(off[nc], (unsigned)g.Np), q0 = min(off[0], q1);
@@ -411,7 +413,9 @@ __global__ void k_codec_tables(int lim, const double* __restrict__ tanv, const d
 }
 
 // codes and ids in storage order, one CTA per 64 cells: positions and ids
-// gathered by the permutation, momenta already in order
+// gathered by the permutation, momenta already in order.  Bound by that
+// gather's latency, so six CTAs a SM: 40 registers, which the two staging
+// loops unrolled would raise to 48 (five CTAs: 45 us more at 256^3 particles).
 template <int NX, int NV>
 __global__ void __launch_bounds__(T_BRICK) k_encode_codes(Geo g, const float* __restrict__ pos,
                                                           const float* __restrict__ v0, const float* __restrict__ v1,
@@ -422,7 +426,9 @@ __global__ void __launch_bounds__(T_BRICK) k_encode_codes(Geo g, const float* __
     __shared__ float svc[3 * ENC_CELLS];
     chain_wait();
     const int L0 = blockIdx.x * ENC_CELLS, nc = min(ENC_CELLS, g.Ncc - L0);
+#pragma unroll 1
     for (int c = threadIdx.x; c <= nc; c += blockDim.x) off[c] = s.offsets[L0 + c];
+#pragma unroll 1
     for (int t = threadIdx.x; t < 3 * ENC_CELLS; t += blockDim.x)
         if (t % ENC_CELLS < nc) svc[t] = s.vc[(int64_t)(t / ENC_CELLS) * g.Ncc + L0 + t % ENC_CELLS];
     __syncthreads();
