@@ -195,14 +195,19 @@ __global__ void k_encode_keys(Geo g, const float* __restrict__ pos, unsigned* __
     }
     const unsigned k = (unsigned)cell_rank(g, cell[0], cell[1], cell[2]);
     key[i] = k;
-    // one atomic per run of lanes with one cell (neighbours in lattice order)
-    const unsigned act = __activemask(), lane = threadIdx.x & 31;      // a prefix of the warp
+    // one atomic per run of lanes with one cell (neighbours in lattice order).
+    // The lanes here are the warp's first `live`, whichever way each of them
+    // took through pos_bin: the mask follows from the index, and the shuffle
+    // and the ballot bring the lanes together.
+    const int lane = threadIdx.x & 31;
+    const int live = (int)min(g.Np - (i - lane), (int64_t)32);
+    const unsigned act = 0xffffffffu >> (32 - live);
     const unsigned left = __shfl_up_sync(act, k, 1);
     const unsigned heads = __ballot_sync(act, lane == 0 || left != k);
     if ((heads >> lane) & 1u) {
         const unsigned after = lane == 31 ? 0u : heads & (0xfffffffeu << lane);
-        const int end = after ? __ffs(after) - 1 : __popc(act);
-        atomicAdd(&counts[k], (unsigned)(end - (int)lane));
+        const int end = after ? __ffs(after) - 1 : live;
+        atomicAdd(&counts[k], (unsigned)(end - lane));
     }
     if (bad) atomicOr(flags, ERR_NONFINITE);
 }
