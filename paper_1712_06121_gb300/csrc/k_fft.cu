@@ -953,6 +953,11 @@ __global__ void __launch_bounds__(PK_WARPS * 32) k_pk_bin(const float* __restric
 // shells that can hold modes: up to the corner |n| = sqrt(3) N / 2 < 7 N / 8
 __host__ __device__ __forceinline__ int pk_used_bins(int N, int nbins) { return min(nbins, 7 * N / 8); }
 
+// window weights, and each warp's sums of nb bins
+size_t pk_bytes(int N, int nb) {
+    return (size_t)(N / 2 + 1) * sizeof(float2) + (size_t)PK_WARPS * nb * (2 * sizeof(float2) + sizeof(unsigned));
+}
+
 // one warp per bin: the blocks' sums in a fixed order; bins from nb on lie
 // beyond the mesh's corner and hold no mode
 __global__ void k_pk_reduce(const double* __restrict__ part, int nblocks, int nb, int nbins, double pfac, double kfund,
@@ -1154,9 +1159,10 @@ int pk_blocks(int N) {
 
 void launch_pk_bin(const FftPlan& p, const float* mesh, int S, int nbins, double* part, cudaStream_t st) {
     const int nb = pk_used_bins(p.N, nbins);
-    const size_t sm = (size_t)(p.N / 2 + 1) * sizeof(float2) + (size_t)PK_WARPS * nb * (2 * sizeof(float2) + 4);
-    if (sm > 48 * 1024) cudaFuncSetAttribute(k_pk_bin, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    k_pk_bin<<<pk_blocks(p.N), PK_WARPS * 32, sm, st>>>(mesh, p.N, S, nb, nbins, p.wpk, part);
+    // the limit is the kernel's, not this launch's: always the largest mesh's, so
+    // that a call on another thread cannot lower it between here and the launch
+    cudaFuncSetAttribute(k_pk_bin, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pk_bytes(1024, pk_used_bins(1024, 1024)));
+    k_pk_bin<<<pk_blocks(p.N), PK_WARPS * 32, pk_bytes(p.N, nb), st>>>(mesh, p.N, S, nb, nbins, p.wpk, part);
 }
 
 void launch_pk_reduce(const FftPlan& p, const double* part, int nbins, double pfac, double kfund, double* k, double* pk,
