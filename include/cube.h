@@ -332,10 +332,11 @@ cube_status cube_debug_force(cube_ctx* ctx, float* force);
    rebuild it, from a fixed FP32 approximation and a one-byte correction, and
    compared with the full table of the current store's codec, for every k in
    [-lim, lim]; and the codes of the offsets at and just below every threshold
-   of Eq. nu, k in [1, lim], are compared with k and k - 1.  out2[0] = entries
-   and thresholds that differ (0: the kernels see the exact tables), out2[1] =
-   entries kept as "read the full table" (correction out of range).  `out2` is
-   host memory.  Synchronises.
+   of Eq. nu, k in [1, lim], are compared with k and k - 1, those of a NaN, of
+   -infinity and of 0 with 0, -lim and 0.  out2[0] = entries and codes that
+   differ (0: the kernels see the exact tables), out2[1] = entries kept as
+   "read the full table" (correction out of range).  `out2` is host memory.
+   Synchronises.
    Errors: CUBE_E_ARG (NULL, or codes other than 2-byte velocities),
    CUBE_E_STATE (no store). */
 cube_status cube_debug_velocity_tables(cube_ctx* ctx, int64_t* out2);

@@ -297,7 +297,8 @@ struct VelTables {
 // half-integer.  There, 3% of the codes, |d| is compared with the exact
 // threshold: one table read, all three axes' in flight together, where a
 // search from a coarser guess reads two per code one code after the other.
-// Halves away from zero, |nu| <= lim.  1.03 M particles x2v2 (1728 bricks), with
+// Halves away from zero, |nu| <= lim, 0 for a NaN (as an offset that reaches no
+// threshold).  1.03 M particles x2v2 (1728 bricks), with
 // the two-threshold search -> this: pass A 108 -> 69 us, pass B 55 -> 38 us.
 constexpr float kNuMargin = 1.0f / 64.0f;
 __device__ __forceinline__ float nu_value(float a, float s, float m_over_pi, float half_m) {
@@ -336,7 +337,8 @@ __device__ __forceinline__ void nu_codes3(const float* d, const float* __restric
     }
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-        const int v = min(j[k] + ((near[k] ? fabsf(d[k]) >= t[k] : up[k]) ? 1 : 0), lim);
+        int v = min(j[k] + ((near[k] ? fabsf(d[k]) >= t[k] : up[k]) ? 1 : 0), lim);
+        if (j[k] > lim) v = 0;                                   // y is not a number (else y <= lim + 1/2)
         nu[k] = d[k] < 0.0f ? -v : v;
     }
 }

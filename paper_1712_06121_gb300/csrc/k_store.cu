@@ -1826,7 +1826,7 @@ __global__ void k_zero_slot_words(unsigned* p, Batch bt) {
 }
 
 // every entry of the 2-byte decode table as VelTables rebuilds it, and the
-// codes of nu_codes3 at and just below every threshold, against the tables
+// codes of nu_codes3 at and just below every threshold, of a NaN, of infinity and of 0, against the tables
 __global__ void k_check_vel_tables(int lim, CodecDev c, long long* out2) {
     const VelTables vt = vel_tables<2>(c, lim);
     long long bad = 0, whole = 0;
@@ -1840,6 +1840,11 @@ __global__ void k_check_vel_tables(int lim, CodecDev c, long long* out2) {
             int nu[3];
             nu_codes3(d, c.thr, lim, c.est[0], c.est[1], nu);
             bad += nu[0] != k || nu[1] != -k || nu[2] != k - 1;
+        } else {
+            const float nan = __int_as_float(0x7fffffff), inf = __int_as_float(0x7f800000), d[3] = {nan, -inf, 0.0f};
+            int nu[3];
+            nu_codes3(d, c.thr, lim, c.est[0], c.est[1], nu);
+            bad += nu[0] != 0 || nu[1] != -lim || nu[2] != 0;
         }
     }
     block_sum_to(bad, &out2[0]);
