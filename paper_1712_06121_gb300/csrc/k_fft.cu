@@ -787,44 +787,86 @@ __global__ void k_grad_max(const float* __restrict__ phig, int N, unsigned* __re
 // weights, weight * |n| and weight * |delta_k|^2 / W^2.
 //
 // FP64 issues at 1/64 of the FP32 rate here, and FP64 shared atomics are a
-// compare-and-swap loop, so neither is in the loop: sums are pairs of floats
-// (value + error term, the two-sum of Knuth and the FMA product of Dekker /
-// Ogita, Rump and Oishi: about 2^-47 relative), converted to FP64 once per
-// CTA.  A warp takes the rows (|ky|, |kz|) that share their weights and
-// shells, up to four of them (+-ky, +-kz), 32 consecutive kx at a time; along
-// kx the shell index never decreases, so equal shells are runs of lanes: a
-// segmented scan adds each run and its last lane alone adds it to the warp's
-// own bins, without atomics and in a fixed order.  Rows are left as soon as
-// they leave the last shell.  512^3 mesh, 256 bins: 4.23 ms with FP64 sums and
-// shared atomics -> 0.136 ms; the reduction over blocks 0.170 ms (one thread
-// per bin) -> 0.012 ms (one
-// warp per bin).
+// compare-and-swap loop, so neither is in the loop: sums are triples of floats
+// (the exact rounding errors of the values in a second word, those of the
+// second in a third: the two-sum of Knuth and the FMA product, cascaded as in
+// Ogita, Rump and Oishi's DotK, about 2^-70 relative), converted to FP64 once
+// per CTA, so no sum has fewer bits than in FP64.  Largest error over meshes of
+// 16^3 to 512^3 with known modes, |k| / P: FP64 atomics 1.8e-15 / 1.7e-15, pairs
+// of floats (2^-47 an addition) 1.3e-15 / 6.7e-15, triples 4.1e-16 / 3.7e-16.
+// The modes are scaled by 2^12, which keeps the error words in range for every
+// mode from 2^-62 to 2^30 (a mesh of mean 1 has none larger).  A warp takes the
+// rows (|ky|, |kz|) that share their weights and shells, up to four of them
+// (+-ky, +-kz), 32 consecutive kx at a time; along kx the shell index never decreases, so equal shells are
+// runs of lanes: a segmented scan adds each run and its last lane alone adds it
+// to the warp's own bins, without atomics and in a fixed order.  Rows are left
+// as soon as they leave the last shell.  512^3 mesh, 256 bins: 4.23 ms with
+// FP64 sums and shared atomics -> 0.185 ms (pairs: 0.136 ms), 65% of the issue
+// slots; the reduction over blocks 0.170 ms (one thread per bin) -> 0.012 ms
+// (one warp per bin).
 constexpr int PK_WARPS = 8;
+constexpr float PK_SCALE = 4096.0f;
 
-// (h, l) += (bh, bl)
-__device__ __forceinline__ void pair_add(float& h, float& l, float bh, float bl) {
-    const float s = __fadd_rn(h, bh), z = __fsub_rn(s, h);
-    const float e = __fadd_rn(__fsub_rn(h, __fsub_rn(s, z)), __fsub_rn(bh, z));
-    const float t = __fadd_rn(e, __fadd_rn(l, bl));
-    h = __fadd_rn(s, t);
-    l = __fsub_rn(t, __fsub_rn(h, s));
+// a sum as h + l + m, and two of them side by side (float2)
+struct Triple {
+    float h, l, m;
+};
+struct Triple2 {
+    float2 h, l, m;
+};
+// a + b = a + (returned error), exactly
+__device__ __forceinline__ float2 two_sum(float2& a, float2 b) {
+    const float2 s = padd(a, b), z = psub(s, a);
+    const float2 e = padd(psub(a, psub(s, z)), psub(b, z));
+    a = s;
+    return e;
 }
-// (h, l) += x^2
-__device__ __forceinline__ void pair_add_square(float& h, float& l, float x) {
-    const float q = __fmul_rn(x, x);
-    const float s = __fadd_rn(h, q), z = __fsub_rn(s, h);
-    const float e = __fadd_rn(__fsub_rn(h, __fsub_rn(s, z)), __fsub_rn(q, z));
-    l = __fadd_rn(l, __fadd_rn(e, __fmaf_rn(x, x, -q)));
-    h = s;
+__device__ __forceinline__ float two_sum(float& a, float b) {
+    const float s = __fadd_rn(a, b), z = __fsub_rn(s, a);
+    const float e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, z)), __fsub_rn(b, z));
+    a = s;
+    return e;
 }
-__device__ __forceinline__ float2 pair_mul(float2 a, float2 b) {
-    const float p = __fmul_rn(a.x, b.x);
-    float e = __fmaf_rn(a.x, b.x, -p);
-    e = __fmaf_rn(a.x, b.y, e);
-    e = __fmaf_rn(a.y, b.x, e);
-    const float h = __fadd_rn(p, e);
-    return make_float2(h, __fsub_rn(e, __fsub_rn(h, p)));
+__device__ __forceinline__ void add(Triple2& t, const Triple2& b) {
+    const float2 e0 = two_sum(t.h, b.h);
+    const float2 e1 = two_sum(t.l, b.l);
+    const float2 e2 = two_sum(t.l, e0);
+    t.m = padd(t.m, padd(b.m, padd(e1, e2)));
 }
+__device__ __forceinline__ void add(Triple& t, const Triple& b) {
+    const float e0 = two_sum(t.h, b.h);
+    const float e1 = two_sum(t.l, b.l);
+    const float e2 = two_sum(t.l, e0);
+    t.m = __fadd_rn(t.m, __fadd_rn(b.m, __fadd_rn(e1, e2)));
+}
+// t += x^2 (the square exactly: q and its error)
+__device__ __forceinline__ void add_square(Triple2& t, float2 x) {
+    const float2 q = pmul(x, x), e = pfma(x, x, make_float2(-q.x, -q.y));
+    const float2 e0 = two_sum(t.h, q);
+    const float2 e1 = two_sum(t.l, e);
+    const float2 e2 = two_sum(t.l, e0);
+    t.m = padd(t.m, padd(e1, e2));
+}
+// a b: the products down to the third word, their errors down to the second
+__device__ __forceinline__ Triple mul(const Triple& a, const Triple& b) {
+    Triple r;
+    r.h = __fmul_rn(a.h, b.h);
+    r.l = __fmaf_rn(a.h, b.h, -r.h);
+    const float p = __fmul_rn(a.h, b.l), q = __fmul_rn(a.l, b.h);
+    float m = __fadd_rn(__fmaf_rn(a.h, b.l, -p), __fmaf_rn(a.l, b.h, -q));
+    m = __fmaf_rn(a.l, b.l, __fmaf_rn(a.h, b.m, __fmaf_rn(a.m, b.h, m)));
+    const float e0 = two_sum(r.l, p);
+    const float e1 = two_sum(r.l, q);
+    r.m = __fadd_rn(m, __fadd_rn(e0, e1));
+    return r;
+}
+__device__ __forceinline__ Triple triple(double x) {
+    const float h = (float)x;
+    const double d = x - (double)h;
+    const float l = (float)d;
+    return Triple{h, l, (float)(d - (double)l)};
+}
+__device__ __forceinline__ double value(const Triple& t) { return (double)t.h + ((double)t.l + (double)t.m); }
 
 // shell of the integer n2 = |n|^2 <= 3 (N / 2)^2: |n| is never within 1.4e-4 of
 // a half-integer (n2 = i^2 + i lies 1/8 / i below one) and the correctly
@@ -837,25 +879,21 @@ __device__ __forceinline__ int pk_shell(float n2, float* root) {
 __global__ void __launch_bounds__(PK_WARPS * 32) k_pk_bin(const float* __restrict__ mesh, int N, int S, int nb,
                                                           int nbins, const double* __restrict__ wpk,
                                                           double* __restrict__ part) {
-    extern __shared__ float2 pk_smem[];
+    extern __shared__ Triple pk_smem[];
     const int M = N / 2 + 1, Sc = S / 2;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    float2* wt = pk_smem;                                        // [M] window weights as pairs
-    float2* sp = wt + M;                                         // [PK_WARPS][nb] power
-    float2* sk = sp + PK_WARPS * nb;                             // [PK_WARPS][nb] |n|
+    Triple* wt = pk_smem;                                        // [M] window weights
+    Triple* sp = wt + M;                                         // [PK_WARPS][nb] power
+    Triple* sk = sp + PK_WARPS * nb;                             // [PK_WARPS][nb] |n|
     unsigned* sc = reinterpret_cast<unsigned*>(sk + PK_WARPS * nb);   // [PK_WARPS][nb] weights
-    for (int i = threadIdx.x; i < M; i += blockDim.x) {
-        const double w = wpk[i];
-        const float h = (float)w;
-        wt[i] = make_float2(h, (float)(w - (double)h));
-    }
+    for (int i = threadIdx.x; i < M; i += blockDim.x) wt[i] = triple(wpk[i]);
     for (int i = threadIdx.x; i < PK_WARPS * nb; i += blockDim.x) {
-        sp[i] = sk[i] = make_float2(0.0f, 0.0f);
+        sp[i] = sk[i] = Triple{0.0f, 0.0f, 0.0f};
         sc[i] = 0u;
     }
     __syncthreads();
-    float2* wp = sp + warp * nb - 1;                             // bins from shell 1
-    float2* wk = sk + warp * nb - 1;
+    Triple* wp = sp + warp * nb - 1;                             // bins from shell 1
+    Triple* wk = sk + warp * nb - 1;
     unsigned* wc = sc + warp * nb - 1;
     const float2* base = reinterpret_cast<const float2*>(mesh);
     const int nw = gridDim.x * PK_WARPS;
@@ -869,7 +907,7 @@ __global__ void __launch_bounds__(PK_WARPS * 32) k_pk_bin(const float* __restric
         const float2* r3 = base + ((int64_t)bz * N + ay) * Sc;
         const float rows = (ry ? 2.0f : 1.0f) * (rz ? 2.0f : 1.0f);
         const float c2 = (float)(a * a + b * b);
-        const float2 wab = pair_mul(wt[a], wt[b]);
+        const Triple wab = mul(wt[a], wt[b]);
         const float2 zero = make_float2(0.0f, 0.0f);
         float2 n0, n1, n2v, n3;
         auto fetch = [&](int kx) {
@@ -886,24 +924,27 @@ __global__ void __launch_bounds__(PK_WARPS * 32) k_pk_bin(const float* __restric
             const float2 v0 = n0, v1 = n1, v2 = n2v, v3 = n3;
             const int kx = kx0 + lane;
             if (kx0 + 32 < M) fetch(kx + 32);
-            float ph = 0.0f, pl = 0.0f;
-            pair_add_square(ph, pl, v0.x);
-            pair_add_square(ph, pl, v0.y);
-            pair_add_square(ph, pl, v1.x);
-            pair_add_square(ph, pl, v1.y);
-            pair_add_square(ph, pl, v2.x);
-            pair_add_square(ph, pl, v2.y);
-            pair_add_square(ph, pl, v3.x);
-            pair_add_square(ph, pl, v3.y);
+            // real and imaginary parts side by side, then together
+            const float2 sc2 = pk2(PK_SCALE);
+            const float2 y = pmul(sc2, v0), y2 = pmul(y, y);
+            Triple2 s2{y2, pfma(y, y, make_float2(-y2.x, -y2.y)), zero};
+            if (ry) add_square(s2, pmul(sc2, v1));
+            if (rz) add_square(s2, pmul(sc2, v2));
+            if (ry && rz) add_square(s2, pmul(sc2, v3));
+            Triple p{s2.h.x, s2.l.x, s2.m.x};
+            add(p, Triple{s2.h.y, s2.l.y, s2.m.y});
+            p = mul(p, wt[min(kx, M - 1)]);
             const float mult = kx == 0 || kx == N / 2 ? 1.0f : 2.0f;
-            const float2 p = pair_mul(make_float2(ph, pl), wt[min(kx, M - 1)]);
-            ph = p.x * mult;
-            pl = p.y * mult;
             const float q2 = c2 + (float)(kx * kx);              // exact: < 2^24
             int shell = pk_shell(q2, &root);
             if (kx >= M) shell = 0x7fffffff;
-            const float rl = shell > 0 ? __fdividef(__fmaf_rn(-root, root, q2), 2.0f * root) : 0.0f;
-            float kh = root * mult, kl = rl * mult;
+            // |n| = root + l + x: q2 - root^2 is exact, then (root + l + x)^2 = q2
+            const float inv = shell > 0 ? __fdividef(0.5f, root) : 0.0f;
+            const float d = __fmaf_rn(-root, root, q2), l = __fmul_rn(d, inv);
+            const float x = __fmul_rn(__fmaf_rn(-2.0f * root, l, d) - __fmul_rn(l, l), inv);
+            // power and |n| side by side
+            const float2 mu = pk2(mult);
+            Triple2 t{pmul(mu, make_float2(p.h, root)), pmul(mu, make_float2(p.l, l)), pmul(mu, make_float2(p.m, x))};
             // runs of equal shells
             const int before = __shfl_up_sync(0xffffffffu, shell, 1);
             const unsigned heads = __ballot_sync(0xffffffffu, lane == 0 || shell != before);
@@ -911,22 +952,20 @@ __global__ void __launch_bounds__(PK_WARPS * 32) k_pk_bin(const float* __restric
             for (int o = 1; o < 32; o <<= 1) {
                 const bool in = lane - o >= head;
                 if (!__any_sync(0xffffffffu, in)) break;         // no run is longer than o
-                const float a0 = __shfl_up_sync(0xffffffffu, ph, o), a1 = __shfl_up_sync(0xffffffffu, pl, o);
-                const float b0 = __shfl_up_sync(0xffffffffu, kh, o), b1 = __shfl_up_sync(0xffffffffu, kl, o);
-                if (in) {
-                    pair_add(ph, pl, a0, a1);
-                    pair_add(kh, kl, b0, b1);
-                }
+                auto up = [&](float2 v) {
+                    return make_float2(__shfl_up_sync(0xffffffffu, v.x, o), __shfl_up_sync(0xffffffffu, v.y, o));
+                };
+                const Triple2 u{up(t.h), up(t.l), up(t.m)};
+                if (in) add(t, u);
             }
             const bool tail = lane == 31 || ((heads >> (lane + 1)) & 1u);
             if (tail && shell >= 1 && shell <= nb) {
-                const float2 w = pair_mul(make_float2(ph, pl), wab);
-                float2 acc = wp[shell];
-                pair_add(acc.x, acc.y, w.x, w.y);
-                wp[shell] = acc;
-                acc = wk[shell];
-                pair_add(acc.x, acc.y, kh * rows, kl * rows);
-                wk[shell] = acc;
+                const Triple w = mul(Triple{t.h.x, t.l.x, t.m.x}, wab), ap = wp[shell], ak = wk[shell];
+                Triple2 acc{make_float2(ap.h, ak.h), make_float2(ap.l, ak.l), make_float2(ap.m, ak.m)};
+                add(acc, Triple2{make_float2(w.h, rows * t.h.y), make_float2(w.l, rows * t.l.y),
+                                 make_float2(w.m, rows * t.m.y)});
+                wp[shell] = Triple{acc.h.x, acc.l.x, acc.m.x};
+                wk[shell] = Triple{acc.h.y, acc.l.y, acc.m.y};
                 const int len = lane - head + 1;
                 const int cnt = 2 * len - (kx0 + head == 0) - (kx == N / 2);
                 wc[shell] += (unsigned)cnt * (unsigned)rows;
@@ -937,16 +976,16 @@ __global__ void __launch_bounds__(PK_WARPS * 32) k_pk_bin(const float* __restric
     __syncthreads();
     double* out = part + (int64_t)blockIdx.x * 3 * nbins;
     for (int i = threadIdx.x; i < nb; i += blockDim.x) {
-        double c = 0.0, k = 0.0, p = 0.0;
+        Triple2 s{make_float2(0.0f, 0.0f), make_float2(0.0f, 0.0f), make_float2(0.0f, 0.0f)};
+        double c = 0.0;
         for (int w = 0; w < PK_WARPS; ++w) {
-            const float2 vk = sk[w * nb + i], vp = sp[w * nb + i];
+            const Triple vp = sp[w * nb + i], vk = sk[w * nb + i];
             c += (double)sc[w * nb + i];
-            k += (double)vk.x + (double)vk.y;
-            p += (double)vp.x + (double)vp.y;
+            add(s, Triple2{make_float2(vp.h, vk.h), make_float2(vp.l, vk.l), make_float2(vp.m, vk.m)});
         }
         out[i] = c;
-        out[nbins + i] = k;
-        out[2 * nbins + i] = p;
+        out[nbins + i] = value(Triple{s.h.y, s.l.y, s.m.y});
+        out[2 * nbins + i] = value(Triple{s.h.x, s.l.x, s.m.x}) * (1.0 / ((double)PK_SCALE * PK_SCALE));
     }
 }
 
@@ -955,7 +994,7 @@ __host__ __device__ __forceinline__ int pk_used_bins(int N, int nbins) { return 
 
 // window weights, and each warp's sums of nb bins
 size_t pk_bytes(int N, int nb) {
-    return (size_t)(N / 2 + 1) * sizeof(float2) + (size_t)PK_WARPS * nb * (2 * sizeof(float2) + sizeof(unsigned));
+    return (size_t)(N / 2 + 1) * sizeof(Triple) + (size_t)PK_WARPS * nb * (2 * sizeof(Triple) + sizeof(unsigned));
 }
 
 // one warp per bin: the blocks' sums in a fixed order; bins from nb on lie

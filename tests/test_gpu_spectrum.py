@@ -1,5 +1,6 @@
 """The power spectrum's binning beyond 300 shells, from several threads and
 against sums of known modes."""
+import math
 import threading
 
 import numpy as np
@@ -96,3 +97,45 @@ def test_spectra_from_several_threads(cube):
     finally:
         for c, _ in ctxs:
             cube.cube_destroy(c)
+
+
+# All particles on the node at the origin: every mode is that node's density,
+# so the shells' sums are known to more bits than FP64 keeps.  Roundings on the
+# way, of 2^-53 each and all sums of positive terms: one where a block's sums
+# become FP64, ceil(blocks / 32) + 5 additions over the blocks, four in the
+# final factors and quotient (blocks: of eight rows (|ky|, |kz|), 456 at most);
+# the window weights are the host's, from the same expression.
+@pytest.mark.parametrize("nf,n_bins", [(16, 13), (48, 24), (192, 150)])
+def test_binning_keeps_every_bit_of_fp64(cube, nf, n_bins):
+    n, box = 100003, 50.0
+    prm = cube.make_params(nf, n, x_bytes=4, v_bytes=4, id_bytes=0, box=box)
+    ctx = cube.cube_create(prm, torch.cuda.current_stream())
+    try:
+        cube.cube_encode(ctx, np.zeros((3, n), np.float32), np.zeros((3, n), np.float32), None, 0.02, 0.5)
+        rho = np.empty((nf, nf, nf), np.float32)
+        cube.cube_density(ctx, rho)
+        assert np.count_nonzero(rho) == 1 and rho[0, 0, 0] > 0
+        k, p, m = _spectrum(cube, ctx, n_bins)
+    finally:
+        cube.cube_destroy(ctx)
+    real = np.longdouble
+    h = nf // 2
+    sinc = [1.0] + [math.sin(math.pi * i / nf) / (math.pi * i / nf) for i in range(1, h + 1)]
+    w = np.array([math.pow(s, -4.0) for s in sinc]).astype(real)
+    mult = np.where((np.arange(h + 1) == 0) | (np.arange(h + 1) == h), 1, 2)
+    i2 = np.arange(h + 1, dtype=np.int64) ** 2
+    n2 = (i2[:, None, None] + i2[:, None] + i2).ravel()
+    count = (mult[:, None, None] * mult[:, None] * mult).ravel()
+    root = np.sqrt(n2.astype(real))
+    weight = (w[:, None, None] * w[:, None] * w).ravel()
+    shell = np.floor(root.astype(np.float64) + 0.5).astype(np.int64)
+    blocks = min(456, ((h + 1) ** 2 + 7) // 8)
+    tol = (1 + -(-blocks // 32) + 5 + 4) * 2.0 ** -53
+    for i in range(1, n_bins + 1):
+        at = shell == i
+        modes = int(count[at].sum())
+        assert m[i - 1] == modes
+        want_k = 2 * real(math.pi) / real(box) * (count[at] * root[at]).sum() / modes
+        want_p = real(box) ** 3 / real(nf) ** 6 * real(rho[0, 0, 0]) ** 2 * (count[at] * weight[at]).sum() / modes
+        assert abs(real(k[i - 1]) / want_k - 1) <= tol, (i, k[i - 1], want_k)
+        assert abs(real(p[i - 1]) / want_p - 1) <= tol, (i, p[i - 1], want_p)
