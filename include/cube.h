@@ -344,13 +344,14 @@ cube_status cube_debug_velocity_tables(cube_ctx* ctx, int64_t* out2);
 /* ---------------------------------------------------------------- tracing */
 
 /* Kernel phases of one cube_pm_step, in launch order:
-   0 setup (clears the new-store counters; no kernel), 1 deposit (CIC density),
+   0 setup (no kernel), 1 deposit (CIC density; clears the new-store counters),
    2 fft_x_r2c, 3 fft_y_fwd, 4 fft_z_green (z forward, Green's function, z
    inverse), 5 fft_y_inv, 6 fft_x_c2r, 7 pass_a (decode, force gather, kick,
-   drift, per-brick histograms of the new cells), 8 codec (next codec scale
-   and tables), 9 scan (of the histograms in cell-major, brick-minor order:
-   per-brick starts), 10 cells (new counts, offsets and v_c),
-   11 pass_b (stable scatter and encode).  Section 2.3.3 places such timing
+   drift, per-brick histograms of the new cells), 8 codec (next codec scale;
+   sums of the histograms' tiles), 9 scan (of the tile sums: stores of more
+   than 8192 tiles, else no kernel), 10 cells (the histograms' scan in
+   cell-major, brick-minor order: per-brick starts; new counts, offsets and
+   v_c; next codec tables), 11 pass_b (stable scatter and encode).  Section 2.3.3 places such timing
    statistics in the code's final stage. */
 #define CUBE_PHASES 12
 

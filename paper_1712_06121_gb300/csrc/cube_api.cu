@@ -757,7 +757,8 @@ cube_status cube_encode(cube_ctx* c, const float* pos, const float* vel, const u
 
 // kernels launched per phase of a step (see cube_phase_name): the codec
 // phase's kernel also sums the scan's tiles, the cells phase's kernel scans
-// them and builds the codec tables
+// them and builds the codec tables; the scan phase has kernels of its own only
+// for stores of many tiles (step_scan_launches)
 const int kPhaseKernels[CUBE_PHASES] = {0, 1, 1, 1, 1, 1, 1, 1, 1, 0, 1, 1};
 const char* kPhaseNames[CUBE_PHASES] = {"setup", "deposit", "fft_x_r2c", "fft_y_fwd", "fft_z_green", "fft_y_inv",
                                         "fft_x_c2r", "pass_a", "codec", "scan", "cells", "pass_b"};
@@ -857,13 +858,14 @@ cube_status cube_pm_step(cube_ctx* c, double a_from, double a_to) {
     mark(c, 8);
     launch_step_sums(g, w, ratio, c->codec[kn].sigma, c->scan_tmp, c->st);
     mark(c, 9);
+    launch_step_scan(g, c->scan_tmp, c->st);
     mark(c, 10);
     launch_step_cells(g, w, c->offsets[kn], c->vc[kn], c->tanv, c->tanh_, c->codec[kn], c->scan_tmp, c->st);
     mark(c, 11);
     launch_passB(g, c->store(k), c->store(kn), c->codec[k], c->codec[kn], dc, w, c->st);
     mark(c, 12);
     CK(cudaEventRecord(c->ev1, c->st));
-    c->launches += 4;
+    c->launches += 4 + step_scan_launches(g);
     if (c->prof_steps < c->prof_max) c->prof_steps += 1;
     CK(cudaGetLastError());
     c->cur = kn;
@@ -1443,7 +1445,7 @@ cube_status cube_profile_read(cube_ctx* c, double* ms, int32_t* kernels, int32_t
             t += e;
         }
         ms[p] = t;
-        if (kernels) kernels[p] = c->raw ? kPhaseKernelsRaw[p] : kPhaseKernels[p];
+        if (kernels) kernels[p] = c->raw ? kPhaseKernelsRaw[p] : kPhaseKernels[p] + (p == 9 ? step_scan_launches(c->g) : 0);
     }
     if (nsteps) *nsteps = c->prof_steps;
     return CUBE_OK;

@@ -1247,7 +1247,8 @@ __global__ void k_cells(Geo g, StepScratch w, unsigned* __restrict__ off_new, fl
 // A single context's step runs two kernels between its passes, over tiles of
 // whole bricks (16, 64 or 128 of them: at most 4096 histogram slots, eight a
 // thread, and 1024 cells, two a thread): k_step_sums adds each tile's slots up, k_step_cells starts from the
-// sum of the tiles before its own, scans its slots in place and, with the
+// sum of the tiles before its own (of many tiles, where that would add up tiles^2 / 2
+// words, from a scan of the tile sums), scans its slots in place and, with the
 // scanned values in shared memory, finishes the cells of its bricks.  The
 // codec rides along: one block of the first kernel finds the next scale, a few
 // blocks of the second build its tables.  Eight launches before (scale,
@@ -1317,7 +1318,7 @@ __global__ void __launch_bounds__(1024) k_step_sums(Geo g, StepScratch w, double
 __global__ void __launch_bounds__(SC_T) k_step_cells(Geo g, StepScratch w, const unsigned* __restrict__ tsum,
                                                      unsigned* __restrict__ off_new, float* __restrict__ vc_new,
                                                      const double* __restrict__ tanv, const double* __restrict__ tanh_,
-                                                     CodecDev next, int ntab) {
+                                                     CodecDev next, int ntab, bool scanned) {
     chain_wait();
     if ((int)blockIdx.x < ntab) {                            // the next codec's tables
         codec_tables_body(g.nulim, tanv, tanh_, *next.sigma, next.dec, next.thr, next.est,
@@ -1342,7 +1343,9 @@ __global__ void __launch_bounds__(SC_T) k_step_cells(Geo g, StepScratch w, const
             vs[h][d] = c < ncell ? w.vsum_new[(int64_t)d * g.Ncc + L0 + c] : 0;
         }
     unsigned before = 0;
-    for (int j = threadIdx.x; j < tile; j += SC_T) before += tsum[j];
+    if (scanned) before = threadIdx.x == 0 ? tsum[tile] : 0u;
+    else
+        for (int j = threadIdx.x; j < tile; j += SC_T) before += tsum[j];
     unsigned s = 0;
 #pragma unroll
     for (int k = 0; k < SC_ITEMS; ++k) s += v[k];
@@ -2043,7 +2046,22 @@ void launch_cells(const Geo& g, const StepScratch& w, unsigned* off_new, float* 
     launch_chained(k_cells, dim3(nblk(g.Ncc, 256), bt.members), 256, 0, st, g, w, off_new, vc_new, bt);
 }
 
-int step_tmp_words(const Geo& g) { return step_tiles(g); }
+// Beyond STEP_TILES tiles their sums are scanned in two more launches, us of the
+// three (every tile adding up the ones before it / scanned): 4096 tiles 57 /
+// 62, 6912 139 / 141, 16384 319 / 310, 55296 1166 / 1002, 131072 (a mesh of
+// 512^3 at ratio 1, a step of 28 ms) 3470 / 2352.
+constexpr int STEP_TILES = 8192;
+int step_scan_launches(const Geo& g) { return step_tiles(g) > STEP_TILES ? scan_launches(step_tiles(g)) : 0; }
+
+int step_tmp_words(const Geo& g) {
+    const int n = step_tiles(g);
+    return n > STEP_TILES ? n + 1 + scan_tmp_words(n) : n;
+}
+
+void launch_step_scan(const Geo& g, unsigned* tmp, cudaStream_t st) {
+    const int n = step_tiles(g);
+    if (n > STEP_TILES) exclusive_scan(tmp, tmp, n, tmp + n + 1, st);
+}
 
 void launch_step_sums(const Geo& g, const StepScratch& w, double ratio, double* sigma_out, unsigned* tmp,
                       cudaStream_t st) {
@@ -2053,7 +2071,8 @@ void launch_step_sums(const Geo& g, const StepScratch& w, double ratio, double* 
 void launch_step_cells(const Geo& g, const StepScratch& w, unsigned* off_new, float* vc_new, const double* tanv,
                        const double* tanh, const CodecDev& next, const unsigned* tmp, cudaStream_t st) {
     const int ntab = g.nnu == 1 ? 1 : nblk(g.nulim + 2, SC_T);
-    launch_chained(k_step_cells, dim3(ntab + step_tiles(g)), SC_T, 0, st, g, w, tmp, off_new, vc_new, tanv, tanh, next, ntab);
+    launch_chained(k_step_cells, dim3(ntab + step_tiles(g)), SC_T, 0, st, g, w, tmp, off_new, vc_new, tanv, tanh, next, ntab,
+                   step_tiles(g) > STEP_TILES);
 }
 
 // `words` of a CTA's brick tables after the staged 1-byte codec tables

@@ -206,11 +206,13 @@ void launch_passA(const Geo& g, const StoreDev& s, const float* phig, const CUte
 // a batch step's cleared scratch (momentum sums, migration words) of its stepped members
 void launch_batch_clear(const Geo& g, long long* vsum, int* maxmig, cudaStream_t st, const Batch& bt);
 // a single context's kernels between the passes: the histograms' tile sums and
-// the next codec scale, then the scanned histograms, the new cells' counts,
+// the next codec scale, the tile sums' scan (many tiles only), then the scanned histograms, the new cells' counts,
 // offsets and v_c, and the next codec's tables.  tmp: step_tmp_words words
 int step_tmp_words(const Geo& g);
 void launch_step_sums(const Geo& g, const StepScratch& w, double ratio, double* sigma_out, unsigned* tmp,
                       cudaStream_t st);
+int step_scan_launches(const Geo& g);
+void launch_step_scan(const Geo& g, unsigned* tmp, cudaStream_t st);
 void launch_step_cells(const Geo& g, const StepScratch& w, unsigned* off_new, float* vc_new, const double* tanv,
                        const double* tanh, const CodecDev& next, const unsigned* tmp, cudaStream_t st);
 // the new cells of a batch, from the scanned histograms
