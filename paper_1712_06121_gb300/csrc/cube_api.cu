@@ -272,6 +272,7 @@ struct cube_ctx {
     unsigned* ghost = nullptr;
     float* part = nullptr;
     int npart = 0;
+    unsigned* ncrowded = nullptr;
     unsigned* flags = nullptr;
     unsigned* line = nullptr;       // pinned, 64 bytes: small read-backs
     int* maxmig = nullptr;
@@ -357,8 +358,10 @@ size_t state_layout(cube_ctx* c, char* base) {
     }
     carve(base, off, c->tanv, (size_t)(g.nulim + 1) * 8);
     carve(base, off, c->tanh_, (size_t)(g.nulim + 2) * 8);
-    // error flags and vmax (one read-back), largest migration, crowded-brick list
-    carve(base, off, c->flags, ((size_t)g.nbricks + 4) * 4);
+    // length of the encode's list of crowded groups; error flags (cleared with it)
+    // and vmax (read back together); largest migration, crowded-brick list
+    carve(base, off, c->ncrowded, ((size_t)g.nbricks + 5) * 4);
+    c->flags = base ? c->ncrowded + 1 : nullptr;
     c->vmax = base ? c->flags + 1 : nullptr;
     c->maxmig = base ? (int*)(c->flags + 2) : nullptr;
     carve(base, off, c->mom, 4 * 8);
@@ -388,7 +391,7 @@ size_t work_layout(cube_ctx* c, char* base) {
     carve(base, off, c->phig, (size_t)phig_nx(g.N) * phig_ny(g.N) * phig_ny(g.N) * 4);
     carve(base, off, c->vsum, 3 * Ncc * 8);
     carve(base, off, c->ghost, ((size_t)g.nbricks * H3 + 1) * 4);
-    c->npart = std::max(g.nbricks, 1024);
+    c->npart = (int)std::max<int64_t>(std::max(g.nbricks, 1024), c->raw ? 0 : encode_partials(g));
     carve(base, off, c->part, (size_t)c->npart * 4);
     carve(base, off, c->scan_tmp,
           (size_t)std::max(scan_tmp_words(std::max<int64_t>(g.Ncc + 1, (int64_t)g.nbricks * H3 + 1)),
@@ -723,8 +726,10 @@ static cube_status encode_impl(cube_ctx* c, const float* pos, const float* vel, 
     if (hid) { CK(cudaMemcpyAsync(sp, id, 4 * Np, cudaMemcpyHostToDevice, c->st)); did = (const unsigned*)sp; }
     c->cur = 0;                          // a fresh store always starts in buffer 0 (batch members stay in step)
     const int k = c->cur;
-    CK(cudaMemsetAsync(c->flags, 0, 4, c->st));
+    CK(cudaMemsetAsync(c->ncrowded, 0, 8, c->st));                // and the flags
     CK(cudaMemsetAsync(c->counts[k], 0, (size_t)g.Ncc * 4, c->st));
+    // (the list of crowded groups goes where the sort's histograms were)
+    const Crowded crowded = encode_crowded(g, c->ncrowded, rtmp, c->vsum, c->part);
     launch_encode_keys(g, dpos, keys, c->counts[k], c->flags, c->st);
     exclusive_scan(c->counts[k], c->offsets[k], g.Ncc, c->scan_tmp, c->st);
     unsigned* spare[3];
@@ -732,12 +737,14 @@ static cube_status encode_impl(cube_ctx* c, const float* pos, const float* vel, 
     // the momenta in storage order take the sort's other arrays
     float* const vsorted[3] = {(float*)spare[0], (float*)spare[1], (float*)spare[2]};
     const StoreDev store = c->store(k);
-    launch_encode_vc(g, dvel, order, store, vsorted, sigma > 0.0 ? nullptr : c->part, c->flags, c->st);
-    launch_sigma_finalize(c->part, sigma > 0.0 ? 0 : encode_groups(g), 3.0 * (double)g.Np, 1.0, sigma > 0.0 ? sigma : 0.0,
-                          c->codec[k].sigma, c->st);
+    int kernels =
+        launch_encode_vc(g, dvel, order, store, vsorted, sigma > 0.0 ? nullptr : c->part, crowded, c->flags, c->st);
+    const int nparts = sigma > 0.0 ? 0 : (int)(crowded.ctas ? encode_partials(g) : encode_groups(g));
+    launch_sigma_finalize(c->part, nparts, 3.0 * (double)g.Np, 1.0, sigma > 0.0 ? sigma : 0.0,
+                          c->codec[k].sigma, true, c->st);
     launch_codec_tables(g.nulim, c->tanv, c->tanh_, c->codec[k], c->st);
-    launch_encode_codes(g, dpos, vsorted, did, order, c->codec[k], store, c->st);
-    c->launches += 1 + scan_launches(g.Ncc) + radix_launches(g.Np, key_bits) + 4;
+    kernels += launch_encode_codes(g, dpos, vsorted, did, order, c->codec[k], store, crowded, c->st);
+    c->launches += 1 + scan_launches(g.Ncc) + radix_launches(g.Np, key_bits) + kernels + 2;
     CK(cudaGetLastError());
     if (sync) CK(cudaStreamSynchronize(c->st));
     c->encoded = true;
@@ -1786,7 +1793,7 @@ cube_status cube_batch_step(cube_batch* b, const double* a_from, const double* a
         launch_batch_clear(g, c0->vsum, c0->maxmig, b->st, bt);
         launch_passA(g, c0->store(k), c0->phig, b->tma ? &b->map : nullptr, c0->codec[k], 0.0f, 0.0f, w, nodbg,
                      b->st, bt);
-        launch_sigma_finalize(c0->part, g.nbricks, 3.0 * (double)g.Np, 1.0, 0.0, c0->codec[kn].sigma, b->st, bt);
+        launch_sigma_finalize(c0->part, g.nbricks, 3.0 * (double)g.Np, 1.0, 0.0, c0->codec[kn].sigma, false, b->st, bt);
         launch_codec_tables(g.nulim, c0->tanv, c0->tanh_, c0->codec[kn], b->st, bt);
         exclusive_scan(c0->ghost, c0->ghost, (int64_t)g.nbricks * (g.Bh * g.Bh * g.Bh), c0->scan_tmp, b->st, bt);
         launch_cells(g, w, c0->offsets[kn], c0->vc[kn], b->st, bt);

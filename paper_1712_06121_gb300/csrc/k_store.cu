@@ -212,119 +212,237 @@ __global__ void k_encode_keys(Geo g, const float* __restrict__ pos, unsigned* __
     if (bad) atomicOr(flags, ERR_NONFINITE);
 }
 
-// Cells of a CTA of the two kernels below: consecutive in storage order, so
-// their particles are too, whatever the brick (the encode of 128^3 particles
-// in bricks of one cell: 482 us with a CTA a brick -> 184; of 64 cells 183)
+// Cells of a CTA of k_encode_vc and k_encode_codes: consecutive in storage order, so their
+// particles are too, whatever the brick (the encode of 128^3 particles in bricks
+// of one cell: 482 us with a CTA a brick -> 184; of 64 cells 183)
 constexpr int ENC_CELLS = 64;
 
+// A CTA's 64 cells may hold any number of particles (a halo in a cell).  Groups
+// of more than ENC_BIG are cut at the multiples of ENC_RUN in storage order, and
+// the runs taken by CTAs of their own from a list, so that no CTA works on more
+// than ENC_BIG particles and no thread adds the squares of more than 64.  A run's
+// slot is 2 c if it begins at c ENC_RUN and 2 c + 1 if its group begins inside
+// that run: no two share one, and the scale's sum does not depend on the list's
+// order.  Encode of 128^3 particles, a fifth of them in one cell: 4285 us by one CTA a
+// group (695 with the global atomics before it) -> 335; of 256^3, 5% in one
+// cell: 9065 (2134) -> 1160.  The three launches that find an empty list: 5 of
+// 250 us, 14 of 1087.
+constexpr unsigned ENC_RUN = 8192, ENC_BIG = 2 * ENC_RUN;
+__host__ __device__ __forceinline__ int64_t crowded_slots(const Geo& g) { return 2 * (g.Np / ENC_RUN + 1); }
+
+// the offsets of group G's cells in shared memory, off[0 .. *nc], and its
+// particles [*q0, *q1)
+__device__ __forceinline__ void stage_group(const Geo& g, const unsigned* __restrict__ offsets, int G, unsigned* off,
+                                            int* nc, unsigned* q0, unsigned* q1) {
+    const int L0 = G * ENC_CELLS;
+    *nc = min(ENC_CELLS, g.Ncc - L0);
+#pragma unroll 1
+    for (int c = threadIdx.x; c <= *nc; c += blockDim.x) off[c] = offsets[L0 + c];
+    __syncthreads();
+    *q1 = min(off[*nc], (unsigned)g.Np);
+    *q0 = min(off[0], *q1);
+}
+__device__ __forceinline__ void cut_to_run(unsigned slot, unsigned* q0, unsigned* q1) {
+    const unsigned c = slot >> 1;
+    *q0 = max(*q0, c * ENC_RUN);
+    *q1 = min(*q1, (c + 1) * ENC_RUN);
+}
+
+// a crowded group's runs appended to the list and its cells' sums cleared, by its CTA
+__device__ void list_runs(const Geo& g, const Crowded& cr, int G, int nc, unsigned q0, unsigned q1) {
+    const unsigned c0 = q0 / ENC_RUN, n = (q1 - 1) / ENC_RUN - c0 + 1;
+    __shared__ unsigned at;
+    if (threadIdx.x == 0) at = atomicAdd(cr.count, n);
+    for (int t = threadIdx.x; t < 3 * ENC_CELLS; t += blockDim.x)
+        if (t % ENC_CELLS < nc) cr.vsum[(int64_t)(t / ENC_CELLS) * g.Ncc + G * ENC_CELLS + t % ENC_CELLS] = 0;
+    __syncthreads();
+    for (unsigned k = threadIdx.x; k < n; k += blockDim.x)
+        cr.item[at + k] = make_uint2(G, 2 * (c0 + k) + (q0 > (c0 + k) * ENC_RUN ? 1u : 0u));
+}
+
 // One CTA per 64 cells of the sorted order: the particles' momenta are gathered
-// once, written in storage order for the kernels that follow, and added up
-// per cell in shared memory (exact fixed point); then v_c, and the cells' sum
-// of squared offsets for a measured codec scale.  256^3 particles x1v1: this
-// 273 us and k_encode_codes 231, where 64-bit global atomics per particle, the
-// measurement and the final gather took 215 + 28 + 58 + 398 us in four kernels;
-// the whole encode with its sort 1540 -> 1129 us.
-__global__ void __launch_bounds__(T_BRICK) k_encode_vc(Geo g, const float* __restrict__ vel,
-                                                       const unsigned* __restrict__ perm, StoreDev s, float* v0,
-                                                       float* v1, float* v2, float* __restrict__ part,
-                                                       unsigned* flags) {
+// once, written in storage order for the kernels that follow, and added up per
+// cell in shared memory (exact fixed point); then v_c, and the cells' sum of
+// squared offsets for a measured codec scale.  Crowded groups are only listed;
+// the same kernel with RUNS then adds up their runs, CTA by CTA of the list, and
+// k_encode_crowded finishes them.  (In one launch, the list's idle CTAs leave
+// the groups unevenly over the SMs: 78 to 92 us against 66 for 512 groups of 4096
+// particles.)  256^3 particles x1v1: this 182 us and k_encode_codes 203, where
+// 64-bit global atomics per particle, the measurement and the final gather took
+// 215 + 28 + 58 + 398 us in four kernels; the whole encode with its sort 1540 ->
+// 1087 us.
+template <bool RUNS>
+__global__ void __launch_bounds__(T_BRICK, 6) k_encode_vc(Geo g, const float* __restrict__ vel,
+                                                          const unsigned* __restrict__ perm, StoreDev s, float* v0,
+                                                          float* v1, float* v2, float* __restrict__ part, Crowded cr,
+                                                          unsigned* flags) {
     __shared__ unsigned off[ENC_CELLS + 1];
     __shared__ unsigned vs[3 * ENC_CELLS * 2];               // {low, high} words
     __shared__ float svc[3 * ENC_CELLS];
     __shared__ double red[32];
     chain_wait();
-    const int L0 = blockIdx.x * ENC_CELLS, nc = min(ENC_CELLS, g.Ncc - L0);
-#pragma unroll 1
-    for (int c = threadIdx.x; c <= nc; c += blockDim.x) off[c] = s.offsets[L0 + c];
-#pragma unroll 1
-    for (int t = threadIdx.x; t < 6 * ENC_CELLS; t += blockDim.x) vs[t] = 0u;
-    __syncthreads();
-    const unsigned q1 = min(off[nc], (unsigned)g.Np), q0 = min(off[0], q1);
-    unsigned p0, p1;
-    brick_share(q0, q1, &p0, &p1);
     const unsigned lane = threadIdx.x & 31;
     float* vo[3] = {v0, v1, v2};
     const float* vi[3] = {vel, vel + g.Np, vel + 2 * g.Np};
     bool bad = false;
-    // 64 particles of the warp at a time, their loads in flight together
-    float v[2][3];
-    int cell[2] = {0, 0};
-    int c0 = p0 < p1 ? upper_cell(off, nc, p0) : 0;
-    for (unsigned base = p0; base < p1; base += 64) {
-        unsigned i[2];
+    const int nrun = RUNS ? (int)*cr.count : 0;
+    for (int k = blockIdx.x; !RUNS || k < nrun; k += gridDim.x) {
+        const uint2 item = RUNS ? cr.item[k] : make_uint2(blockIdx.x, 0u);
+        const int G = (int)item.x, L0 = G * ENC_CELLS;
+        if (RUNS) __syncthreads();                           // the last run's sums have been read
+#pragma unroll 1
+        for (int t = threadIdx.x; t < 6 * ENC_CELLS; t += blockDim.x) vs[t] = 0u;
+        int nc;
+        unsigned q0, q1, p0, p1;
+        stage_group(g, s.offsets, G, off, &nc, &q0, &q1);
+        if (RUNS) cut_to_run(item.y, &q0, &q1);
+        if (!RUNS && cr.ctas > 0) {
+            if (part && threadIdx.x == 0)
+                for (int64_t i = G; i < crowded_slots(g); i += gridDim.x) cr.part[i] = 0.0f;
+            if (q1 - q0 > ENC_BIG) {
+                if (part && threadIdx.x == 0) part[G] = 0.0f;
+                list_runs(g, cr, G, nc, q0, q1);
+                return;
+            }
+        }
+        brick_share(q0, q1, &p0, &p1);
+        // 64 particles of the warp at a time, their loads in flight together
+        float v[2][3];
+        int cell[2] = {0, 0};
+        int c0 = p0 < p1 ? upper_cell(off, nc, p0) : 0;
+        for (unsigned base = p0; base < p1; base += 64) {
+            unsigned i[2];
 #pragma unroll
-        for (int h = 0; h < 2; ++h) i[h] = base + 32 * h + lane < p1 ? perm[base + 32 * h + lane] : 0xffffffffu;
+            for (int h = 0; h < 2; ++h) i[h] = base + 32 * h + lane < p1 ? perm[base + 32 * h + lane] : 0xffffffffu;
 #pragma unroll
-        for (int h = 0; h < 2; ++h)
+            for (int h = 0; h < 2; ++h)
 #pragma unroll
-            for (int d = 0; d < 3; ++d) v[h][d] = i[h] < (unsigned)g.Np ? vi[d][i[h]] : 0.0f;
+                for (int d = 0; d < 3; ++d) v[h][d] = i[h] < (unsigned)g.Np ? vi[d][i[h]] : 0.0f;
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const unsigned j = base + 32 * h + lane;
-            int cnext;
-            cell[h] = warp_cells(off, nc, base + 32 * h, c0, &cnext);
-            c0 = cnext;
-            if (j < p1)
+            for (int h = 0; h < 2; ++h) {
+                const unsigned j = base + 32 * h + lane;
+                int cnext;
+                cell[h] = warp_cells(off, nc, base + 32 * h, c0, &cnext);
+                c0 = cnext;
+                if (j < p1)
+#pragma unroll
+                    for (int d = 0; d < 3; ++d) {
+                        if (!isfinite(v[h][d])) {
+                            bad = true;
+                            v[h][d] = 0.0f;
+                        }
+                        vo[d][j] = v[h][d];
+                        smem_add_u64(&vs[2 * (d * ENC_CELLS + cell[h])], (unsigned long long)vel_fix(v[h][d]));
+                    }
+            }
+        }
+        __syncthreads();
+        for (int t = threadIdx.x; t < 3 * ENC_CELLS; t += blockDim.x) {
+            const int d = t / ENC_CELLS, c = t % ENC_CELLS;
+            if (c >= nc) continue;
+            const unsigned long long sum = ((unsigned long long)vs[2 * t + 1] << 32) | vs[2 * t];
+            const int64_t at = (int64_t)d * g.Ncc + L0 + c;
+            if (RUNS) {
+                if (sum) atomicAdd(reinterpret_cast<unsigned long long*>(&cr.vsum[at]), sum);
+            } else {
+                const float m = vel_unfix_mean((long long)sum, off[c + 1] - off[c]);
+                svc[t] = m;
+                s.vc[at] = m;
+            }
+        }
+        if (RUNS) continue;
+        if (part) {
+            __syncthreads();
+            float acc = 0.0f;
+            auto add = [&](const float* x, int c) {
 #pragma unroll
                 for (int d = 0; d < 3; ++d) {
-                    if (!isfinite(v[h][d])) {
-                        bad = true;
-                        v[h][d] = 0.0f;
-                    }
-                    vo[d][j] = v[h][d];
-                    smem_add_u64(&vs[2 * (d * ENC_CELLS + cell[h])], (unsigned long long)vel_fix(v[h][d]));
+                    const float e = x[d] - svc[d * ENC_CELLS + c];
+                    acc = __fmaf_rn(e, e, acc);
                 }
+            };
+            if (p1 - p0 <= 64) {                             // the share is still in registers
+#pragma unroll
+                for (int h = 0; h < 2; ++h)
+                    if (p0 + 32 * h + lane < p1) add(v[h], cell[h]);
+            } else {
+                c0 = upper_cell(off, nc, p0);
+                for (unsigned base = p0; base < p1; base += 32) {
+                    const unsigned j = base + lane;
+                    int cnext;
+                    const int c = warp_cells(off, nc, base, c0, &cnext);
+                    c0 = cnext;
+                    if (j < p1) {
+                        const float x[3] = {vo[0][j], vo[1][j], vo[2][j]};
+                        add(x, c);
+                    }
+                }
+            }
+            const double t = block_sum_double((double)acc, red);
+            if (threadIdx.x == 0) part[G] = (float)t;
         }
+        break;
     }
-    __syncthreads();
-    for (int t = threadIdx.x; t < 3 * ENC_CELLS; t += blockDim.x) {
-        const int d = t / ENC_CELLS, c = t % ENC_CELLS;
-        if (c >= nc) continue;
-        const long long sum = (long long)(((unsigned long long)vs[2 * t + 1] << 32) | vs[2 * t]);
-        const float m = vel_unfix_mean(sum, off[c + 1] - off[c]);
-        svc[t] = m;
-        s.vc[(int64_t)d * g.Ncc + L0 + c] = m;
-    }
-    if (part) {
+    if (bad) atomicOr(flags, ERR_NONFINITE);
+}
+
+// the crowded groups' v_c (written by a group's first run) and their runs' sums
+// of squared offsets, each in its slot
+__global__ void __launch_bounds__(T_BRICK) k_encode_crowded(Geo g, StoreDev s, const float* v0, const float* v1,
+                                                            const float* v2, bool measure, Crowded cr) {
+    __shared__ unsigned off[ENC_CELLS + 1];
+    __shared__ float svc[3 * ENC_CELLS];
+    __shared__ double red[32];
+    chain_wait();
+    const unsigned lane = threadIdx.x & 31, nrun = *cr.count;
+    for (unsigned k = blockIdx.x; k < nrun; k += gridDim.x) {
+        const uint2 item = cr.item[k];
+        int nc;
+        unsigned q0, q1, p0, p1;
+        __syncthreads();                                     // the last run's tables have been read
+        stage_group(g, s.offsets, (int)item.x, off, &nc, &q0, &q1);
+        const bool first = item.y >> 1 == q0 / ENC_RUN;
+        cut_to_run(item.y, &q0, &q1);
+        for (int t = threadIdx.x; t < 3 * ENC_CELLS; t += blockDim.x) {
+            const int d = t / ENC_CELLS, c = t % ENC_CELLS;
+            if (c >= nc) continue;
+            const int64_t at = (int64_t)d * g.Ncc + (int)item.x * ENC_CELLS + c;
+            const float m = vel_unfix_mean(cr.vsum[at], off[c + 1] - off[c]);
+            svc[t] = m;
+            if (first) s.vc[at] = m;
+        }
+        if (!measure) continue;
         __syncthreads();
+        brick_share(q0, q1, &p0, &p1);
         float acc = 0.0f;
-        auto add = [&](const float* x, int c) {
+        int c0 = p0 < p1 ? upper_cell(off, nc, p0) : 0;
+        for (unsigned base = p0; base < p1; base += 32) {
+            const unsigned j = base + lane;
+            int cnext;
+            const int c = warp_cells(off, nc, base, c0, &cnext);
+            c0 = cnext;
+            if (j >= p1) continue;
+            const float x[3] = {v0[j], v1[j], v2[j]};
 #pragma unroll
             for (int d = 0; d < 3; ++d) {
                 const float e = x[d] - svc[d * ENC_CELLS + c];
                 acc = __fmaf_rn(e, e, acc);
             }
-        };
-        if (p1 - p0 <= 64) {                                 // the share is still in registers
-#pragma unroll
-            for (int h = 0; h < 2; ++h)
-                if (p0 + 32 * h + lane < p1) add(v[h], cell[h]);
-        } else {
-            c0 = upper_cell(off, nc, p0);
-            for (unsigned base = p0; base < p1; base += 32) {
-                const unsigned j = base + lane;
-                int cnext;
-                const int c = warp_cells(off, nc, base, c0, &cnext);
-                c0 = cnext;
-                if (j < p1) {
-                    const float x[3] = {vo[0][j], vo[1][j], vo[2][j]};
-                    add(x, c);
-                }
-            }
         }
         const double t = block_sum_double((double)acc, red);
-        if (threadIdx.x == 0) part[blockIdx.x] = (float)t;
+        if (threadIdx.x == 0) cr.part[item.y] = (float)t;
     }
-    if (bad) atomicOr(flags, ERR_NONFINITE);
 }
 
 // The codec scale from the partial sums of squared offsets, by a block of 1024
 // threads: strided FP32 sums per thread (coalesced loads, fixed order), then a
-// fixed tree in FP64
+// fixed tree in FP64.  COMP: the additions' errors are added up beside them
+// (the encode's many partial sums, of which it once had one a thread)
+template <bool COMP>
 __device__ __forceinline__ void sigma_body(const float* __restrict__ part, int nparts, double count, double ratio,
                                            double fixed, double* sigma_out) {
     __shared__ double sh[32];
-    float acc = 0.0f;
+    float acc = 0.0f, low = 0.0f;
     for (int i = threadIdx.x; i < nparts; i += 16 * blockDim.x) {
         float v[16];                                     // 16 loads in flight, added in order
 #pragma unroll
@@ -333,15 +451,23 @@ __device__ __forceinline__ void sigma_body(const float* __restrict__ part, int n
             v[k] = j < nparts ? part[j] : 0.0f;
         }
 #pragma unroll
-        for (int k = 0; k < 16; ++k) acc += v[k];        // (+ 0 past the end changes nothing: acc >= 0)
+        for (int k = 0; k < 16; ++k) {                   // (+ 0 past the end changes nothing: acc >= 0)
+            const float t = __fadd_rn(acc, v[k]);
+            if (COMP) {                                  // Knuth's two-sum
+                const float z = __fsub_rn(t, acc);
+                low += __fadd_rn(__fsub_rn(acc, __fsub_rn(t, z)), __fsub_rn(v[k], z));
+            }
+            acc = t;
+        }
     }
-    double s = block_sum_double((double)acc, sh);
+    double s = block_sum_double((double)acc + (double)low, sh);
     if (threadIdx.x == 0) {
         double x = fixed > 0.0 ? fixed : sqrt(s / count) * ratio;
         *sigma_out = snap_sigma_dev(x);
     }
 }
 
+template <bool COMP>
 __global__ void k_sigma_finalize(const float* __restrict__ part, int nparts, double count, double ratio,
                                  double fixed, double* sigma_out, Batch bt) {
     chain_wait();
@@ -351,7 +477,7 @@ __global__ void k_sigma_finalize(const float* __restrict__ part, int nparts, dou
         ratio = bt.ms[slot].ratio;
     }
     const int m = slot_member(bt, slot);
-    sigma_body(moved(part, m * bt.stride), nparts, count, ratio, fixed, moved(sigma_out, m * bt.stride));
+    sigma_body<COMP>(moved(part, m * bt.stride), nparts, count, ratio, fixed, moved(sigma_out, m * bt.stride));
 }
 
 // decode table, thresholds, scale constants and (1-byte codes,
@@ -417,74 +543,82 @@ __global__ void k_codec_tables(int lim, const double* __restrict__ tanv, const d
                       moved(est, o), moved(vtab, o), moved(vdel, o), blockIdx.x, gridDim.x);
 }
 
-// codes and ids in storage order, one CTA per 64 cells: positions and ids
-// gathered by the permutation, momenta already in order.  Bound by that
-// gather's latency, so six CTAs a SM: 40 registers, which the two staging
-// loops unrolled would raise to 48 (five CTAs: 45 us more at 256^3 particles).
-template <int NX, int NV>
+// codes and ids in storage order, one CTA per 64 cells (RUNS: per listed run of
+// a crowded group): positions and ids gathered by the permutation, momenta
+// already in order.  Bound by that gather's latency, so six CTAs a SM: 40
+// registers, which the two staging loops unrolled would raise to 48 (five CTAs:
+// 45 us more at 256^3 particles).
+template <int NX, int NV, bool RUNS>
 __global__ void __launch_bounds__(T_BRICK) k_encode_codes(Geo g, const float* __restrict__ pos,
                                                           const float* __restrict__ v0, const float* __restrict__ v1,
                                                           const float* __restrict__ v2,
                                                           const unsigned* __restrict__ id_in,
-                                                          const unsigned* __restrict__ perm, CodecDev cd, StoreDev s) {
+                                                          const unsigned* __restrict__ perm, CodecDev cd, StoreDev s,
+                                                          Crowded cr) {
     __shared__ unsigned off[ENC_CELLS + 1];
     __shared__ float svc[3 * ENC_CELLS];
     chain_wait();
-    const int L0 = blockIdx.x * ENC_CELLS, nc = min(ENC_CELLS, g.Ncc - L0);
-#pragma unroll 1
-    for (int c = threadIdx.x; c <= nc; c += blockDim.x) off[c] = s.offsets[L0 + c];
-#pragma unroll 1
-    for (int t = threadIdx.x; t < 3 * ENC_CELLS; t += blockDim.x)
-        if (t % ENC_CELLS < nc) svc[t] = s.vc[(int64_t)(t / ENC_CELLS) * g.Ncc + L0 + t % ENC_CELLS];
-    __syncthreads();
-    const unsigned q1 = min(off[nc], (unsigned)g.Np);
-    unsigned p0, p1;
-    brick_share(min(off[0], q1), q1, &p0, &p1);
-    if (p0 >= p1) return;
     constexpr int nbits = 8 * NX, half = 1 << (nbits - 1), mask = (1 << nbits) - 1;
     const float scale = ldexpf(1.0f, nbits - g.r);
-    const int key0 = NV == 1 ? __float_as_int(cd.est[2]) : 0;
     const unsigned lane = threadIdx.x & 31;
     const CodeRows<NX> chi(s.chi, g.Np);
     const CodeRows<NV> nu_r(s.nu, g.Np);
     const float* vi[3] = {v0, v1, v2};
     const float* xi[3] = {pos, pos + g.Np, pos + 2 * g.Np};
-    int c0 = upper_cell(off, nc, p0);
-    for (unsigned base = p0; base < p1; base += 64) {       // 64 particles' loads in flight
-        float x[2][3], v[2][3];
-        unsigned i[2], pid[2] = {0, 0};
+    const int nrun = RUNS ? (int)*cr.count : 0;
+    for (int k = blockIdx.x; !RUNS || k < nrun; k += gridDim.x) {
+        const uint2 item = RUNS ? cr.item[k] : make_uint2(blockIdx.x, 0u);
+        const int L0 = (int)item.x * ENC_CELLS;
+        if (RUNS) __syncthreads();                           // the last run's tables have been read
+#pragma unroll 1
+        for (int t = threadIdx.x; t < 3 * ENC_CELLS; t += blockDim.x)
+            if (L0 + t % ENC_CELLS < g.Ncc) svc[t] = s.vc[(int64_t)(t / ENC_CELLS) * g.Ncc + L0 + t % ENC_CELLS];
+        int nc;
+        unsigned q0, q1, p0, p1;
+        stage_group(g, s.offsets, (int)item.x, off, &nc, &q0, &q1);
+        if (RUNS) cut_to_run(item.y, &q0, &q1);
+        else if (q1 - q0 > ENC_BIG) return;
+        brick_share(q0, q1, &p0, &p1);
+        if (!RUNS && p0 >= p1) return;
+        const int key0 = NV == 1 ? __float_as_int(cd.est[2]) : 0;
+        int c0 = p0 < p1 ? upper_cell(off, nc, p0) : 0;
+        for (unsigned base = p0; base < p1; base += 64) {   // 64 particles' loads in flight
+            float x[2][3], v[2][3];
+            unsigned i[2], pid[2] = {0, 0};
 #pragma unroll
-        for (int h = 0; h < 2; ++h) i[h] = base + 32 * h + lane < p1 ? perm[base + 32 * h + lane] : 0xffffffffu;
+            for (int h = 0; h < 2; ++h) i[h] = base + 32 * h + lane < p1 ? perm[base + 32 * h + lane] : 0xffffffffu;
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const bool ok = i[h] < (unsigned)g.Np;
+            for (int h = 0; h < 2; ++h) {
+                const bool ok = i[h] < (unsigned)g.Np;
 #pragma unroll
-            for (int d = 0; d < 3; ++d) {
-                x[h][d] = ok ? xi[d][i[h]] : 0.0f;
-                v[h][d] = ok ? vi[d][base + 32 * h + lane] : 0.0f;
+                for (int d = 0; d < 3; ++d) {
+                    x[h][d] = ok ? xi[d][i[h]] : 0.0f;
+                    v[h][d] = ok ? vi[d][base + 32 * h + lane] : 0.0f;
+                }
+                if (s.id && ok) pid[h] = id_in ? id_in[i[h]] : i[h];
             }
-            if (s.id && ok) pid[h] = id_in ? id_in[i[h]] : i[h];
-        }
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const unsigned j = base + 32 * h + lane;
-            int cnext;
-            const int c = warp_cells(off, nc, base + 32 * h, c0, &cnext);
-            c0 = cnext;
-            if (j >= p1) continue;
-            float dd[3];
-            int nu[3];
+            for (int h = 0; h < 2; ++h) {
+                const unsigned j = base + 32 * h + lane;
+                int cnext;
+                const int c = warp_cells(off, nc, base + 32 * h, c0, &cnext);
+                c0 = cnext;
+                if (j >= p1) continue;
+                float dd[3];
+                int nu[3];
 #pragma unroll
-            for (int d = 0; d < 3; ++d) {
-                chi.put(d, j, (pos_bin(x[h][d], scale, g.Nc << nbits) & mask) - half);
-                dd[d] = v[h][d] - svc[d * ENC_CELLS + c];
-                if (NV == 1) nu[d] = nu_from_table(dd[d], cd.thr, cd.vtab, key0, g.nulim);
+                for (int d = 0; d < 3; ++d) {
+                    chi.put(d, j, (pos_bin(x[h][d], scale, g.Nc << nbits) & mask) - half);
+                    dd[d] = v[h][d] - svc[d * ENC_CELLS + c];
+                    if (NV == 1) nu[d] = nu_from_table(dd[d], cd.thr, cd.vtab, key0, g.nulim);
+                }
+                if (NV == 2) nu_codes3(dd, cd.thr, g.nulim, cd.est[0], cd.est[1], nu);
+#pragma unroll
+                for (int d = 0; d < 3; ++d) nu_r.put(d, j, nu[d]);
+                if (s.id) store_pid(s.id, j, g.nid, pid[h]);
             }
-            if (NV == 2) nu_codes3(dd, cd.thr, g.nulim, cd.est[0], cd.est[1], nu);
-#pragma unroll
-            for (int d = 0; d < 3; ++d) nu_r.put(d, j, nu[d]);
-            if (s.id) store_pid(s.id, j, g.nid, pid[h]);
         }
+        if (!RUNS) break;
     }
 }
 
@@ -1283,7 +1417,7 @@ __global__ void __launch_bounds__(1024) k_step_sums(Geo g, StepScratch w, double
                                                     unsigned* __restrict__ tsum) {
     chain_wait();
     if (blockIdx.x == 0) {
-        sigma_body(w.part, g.nbricks, 3.0 * (double)g.Np, ratio, 0.0, sigma_out);
+        sigma_body<false>(w.part, g.nbricks, 3.0 * (double)g.Np, ratio, 0.0, sigma_out);
         return;
     }
     __shared__ unsigned sw[32];
@@ -1917,6 +2051,14 @@ static inline unsigned brick_threads(const Geo& g) { return std::max(32, std::mi
 
 static inline int nblk(int64_t n, int t) { return (int)((n + t - 1) / t); }
 
+// scratch of the crowded groups; none where no group can be crowded
+Crowded encode_crowded(const Geo& g, unsigned* count, unsigned* items, long long* vsum, float* part) {
+    return Crowded{count, reinterpret_cast<uint2*>(items), vsum, part + encode_groups(g),
+                   g.Np > ENC_BIG ? (int)std::min<int64_t>(crowded_slots(g), 4 * g.nsm) : 0};
+}
+
+int64_t encode_partials(const Geo& g) { return encode_groups(g) + crowded_slots(g); }
+
 void launch_encode_keys(const Geo& g, const float* pos, unsigned* key, unsigned* counts, unsigned* flags,
                         cudaStream_t st) {
     const dim3 grid(nblk(g.Np, 256));
@@ -1926,15 +2068,22 @@ void launch_encode_keys(const Geo& g, const float* pos, unsigned* key, unsigned*
 
 int encode_groups(const Geo& g) { return nblk(g.Ncc, ENC_CELLS); }
 
-void launch_encode_vc(const Geo& g, const float* vel, const unsigned* perm, const StoreDev& s, float* const* vsorted,
-                      float* part, unsigned* flags, cudaStream_t st) {
-    launch_chained(k_encode_vc, dim3(encode_groups(g)), T_BRICK, 0, st, g, vel, perm, s, vsorted[0], vsorted[1], vsorted[2],
-                   part, flags);
+int launch_encode_vc(const Geo& g, const float* vel, const unsigned* perm, const StoreDev& s, float* const* vsorted,
+                     float* part, const Crowded& cr, unsigned* flags, cudaStream_t st) {
+    launch_chained(k_encode_vc<false>, dim3(encode_groups(g)), T_BRICK, 0, st, g, vel, perm, s, vsorted[0], vsorted[1],
+                   vsorted[2], part, cr, flags);
+    if (cr.ctas == 0) return 1;
+    launch_chained(k_encode_vc<true>, dim3(cr.ctas), T_BRICK, 0, st, g, vel, perm, s, vsorted[0], vsorted[1], vsorted[2],
+                   part, cr, flags);
+    launch_chained(k_encode_crowded, dim3(cr.ctas), T_BRICK, 0, st, g, s, vsorted[0], vsorted[1], vsorted[2],
+                   part != nullptr, cr);
+    return 3;
 }
 
 void launch_sigma_finalize(const float* part, int nparts, double count, double ratio, double fixed,
-                           double* sigma_out, cudaStream_t st, const Batch& bt) {
-    launch_chained(k_sigma_finalize, dim3(bt.members), 1024, 0, st, part, nparts, count, ratio, fixed, sigma_out, bt);
+                           double* sigma_out, bool comp, cudaStream_t st, const Batch& bt) {
+    launch_chained(comp ? k_sigma_finalize<true> : k_sigma_finalize<false>, dim3(bt.members), 1024, 0, st, part, nparts,
+                   count, ratio, fixed, sigma_out, bt);
 }
 
 void launch_codec_tables(int nulim, const double* tanv, const double* tanh_, const CodecDev& c, cudaStream_t st,
@@ -1946,16 +2095,24 @@ void launch_codec_tables(int nulim, const double* tanv, const double* tanh_, con
                                                                           one ? nullptr : c.vdel, bt);
 }
 
-void launch_encode_codes(const Geo& g, const float* pos, const float* const* vsorted, const unsigned* id_in,
-                         const unsigned* perm, const CodecDev& c, const StoreDev& s, cudaStream_t st) {
-    const dim3 grid(encode_groups(g));
-    auto go = [&](auto kernel) {
-        launch_chained(kernel, grid, T_BRICK, 0, st, g, pos, vsorted[0], vsorted[1], vsorted[2], id_in, perm, c, s);
-    };
-    if (g.nchi == 1 && g.nnu == 1) go(k_encode_codes<1, 1>);
-    else if (g.nchi == 1) go(k_encode_codes<1, 2>);
-    else if (g.nnu == 1) go(k_encode_codes<2, 1>);
-    else go(k_encode_codes<2, 2>);
+template <int NX, int NV>
+static int encode_codes(const Geo& g, const float* pos, const float* const* vsorted, const unsigned* id_in,
+                        const unsigned* perm, const CodecDev& c, const StoreDev& s, const Crowded& cr, cudaStream_t st) {
+    launch_chained(k_encode_codes<NX, NV, false>, dim3(encode_groups(g)), T_BRICK, 0, st, g, pos, vsorted[0], vsorted[1],
+                   vsorted[2], id_in, perm, c, s, cr);
+    if (cr.ctas == 0) return 1;
+    launch_chained(k_encode_codes<NX, NV, true>, dim3(cr.ctas), T_BRICK, 0, st, g, pos, vsorted[0], vsorted[1],
+                   vsorted[2], id_in, perm, c, s, cr);
+    return 2;
+}
+
+int launch_encode_codes(const Geo& g, const float* pos, const float* const* vsorted, const unsigned* id_in,
+                        const unsigned* perm, const CodecDev& c, const StoreDev& s, const Crowded& cr,
+                        cudaStream_t st) {
+    if (g.nchi == 1 && g.nnu == 1) return encode_codes<1, 1>(g, pos, vsorted, id_in, perm, c, s, cr, st);
+    if (g.nchi == 1) return encode_codes<1, 2>(g, pos, vsorted, id_in, perm, c, s, cr, st);
+    if (g.nnu == 1) return encode_codes<2, 1>(g, pos, vsorted, id_in, perm, c, s, cr, st);
+    return encode_codes<2, 2>(g, pos, vsorted, id_in, perm, c, s, cr, st);
 }
 
 void launch_max_speed(const Geo& g, const StoreDev& s, const CodecDev& c, unsigned* vmax_bits, cudaStream_t st,

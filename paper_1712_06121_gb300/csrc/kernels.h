@@ -178,21 +178,38 @@ __host__ __device__ __forceinline__ StepScratch moved(const StepScratch& w, size
 // a batch of one: a single context's launch
 constexpr Batch kSingle{1, 0, nullptr, nullptr};
 
+// Groups of cells that the encode splits over several CTAs (k_store.cu): the
+// list of their runs, {group, slot}, and its length (cleared by the caller); their cells' momentum sums
+// [3][Ncc]; the runs' sums of squared offsets, by slot.  ctas: CTAs for
+// the list (0: no group can be crowded, and nothing else is used)
+struct Crowded {
+    unsigned* count;
+    uint2* item;
+    long long* vsum;
+    float* part;
+    int ctas;
+};
+// items: two words a slot, 4 (Np / 8192 + 1) in all; part: encode_partials(g) words
+Crowded encode_crowded(const Geo& g, unsigned* count, unsigned* items, long long* vsum, float* part);
+int64_t encode_partials(const Geo& g);
 // sort keys (cell ranks) and cell counts of float positions
 void launch_encode_keys(const Geo& g, const float* pos, unsigned* key, unsigned* counts, unsigned* flags,
                         cudaStream_t st);
 // the particles' momenta in storage order (three rows of Np), v_c of every
 // cell, and (part not null) the sums of squared offsets from v_c of
-// encode_groups runs of cells
+// encode_groups runs of cells; the kernels launched
 int encode_groups(const Geo& g);
-void launch_encode_vc(const Geo& g, const float* vel, const unsigned* perm, const StoreDev& s, float* const* vsorted,
-                      float* part, unsigned* flags, cudaStream_t st);
+int launch_encode_vc(const Geo& g, const float* vel, const unsigned* perm, const StoreDev& s, float* const* vsorted,
+                     float* part, const Crowded& cr, unsigned* flags, cudaStream_t st);
+// (comp: many partial sums, added with their errors)
 void launch_sigma_finalize(const float* part, int nparts, double count, double ratio, double fixed,
-                           double* sigma_out, cudaStream_t st, const Batch& bt = Batch{1, 0, nullptr, nullptr});
+                           double* sigma_out, bool comp, cudaStream_t st,
+                           const Batch& bt = Batch{1, 0, nullptr, nullptr});
 void launch_codec_tables(int nulim, const double* tanv, const double* tanh, const CodecDev& c, cudaStream_t st,
                          const Batch& bt = Batch{1, 0, nullptr, nullptr});
-void launch_encode_codes(const Geo& g, const float* pos, const float* const* vsorted, const unsigned* id_in,
-                         const unsigned* perm, const CodecDev& c, const StoreDev& s, cudaStream_t st);
+int launch_encode_codes(const Geo& g, const float* pos, const float* const* vsorted, const unsigned* id_in,
+                         const unsigned* perm, const CodecDev& c, const StoreDev& s, const Crowded& cr,
+                         cudaStream_t st);
 void launch_decode(const Geo& g, const StoreDev& s, const CodecDev& c, float* pos, float* vel, unsigned* id,
                    cudaStream_t st);
 // (step: the step's scratch that pass A accumulates into, cleared by the way, or null)
