@@ -702,12 +702,15 @@ __global__ void __launch_bounds__(T_BRICK) k_decode(Geo g, StoreDev s, CodecDev 
 // so a cell's largest |p| along an axis is at its smallest or largest code:
 // LPC lanes a cell take both over the cell's particles and two codes are
 // decoded, not every particle's.  Cells of more than 8 LPC particles (haloes)
-// are finished by their whole warp, so that no lane runs alone.  A warp's
+// are finished by their whole warp, so that no lane runs alone, and cells of
+// more than SPEED_BIG by the whole CTA (128^3 particles, a fifth of them in one
+// cell: 1566 us by a warp, 798 by a CTA a brick and a decode per particle -> 158).  A warp's
 // life is a chain of loads (offsets, codes, table): LPC = 8 gives small stores
 // their warps (one wave holds 64 of them per SM), LPC = 2 keeps large ones to
 // few waves.  The call with its read-backs (25 us of
 // them host and copies), 192^3 particles x1v1, clustered: 73 us with a CTA a
 // brick, a search and a decode per particle -> 55 us; 32^3: 29.7 -> 26.4 us.
+constexpr unsigned SPEED_BIG = 2048;
 template <int NV, int LPC>
 __global__ void __launch_bounds__(T_BRICK) k_max_speed(Geo g, StoreDev s, CodecDev cd,
                                                        unsigned* __restrict__ vmax_bits, Batch bt) {
@@ -743,7 +746,8 @@ __global__ void __launch_bounds__(T_BRICK) k_max_speed(Geo g, StoreDev s, CodecD
                 hi[d] = max(hi[d], v);
             }
     }
-    for (unsigned more = __ballot_sync(0xffffffffu, sub == 0 && e < i1); more; more &= more - 1) {
+    const bool big = i1 - i0 > SPEED_BIG;
+    for (unsigned more = __ballot_sync(0xffffffffu, sub == 0 && e < i1 && !big); more; more &= more - 1) {
         const int src = __ffs(more) - 1;
         const unsigned a = __shfl_sync(0xffffffffu, e, src), z = __shfl_sync(0xffffffffu, i1, src);
         int wl[3] = {kNone, kNone, kNone}, wh[3] = {-kNone, -kNone, -kNone};
@@ -778,6 +782,33 @@ __global__ void __launch_bounds__(T_BRICK) k_max_speed(Geo g, StoreDev s, CodecD
             const int v = max(-g.nulim, min(g.nulim, sub ? hi[d] : lo[d]));
             m = fmaxf(m, fabsf(vc[d] + cd.dec[v + g.nulim]));
         }
+    if (__syncthreads_or(big)) {                             // the rest of the CTA's big cells, one after the other
+        __shared__ int list[T_BRICK / LPC], nbig;
+        if (threadIdx.x == 0) nbig = 0;
+        __syncthreads();
+        if (big && sub == 0) list[atomicAdd(&nbig, 1)] = L;
+        __syncthreads();
+        for (int k = 0; k < nbig; ++k) {
+            const int C = list[k];
+            const unsigned z = min(s.offsets[C + 1], (unsigned)g.Np);
+            int wl[3] = {kNone, kNone, kNone}, wh[3] = {-kNone, -kNone, -kNone};
+#pragma unroll 4
+            for (unsigned i = s.offsets[C] + 8u * LPC + threadIdx.x; i < z; i += T_BRICK)
+#pragma unroll
+                for (int d = 0; d < 3; ++d) {
+                    const int v = nu.get(d, i);
+                    wl[d] = min(wl[d], v);
+                    wh[d] = max(wh[d], v);
+                }
+            // each warp's own extremes (it has some: SPEED_BIG is larger than a round)
+#pragma unroll
+            for (int d = 0; d < 3; ++d) {
+                const int l = __reduce_min_sync(0xffffffffu, wl[d]), h = __reduce_max_sync(0xffffffffu, wh[d]);
+                const int v = max(-g.nulim, min(g.nulim, lane & 1 ? h : l));
+                if (lane < 2) m = fmaxf(m, fabsf(s.vc[(int64_t)d * g.Ncc + C] + cd.dec[v + g.nulim]));
+            }
+        }
+    }
     block_max_to(__float_as_uint(m), vmax_bits);
 }
 

@@ -98,3 +98,46 @@ def test_encode_does_not_wait_for_a_crowd(cube):
         assert t[1] < 6 * t[0], t
     finally:
         cube.cube_destroy(ctx)
+
+
+# cells on either side of the 2048 particles that a warp finishes alone, several
+# of them in one CTA's share, the largest momentum anywhere in a crowd; every
+# code width, alone and in a batch.  The decoded values' own maximum, exactly.
+@pytest.mark.parametrize("vb", [1, 2])
+@pytest.mark.parametrize("crowds", [[(2048, 5.0, 0.9)], [(2049, 5.0, 0.9)],
+                                    [(30000, 4.1, 3.8), (2500, 8.1, 3.8), (2040, 20.1, 3.8), (9000, 40.1, 7.8)]])
+def test_largest_momentum_of_crowded_cells(cube, vb, crowds):
+    n, nf = 60000, 48
+    prm = cube.make_params(nf, n, v_bytes=vb, box=50.0)
+    batch = cube.cube_batch_create([prm] * 2, torch.cuda.current_stream())
+    ctx = cube.cube_create(prm, torch.cuda.current_stream())
+    try:
+        pos, vel, ids = _crowd(n, nf, 1712216, crowds)
+        crowd = np.flatnonzero((np.abs(pos - 5.5) < 2.0).all(axis=0))
+        members = [ctx, cube.cube_batch_member(batch, 0), cube.cube_batch_member(batch, 1)]
+        for k, c in enumerate(members):
+            v = vel.copy()
+            v[k, crowd[(k + 1) * len(crowd) // 4]] = (3.0, -2.5, 2.75)[k]
+            cube.cube_encode(c, pos, v, ids, 0.02, 0.5)
+            out = [np.empty((3, n), np.float32) for _ in range(2)]
+            cube.cube_decode(c, *out)
+            assert cube.cube_max_speed(c) == np.abs(out[1]).max()
+    finally:
+        cube.cube_destroy(ctx)
+        cube.cube_batch_destroy(batch)
+
+
+# a fifth of 128^3 particles in one cell, against particles anywhere: 16 times
+# with a CTA a brick, 47 times with a warp for the crowd
+def test_largest_momentum_does_not_wait_for_a_warp(cube):
+    n, nf = 128 ** 3, 256
+    prm = cube.make_params(nf, n, box=50.0)
+    ctx = cube.cube_create(prm, torch.cuda.current_stream())
+    try:
+        t = []
+        for crowds in ([], [(n // 5, 41.0, 0.9)]):
+            cube.cube_encode(ctx, *_crowd(n, nf, 1712215, crowds), 0.02, 0.0)
+            t.append(_us(lambda: cube.cube_max_speed(ctx)))
+        assert t[1] < 24 * t[0], t
+    finally:
+        cube.cube_destroy(ctx)
