@@ -68,27 +68,6 @@ __device__ __forceinline__ void brick_share(unsigned q0, unsigned q1, unsigned* 
     *p1 = min(q1, *p0 + share);
 }
 
-// brick offsets, v_c of the brick and (1-byte codes) the decode table in
-// shared memory, [nbc + 1], [3][nbc], [2 lim + 1], by asynchronous copies:
-// complete after cp_async_wait_all() and a barrier
-struct BrickTables {
-    unsigned* off;
-    float* vc;
-    float* dec;
-};
-template <int NV>
-__device__ __forceinline__ BrickTables stage_brick(const Geo& g, const StoreDev& s, const CodecDev& c, int L0,
-                                                   unsigned* smem) {
-    const int nbc = g.B * g.B * g.B;
-    BrickTables t{smem, reinterpret_cast<float*>(smem + nbc + 1), reinterpret_cast<float*>(smem + 4 * nbc + 1)};
-    for (int i = threadIdx.x; i <= nbc; i += blockDim.x) cp_async4(&t.off[i], &s.offsets[L0 + i]);
-    for (int i = threadIdx.x; i < 3 * nbc; i += blockDim.x)
-        cp_async4(&t.vc[i], &s.vc[(int64_t)(i >> (3 * g.lB)) * g.Ncc + L0 + (i & (nbc - 1))]);
-    if (NV == 1)
-        for (int i = threadIdx.x; i < 2 * g.nulim + 1; i += blockDim.x) cp_async4(&t.dec[i], &c.dec[i]);
-    return t;
-}
-
 // the decode table of 2-byte codes through its corrections
 template <int NV>
 __device__ __forceinline__ VelTables vel_tables(const CodecDev& c, int lim) {
@@ -631,15 +610,32 @@ __global__ void __launch_bounds__(T_BRICK) k_encode_codes(Geo g, const float* __
 // loads, so a warp's first 64 particles are requested beside the brick's
 // tables and the rest 64 at a time.  256^3 particles x1v1: 0.342 ms with FP64
 // positions, a search per particle and tables in global memory -> 0.164 ms.
-template <int NX, int NV>
+// A CTA takes 64 consecutive cells whatever the brick: one of side 4, eight of
+// side 2 or 64 of side 1, whose cells' coordinates are staged (!B4).  128^3
+// particles in bricks of one cell: 682 us with 256 threads a brick, 157 with 32 -> 45; with a
+// fifth of them in one cell 2962, 6212 -> 803.  (The staging loops are not unrolled:
+// 172 us instead of 163 at 256^3.)
+constexpr int DEC_CELLS = 64;
+template <int NX, int NV, bool B4>
 __global__ void __launch_bounds__(T_BRICK) k_decode(Geo g, StoreDev s, CodecDev cd, float* __restrict__ pos,
                                                     float* __restrict__ vel, unsigned* __restrict__ id) {
-    extern __shared__ unsigned brick_sm[];
+    __shared__ unsigned off[DEC_CELLS + 1];
+    __shared__ float svc[3 * DEC_CELLS];
+    __shared__ float dec[NV == 1 ? 255 : 1];
+    __shared__ unsigned where[B4 ? 1 : DEC_CELLS];            // x + 2^10 (y + 2^10 z) of the cells
     chain_wait();
-    const int nbc = g.B * g.B * g.B, lim = g.nulim;
-    const int L0 = blockIdx.x * nbc;
-    const BrickTables bt = stage_brick<NV>(g, s, cd, L0, brick_sm);
-    const unsigned q1 = min(s.offsets[L0 + nbc], (unsigned)g.Np), q0 = min(s.offsets[L0], q1);
+    const int lim = g.nulim;
+    const int L0 = blockIdx.x * DEC_CELLS, nc = B4 ? DEC_CELLS : min(DEC_CELLS, g.Ncc - L0);
+#pragma unroll 1
+    for (int i = threadIdx.x; i <= nc; i += blockDim.x) cp_async4(&off[i], &s.offsets[L0 + i]);
+#pragma unroll 1
+    for (int i = threadIdx.x; i < 3 * DEC_CELLS; i += blockDim.x)
+        if (B4 || i % DEC_CELLS < nc)
+            cp_async4(&svc[i], &s.vc[(int64_t)(i / DEC_CELLS) * g.Ncc + L0 + i % DEC_CELLS]);
+    if (NV == 1)
+#pragma unroll 1
+        for (int i = threadIdx.x; i < 2 * lim + 1; i += blockDim.x) cp_async4(&dec[i], &cd.dec[i]);
+    const unsigned q1 = min(s.offsets[L0 + nc], (unsigned)g.Np), q0 = min(s.offsets[L0], q1);
     unsigned p0, p1;
     brick_share(q0, q1, &p0, &p1);
     const unsigned lane = threadIdx.x & 31;
@@ -661,31 +657,38 @@ __global__ void __launch_bounds__(T_BRICK) k_decode(Geo g, StoreDev s, CodecDev 
         }
     };
     load(p0);
+    int b[3];
+    if (!B4 && (int)threadIdx.x < nc) {
+        const int L = L0 + (int)threadIdx.x, lc = L & ((1 << (3 * g.lB)) - 1), bm = g.B - 1;
+        brick_coords(g, L >> (3 * g.lB), &b[0], &b[1], &b[2]);
+        where[threadIdx.x] = (unsigned)((b[0] << g.lB) + (lc & bm)) |
+                             (unsigned)((b[1] << g.lB) + ((lc >> g.lB) & bm)) << 10 |
+                             (unsigned)((b[2] << g.lB) + (lc >> (2 * g.lB))) << 20;
+    }
     cp_async_wait_all();
     __syncthreads();
     if (p0 >= p1) return;
     const VelTables vt = vel_tables<NV>(cd, lim);
-    int b[3];
-    brick_coords(g, blockIdx.x, &b[0], &b[1], &b[2]);
+    if (B4) brick_coords(g, blockIdx.x, &b[0], &b[1], &b[2]);
     constexpr int nbits = 8 * NX, half = 1 << (nbits - 1);
     const float pscale = ldexpf(1.0f, g.r - nbits - 1);
-    int c0 = upper_cell(bt.off, nbc, p0);
+    int c0 = upper_cell(off, nc, p0);
     for (unsigned base = p0;;) {
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             const unsigned i = base + 32 * h + lane;
             int cnext;
-            const int lc = warp_cells(bt.off, nbc, base + 32 * h, c0, &cnext);
+            const int lc = warp_cells(off, nc, base + 32 * h, c0, &cnext);
             c0 = cnext;
             if (i < p1) {
 #pragma unroll
                 for (int d = 0; d < 3; ++d) {
-                    const int c = (b[d] << g.lB) + ((lc >> (d * g.lB)) & (g.B - 1));
+                    const int c = B4 ? 4 * b[d] + ((lc >> (2 * d)) & 3) : (int)((where[lc] >> (10 * d)) & 1023u);
                     const unsigned q = ((unsigned)c << (nbits + 1)) + (unsigned)(2 * (x[h][d] + half) + 1);
                     const float f = NX == 1 ? __uint_as_float(0x4B000000u | q) - 8388608.0f : u32_to_float_rn(q);
                     pos[d * g.Np + i] = f * pscale;
                     const int k = max(-lim, min(lim, v[h][d]));
-                    vel[d * g.Np + i] = bt.vc[(d << (3 * g.lB)) + lc] + (NV == 1 ? bt.dec[k + lim] : vt.dec(k));
+                    vel[d * g.Np + i] = svc[d * DEC_CELLS + lc] + (NV == 1 ? dec[k + lim] : vt.dec(k));
                 }
                 if (id) id[i] = pid[h];
             }
@@ -2076,10 +2079,6 @@ void launch_batch_clear(const Geo& g, long long* vsum, int* maxmig, cudaStream_t
                    vsum, maxmig, bt);
 }
 
-// threads of a decode CTA: four a cell, a warp at least (128^3 particles in
-// bricks of one cell: 673 us with 256 -> 151; of eight 127 -> 41)
-static inline unsigned brick_threads(const Geo& g) { return std::max(32, std::min(T_BRICK, 4 * g.B * g.B * g.B)); }
-
 static inline int nblk(int64_t n, int t) { return (int)((n + t - 1) / t); }
 
 // scratch of the crowded groups; none where no group can be crowded
@@ -2159,18 +2158,20 @@ void launch_max_speed(const Geo& g, const StoreDev& s, const CodecDev& c, unsign
     else launch_chained(k_max_speed<2, 2>, grid, T_BRICK, 0, st, g, s, c, vmax_bits, bt);
 }
 
-// a brick's offsets, v_c and (1-byte codes) decode table
-static size_t brick_smem(const Geo& g) {
-    return (size_t)(4 * g.B * g.B * g.B + 1 + (g.nnu == 1 ? 2 * g.nulim + 1 : 0)) * 4;
+template <int NX, int NV>
+static void decode(const Geo& g, const StoreDev& s, const CodecDev& c, float* pos, float* vel, unsigned* id,
+                   cudaStream_t st) {
+    const dim3 grid(nblk(g.Ncc, DEC_CELLS));
+    if (g.B == 4) launch_chained(k_decode<NX, NV, true>, grid, T_BRICK, 0, st, g, s, c, pos, vel, id);
+    else launch_chained(k_decode<NX, NV, false>, grid, T_BRICK, 0, st, g, s, c, pos, vel, id);
 }
 
 void launch_decode(const Geo& g, const StoreDev& s, const CodecDev& c, float* pos, float* vel, unsigned* id,
                    cudaStream_t st) {
-    const size_t sm = brick_smem(g);
-    if (g.nchi == 1 && g.nnu == 1) launch_chained(k_decode<1, 1>, dim3(g.nbricks), brick_threads(g), sm, st, g, s, c, pos, vel, id);
-    else if (g.nchi == 1) launch_chained(k_decode<1, 2>, dim3(g.nbricks), brick_threads(g), sm, st, g, s, c, pos, vel, id);
-    else if (g.nnu == 1) launch_chained(k_decode<2, 1>, dim3(g.nbricks), brick_threads(g), sm, st, g, s, c, pos, vel, id);
-    else launch_chained(k_decode<2, 2>, dim3(g.nbricks), brick_threads(g), sm, st, g, s, c, pos, vel, id);
+    if (g.nchi == 1 && g.nnu == 1) decode<1, 1>(g, s, c, pos, vel, id, st);
+    else if (g.nchi == 1) decode<1, 2>(g, s, c, pos, vel, id, st);
+    else if (g.nnu == 1) decode<2, 1>(g, s, c, pos, vel, id, st);
+    else decode<2, 2>(g, s, c, pos, vel, id, st);
 }
 
 static size_t deposit_smem(const Geo& g) {

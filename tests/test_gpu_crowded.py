@@ -141,3 +141,44 @@ def test_largest_momentum_does_not_wait_for_a_warp(cube):
         assert t[1] < 24 * t[0], t
     finally:
         cube.cube_destroy(ctx)
+
+
+# decode of bricks of one, 8 and 64 cells, 64 cells a CTA: a last CTA of 24
+# cells, crowds within and across its shares, every code width
+@pytest.mark.parametrize("nf,ratio,brick,xb,vb", [(24, 4, 1, 1, 1), (24, 4, 1, 2, 2), (48, 4, 2, 1, 2), (64, 2, 2, 2, 1),
+                                                  (48, 4, 4, 2, 2), (32, 8, 1, 1, 1)])
+def test_decode_of_any_brick_matches_oracle(cube, nf, ratio, brick, xb, vb):
+    n = 30011
+    pos, vel, ids = _crowd(n, nf, 1712217, [(12000, 5.0, 0.9), (5000, 8.0, 9.0)])
+    prm = cube.make_params(nf, n, ratio=ratio, brick=brick, x_bytes=xb, v_bytes=vb, box=50.0, omega_m=0.3, omega_l=0.7)
+    ctx = cube.cube_create(prm, torch.cuda.current_stream())
+    try:
+        cube.cube_encode(ctx, pos, vel, ids, 0.02, 0.5)
+        g = read_store(cube, ctx)
+        ref = pm.encode(oracle_params(pm, prm, brick), pos, vel, ids, 0.02, g["sigma"], snap=False)
+        out = [np.empty((3, n), np.float32) for _ in range(2)] + [np.empty(n, np.uint32)]
+        cube.cube_decode(ctx, *out)
+        rp, rv = pm.decode(ref)[:2]
+        assert np.array_equal(out[0], rp.astype(np.float32))
+        assert np.array_equal(out[2], ref.ids)
+        # v_c and the FP32 table entry are each rounded once, and their sum
+        assert np.all(np.abs(out[1] - rv) <= 2.0 ** -23 * (np.abs(ref.vc).max() + np.abs(rv)))
+    finally:
+        cube.cube_destroy(ctx)
+
+
+# a fifth of 128^3 particles in one cell: bricks of one cell take as long as
+# bricks of 64 (one warp for the crowd took 7 times as long)
+def test_decode_of_a_crowd_does_not_depend_on_the_brick(cube):
+    n, nf = 128 ** 3, 256
+    t = []
+    for brick in (4, 2, 1):
+        prm = cube.make_params(nf, n, brick=brick, box=50.0)
+        ctx = cube.cube_create(prm, torch.cuda.current_stream())
+        try:
+            cube.cube_encode(ctx, *_crowd(n, nf, 1712215, [(n // 5, 41.0, 0.9)]), 0.02, 0.0)
+            p, v = torch.empty((3, n), device="cuda"), torch.empty((3, n), device="cuda")
+            t.append(_us(lambda: cube.cube_decode(ctx, p, v, None)))
+        finally:
+            cube.cube_destroy(ctx)
+    assert max(t) < 2.5 * t[0], t
