@@ -532,8 +532,8 @@ cube_status cube_batch_member(cube_batch* batch, int32_t i, cube_ctx** out);
    out.  Members stepped together must have taken the same number of steps
    since they were encoded (a member that sat a step out continues alone with
    cube_pm_step).  Host arrays [members].  Enqueues 16 kernel launches for
-   the whole batch (a context stepped alone launches the same kernels once
-   per step), 6 of them the mesh half, which is skipped for members whose
+   the whole batch (a context stepped alone launches 10 per step, two of which
+   do the work of the batch's eight between the passes), 6 of them the mesh half, which is skipped for members whose
    potential cube_batch_solve already enqueued.  For meshes up to 256^3 each
    half is captured as a CUDA graph on the second step with the same store
    parity and number of moving members, and replayed on later ones.  Errors: CUBE_E_ARG,

@@ -43,15 +43,6 @@ __device__ __forceinline__ void mbar_expect_tx(unsigned long long* bar, unsigned
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(bar)), "r"(bytes)
                  : "memory");
 }
-__device__ __forceinline__ bool mbar_test(unsigned long long* bar, unsigned parity) {
-    unsigned done;
-    asm volatile(
-        "{\n .reg .pred p;\n mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
-        : "=r"(done)
-        : "r"(smem_addr(bar)), "r"(parity)
-        : "memory");
-    return done != 0;
-}
 // one potentially blocking test: the thread is suspended until the phase
 // completes or about `hint_ns` nanoseconds pass (the hardware may wake it
 // earlier); true if the phase completed
@@ -72,17 +63,6 @@ __device__ __forceinline__ bool mbar_wait_bounded(unsigned long long* bar, unsig
         if (mbar_try_wait(bar, parity, 100000u)) return true;
     return false;
 }
-// 3-D tiled TMA load of the tensor map's box at (x, y, z) into shared memory,
-// completing on `bar`
-__device__ __forceinline__ void tma_load_3d(void* dst, const void* tmap, int x, int y, int z,
-                                            unsigned long long* bar) {
-    asm volatile(
-        "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], "
-        "[%5];" ::"r"(smem_addr(dst)),
-        "l"(tmap), "r"(x), "r"(y), "r"(z), "r"(smem_addr(bar))
-        : "memory");
-}
-
 // 4-D tiled TMA load (x, y, z, member) of the tensor map's box, completing on `bar`
 __device__ __forceinline__ void tma_load_4d(void* dst, const void* tmap, int x, int y, int z, int w,
                                             unsigned long long* bar) {
@@ -132,11 +112,6 @@ __host__ __device__ __forceinline__ int cell_rank(const Geo& g, int cx, int cy, 
     const int m = g.B - 1;
     const int bx = cx >> g.lB, by = cy >> g.lB, bz = cz >> g.lB;
     return ((bx + g.nb * (by + g.nb * bz)) << (3 * g.lB)) + (cx & m) + ((cy & m) << g.lB) + ((cz & m) << (2 * g.lB));
-}
-
-__host__ __device__ __forceinline__ int wrapi(int v, int n) {
-    v %= n;
-    return v < 0 ? v + n : v;
 }
 
 // periodic wrap of a coordinate known to lie in [-n, 2n)
@@ -252,8 +227,10 @@ struct VelApprox {
 // tan(k pi / M) gamma for 0 <= 2 k < M in FP32 to a few ulps: the angle, or
 // above pi/4 its complement (M - 2k) pi / (2M) (tan = 1 / tan of the
 // complement), lies in [0, pi/4], where the polynomial of Abramowitz & Stegun
-// 4.3.101 is within 2e-8.  Explicitly rounded operations only, so every kernel
-// gets the same bits.
+// 4.3.101 is within 2e-8.  Every kernel gets the same bits: the products and sums
+// are explicitly rounded, so none is contracted with another, and the quotient is
+// one approximate division, whose rounding is not specified but is the same
+// instruction everywhere (its result is only taken as bits).
 __device__ __forceinline__ float tan_steps(int k, const VelApprox& va) {
     const bool cot = 4 * k > va.M;
     const int mm = cot ? va.M - 2 * k : 2 * k;                 // < 2^16
@@ -455,30 +432,17 @@ __device__ __forceinline__ int load_nu(const void* base, int64_t idx, int lim) {
     return max(-lim, min(lim, load_code<NB>(base, idx)));
 }
 
-template <int NB>
-__device__ __forceinline__ void store_code(void* base, int64_t idx, int v) {
-    if (NB == 1) reinterpret_cast<int8_t*>(base)[idx] = (int8_t)v;
-    else reinterpret_cast<int16_t*>(base)[idx] = (int16_t)v;
-}
-
 // Asynchronous global -> shared copies (cp.async): all copies of a tile are
 // issued before any is waited for, so the tile's load latency is paid once.
 __device__ __forceinline__ void cp_async4(void* smem, const void* gmem) {
     const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4;\n" ::"r"(s), "l"(gmem) : "memory");
 }
-__device__ __forceinline__ void cp_async8(void* smem, const void* gmem) {
-    const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(s), "l"(gmem) : "memory");
-}
 __device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
     const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(s), "l"(gmem) : "memory");
 }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-// wait until at most one committed group (the most recent) is still in flight
-__device__ __forceinline__ void cp_async_wait_prev() { asm volatile("cp.async.wait_group 1;\n" ::: "memory"); }
 
 // 64-bit add into shared memory from 32-bit atomics: the low word's
 // wrap-arounds are carried into the high word, so the final value is the

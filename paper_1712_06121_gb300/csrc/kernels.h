@@ -20,8 +20,8 @@ namespace cube {
 // chain_wait() before it touches anything that an earlier kernel of the stream
 // reads or writes (tables uploaded once at creation may be read before), and
 // before it returns, so completion stays transitive along the chain.  Steps of
-// 32^3, 64^3 (x1v2), 128^3 and 256^3 particles: runs 766 -> 652, 640 -> 533, 1787
-// -> 1672 and 6683 -> 6605 us.  (An early griddepcontrol.launch_dependents
+// 32^3, 64^3 (x1v2), 128^3 and 256^3 particles: runs 766 -> 636, 640 -> 519, 1787
+// -> 1656 and 6683 -> 6599 us.  (An early griddepcontrol.launch_dependents
 // lets the successor's waiting CTAs take the slots of the running kernel: 7535
 // us at 256^3.)
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
