@@ -246,10 +246,10 @@ __device__ void list_runs(const Geo& g, const Crowded& cr, int G, int nc, unsign
 // the same kernel with RUNS then adds up their runs, CTA by CTA of the list, and
 // k_encode_crowded finishes them.  (In one launch, the list's idle CTAs leave
 // the groups unevenly over the SMs: 78 to 92 us against 66 for 512 groups of 4096
-// particles.)  256^3 particles x1v1: this 182 us and k_encode_codes 203, where
-// 64-bit global atomics per particle, the measurement and the final gather took
-// 215 + 28 + 58 + 398 us in four kernels; the whole encode with its sort 1540 ->
-// 1087 us.
+// particles.)  Six CTAs a SM, as k_encode_codes.  256^3 particles x1v1: this 182
+// us and k_encode_codes 203, where 64-bit global atomics per particle, the
+// measurement and the final gather took 215 + 28 + 58 + 398 us in four kernels;
+// the whole encode with its sort 1540 -> 1087 us.
 template <bool RUNS>
 __global__ void __launch_bounds__(T_BRICK, 6) k_encode_vc(Geo g, const float* __restrict__ vel,
                                                           const unsigned* __restrict__ perm, StoreDev s, float* v0,
